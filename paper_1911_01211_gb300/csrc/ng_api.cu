@@ -17,6 +17,7 @@
 #include "ng_tvfft.h"
 #include "ng_gw.cuh"
 #include "ng_vie2_launch.h"
+#include "ng_histclose.cuh"
 #include "ng_adjoint_types.h"
 #include <cmath>
 
@@ -98,6 +99,8 @@ struct ng_ctx {
     int bulk_split = NG_BULK_AUTO;   // one thread or one warp per bulk item (ng_set_bulk_split)
     void* ws_tvq = nullptr;          // FFT correlation of the source, [m][a][b][kb]
     size_t ws_tvq_bytes = 0;
+    void* ws_hist = nullptr;         // digit-product history sums: row vectors, digits, unit sums
+    size_t ws_hist_bytes = 0;
     void* ws_tw = nullptr;           // twiddle table of length tw_L
     size_t ws_tw_bytes = 0;
     int tw_L = 0;
@@ -297,6 +300,40 @@ ng_status prep_tvfft(ng_ctx* c, const Grid& g, int n, const HermV& G, const Herm
     return NG_OK;
 }
 
+// Whether the history sums of step n run as digit products (ng_hist.cu): nf = 1, groups of 8 problems,
+// and work = nb (2 n^2 + 2 n ntau + ntau^2) multiply-adds (history, and the left-mixing source that the warp
+// form sums directly) above 8e6, or 16e6 where the warp form is the alternative: the launches of the digit
+// products take about 100 us for any size.  Whole steps, FP64 kernels / digit products in us, at
+// work / 1e6: one thread per item 512 problems 28730 / 10370 (3.9e3), 64 problems 344 / 233 (13), 100 problems
+// 181 / 198 (6.5); one warp per item 8 problems 320 / 211 (24), 12 problems 255 / 239 (16), 16 problems 186 / 229 (9.3).
+bool hist_applies(const ng_ctx* c, const Grid& g, int n) {
+    if (g.nf != 1 || g.nb < NGH_KG || c->bulk_split != NG_BULK_AUTO || n < 2 * g.k + 2) return false;
+    const double N = n, T = g.ntau, work = g.nb * (2.0 * N * (N + T) + T * T);
+    return work >= ((double)g.nb * (2.0 * N + T) < 128.0 * c->sms ? 16e6 : 8e6);
+}
+// *w describes the sums; *ok = false without room for the workspace: the step keeps the FP64 kernels
+ng_status hist_sums(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV& S, const HermV& Scc, HistWs* w, bool* ok,
+                    cudaStream_t s) {
+    const int nv = (S.ret.ldk == 1 && Scc.les.ldk == 1 && S.tv.ldk == 1) ? 1 : g.nb;
+    *ok = false;
+    const size_t need = hist_ws_bytes(g.nt, g.ntau, g.nb, nv);
+    if (c->ws_hist_bytes < need && ensure(c, &c->ws_hist, &c->ws_hist_bytes, need)) return NG_OK;   // no room: FP64 kernels
+    *w = hist_ws_layout(c->ws_hist, g.nt, n, g.ntau, g.k, g.nb, nv);
+    HistRow r{S.ret.p + tri(n) * S.ret.ldk, Scc.les.p + tri(n) * Scc.les.ldk,
+              S.tv.p + (int64_t)n * (g.ntau + 1) * S.tv.ldk, S.ret.ldk, Scc.les.ldk, S.tv.ldk};
+    const unsigned chunks = (unsigned)(w->lenp / NGH_BLK);
+    if (nv == 1) k_hist_vec<1><<<dim3(chunks, 1, NGH_NVEC), 256, 0, s>>>(*w, r);
+    else k_hist_vec<8><<<dim3(chunks, nblocks(nv, 8), NGH_NVEC), 256, 0, s>>>(*w, r);
+    ng_status st = check_launch(c, "k_hist_vec");
+    if (st) return st;
+    if (hist_launch(*w, G.ret.p, G.les.p, G.tv.p, c->sms, c->d_status, s) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(c, NG_ECUDA, "launch of k_hist_mma failed");
+    }
+    *ok = true;
+    return NG_OK;
+}
+
 // the boundary of step n in three launches, its (A)-row sums over (row, problem, chunk) blocks;
 // pre_done: the retarded start-up ran in the leading warps of the bulk launch
 template <int D>
@@ -330,7 +367,9 @@ ng_status launch_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const
     // small batches: one warp per item when one thread per item would not give each SM a block;
     // the warp form splits the left-mixing source over its lanes instead of the FFT pre-pass
     const int64_t items = it_les + it_tv + it_ret;
-    const bool warp = c->bulk_split == NG_BULK_WARP || (c->bulk_split == NG_BULK_AUTO && items < (int64_t)c->sms * thr);
+    const bool digits = hist_applies(c, g, n);
+    const bool warp = c->bulk_split == NG_BULK_WARP ||
+                      (c->bulk_split == NG_BULK_AUTO && !digits && items < (int64_t)c->sms * thr);
     // small batches: the boundary's (A)-row sums spread over (row, problem, chunk) blocks, and
     // with the warp bulk its retarded start-up in the bulk launch's leading warps
     const int nq = (n <= 2 * k) ? n : k + 1;
@@ -343,7 +382,13 @@ ng_status launch_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const
     long e0 = prof_pair(c, 0);
     if (e0 >= 0) cudaEventRecord(c->ev_pool[e0], s);
     if ((sm = launch_minv<D>(c, g, n, S, eps, s))) return sm;
-    if (warp) {
+    bool hist = false;   // their sums are per unit and problem: k_hist_close finishes the items
+    HistWs hw;
+    if (D == 1 && digits && (sm = hist_sums(c, g, n, G, S, S, &hw, &hist, s))) return sm;
+    if (hist) {
+        k_hist_close<<<b_les + b_tv + b_ret, thr, 0, s>>>(g, n, G, S, hw, (const cplx*)c->ws_minv, b_les, b_tv, tvq,
+                                                          c->d_status);
+    } else if (warp) {
         k_step_bulk_w<D><<<nblocks((w_pre + items) * 32, thr), thr, 0, s>>>(g, n, G, S, eps, (const cplx*)c->ws_minv,
                                                                            w_pre, it_les, it_tv, it_ret, c->d_status);
     } else {
@@ -444,6 +489,9 @@ template <int D>
 ng_status launch_timestepdf(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV& S, const FuncV& eps,
                             cudaStream_t s) {
     ng_status st;
+    // the digit products are exact and read half the bytes of the double-float sums (16 B per element for
+    // two multiply-adds): a step of 256 problems, n = 900, ntau = 400: 2.08 -> 1.92 ms
+    if (hist_applies(c, g, n)) return launch_timestep<D>(c, g, n, G, S, eps, s);
     if ((st = update_shadow_df(c, c->dfG, g, G, n, false, s))) return st;
     if ((st = update_shadow_df(c, c->dfS, g, S, n, true, s))) return st;
     const int k = g.k, thr = 128;
@@ -670,6 +718,7 @@ ng_status launch_vie2_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV&
 // one warp per vie2 bulk item: forced, or for batches with fewer items than 128 per SM
 bool vie2_warp(const ng_ctx* c, const Grid& g, int n) {
     const int64_t items = (int64_t)g.nb * ((n - 1) + (g.ntau + 1) + n);
+    if (hist_applies(c, g, n)) return false;
     return c->bulk_split == NG_BULK_WARP || (c->bulk_split == NG_BULK_AUTO && items < (int64_t)c->sms * 128);
 }
 
@@ -1051,6 +1100,7 @@ void ng_destroy(ng_ctx* c) {
     cudaFree(c->ws_usrc);
     cudaFree(c->ws_tvq);
     cudaFree(c->ws_tw);
+    cudaFree(c->ws_hist);
     delete c;
 }
 
@@ -1064,6 +1114,7 @@ ng_status ng_status_sync(ng_ctx* c, void* stream, int* flags) {
     CUDA_TRY(c, cudaMemset(c->d_status, 0, sizeof(int)));
     if (flags) *flags = f;
     if (f & NGF_NONFINITE) return fail(c, NG_ENONFINITE, "device reported non-finite values (flags %d)", f);
+    if (f & NGF_TIMEOUT) return fail(c, NG_ETIMEOUT, "a kernel's wait for its copies ran out (flags %d)", f);
     if (f & NGF_SINGULAR) return fail(c, NG_ESINGULAR, "device reported a singular matrix (flags %d)", f);
     return NG_OK;
 }
@@ -1234,7 +1285,10 @@ ng_status ng_vie2_timestep(ng_ctx* c, const ng_grid* grid, int tstp, ng_herm G, 
     const cplx* tvq = nullptr;
     const bool w = vie2_warp(c, g, tstp);
     if (!w && (st = prep_tvfft(c, g, tstp, Gv, Fv, (cudaStream_t)stream, &tvq))) return st;
-    if (vie2_step_launch(g, tstp, Gv, Fv, Fccv, Qv, tvq, w, c->d_status, (cudaStream_t)stream) !=
+    bool hist = false;
+    HistWs hw;
+    if (!w && hist_applies(c, g, tstp) && (st = hist_sums(c, g, tstp, Gv, Fv, Fccv, &hw, &hist, (cudaStream_t)stream))) return st;
+    if (vie2_step_launch(g, tstp, Gv, Fv, Fccv, Qv, tvq, w, hist ? &hw : nullptr, c->d_status, (cudaStream_t)stream) !=
         cudaSuccess) {
         cudaGetLastError();
         return fail(c, NG_ECUDA, "launch of the vie2 time-step kernels failed");
@@ -1569,7 +1623,11 @@ static ng_status run_2b_impl(ng_ctx* c, const ng_grid* grid, ng_herm G, ng_herm 
                 const cplx* tvq = nullptr;
                 const bool w = vie2_warp(c, gw->gb, n);
                 if (!w && (r = prep_tvfft(c, gw->gb, n, gw->X, gw->K, s, &tvq, false))) return r;
-                e = vie2_step_launch(gw->gb, n, gw->X, gw->K, gw->Kcc, gw->P, tvq, w, c->d_status, s);
+                bool hist = false;
+                HistWs hw;
+                if (!w && hist_applies(c, gw->gb, n) && (r = hist_sums(c, gw->gb, n, gw->X, gw->K, gw->Kcc, &hw, &hist, s)))
+                    return r;
+                e = vie2_step_launch(gw->gb, n, gw->X, gw->K, gw->Kcc, gw->P, tvq, w, hist ? &hw : nullptr, c->d_status, s);
             }
         }
         if (e != cudaSuccess) {

@@ -291,3 +291,4 @@ __device__ __forceinline__ double gw(const NgWeights& W, int n, int j) {
 // status word bits
 #define NGF_NONFINITE 1
 #define NGF_SINGULAR 2
+#define NGF_TIMEOUT 4

@@ -19,6 +19,7 @@
 //             G^<(n,l) = -[G^<(l,n)]^dagger of the column just computed.
 #pragma once
 
+#include "ng_hist.cuh"
 #include "ng_step.cuh"
 #include "ng_stepsplit.cuh"
 
@@ -341,6 +342,57 @@ __global__ void __launch_bounds__(128, D == 1 ? 6 : 1)
         if (!mfinite<D>(y)) atomicOr(status, NGF_NONFINITE);
         st<D>(G.les, tri(n) + m, kb, y);
     }
+}
+
+// The same items with their history sums from the digit products (nf = 1; w: unit sums for the row
+// vectors of F and Fcc).
+static __global__ void __launch_bounds__(128)
+    k_v2_hist_close(Grid g, int n, HermV G, HermV F, HermV Fcc, HermV Q, HistWs w, int nb_tv, int nb_les, const cplx* tvq,
+                    int* status) {
+    const NgWeights& W = c_W[g.k - 1];
+    const int k = W.k;
+    int blk = blockIdx.x, task;
+    if (blk < nb_les) task = 0;
+    else if ((blk -= nb_les) < nb_tv) task = 1;
+    else { blk -= nb_tv; task = 2; }
+    const int64_t item = (int64_t)blk * blockDim.x + threadIdx.x;
+    const int kb = (int)(item % g.nb);
+    const int64_t col = item / g.nb;
+    const int ncol = task == 0 ? n - 1 : (task == 1 ? g.ntau + 1 : n);
+    if (col >= ncol) return;
+    const int m = task == 0 ? (int)col + 1 : (int)col;
+    const cplx fnn = ld<1>(F.ret, tri(n) + n, kb).v[0][0];
+    cplx rhs;
+    double wd = gw(W, n, n);
+    if (task == 0) {
+        cplx c1, c3, hist;
+        const int kv = w.nv == 1 ? 0 : kb;
+        hist_les_sums(W, w, G, Fcc.les.p + tri(n) * Fcc.les.ldk, Fcc.les.ldk, w.vec + ((int64_t)w.nv + kv) * w.lenp, n, m, kb,
+                      c1, c3, hist);
+        rhs = csub(ld<1>(Q.les, tri(n) + m, kb).v[0][0], cscal(g.h, cadd(c1, hist)));
+        rhs = csub(rhs, cmul(make_double2(0.0, (double)g.sig * g.htau), c3));
+    } else if (task == 1) {
+        rhs = csub(gtv<1>(Q, g, n, m, kb).v[0][0], v2_ctv23<1>(W, g, G, F, n, m, kb, tvq).v[0][0]);
+        rhs = csub(rhs, cscal(g.h, hist_tv_sum(w, m, kb)));
+    } else {
+        const int L = n - m;
+        cplx acc = cz();
+        if (L > k) {
+            acc = hist_ret_sum(W, w, G, F, n, m, kb);
+            wd = gw(W, L, L);
+        } else {
+            for (int j = 1; j <= k; ++j)
+                acc = cfma(cscal(W.greg[L][j], ld<1>(F.ret, tri(n) + n - j, kb).v[0][0]), gretx<1>(G, n - j, m, kb).v[0][0], acc);
+            wd = W.greg[L][0];
+        }
+        rhs = csub(ld<1>(Q.ret, tri(n) + m, kb).v[0][0], cscal(g.h, acc));
+    }
+    const cplx M = make_double2(1.0 + g.h * wd * fnn.x, g.h * wd * fnn.y);
+    if (cabs2(M) == 0.0) atomicOr(status, NGF_SINGULAR);
+    const cplx Mi = cdiv(cr(1.0), M), y = cmul(rhs, task == 0 ? cconj(Mi) : Mi);
+    if (!cfinite(y)) atomicOr(status, NGF_NONFINITE);
+    const Comp& X = task == 0 ? G.les : (task == 1 ? G.tv : G.ret);
+    X.p[(task == 1 ? (int64_t)n * (g.ntau + 1) + m : tri(n) + m) * X.ldk + kb] = y;
 }
 
 // After the bulk launch, one block per problem: G^R(n,n) = Q^R(n,n), G^<(0,n) from G^tv(n,0),
