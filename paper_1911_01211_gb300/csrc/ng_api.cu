@@ -10,6 +10,7 @@
 #include "ng_slice.cuh"
 #include "ng_step32.cuh"
 #include "ng_stepsplit.cuh"
+#include "ng_bound.cuh"
 #include "ng_obs.cuh"
 #include "ng_ubatch.cuh"
 #include "ng_stepdf.cuh"
@@ -241,7 +242,7 @@ long prof_pair(ng_ctx* c, int kind) {
 double bulk_cmacs(const Grid& g, int n, bool fft = false) {
     const int k = g.k, T = g.ntau;
     auto corr = [&](int L) {   // correction terms of one piece with row length L
-        return L <= k ? (k + 1) * (k + 1) + L + 1 : (L <= 2 * k + 1 ? L + 1 : 2 * (k + 1));
+        return L <= k ? (k + 1) * (k + 1) + L + 1 : (L <= 2 * k + 1 ? L + 1 : (T - L <= k ? k - (T - L) + 1 : 0));
     };
     double per_tv = 0.0;
     for (int m = 0; m <= T; ++m) {
@@ -287,11 +288,11 @@ ng_status prep_tvfft(ng_ctx* c, const Grid& g, int n, const HermV& G, const Herm
         if (tvfft_twiddles((cplx*)c->ws_tw, L, s) != cudaSuccess) return check_launch(c, "k_twiddle");
         c->tw_L = L;
     }
-    const size_t need = sizeof(cplx) * (size_t)(g.ntau + 1) * g.nf * g.nf * g.nb;
+    const size_t need = tvfft_out_bytes(g, S.tv.ldk);
     if ((st = ensure(c, &c->ws_tvq, &c->ws_tvq_bytes, need))) return st;
     long e = prof ? prof_pair(c, 2) : -1;
     if (e >= 0) cudaEventRecord(c->ev_pool[e], s);
-    if (tvfft_launch(g, n, S.tv, G.mat, (const cplx*)c->ws_tw, (cplx*)c->ws_tvq, s) != cudaSuccess) {
+    if (tvfft_launch(g, c->W, n, S.tv, G.mat, (const cplx*)c->ws_tw, (cplx*)c->ws_tvq, s) != cudaSuccess) {
         cudaGetLastError();
         return fail(c, NG_ECUDA, "launch of k_tvsrc_fft failed");
     }
@@ -356,6 +357,48 @@ ng_status boundary_spread(ng_ctx* c, const Grid& g, int n, const HermV& G, const
     return check_launch(c, "k_bnd_fin");
 }
 
+// The boundary with one lane per problem: nf = 1, batches of 16 and more, n > 2k.  pre_done: the retarded
+// start-up ran with the bulk launch.  Below 16 problems most lanes would be idle and the per-problem forms
+// stay.
+bool bnd1_applies(const Grid& g, int n) { return g.nf == 1 && g.nb >= 16 && n > 2 * g.k; }
+ng_status boundary1(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV& S, const FuncV& eps, bool pre_done,
+                    cudaStream_t s) {
+    ng_status st;
+    const int J = std::max(n, g.ntau) + 1, groups = (g.nb + 31) / 32;
+    // two blocks a SM, chunks of four indices (one a warp) or more, at most 48 partial sums to add
+    const int want = std::min(48, std::max(1, (2 * c->sms + groups - 1) / groups));
+    const int len = std::max(4, (J + want - 1) / want), nchunk = (J + len - 1) / len;
+    if ((st = ensure(c, &c->ws_bnd, &c->ws_bnd_bytes, sizeof(cplx) * (size_t)nchunk * 2 * NG_B1_ROWS * g.nb))) return st;
+    if (!pre_done) {
+        k_bnd_pre<1><<<g.nb, 32, 0, s>>>(g, n, G, S, eps, c->d_status);
+        if ((st = check_launch(c, "k_bnd_pre"))) return st;
+    }
+    const dim3 grid(groups, nchunk);
+    if (S.ret.ldk == 1 && S.les.ldk == 1 && S.tv.ldk == 1)
+        k_bnd1_sums<true><<<grid, 128, 0, s>>>(g, n, G, S, len, (cplx*)c->ws_bnd);
+    else
+        k_bnd1_sums<false><<<grid, 128, 0, s>>>(g, n, G, S, len, (cplx*)c->ws_bnd);
+    if ((st = check_launch(c, "k_bnd1_sums"))) return st;
+    k_bnd1_fin<<<groups, 32 * NG_B1_WARPS, 0, s>>>(g, n, G, S, eps, nchunk, (const cplx*)c->ws_bnd, c->d_status);
+    return check_launch(c, "k_bnd1_fin");
+}
+
+// the whole boundary of a batch after its bulk launch
+template <int D>
+ng_status boundary_batch(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV& S, const FuncV& eps, cudaStream_t s) {
+    ng_status st;
+    const long e = prof_pair(c, 1);
+    if (e >= 0) cudaEventRecord(c->ev_pool[e], s);
+    if (D == 1 && bnd1_applies(g, n)) {
+        st = boundary1(c, g, n, G, S, eps, false, s);
+    } else {
+        k_step_boundary<D><<<g.nb, NG_BND_THREADS, 0, s>>>(g, n, G, S, eps, c->d_status);
+        st = check_launch(c, "k_step_boundary");
+    }
+    if (e >= 0) cudaEventRecord(c->ev_pool[e + 1], s);
+    return st;
+}
+
 template <int D>
 ng_status launch_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV& S, const FuncV& eps,
                           cudaStream_t s) {
@@ -375,7 +418,8 @@ ng_status launch_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const
     const int nq = (n <= 2 * k) ? n : k + 1;
     const bool spread = c->bulk_split == NG_BULK_WARP ||
                         (c->bulk_split == NG_BULK_AUTO && (int64_t)nq * g.nb < 2 * (int64_t)c->sms);
-    const int64_t w_pre = (warp && spread) ? g.nb : 0;
+    const bool lanes = D == 1 && c->bulk_split == NG_BULK_AUTO && bnd1_applies(g, n);
+    const int64_t w_pre = (warp && (spread || lanes)) ? g.nb : 0;
     const cplx* tvq = nullptr;
     ng_status sm = warp ? NG_OK : prep_tvfft(c, g, n, G, S, s, &tvq);
     if (sm) return sm;
@@ -385,9 +429,10 @@ ng_status launch_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const
     bool hist = false;   // their sums are per unit and problem: k_hist_close finishes the items
     HistWs hw;
     if (D == 1 && digits && (sm = hist_sums(c, g, n, G, S, S, &hw, &hist, s))) return sm;
+    const int pre = hist && lanes ? (int)nblocks(g.nb, thr / 32) : 0;   // leading blocks: the retarded start-up
     if (hist) {
-        k_hist_close<<<b_les + b_tv + b_ret, thr, 0, s>>>(g, n, G, S, hw, (const cplx*)c->ws_minv, b_les, b_tv, tvq,
-                                                          c->d_status);
+        k_hist_close<<<pre + b_les + b_tv + b_ret, thr, 0, s>>>(g, n, G, S, eps, hw, (const cplx*)c->ws_minv, pre, b_les,
+                                                                b_tv, tvq, c->d_status);
     } else if (warp) {
         k_step_bulk_w<D><<<nblocks((w_pre + items) * 32, thr), thr, 0, s>>>(g, n, G, S, eps, (const cplx*)c->ws_minv,
                                                                            w_pre, it_les, it_tv, it_ret, c->d_status);
@@ -403,6 +448,11 @@ ng_status launch_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const
     }
     long e1 = prof_pair(c, 1);
     if (e1 >= 0) cudaEventRecord(c->ev_pool[e1], s);
+    if (lanes) {
+        st = boundary1(c, g, n, G, S, eps, w_pre > 0 || pre > 0, s);
+        if (e1 >= 0) cudaEventRecord(c->ev_pool[e1 + 1], s);
+        return st;
+    }
     if (spread) {
         st = boundary_spread<D>(c, g, n, G, S, eps, w_pre > 0, s);
         if (e1 >= 0) cudaEventRecord(c->ev_pool[e1 + 1], s);
@@ -511,11 +561,7 @@ ng_status launch_timestepdf(ng_ctx* c, const Grid& g, int n, const HermV& G, con
         cudaEventRecord(c->ev_pool[e0 + 1], s);
         c->prof_flops += 8.0 * D * D * D * bulk_cmacs(g, n, tvq != nullptr);
     }
-    long e1 = prof_pair(c, 1);
-    if (e1 >= 0) cudaEventRecord(c->ev_pool[e1], s);
-    k_step_boundary<D><<<g.nb, NG_BND_THREADS, 0, s>>>(g, n, G, S, eps, c->d_status);
-    if (e1 >= 0) cudaEventRecord(c->ev_pool[e1 + 1], s);
-    return check_launch(c, "k_step_boundary");
+    return boundary_batch<D>(c, g, n, G, S, eps, s);
 }
 
 template <int D>
@@ -551,11 +597,7 @@ ng_status launch_timestep32(ng_ctx* c, const Grid& g, int n, const HermV& G, con
         cudaEventRecord(c->ev_pool[e0 + 1], s);
         c->prof_flops += 8.0 * D * D * D * bulk_cmacs(g, n, tvq != nullptr);
     }
-    long e1 = prof_pair(c, 1);
-    if (e1 >= 0) cudaEventRecord(c->ev_pool[e1], s);
-    k_step_boundary<D><<<g.nb, NG_BND_THREADS, 0, s>>>(g, n, G, S, eps, c->d_status);
-    if (e1 >= 0) cudaEventRecord(c->ev_pool[e1 + 1], s);
-    return check_launch(c, "k_step_boundary");
+    return boundary_batch<D>(c, g, n, G, S, eps, s);
 }
 
 // Matsubara solve.  refine_steps = 0: exact solve by a fresh LU of the current operator (the

@@ -45,6 +45,15 @@ __host__ __device__ __forceinline__ cplx cdiv(cplx a, cplx b) {
     double r = b.x / b.y, den = b.x * r + b.y;
     return make_double2((a.x * r + a.y) / den, (a.y * r - a.x) / den);
 }
+// 1 / z by the conjugate over |z|^2 on a power-of-two scale: one division, where cdiv's quotients take
+// three (an FP64 instruction occupies a quarter SM for 64 clocks on this part)
+__device__ __forceinline__ cplx cinv(cplx z) {
+    const int e = max(__double2hiint(z.x) >> 20 & 2047, __double2hiint(z.y) >> 20 & 2047);
+    if (e == 2047) return cdiv(cr(1.0), z);   // non-finite: as cdiv
+    const double s = __hiloint2double(min(max(2046 - e, 1), 2045) << 20, 0);
+    const double x = z.x * s, y = z.y * s, r = 1.0 / fma(x, x, y * y) * s;
+    return make_double2(x * r, -y * r);
+}
 __host__ __device__ __forceinline__ bool cfinite(cplx a) { return isfinite(a.x) && isfinite(a.y); }
 
 // ---------------------------------------------------------------------------------------
@@ -161,7 +170,11 @@ __host__ __device__ __forceinline__ Mat<D> minv(const Mat<D>& x, int* sing) {
     if (D == 1) {
         Mat<D> r;
         if (cabs2(x.v[0][0]) == 0.0) *sing = 1;
+#ifdef __CUDA_ARCH__
+        r.v[0][0] = cinv(x.v[0][0]);
+#else
         r.v[0][0] = cdiv(cr(1.0), x.v[0][0]);
+#endif
         return r;
     }
     Mat<D> a = x, r = meye<D>(cr(1.0));

@@ -2,14 +2,24 @@
 #pragma once
 
 #include "ng_hist.cuh"
+#include "ng_stepsplit.cuh"
 
 // Items as in k_step_bulk (nf = 1): lesser m = 1..n-k-1, left-mixing m = 0..ntau, retarded
-// m = 0..n-k-1; problem fastest.
-static __global__ void __launch_bounds__(128) k_hist_close(Grid g, int n, HermV G, HermV S, HistWs w, const cplx* minv_ws,
-                                                    int nb_les, int nb_tv, const cplx* tvq, int* status) {
+// m = 0..n-k-1; problem fastest.  The first nb_pre blocks run the boundary's retarded start-up, a warp
+// per problem: it reads only the self-energy and eps and writes G^R(n, n-k..n), which no item reads.
+static __global__ void __launch_bounds__(128) k_hist_close(Grid g, int n, HermV G, HermV S, FuncV eps, HistWs w,
+                                                           const cplx* minv_ws, int nb_pre, int nb_les, int nb_tv,
+                                                           const cplx* tvq, int* status) {
     const NgWeights& W = c_W[g.k - 1];
     const int k = W.k;
     int blk = blockIdx.x, task;
+    if (blk < nb_pre) {
+        __shared__ cplx sh[4][bnd_pre_scratch<1>()];
+        const int warp = threadIdx.x >> 5, kb = blk * 4 + warp;
+        if (kb < g.nb) bnd_pre_warp<1>(W, g, n, G, S, eps, kb, sh[warp], threadIdx.x & 31, status);
+        return;
+    }
+    blk -= nb_pre;
     if (blk < nb_les) task = 0;
     else if ((blk -= nb_les) < nb_tv) task = 1;
     else { blk -= nb_tv; task = 2; }

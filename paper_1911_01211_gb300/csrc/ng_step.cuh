@@ -95,53 +95,58 @@ __device__ Mat<D> q_tv(const NgWeights& W, const Grid& g, const HermV& G, const 
     return mscal<D>(g.htau, mmuli<D>(mscal<D>(-1.0, madd<D>(c2, c3))));
 }
 
-// The same source from the unit-weight correlation F(m) of the FFT pre-pass (ng_tvfft.cu):
-// q(m) = -i h_tau [F(m) + the difference between the quadrature of Eqs. ctv2, ctv3 and unit
-// weights], i.e. (w - 1) terms at the Gregory ends of each piece (rows longer than 2k+1), every
-// term of short rows, and the boundary (R) formulas minus their unit-weight sums for m <= k and
-// m >= ntau - k.  Q: [m][a][b][kb] with ldk = nb.
+// The same source from the correlation F(m) of the FFT pre-pass (ng_tvfft.cu), whose end weights
+// reproduce the quadrature of Eqs. ctv2, ctv3 but for the columns next to either end of the tau axis:
+// q(m) = -i h_tau [F(m) + quadrature - F's terms] there (short rows, the boundary (R) formulas, and the
+// weights of the other end).  Q: [m][a][b][kb] with ldk = nb.
 template <int D>
 __device__ Mat<D> q_tv_fft(const NgWeights& W, const Grid& g, const HermV& G, const HermV& S, int n, int m, int kb,
                            const cplx* Q) {
     const int k = W.k, T = g.ntau;
     const double xi = (double)g.sig;
-    Mat<D> c2 = mzero<D>(), c3 = mzero<D>();   // corrections, C2 without its factor xi
-    // C2: sum_l w_{m,l} S(m-l) G^M(T-l)
-    auto t2 = [&](int l, double dw) { mfma<D>(c2, mscal<D>(dw, gtv<D>(S, g, n, m - l, kb)), gmat<D>(G, T - l, kb)); };
-    if (m <= k) {
-        for (int j = 0; j <= k; ++j) {
-            Mat<D> gm = gmat<D>(G, T - j, kb);
-            for (int l = 0; l <= k; ++l) mfma<D>(c2, mscal<D>(W.R[m][j][l], gtv<D>(S, g, n, l, kb)), gm);
-        }
-        for (int l = 0; l <= m; ++l) t2(l, -1.0);
-    } else if (m <= 2 * k + 1) {
-        for (int l = 0; l <= m; ++l) t2(l, W.greg[m][l] - 1.0);
-    } else {
-        for (int l = 0; l <= k; ++l) t2(l, W.omega[l] - 1.0);
-        for (int l = m - k; l <= m; ++l) t2(l, W.omega[m - l] - 1.0);
-    }
-    // C3: sum_l w_{T-m,l} S(m+l) G^M(l)
-    const int L3 = T - m;
-    auto t3 = [&](int l, double dw) { mfma<D>(c3, mscal<D>(dw, gtv<D>(S, g, n, m + l, kb)), gmat<D>(G, l, kb)); };
-    if (L3 <= k) {
-        for (int j = 0; j <= k; ++j) {
-            Mat<D> gm = gmat<D>(G, j, kb);
-            for (int l = 0; l <= k; ++l) mfma<D>(c3, mscal<D>(W.R[L3][j][l], gtv<D>(S, g, n, T - l, kb)), gm);
-        }
-        for (int l = 0; l <= L3; ++l) t3(l, -1.0);
-    } else if (L3 <= 2 * k + 1) {
-        for (int l = 0; l <= L3; ++l) t3(l, W.greg[L3][l] - 1.0);
-    } else {
-        for (int l = 0; l <= k; ++l) t3(l, W.omega[l] - 1.0);
-        for (int l = L3 - k; l <= L3; ++l) t3(l, W.omega[L3 - l] - 1.0);
-    }
     Mat<D> F;
 #pragma unroll
     for (int a = 0; a < D; ++a)
 #pragma unroll
         for (int b = 0; b < D; ++b) F.v[a][b] = Q[((int64_t)m * (D * D) + a * D + b) * g.nb + kb];
-    Mat<D> v = madd<D>(F, madd<D>(mscal<D>(xi, c2), c3));
-    return mscal<D>(g.htau, mmuli<D>(mscal<D>(-1.0, v)));
+    if (min(m, T - m) <= 2 * k + 1) {
+        Mat<D> c2 = mzero<D>(), c3 = mzero<D>();   // corrections, C2 without its factor xi
+        auto om = [&](int l) { return l <= k ? W.omega[l] : 1.0; };
+        auto ws = [&](int j) { return om(min(j, T - j)); };   // F's weight of S(j)
+        // C2: sum_l w_{m,l} S(m-l) G^M(T-l)
+        auto t2 = [&](int l, double w) {
+            mfma<D>(c2, mscal<D>(w - om(l) * ws(m - l), gtv<D>(S, g, n, m - l, kb)), gmat<D>(G, T - l, kb));
+        };
+        if (m <= k) {
+            for (int j = 0; j <= k; ++j) {
+                Mat<D> gm = gmat<D>(G, T - j, kb);
+                for (int l = 0; l <= k; ++l) mfma<D>(c2, mscal<D>(W.R[m][j][l], gtv<D>(S, g, n, l, kb)), gm);
+            }
+            for (int l = 0; l <= m; ++l) t2(l, 0.0);
+        } else if (m <= 2 * k + 1) {
+            for (int l = 0; l <= m; ++l) t2(l, W.greg[m][l]);
+        } else {
+            for (int l = 0; l <= m - T + k; ++l) t2(l, gw(W, m, l));   // the weights of the end j = T
+        }
+        // C3: sum_l w_{T-m,l} S(m+l) G^M(l)
+        const int L3 = T - m;
+        auto t3 = [&](int l, double w) {
+            mfma<D>(c3, mscal<D>(w - om(l) * ws(m + l), gtv<D>(S, g, n, m + l, kb)), gmat<D>(G, l, kb));
+        };
+        if (L3 <= k) {
+            for (int j = 0; j <= k; ++j) {
+                Mat<D> gm = gmat<D>(G, j, kb);
+                for (int l = 0; l <= k; ++l) mfma<D>(c3, mscal<D>(W.R[L3][j][l], gtv<D>(S, g, n, T - l, kb)), gm);
+            }
+            for (int l = 0; l <= L3; ++l) t3(l, 0.0);
+        } else if (L3 <= 2 * k + 1) {
+            for (int l = 0; l <= L3; ++l) t3(l, W.greg[L3][l]);
+        } else {
+            for (int l = 0; l <= k - m; ++l) t3(l, gw(W, L3, l));      // the weights of the end j = 0
+        }
+        F = madd<D>(F, madd<D>(mscal<D>(xi, c2), c3));
+    }
+    return mscal<D>(g.htau, mmuli<D>(mscal<D>(-1.0, F)));
 }
 
 // Partial sums of the (A)-source of the lesser column, -i (C^<_2 + C^<_3)[Sigma,1,G](m,n)
@@ -307,7 +312,7 @@ __device__ inline int dense_solve(cplx* A, int N, cplx* B, int nrhs) {
             for (int j = 0; j < N; ++j) { cplx t = A[c * N + j]; A[c * N + j] = A[p * N + j]; A[p * N + j] = t; }
             for (int j = 0; j < nrhs; ++j) { cplx t = B[c * nrhs + j]; B[c * nrhs + j] = B[p * nrhs + j]; B[p * nrhs + j] = t; }
         }
-        cplx inv = cdiv(cr(1.0), A[c * N + c]);
+        cplx inv = cinv(A[c * N + c]);
         for (int r = c + 1; r < N; ++r) {
             cplx f = cmul(A[r * N + c], inv);
             if (f.x == 0.0 && f.y == 0.0) continue;
@@ -316,7 +321,7 @@ __device__ inline int dense_solve(cplx* A, int N, cplx* B, int nrhs) {
         }
     }
     for (int c = N - 1; c >= 0; --c) {
-        cplx inv = cdiv(cr(1.0), A[c * N + c]);
+        cplx inv = cinv(A[c * N + c]);
         for (int j = 0; j < nrhs; ++j) {
             cplx s = B[c * nrhs + j];
             for (int q = c + 1; q < N; ++q) s = csub(s, cmul(A[c * N + q], B[q * nrhs + j]));
@@ -337,20 +342,20 @@ __device__ inline int dense_solve(cplx* A, int N, cplx* B, int nrhs) {
 __device__ inline int warp_dense_solve(cplx* A, int N, cplx* B, int nrhs, cplx* f, int lane) {
     const unsigned full = 0xffffffffu;
     for (int c = 0; c < N; ++c) {
-        double best = -1.0;
+        // squares of magnitudes compare as their bits, without the FP64 pipe
+        long long best = -1;
         int p = N;
         for (int r = c + lane; r < N; r += 32) {
-            const double v = cabs2(A[r * N + c]);
+            const long long v = __double_as_longlong(cabs2(A[r * N + c]));
             if (v > best) { best = v; p = r; }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            const double bo = __shfl_xor_sync(full, best, o);
+            const long long bo = __shfl_xor_sync(full, best, o);
             const int po = __shfl_xor_sync(full, p, o);
             if (bo > best || (bo == best && po < p)) { best = bo; p = po; }
         }
-        if (best == 0.0) return 1;
-        if (p >= N) p = c;   // no comparable entry (NaN column): keep the row, as dense_solve does
+        if (best == 0) return 1;
         if (p != c) {
             for (int j = lane; j < N; j += 32) {
                 const cplx t = A[c * N + j]; A[c * N + j] = A[p * N + j]; A[p * N + j] = t;
@@ -360,21 +365,22 @@ __device__ inline int warp_dense_solve(cplx* A, int N, cplx* B, int nrhs, cplx* 
             }
         }
         __syncwarp();
-        const cplx inv = cdiv(cr(1.0), A[c * N + c]);
+        const cplx inv = cinv(A[c * N + c]);
         for (int r = c + 1 + lane; r < N; r += 32) f[r] = cmul(A[r * N + c], inv);
         __syncwarp();
-        const int wa = N - c, w = wa + nrhs, cnt = (N - c - 1) * w;
+        if (lane == 0) A[c * N + c] = inv;   // for the back substitution (the factors in f are taken)
+        const int wa = N - c - 1, w = wa + nrhs, cnt = (N - c - 1) * w;
         for (int e = lane; e < cnt; e += 32) {
             const int r = c + 1 + e / w, j = e % w;
             const cplx fr = f[r];
             if (fr.x == 0.0 && fr.y == 0.0) continue;
-            if (j < wa) A[r * N + c + j] = csub(A[r * N + c + j], cmul(fr, A[c * N + c + j]));
+            if (j < wa) A[r * N + c + 1 + j] = csub(A[r * N + c + 1 + j], cmul(fr, A[c * N + c + 1 + j]));
             else B[r * nrhs + j - wa] = csub(B[r * nrhs + j - wa], cmul(fr, B[c * nrhs + j - wa]));
         }
         __syncwarp();
     }
     for (int c = N - 1; c >= 0; --c) {
-        const cplx inv = cdiv(cr(1.0), A[c * N + c]);
+        const cplx inv = A[c * N + c];
         for (int j = lane; j < nrhs; j += 32) B[c * nrhs + j] = cmul(B[c * nrhs + j], inv);
         __syncwarp();
         for (int e = lane; e < c * nrhs; e += 32) {

@@ -13,6 +13,10 @@ size_t tvfft_smem_bytes(int nf, int ntau);
 bool tvfft_supported(int nf, int ntau);
 // tw[p] = exp(-2 pi i p / L), p = 0..L/2-1
 cudaError_t tvfft_twiddles(cplx* tw, int L, cudaStream_t s);
-// Q[(m nf^2 + a nf + b) nb + kb] = the unit-weight correlation F_ab(m) of step n, every problem
-cudaError_t tvfft_launch(const Grid& g, int n, const Comp& Stv, const Comp& Gmat, const cplx* tw, cplx* Q,
+// whether the row of S (ldk = 1: shared by the batch) is transformed once for all problems, and the bytes
+// of Q with those spectra behind it
+bool tvfft_shared(const Grid& g, int ldk);
+size_t tvfft_out_bytes(const Grid& g, int ldk);
+// Q[(m nf^2 + a nf + b) nb + kb] = the correlation F_ab(m) of step n, every problem; W: weights of order g.k
+cudaError_t tvfft_launch(const Grid& g, const NgWeights& W, int n, const Comp& Stv, const Comp& Gmat, const cplx* tw, cplx* Q,
                          cudaStream_t s);

@@ -57,6 +57,8 @@ def _check(a, b):
 DYSON = [  # nk, n, ntau, k, shared
     (29, 384, 300, 5, True), (33, 129, 640, 4, True), (203, 13, 400, 5, True), (130, 128, 127, 3, False),
     (31, 400, 127, 2, False), (17, 600, 129, 1, True), (40, 144, 383, 5, False), (8, 770, 639, 5, True),
+    # below the line: one warp per item, the boundary with one lane per problem (16 problems and more)
+    (16, 11, 12, 5, True), (33, 12, 25, 4, False), (47, 30, 16, 1, True), (31, 64, 40, 3, True),
 ]
 
 
@@ -135,3 +137,23 @@ def test_non_finite(ng, where, value):
         s = torch.where(fx, x.abs(), torch.zeros_like(x.abs())).amax(0)
         # a problem without any finite element has nothing to compare
         assert (d.amax(0) <= TOL * torch.where(s > 0, s, torch.ones_like(s))).all()
+
+
+@pytest.mark.parametrize("nk,shared", [(3, True), (64, True), (65, False)])
+@pytest.mark.parametrize("T,k", [(4, 1), (12, 5), (13, 5), (24, 5), (25, 4), (40, 5), (127, 3)])
+def test_fft_source_edges(ng, nk, shared, T, k):
+    """The left-mixing row with its Matsubara source by FFT against the direct sums, where most or all
+    columns lie next to an end of the tau axis; with the self-energy's spectra shared and not."""
+    n = 2 * k + 3
+    g = ng.Grid(nt=n, ntau=T, nf=1, nbatch=nk, korder=k, h=0.02, beta=4.0, mu=0.1)
+    G, S, eps = ng.Herm(g), ng.Herm(g, ldk=1 if shared else None), ng.Func(g)
+    _random(G, 7, 0.3)
+    _random(S, 8, 1.0)
+    ctx = ng.Context(k)
+    ctx.set_bulk_split(ng.NG_BULK_THREAD)
+    out = []
+    for src in (ng.NG_TVSRC_DIRECT, ng.NG_TVSRC_AUTO):
+        ctx.set_tv_source(src)
+        ctx.dyson_timestep(g, n, G, S, eps)
+        out.append({q: v.clone() for q, v in _slice(G, g, n).items()})
+    _check(*out)
