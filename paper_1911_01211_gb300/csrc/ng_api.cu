@@ -600,65 +600,78 @@ ng_status launch_timestep32(ng_ctx* c, const Grid& g, int n, const HermV& G, con
     return boundary_batch<D>(c, g, n, G, S, eps, s);
 }
 
-// Matsubara solve.  refine_steps = 0: exact solve by a fresh LU of the current operator (the
-// factors and row interchanges are kept).  refine_steps > 0 (driver only, after a fresh LU of
-// the same grid): iterative refinement of the current G^M against the current operator with
-// the kept factors, at most refine_steps steps; *refined_ok reports convergence of the
-// refinement (update sum below ref_tol); otherwise the caller falls back to a fresh LU.
-// LU solve of nb augmented systems [A | B] (N x (N + nrhs)) in ws_A: one block per problem for
-// batches that fill the SMs (or when several solves run concurrently on streams, spread =
-// false), else column by column with the rank-1 updates over the whole GPU (the same factors
-// bitwise)
-ng_status lu_solve(ng_ctx* c, int N, int nrhs, int nb, cplx* ws_A, int* ws_piv, cudaStream_t s, bool spread = true) {
-    ng_status st;
-    if (!spread || 4 * (int64_t)nb >= c->sms) {
-        const size_t smem = sizeof(cplx) * (size_t)(2 * N + nrhs) + NG_LU_THREADS * (sizeof(double) + sizeof(int));
-        CUDA_TRY(c, cudaFuncSetAttribute(k_lu_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_lu_solve<<<nb, NG_LU_THREADS, smem, s>>>(N, nrhs, ws_A, ws_piv, c->d_status);
-        return check_launch(c, "k_lu_solve");
-    }
-    for (int col = 0; col < N; ++col) {
-        k_lu_col<<<nb, NG_LU_THREADS, 0, s>>>(N, nrhs, ws_A, ws_piv, col, c->d_status);
-        const int64_t items = (int64_t)(N - col - 1) * (N + nrhs - col - 1);
-        if (items > 0) k_lu_rank1<<<dim3(nblocks(items, 256), nb), 256, 0, s>>>(N, nrhs, ws_A, col);
-        if (col % 256 == 0 && (st = check_launch(c, "k_lu_col/k_lu_rank1"))) return st;
-    }
-    k_lu_backsub<<<nb, NG_LU_THREADS, 0, s>>>(N, nrhs, ws_A);
-    return check_launch(c, "k_lu_backsub");
+// LU solve of nb augmented systems [A | B] (N x (N + nrhs)) in ws_A, one block per problem.  Panels as wide
+// as shared memory allows: 16 columns up to 800 unknowns, 8 up to 1600.
+template <int PB>
+ng_status lu_solve_p(ng_ctx* c, int N, int nrhs, int nb, cplx* ws_A, int* ws_piv, cudaStream_t s) {
+    const size_t smem = sizeof(cplx) * ((size_t)N * PB + NG_LU_TRI * nrhs);
+    CUDA_TRY(c, cudaFuncSetAttribute(k_lu_solve<PB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_lu_solve<PB><<<nb, NG_LU_THREADS, smem, s>>>(N, nrhs, ws_A, ws_piv, c->d_status);
+    return check_launch(c, "k_lu_solve");
+}
+ng_status lu_solve(ng_ctx* c, int N, int nrhs, int nb, cplx* ws_A, int* ws_piv, cudaStream_t s) {
+    if (N <= 800) return lu_solve_p<16>(c, N, nrhs, nb, ws_A, ws_piv, s);
+    if (N <= 1600) return lu_solve_p<8>(c, N, nrhs, nb, ws_A, ws_piv, s);
+    if (N <= 3200) return lu_solve_p<4>(c, N, nrhs, nb, ws_A, ws_piv, s);
+    return lu_solve_p<2>(c, N, nrhs, nb, ws_A, ws_piv, s);
+}
+
+// The discretised Matsubara equation X = g + [K * X]^M for the right-hand sides and kernels in ws (as laid out
+// by mat_ws): refine_steps = 0: a fresh solve; > 0: refinement of the current G^M with what the last fresh solve
+// kept in ws (its LU factors, or the inverse), at most refine_steps steps; *refined_ok reports convergence (update
+// sum below ref_tol), otherwise the caller solves afresh.  Few problems (less than a quarter of the SMs)
+// keep the inverse (k_gj_step) unless the solves run side by side on streams (spread = false): one block per
+// problem would leave the GPU idle.
+struct MatWs {
+    cplx *g, *K, *r, *A, *A2;
+    int* piv;
+    unsigned long long* keys;
+};
+bool mat_inverse(const ng_ctx* c, int N, int nb, bool spread) { return spread && 4 * (int64_t)nb < c->sms && N < 0xffff; }
+size_t mat_ws(void* base, int T, int D, int nb, bool inverse, MatWs* w) {
+    const size_t N = (size_t)(T + 1) * D, b_g = (size_t)nb * N * D, b_A = (size_t)nb * N * (N + D);
+    cplx* p = (cplx*)base;
+    w->g = p;
+    w->K = p + b_g;
+    w->r = p + 2 * b_g;
+    w->A = p + 3 * b_g;
+    w->A2 = w->A + b_A;
+    w->piv = (int*)(w->A + (inverse ? 2 : 1) * b_A);
+    const size_t b_piv = (sizeof(int) * (size_t)nb * N + 255) / 256 * 256;
+    w->keys = (unsigned long long*)((char*)w->piv + b_piv);
+    return sizeof(cplx) * (3 * b_g + (inverse ? 2 : 1) * b_A) + b_piv + (inverse ? 8 * (size_t)nb * (N + 1) : 0) + 256;
 }
 
 template <int D>
-ng_status launch_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S, const FuncV& eps, cudaStream_t s,
-                     int refine_steps = 0, double ref_tol = 0.0, bool* refined_ok = nullptr, void* ws_ext = nullptr) {
+ng_status mat_solve(ng_ctx* c, const Grid& g, const HermV& G, const MatWs& w, bool inverse, cudaStream_t s, int refine_steps,
+                    double ref_tol, bool* refined_ok) {
     const int T = g.ntau, N = (T + 1) * D, ld = N + D;
-    const size_t b_g = sizeof(cplx) * (size_t)g.nb * (T + 1) * D * D;
-    const size_t b_A = sizeof(cplx) * (size_t)g.nb * N * ld;
-    const size_t b_piv = sizeof(int) * (size_t)g.nb * N + 256;
-    ng_status st = NG_OK;
-    if (!ws_ext && (st = ensure(c, &c->ws_mat, &c->ws_mat_bytes, 3 * b_g + b_A + b_piv))) return st;
-    cplx* ws_g = (cplx*)(ws_ext ? ws_ext : c->ws_mat);
-    cplx* ws_K = ws_g + b_g / sizeof(cplx);
-    cplx* ws_r = ws_K + b_g / sizeof(cplx);
-    cplx* ws_A = ws_r + b_g / sizeof(cplx);
-    int* ws_piv = (int*)(ws_A + b_A / sizeof(cplx));
     const int64_t items = (int64_t)(T + 1) * g.nb;
-    k_mat_g<D><<<nblocks(items, 128), 128, 0, s>>>(g, eps, ws_g);
-    if ((st = check_launch(c, "k_mat_g"))) return st;
-    k_mat_K<D><<<nblocks(items, 128), 128, 0, s>>>(g, S, ws_g, ws_K);
-    if ((st = check_launch(c, "k_mat_K"))) return st;
+    const bool warp = D <= 4 && items < (int64_t)c->sms * 128;   // as for the bulk items: a warp per item where threads are few
+    const dim3 rows(nblocks((int64_t)N * D * 32, 128), g.nb);
+    const cplx* inv = N % 2 ? w.A2 : w.A;   // where the last of N passes ends
+    ng_status st = NG_OK;
+    auto refine = [&](double* dsum) -> ng_status {
+        if constexpr (D <= 4) {
+            if (warp) k_mat_resid_w<D><<<nblocks(items * 32, 128), 128, 0, s>>>(g, w.g, w.K, G, w.r);
+        }
+        if (!warp) k_mat_resid<D><<<nblocks(items, 128), 128, 0, s>>>(g, w.g, w.K, G, w.r);
+        ng_status e = check_launch(c, "k_mat_resid");
+        if (e) return e;
+        CUDA_TRY(c, cudaMemsetAsync(dsum, 0, sizeof(double), s));
+        if (inverse) k_gj_apply<true><<<rows, 128, 0, s>>>(N, ld, D, inv, w.piv, w.r, G, dsum, c->d_status);
+        else k_lu_resolve<<<g.nb, NG_LU_THREADS, 0, s>>>(g, N, D, w.A, w.piv, w.r, G, dsum);
+        return check_launch(c, "Matsubara refinement");
+    };
     if (refine_steps > 0) {
         *refined_ok = false;
         double prev = 1e300;
         for (int r = 0; r < refine_steps; ++r) {
-            k_mat_resid<D><<<nblocks(items, 128), 128, 0, s>>>(g, ws_g, ws_K, G, ws_r);
-            if ((st = check_launch(c, "k_mat_resid"))) return st;
-            CUDA_TRY(c, cudaMemsetAsync(c->d_scalar, 0, sizeof(double), s));
-            k_lu_resolve<<<g.nb, NG_LU_THREADS, 0, s>>>(g, N, D, ws_A, ws_piv, ws_r, G, c->d_scalar);
-            if ((st = check_launch(c, "k_lu_resolve"))) return st;
+            if ((st = refine(c->d_scalar))) return st;
             double dsum = 0.0;
             CUDA_TRY(c, cudaMemcpyAsync(&dsum, c->d_scalar, sizeof(double), cudaMemcpyDeviceToHost, s));
             CUDA_TRY(c, cudaStreamSynchronize(s));
-            if (!(dsum == dsum)) return NG_OK;               // non-finite: fall back
+            if (!(dsum == dsum)) return NG_OK;               // non-finite: a fresh solve follows
             if (dsum == 0.0 || dsum > 0.5 * prev) {           // at the round-off floor, or stalled
                 *refined_ok = dsum < ref_tol;
                 return NG_OK;
@@ -667,12 +680,45 @@ ng_status launch_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S, c
         }
         return NG_OK;
     }
-    const int64_t ab = (int64_t)(T + 1) * (T + 2) * g.nb;
-    k_mat_assemble<D><<<nblocks(ab, 256), 256, 0, s>>>(g, ws_g, ws_K, ws_A);
+    k_mat_assemble<D><<<nblocks((int64_t)(T + 1) * (T + 2) * g.nb, 256), 256, 0, s>>>(g, w.g, w.K, w.A);
     if ((st = check_launch(c, "k_mat_assemble"))) return st;
-    if ((st = lu_solve(c, N, D, g.nb, ws_A, ws_piv, s, ws_ext == nullptr))) return st;
-    k_mat_store<D><<<nblocks(items, 128), 128, 0, s>>>(g, ws_A, G, c->d_status);
-    return check_launch(c, "k_mat_store");
+    if (!inverse) {
+        if ((st = lu_solve(c, N, D, g.nb, w.A, w.piv, s))) return st;
+        k_mat_store<D><<<nblocks(items, 128), 128, 0, s>>>(g, w.A, G, c->d_status);
+        return check_launch(c, "k_mat_store");
+    }
+    CUDA_TRY(c, cudaMemsetAsync(w.keys, 0, 8 * (size_t)g.nb * (N + 1), s));
+    k_gj_first<<<dim3(nblocks(N, 128), g.nb), 128, 0, s>>>(N, ld, w.A, w.keys, w.piv);
+    const dim3 grid(nblocks(N, 32), nblocks(N, 4 * NG_GJ_ROWS), g.nb);
+    for (int col = 0; col < N; ++col) {
+        k_gj_step<<<grid, 128, 0, s>>>(N, ld, col % 2 ? w.A2 : w.A, col % 2 ? w.A : w.A2, col, w.keys, w.piv, c->d_status);
+        if (col % 256 == 0 && (st = check_launch(c, "k_gj_step"))) return st;
+    }
+    k_gj_apply<false><<<rows, 128, 0, s>>>(N, ld, D, inv, w.piv, w.g, G, nullptr, c->d_status);
+    if ((st = check_launch(c, "k_gj_apply"))) return st;
+    return refine(c->d_scalar);   // the inverse's rounding: one step of refinement
+}
+
+template <int D>
+ng_status launch_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S, const FuncV& eps, cudaStream_t s,
+                     int refine_steps = 0, double ref_tol = 0.0, bool* refined_ok = nullptr, void* ws_ext = nullptr) {
+    const int T = g.ntau, N = (T + 1) * D;
+    const bool inverse = mat_inverse(c, N, g.nb, ws_ext == nullptr);
+    MatWs w;
+    const size_t need = mat_ws(nullptr, T, D, g.nb, inverse, &w);
+    ng_status st = NG_OK;
+    if (!ws_ext && (st = ensure(c, &c->ws_mat, &c->ws_mat_bytes, need))) return st;
+    mat_ws(ws_ext ? ws_ext : c->ws_mat, T, D, g.nb, inverse, &w);
+    const int64_t items = (int64_t)(T + 1) * g.nb;
+    k_mat_g<D><<<nblocks(items, 128), 128, 0, s>>>(g, eps, w.g);
+    if ((st = check_launch(c, "k_mat_g"))) return st;
+    const bool warp = D <= 4 && items < (int64_t)c->sms * 128;
+    if constexpr (D <= 4) {
+        if (warp) k_mat_K_w<D><<<nblocks(items * 32, 128), 128, 0, s>>>(g, S, w.g, w.K);
+    }
+    if (!warp) k_mat_K<D><<<nblocks(items, 128), 128, 0, s>>>(g, S, w.g, w.K);
+    if ((st = check_launch(c, "k_mat_K"))) return st;
+    return mat_solve<D>(c, g, G, w, inverse, s, refine_steps, ref_tol, refined_ok);
 }
 
 template <int D>
@@ -683,6 +729,19 @@ ng_status launch_start(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S,
     ng_status st = NG_OK;
     if (!ws_ext && (st = ensure(c, &c->ws_st, &c->ws_st_bytes, need))) return st;
     cplx* ws = (cplx*)(ws_ext ? ws_ext : c->ws_st);
+    if constexpr (D <= 4) {
+        // one warp per item: the dense solves while the warps fit the GPU at once, the left-mixing row while a thread
+        // per item would leave SMs idle, the lesser columns always (k+1 items per problem)
+        const bool ret_w = g.nb <= 4 * c->sms, tv_w = (int64_t)(g.ntau + 1) * g.nb < (int64_t)c->sms * 128;
+        if (ret_w) k_start_ret_w<D><<<g.nb, 32, 0, s>>>(g, G, S, eps, ws, c->d_status);
+        else k_start_ret<D><<<nblocks(g.nb, 64), 64, 0, s>>>(g, G, S, eps, ws, c->d_status);
+        if ((st = check_launch(c, "k_start_ret"))) return st;
+        if (tv_w) k_start_tv_w<D><<<nblocks((int64_t)(g.ntau + 1) * g.nb * 32, 128), 128, 0, s>>>(g, G, S, ws, c->d_status);
+        else k_start_tv<D><<<nblocks((int64_t)(g.ntau + 1) * g.nb, 128), 128, 0, s>>>(g, G, S, ws, c->d_status);
+        if ((st = check_launch(c, "k_start_tv"))) return st;
+        k_start_les_w<D><<<(unsigned)((k + 1) * g.nb), 128, 0, s>>>(g, G, S, ws, c->d_status);
+        return check_launch(c, "k_start_les");
+    }
     k_start_ret<D><<<nblocks(g.nb, 64), 64, 0, s>>>(g, G, S, eps, ws, c->d_status);
     if ((st = check_launch(c, "k_start_ret"))) return st;
     k_start_tv<D><<<nblocks((int64_t)(g.ntau + 1) * g.nb, 128), 128, 0, s>>>(g, G, S, ws, c->d_status);
@@ -708,53 +767,21 @@ __global__ void k_v2_mat_fill(Grid g, HermV F, HermV Q, cplx* ws_g, cplx* ws_K) 
         }
 }
 
-// refine_steps > 0: refine the current G^M with the LU factors kept in *ws from the previous
-// solve (the operator of a self-consistency loop changes little between iterations), as the
-// Dyson Matsubara solve does; *refined_ok tells whether the residual reached ref_tol
+// refine_steps > 0: refine the current G^M with what the previous solve kept in *ws (the operator of a
+// self-consistency loop changes little between iterations), as the Dyson Matsubara solve does
 template <int D>
 ng_status launch_vie2_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV& F, const HermV& Q, cudaStream_t s,
                           void** ws, size_t* ws_bytes, int refine_steps = 0, double ref_tol = 0.0,
                           bool* refined_ok = nullptr) {
-    const int T = g.ntau, N = (T + 1) * D, ld = N + D;
-    const size_t b_g = sizeof(cplx) * (size_t)g.nb * (T + 1) * D * D;
-    const size_t b_A = sizeof(cplx) * (size_t)g.nb * N * ld;
-    const size_t b_piv = sizeof(int) * (size_t)g.nb * N + 256;
-    ng_status st = NG_OK;
-    if ((st = ensure(c, ws, ws_bytes, 3 * b_g + b_A + b_piv))) return st;
-    cplx* ws_g = (cplx*)*ws;
-    cplx* ws_K = ws_g + b_g / sizeof(cplx);
-    cplx* ws_r = ws_K + b_g / sizeof(cplx);
-    cplx* ws_A = ws_K + 2 * (b_g / sizeof(cplx));
-    int* ws_piv = (int*)(ws_A + b_A / sizeof(cplx));
-    const int64_t items = (int64_t)(T + 1) * g.nb;
-    k_v2_mat_fill<D><<<nblocks(items, 128), 128, 0, s>>>(g, F, Q, ws_g, ws_K);
+    const int T = g.ntau, N = (T + 1) * D;
+    const bool inverse = mat_inverse(c, N, g.nb, true);
+    MatWs w;
+    ng_status st = ensure(c, ws, ws_bytes, mat_ws(nullptr, T, D, g.nb, inverse, &w));
+    if (st) return st;
+    mat_ws(*ws, T, D, g.nb, inverse, &w);
+    k_v2_mat_fill<D><<<nblocks((int64_t)(T + 1) * g.nb, 128), 128, 0, s>>>(g, F, Q, w.g, w.K);
     if ((st = check_launch(c, "k_v2_mat_fill"))) return st;
-    if (refine_steps > 0) {
-        *refined_ok = false;
-        double prev = 1e300;
-        for (int r = 0; r < refine_steps; ++r) {
-            k_mat_resid<D><<<nblocks(items, 128), 128, 0, s>>>(g, ws_g, ws_K, G, ws_r);
-            if ((st = check_launch(c, "k_mat_resid"))) return st;
-            CUDA_TRY(c, cudaMemsetAsync(c->d_scalar, 0, sizeof(double), s));
-            k_lu_resolve<<<g.nb, NG_LU_THREADS, 0, s>>>(g, N, D, ws_A, ws_piv, ws_r, G, c->d_scalar);
-            if ((st = check_launch(c, "k_lu_resolve"))) return st;
-            double dsum = 0.0;
-            CUDA_TRY(c, cudaMemcpyAsync(&dsum, c->d_scalar, sizeof(double), cudaMemcpyDeviceToHost, s));
-            CUDA_TRY(c, cudaStreamSynchronize(s));
-            if (!(dsum == dsum)) return NG_OK;               // non-finite: a fresh solve follows
-            if (dsum == 0.0 || dsum > 0.5 * prev) {           // at the round-off floor, or stalled
-                *refined_ok = dsum < ref_tol;
-                return NG_OK;
-            }
-            prev = dsum;
-        }
-        return NG_OK;
-    }
-    k_mat_assemble<D><<<nblocks((int64_t)(T + 1) * (T + 2) * g.nb, 256), 256, 0, s>>>(g, ws_g, ws_K, ws_A);
-    if ((st = check_launch(c, "k_mat_assemble"))) return st;
-    if ((st = lu_solve(c, N, D, g.nb, ws_A, ws_piv, s))) return st;
-    k_mat_store<D><<<nblocks(items, 128), 128, 0, s>>>(g, ws_A, G, c->d_status);
-    return check_launch(c, "k_mat_store");
+    return mat_solve<D>(c, g, G, w, inverse, s, refine_steps, ref_tol, refined_ok);
 }
 
 // one warp per vie2 bulk item: forced, or for batches with fewer items than 128 per SM
@@ -1047,8 +1074,8 @@ ng_status do_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S, const
 }
 // workspace bytes of one Matsubara solve and of one start-up (nb problems of grid g)
 size_t mat_ws_bytes(const Grid& g) {
-    const size_t D = g.nf, T = g.ntau, N = (T + 1) * D, ld = N + D;
-    return 3 * sizeof(cplx) * g.nb * (T + 1) * D * D + sizeof(cplx) * g.nb * N * ld + sizeof(int) * g.nb * N + 256;
+    MatWs w;
+    return mat_ws(nullptr, g.ntau, g.nf, g.nb, false, &w);
 }
 size_t start_ws_bytes(const Grid& g) {
     const size_t D = g.nf, N = (size_t)g.k * D;
