@@ -11,6 +11,7 @@
 #include "ng_step32.cuh"
 #include "ng_stepsplit.cuh"
 #include "ng_bound.cuh"
+#include "ng_stepq.cuh"
 #include "ng_obs.cuh"
 #include "ng_ubatch.cuh"
 #include "ng_stepdf.cuh"
@@ -301,16 +302,27 @@ ng_status prep_tvfft(ng_ctx* c, const Grid& g, int n, const HermV& G, const Herm
     return NG_OK;
 }
 
-// Whether the history sums of step n run as digit products (ng_hist.cu): nf = 1, groups of 8 problems,
-// and work = nb (2 n^2 + 2 n ntau + ntau^2) multiply-adds (history, and the left-mixing source that the warp
-// form sums directly) above 8e6, or 16e6 where the warp form is the alternative: the launches of the digit
-// products take about 100 us for any size.  Whole steps, FP64 kernels / digit products in us, at
-// work / 1e6: one thread per item 512 problems 28730 / 10370 (3.9e3), 64 problems 344 / 233 (13), 100 problems
-// 181 / 198 (6.5); one warp per item 8 problems 320 / 211 (24), 12 problems 255 / 239 (16), 16 problems 186 / 229 (9.3).
+// Whether the history sums of step n run as digit products (ng_hist.cu): nf = 1, groups of 8 problems, and
+// enough work = nb (2 n^2 + 2 n ntau) multiply-adds, since their launches take about 100 us for any size.
+// Dyson step: against P lanes per item (k_step_bulk_q) the line lies at 14e6, lower for many problems, whose
+// units fill the GPU.  Whole steps, lanes / digit products in us: 16 problems, ntau = 250, n = 300 (5.3e6)
+// 106 / 179, n = 800 (27e6) 308 / 201; 64 problems, ntau = 100, n = 200 (7.7e6) 130 / 168, n = 300 (15e6) 196 / 189;
+// 128 problems, ntau = 400, n = 64 (7.6e6) 185 / 165; 256 problems, ntau = 250, n = 16 (2.2e6) 138 / 118, ntau = 30,
+// n = 64 (3.1e6) 85 / 97.
+bool hist_form(const ng_ctx* c, const Grid& g, int n) {
+    return g.nf == 1 && g.nb >= NGH_KG && c->bulk_split == NG_BULK_AUTO && n >= 2 * g.k + 2;
+}
 bool hist_applies(const ng_ctx* c, const Grid& g, int n) {
-    if (g.nf != 1 || g.nb < NGH_KG || c->bulk_split != NG_BULK_AUTO || n < 2 * g.k + 2) return false;
+    const double work = 2.0 * g.nb * n * ((double)n + g.ntau);
+    return hist_form(c, g, n) &&
+           work >= (g.nb < 128 ? 14e6 : g.nb < 256 ? 7e6 : g.ntau >= 100 ? 1.8e6 : 4e6);
+}
+// vie2 step: against a warp or a thread per item, with the left-mixing source's direct sums (ntau^2 multiply-adds per
+// problem) in the work: 16e6 where the warp form is the alternative, else 8e6.  Step in us, FP64 kernels / digit
+// products: 65 problems, n = 333, ntau = 90 (19e6) 349 / 175; 300 problems, n = 30, ntau = 30 (1.4e6) 60 / 73.
+bool hist_applies_vie2(const ng_ctx* c, const Grid& g, int n) {
     const double N = n, T = g.ntau, work = g.nb * (2.0 * N * (N + T) + T * T);
-    return work >= ((double)g.nb * (2.0 * N + T) < 128.0 * c->sms ? 16e6 : 8e6);
+    return hist_form(c, g, n) && work >= ((double)g.nb * (2.0 * N + T) < 128.0 * c->sms ? 16e6 : 8e6);
 }
 // *w describes the sums; *ok = false without room for the workspace: the step keeps the FP64 kernels
 ng_status hist_sums(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV& S, const HermV& Scc, HistWs* w, bool* ok,
@@ -419,9 +431,19 @@ ng_status launch_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const
     const bool spread = c->bulk_split == NG_BULK_WARP ||
                         (c->bulk_split == NG_BULK_AUTO && (int64_t)nq * g.nb < 2 * (int64_t)c->sms);
     const bool lanes = D == 1 && c->bulk_split == NG_BULK_AUTO && bnd1_applies(g, n);
-    const int64_t w_pre = (warp && (spread || lanes)) ? g.nb : 0;
+    // lanes per item of k_step_bulk_q (0: not used): below 16 problems the warp form's boundary is the faster one, and
+    // above 1000 items a SM a thread per item fills the GPU.  Whole steps in us, warp or thread per item / 8
+    // lanes: 16 problems, ntau = 100, n = 300: 126 / 91; 64 problems, ntau = 100, n = 40: 97 / 62; 256 problems,
+    // ntau = 30, n = 96: 144 / 124 (4 lanes 128); 4 lanes win from 256 items a SM on.
+    int part = 0;
+    if (D == 1 && c->bulk_split == NG_BULK_AUTO && !digits && g.nb >= 16 && items < 1000 * (int64_t)c->sms)
+        part = items < 256 * (int64_t)c->sms ? 8 : 4;
+    const int64_t w_pre = (part ? lanes : warp && (spread || lanes)) ? g.nb : 0;
     const cplx* tvq = nullptr;
-    ng_status sm = warp ? NG_OK : prep_tvfft(c, g, n, G, S, s, &tvq);
+    // its left-mixing source: direct sums while these are below the cost of the FFT's launch (32 problems, ntau = 400,
+    // n = 16: 97 against 103 us; ntau = 900: 260 against 167)
+    const bool direct = part ? (double)g.nb * g.ntau * g.ntau < 6e6 : warp;
+    ng_status sm = direct ? NG_OK : prep_tvfft(c, g, n, G, S, s, &tvq);
     if (sm) return sm;
     long e0 = prof_pair(c, 0);
     if (e0 >= 0) cudaEventRecord(c->ev_pool[e0], s);
@@ -433,6 +455,12 @@ ng_status launch_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const
     if (hist) {
         k_hist_close<<<pre + b_les + b_tv + b_ret, thr, 0, s>>>(g, n, G, S, eps, hw, (const cplx*)c->ws_minv, pre, b_les,
                                                                 b_tv, tvq, c->d_status);
+    } else if (part) {
+        const int c_les = it_les ? n - k - 1 : 0, c_tv = g.ntau + 1, c_ret = n - k, q = 32 / part;
+        const int64_t warps = w_pre + (int64_t)(c_les + c_tv + c_ret) * nblocks(g.nb, q);
+        auto kernel = part == 4 ? k_step_bulk_q<4> : k_step_bulk_q<8>;
+        kernel<<<nblocks(warps * 32, thr), thr, 0, s>>>(g, n, G, S, eps, (const cplx*)c->ws_minv, (int)w_pre, c_les, c_tv,
+                                                        c_ret, tvq, c->d_status);
     } else if (warp) {
         k_step_bulk_w<D><<<nblocks((w_pre + items) * 32, thr), thr, 0, s>>>(g, n, G, S, eps, (const cplx*)c->ws_minv,
                                                                            w_pre, it_les, it_tv, it_ret, c->d_status);
@@ -787,7 +815,7 @@ ng_status launch_vie2_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV&
 // one warp per vie2 bulk item: forced, or for batches with fewer items than 128 per SM
 bool vie2_warp(const ng_ctx* c, const Grid& g, int n) {
     const int64_t items = (int64_t)g.nb * ((n - 1) + (g.ntau + 1) + n);
-    if (hist_applies(c, g, n)) return false;
+    if (hist_applies_vie2(c, g, n)) return false;
     return c->bulk_split == NG_BULK_WARP || (c->bulk_split == NG_BULK_AUTO && items < (int64_t)c->sms * 128);
 }
 
@@ -1356,7 +1384,7 @@ ng_status ng_vie2_timestep(ng_ctx* c, const ng_grid* grid, int tstp, ng_herm G, 
     if (!w && (st = prep_tvfft(c, g, tstp, Gv, Fv, (cudaStream_t)stream, &tvq))) return st;
     bool hist = false;
     HistWs hw;
-    if (!w && hist_applies(c, g, tstp) && (st = hist_sums(c, g, tstp, Gv, Fv, Fccv, &hw, &hist, (cudaStream_t)stream))) return st;
+    if (!w && hist_applies_vie2(c, g, tstp) && (st = hist_sums(c, g, tstp, Gv, Fv, Fccv, &hw, &hist, (cudaStream_t)stream))) return st;
     if (vie2_step_launch(g, tstp, Gv, Fv, Fccv, Qv, tvq, w, hist ? &hw : nullptr, c->d_status, (cudaStream_t)stream) !=
         cudaSuccess) {
         cudaGetLastError();
@@ -1694,7 +1722,7 @@ static ng_status run_2b_impl(ng_ctx* c, const ng_grid* grid, ng_herm G, ng_herm 
                 if (!w && (r = prep_tvfft(c, gw->gb, n, gw->X, gw->K, s, &tvq, false))) return r;
                 bool hist = false;
                 HistWs hw;
-                if (!w && hist_applies(c, gw->gb, n) && (r = hist_sums(c, gw->gb, n, gw->X, gw->K, gw->Kcc, &hw, &hist, s)))
+                if (!w && hist_applies_vie2(c, gw->gb, n) && (r = hist_sums(c, gw->gb, n, gw->X, gw->K, gw->Kcc, &hw, &hist, s)))
                     return r;
                 e = vie2_step_launch(gw->gb, n, gw->X, gw->K, gw->Kcc, gw->P, tvq, w, hist ? &hw : nullptr, c->d_status, s);
             }

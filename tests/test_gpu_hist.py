@@ -1,5 +1,5 @@
 """Time steps whose history sums run as digit products on the tensor cores (nf = 1, at least 8
-problems, at least 1.6e7 multiply-adds) against the FP64 kernels of the same library (NG_BULK_THREAD, themselves
+problems, enough work), and steps with several lanes per item below that, against the FP64 kernels of the same library (NG_BULK_THREAD, themselves
 pinned to the oracle): edges of the 128 x 128 units and 16 x 16 tiles, ragged problem groups, every
 quadrature order, shared and per-problem row functions, scale growth inside a unit, zeros and
 non-finite values.
@@ -55,10 +55,12 @@ def _check(a, b):
 
 
 DYSON = [  # nk, n, ntau, k, shared
-    (29, 384, 300, 5, True), (33, 129, 640, 4, True), (203, 13, 400, 5, True), (130, 128, 127, 3, False),
-    (31, 400, 127, 2, False), (17, 600, 129, 1, True), (40, 144, 383, 5, False), (8, 770, 639, 5, True),
-    # below the line: one warp per item, the boundary with one lane per problem (16 problems and more)
-    (16, 11, 12, 5, True), (33, 12, 25, 4, False), (47, 30, 16, 1, True), (31, 64, 40, 3, True),
+    (29, 384, 300, 5, True), (129, 129, 640, 4, True), (264, 13, 400, 5, True), (130, 128, 127, 3, False),
+    (36, 400, 127, 2, False), (17, 600, 129, 1, True), (131, 144, 383, 5, False), (8, 770, 639, 5, True),
+    # below the line: eight or four lanes per item, the boundary with one lane per problem (16 problems and
+    # more); direct left-mixing source, then by FFT
+    (16, 11, 12, 5, True), (33, 12, 25, 4, False), (47, 30, 16, 1, True), (31, 64, 40, 3, True), (70, 40, 100, 5, True),
+    (300, 60, 30, 2, False), (129, 20, 300, 4, False), (20, 90, 600, 5, True),
 ]
 
 
@@ -92,7 +94,7 @@ def test_vie2_step(ng, nk, n, T, k, fs, ccs, sig):
 def test_scale_growth_and_zeros(ng, grow):
     """History that grows (or falls) by 2^60 along the rows, problems of very different size, and
     problems that are zero."""
-    nk, n, T, k = 40, 300, 100, 5
+    nk, n, T, k = 60, 300, 100, 5
     g = ng.Grid(nt=n, ntau=T, nf=1, nbatch=nk, korder=k, h=0.02, beta=4.0)
     G, S, eps = ng.Herm(g), ng.Herm(g, ldk=1), ng.Func(g)
     _random(G, 3, 0.3)
@@ -102,7 +104,7 @@ def test_scale_growth_and_zeros(ng, grow):
         t *= torch.exp2(grow * 0.3 * row)[:, None, None, None]
     G.tv *= torch.exp2(grow * 0.3 * torch.arange(n + 1, device="cuda").repeat_interleave(T + 1).double())[:, None, None, None]
     for t in G.tensors().values():
-        t *= torch.exp2(15.0 * torch.arange(nk, device="cuda").double() - 300.0)
+        t *= torch.exp2(10.0 * torch.arange(nk, device="cuda").double() - 300.0)
         t[..., 5] = 0
     ctx = ng.Context(k)
     (a, _), (b, _) = _both(ng, ctx, g, n, G, lambda: ctx.dyson_timestep(g, n, G, S, eps))
@@ -118,7 +120,7 @@ def test_scale_growth_and_zeros(ng, grow):
 @pytest.mark.parametrize("value", [float("nan"), float("inf")])
 def test_non_finite(ng, where, value):
     """A non-finite element spoils the items that read it and no others, and sets the status."""
-    nk, n, T, k = 41, 300, 100, 5
+    nk, n, T, k = 61, 300, 100, 5
     g = ng.Grid(nt=n, ntau=T, nf=1, nbatch=nk, korder=k, h=0.02, beta=4.0)
     G, S, eps = ng.Herm(g), ng.Herm(g), ng.Func(g)
     _random(G, 5, 0.3)
