@@ -18,7 +18,7 @@ cudaError_t adj_pass(const AdjStep& a, SliceV Glc, const cplx* U, SliceV cLoc, d
     k_adj_qA<<<nblk((int64_t)(std::max(n, T) + 1) * nb, 128), 128, 0, s>>>(a);
     const int width = std::max(n + 1, T + 1);
     k_adj_sigA<<<dim3(nblk((int64_t)a.nq * width * 32, 128), 4), 128, 0, s>>>(a, width);
-    k_adj_bulk<<<nb, 128, 0, s>>>(a);
+    k_adj_bulk<<<dim3(nb, 2), 128, 0, s>>>(a);
     const unsigned S = NG_ADJ_SPLIT;
     k_adj_tvrow<<<dim3(n, S), 256, 0, s>>>(a);
     k_adj_rrow<<<dim3(n, S), 256, 0, s>>>(a);
@@ -39,7 +39,7 @@ cudaError_t adj_pass(const AdjStep& a, SliceV Glc, const cplx* U, SliceV cLoc, d
 
 cudaError_t adj_predictor(const Grid& g, int n, SliceV cw, cplx* cGr, cplx* cGl, cplx* cGt, cudaStream_t s) {
     k_adj_extrap_diag<<<nblk((int64_t)(2 * (n - g.k) + g.ntau + 1) * g.nb, 128), 128, 0, s>>>(g, n, cw, cGr, cGl, cGt);
-    k_adj_extrap_cols<<<nblk(g.nb, 128), 128, 0, s>>>(g, n, cw, cGr, cGl);
+    k_adj_extrap_cols<<<nblk((int64_t)2 * (n > 2 * g.k ? g.k + 1 : 1) * g.nb, 128), 128, 0, s>>>(g, n, cw, cGr, cGl);
     return cudaGetLastError();
 }
 

@@ -71,16 +71,22 @@ __global__ void __launch_bounds__(128) k_adj_lesA(AdjStep a) {
     const NgWeights& W = c_W[a.g.k - 1];
     const int k = W.k, n = a.n, nb = a.g.nb, kb = blockIdx.x, t = threadIdx.x;
     const double h = a.g.h;
-    __shared__ cplx sc;
+    __shared__ cplx sc, Mis[NG_KMAX + 1];   // conj(M_m)^-1 of the rows: independent of the chain, a lane each
+    __shared__ cplx Ash[NG_KMAX * NG_KMAX], cbs[NG_KMAX], M0s[NG_KMAX + 1], fsh[NG_KMAX];
     cplx* cwl = a.cw.les;
     const int mstep = a.full ? k + 1 : n - k;
+    if (t <= n - mstep) {
+        const int m = mstep + t;
+        cplx e = adj_mf(a, m, kb);
+        e.x -= a.g.mu;
+        cplx M = cadd(cr(W.a[0] / h), cmuli(e));
+        M = cadd(M, cscal(h * gw(W, m, m), cmuli(adj_sigR(a, m, m))));
+        Mis[t] = cconj(cinv(M));
+    }
+    __syncthreads();
     for (int m = n; m >= mstep; --m) {
         if (t == 0) {
-            cplx e = adj_mf(a, m, kb);
-            e.x -= a.g.mu;
-            cplx M = cadd(cr(W.a[0] / h), cmuli(e));
-            M = cadd(M, cscal(h * gw(W, m, m), cmuli(adj_sigR(a, m, m))));
-            const cplx cacc = cmul(cconj(cdiv(cr(1.0), M)), cwl[(int64_t)m * nb + kb]);
+            const cplx cacc = cmul(Mis[m - mstep], cwl[(int64_t)m * nb + kb]);
             a.cA[(int64_t)(m - a.m0) * nb + kb] = cacc;
             // c(eps_m) += -i c(M_m),  c(M_m) = -conj(G^<(m,n)) cacc
             const cplx dm = cmuli(cmul(cconj(a.Gc.les[(int64_t)m * nb + kb]), cacc));
@@ -98,29 +104,32 @@ __global__ void __launch_bounds__(128) k_adj_lesA(AdjStep a) {
         }
         __syncthreads();
     }
-    if (!a.full || t != 0) return;
-    // start-up block m = 1..k (Eq. vdiff_start): sum_{l>=1} M_{m,l} y_l = q_m - M_{m,0} y_0,
+    if (!a.full || t >= 32) return;
+    // start-up block m = 1..k (Eq. vdiff_start), by one warp: sum_{l>=1} M_{m,l} y_l = q_m - M_{m,0} y_0,
     // M_{m,l} = D_{m,l}/h + h s_{m,l} i Sigma~^R(m,l) + delta_{ml} i(eps_m - mu)
-    cplx AH[NG_KMAX * NG_KMAX], cb[NG_KMAX], M0[NG_KMAX + 1];
-    for (int m = 1; m <= k; ++m) {
-        cplx e = adj_mf(a, m, kb);
-        e.x -= a.g.mu;
-        for (int l = 0; l <= k; ++l) {
-            cplx M = cadd(cr(W.D[m][l] / h), cscal(h * W.greg[m][l], cmuli(adj_sigRx(a, m, l))));
-            if (l == m) M = cadd(M, cmuli(e));
-            if (l == 0) M0[m] = M;
-            else AH[(l - 1) * k + (m - 1)] = cconj(M);      // (A^H)[l][m] = conj(A[m][l])
+    for (int p = t; p < k * (k + 1); p += 32) {
+        const int m = 1 + p / (k + 1), l = p % (k + 1);
+        cplx M = cadd(cr(W.D[m][l] / h), cscal(h * W.greg[m][l], cmuli(adj_sigRx(a, m, l))));
+        if (l == m) {
+            cplx e = adj_mf(a, m, kb);
+            e.x -= a.g.mu;
+            M = cadd(M, cmuli(e));
         }
-        cb[m - 1] = cwl[(int64_t)m * nb + kb];
+        if (l == 0) M0s[m] = M;
+        else Ash[(l - 1) * k + (m - 1)] = cconj(M);      // (A^H)[l][m] = conj(A[m][l])
+        if (l == 0) cbs[m - 1] = cwl[(int64_t)m * nb + kb];
     }
-    dense_solve(AH, k, cb, 1);   // a singular system was flagged by the forward step
-    cplx c0 = cz();
-    for (int m = 1; m <= k; ++m) {
-        a.cA[(int64_t)(m - a.m0) * nb + kb] = cb[m - 1];
-        c0 = csub(c0, cmul(cconj(M0[m]), cb[m - 1]));
-        const cplx dm = cmuli(cmul(cconj(a.Gc.les[(int64_t)m * nb + kb]), cb[m - 1]));
+    __syncwarp();
+    warp_dense_solve(Ash, k, cbs, 1, fsh, t);   // a singular system was flagged by the forward step
+    __syncwarp();
+    for (int m = 1 + t; m <= k; m += 32) {
+        a.cA[(int64_t)(m - a.m0) * nb + kb] = cbs[m - 1];
+        const cplx dm = cmuli(cmul(cconj(a.Gc.les[(int64_t)m * nb + kb]), cbs[m - 1]));
         a.cmf[(int64_t)(m + 1) * nb + kb] = cadd(a.cmf[(int64_t)(m + 1) * nb + kb], dm);
     }
+    if (t != 0) return;
+    cplx c0 = cz();
+    for (int m = 1; m <= k; ++m) c0 = csub(c0, cmul(cconj(M0s[m]), cbs[m - 1]));
     cwl[kb] = cadd(cwl[kb], c0);
 }
 
@@ -237,18 +246,60 @@ __global__ void k_adj_sigA(AdjStep a, int width) {
 
 // ======================================================================================
 // 4. Per problem: cotangents of the (B) right-hand sides (ret columns, tv columns, lesser
-//    rows), of M_n, and the retarded (A) block (Eq. MBCVSAMx_cc_start along row n).
+//    rows), of M_n, and, in blocks of their own (blockIdx.y = 1, one warp), the retarded (A) block
+//    (Eq. MBCVSAMx_cc_start along row n), whose k x k solve on one thread took most of this kernel's
+//    62 us (64 problems, n <= 100).
 // ======================================================================================
+__device__ __forceinline__ void adj_retA_w(const AdjStep& a, int kb, int lane) {
+    const NgWeights& W = c_W[a.g.k - 1];
+    const int k = W.k, n = a.n, nb = a.g.nb;
+    const double h = a.g.h;
+    __shared__ cplx AH[NG_KMAX * NG_KMAX], cb[NG_KMAX], f[NG_KMAX];
+    // y_l = G^R(n, n-l), y_0 = -i; sum_{l>=1} y_l Mh[l][j] = -y_0 Mh[0][j], j = 1..k,
+    // Mh[l][j] = D_{j,l}/h + delta_{lj} i(eps_{n-j} - mu) + h s_{j,l} i Sigma~^R(n-l, n-j).
+    // As A y = b with A[j][l] = Mh[l][j]:  c(b) = A^-H c(y), c(A) = -c(b) y^H.
+    for (int p = lane; p < k * k; p += 32) {
+        const int j = 1 + p / k, l = 1 + p % k;
+        cplx Mh = cadd(cr(W.D[j][l] / h), cscal(h * W.greg[j][l], cmuli(adj_sigRx(a, n - l, n - j))));
+        if (l == j) {
+            cplx ej = adj_mf(a, n - j, kb);
+            ej.x -= a.g.mu;
+            Mh = cadd(Mh, cmuli(ej));
+        }
+        AH[(l - 1) * k + (j - 1)] = cconj(Mh);   // (A^H)[l][j] = conj(A[j][l]) = conj(Mh[l][j])
+    }
+    for (int l = 1 + lane; l <= k; l += 32) cb[l - 1] = a.cw.ret[(int64_t)(n - l) * nb + kb];
+    __syncwarp();
+    warp_dense_solve(AH, k, cb, 1, f, lane);
+    __syncwarp();
+    const int K1 = k + 1;
+    for (int p = lane; p < k * K1; p += 32) {
+        const int j = 1 + p / K1, l = p % K1;
+        // c(Mh[l][j]): l >= 1: -c(b_j) conj(y_l); l = 0: b_j = i Mh[0][j] -> -i c(b_j)
+        const cplx cMh = (l == 0) ? cmulmi(cb[j - 1]) : cneg(cmul(cb[j - 1], cconj(a.Gc.ret[(int64_t)(n - l) * nb + kb])));
+        // c(Sigma~^R(n-l, n-j)) += -i h s_{j,l} c(Mh)
+        a.retA[(int64_t)(l * K1 + j) * nb + kb] = cmulmi(cscal(h * W.greg[j][l], cMh));
+        if (l == j) {
+            cplx* q = &a.cmf[(int64_t)(n - j + 1) * nb + kb];
+            *q = cadd(*q, cmulmi(cMh));
+        }
+    }
+}
+
 __global__ void __launch_bounds__(128) k_adj_bulk(AdjStep a) {
     const NgWeights& W = c_W[a.g.k - 1];
     const int k = W.k, n = a.n, nb = a.g.nb, T = a.g.ntau, kb = blockIdx.x, t = threadIdx.x;
     const double h = a.g.h;
     __shared__ cplx red[32];
+    if (blockIdx.y == 1) {
+        if (t < 32) adj_retA_w(a, kb, t);
+        return;
+    }
     cplx e = a.mfc[kb];
     e.x -= a.g.mu;
     cplx M = cadd(cr(W.a[0] / h), cmuli(e));
     M = cadd(M, cscal(h * gw(W, n, n), cmuli(a.Sc.ret[n])));
-    const cplx Minv = cdiv(cr(1.0), M);
+    const cplx Minv = cinv(M);
     const cplx cMinvc = cconj(Minv);
     cplx cMi = cz();   // cotangent of M_n^-1
     for (int m = t; m <= n - k - 1; m += blockDim.x) {
@@ -273,36 +324,6 @@ __global__ void __launch_bounds__(128) k_adj_bulk(AdjStep a) {
     const cplx cM = cneg(cmul(cconj(cmul(Minv, Minv)), cMi));
     a.cmfw[kb] = cadd(a.cmfw[kb], cmulmi(cM));
     a.cMn[kb] = cM;
-    // retarded (A): y_l = G^R(n, n-l), y_0 = -i; sum_{l>=1} y_l Mh[l][j] = -y_0 Mh[0][j], j = 1..k,
-    // Mh[l][j] = D_{j,l}/h + delta_{lj} i(eps_{n-j} - mu) + h s_{j,l} i Sigma~^R(n-l, n-j).
-    // As A y = b with A[j][l] = Mh[l][j]:  c(b) = A^-H c(y), c(A) = -c(b) y^H.
-    cplx AH[NG_KMAX * NG_KMAX], cb[NG_KMAX];
-    for (int j = 1; j <= k; ++j)
-        for (int l = 1; l <= k; ++l) {
-            cplx Mh = cadd(cr(W.D[j][l] / h), cscal(h * W.greg[j][l], cmuli(adj_sigRx(a, n - l, n - j))));
-            if (l == j) {
-                cplx ej = adj_mf(a, n - j, kb);
-                ej.x -= a.g.mu;
-                Mh = cadd(Mh, cmuli(ej));
-            }
-            AH[(l - 1) * k + (j - 1)] = cconj(Mh);   // (A^H)[l][j] = conj(A[j][l]) = conj(Mh[l][j])
-        }
-    for (int l = 1; l <= k; ++l) cb[l - 1] = a.cw.ret[(int64_t)(n - l) * nb + kb];
-    dense_solve(AH, k, cb, 1);
-    const int K1 = k + 1;
-    for (int j = 1; j <= k; ++j) {
-        for (int l = 0; l <= k; ++l) {
-            // c(Mh[l][j]): l >= 1: -c(b_j) conj(y_l); l = 0: b_j = i Mh[0][j] -> -i c(b_j)
-            const cplx cMh = (l == 0) ? cmulmi(cb[j - 1])
-                                      : cneg(cmul(cb[j - 1], cconj(a.Gc.ret[(int64_t)(n - l) * nb + kb])));
-            // c(Sigma~^R(n-l, n-j)) += -i h s_{j,l} c(Mh)
-            a.retA[(int64_t)(l * K1 + j) * nb + kb] = cmulmi(cscal(h * W.greg[j][l], cMh));
-            if (l == j) {
-                cplx* p = &a.cmf[(int64_t)(n - j + 1) * nb + kb];
-                *p = cadd(*p, cmulmi(cMh));
-            }
-        }
-    }
 }
 
 // ======================================================================================
@@ -730,24 +751,24 @@ __global__ void k_adj_extrap_diag(Grid g, int n, SliceV cw, cplx* cGr, cplx* cGl
     }
 }
 
-// columns j <= k of ret and rows j <= k of les (with the hermitian continuation); thread per problem
+// columns j <= k of ret and rows j <= k of les (with the hermitian continuation): thread per (component, j,
+// problem) where no continued element meets another column's (n > 2k), else per (component, problem)
 __global__ void k_adj_extrap_cols(Grid g, int n, SliceV cw, cplx* cGr, cplx* cGl) {
     const NgWeights& W = c_W[g.k - 1];
     const int k = W.k, nb = g.nb, Np = n - 1;
-    const int kb = blockIdx.x * blockDim.x + threadIdx.x;
-    if (kb >= nb) return;
-    for (int j = 0; j <= k; ++j) {
-        const cplx cr_ = cw.ret[(int64_t)j * nb + kb], cl = cw.les[(int64_t)j * nb + kb];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, kb = i % nb, c = i / nb;
+    const bool split = n > 2 * k;
+    const int comp = split ? c / (k + 1) : c, j0 = split ? c % (k + 1) : 0, j1 = split ? j0 : k;
+    if (comp > 1) return;
+    const cplx* src = comp ? cw.les : cw.ret;
+    cplx* dst = comp ? cGl : cGr;
+    for (int j = j0; j <= j1; ++j) {
+        const cplx x = src[(int64_t)j * nb + kb];
         for (int l = 0; l <= k; ++l) {
             const int r = Np - l;
-            const cplx vr = cscal(W.C[l], cr_), vl = cscal(W.C[l], cl);
-            if (j <= r) {
-                cGr[(tri(r) + j) * nb + kb] = cadd(cGr[(tri(r) + j) * nb + kb], vr);
-                cGl[(tri(r) + j) * nb + kb] = cadd(cGl[(tri(r) + j) * nb + kb], vl);
-            } else {
-                cGr[(tri(j) + r) * nb + kb] = csub(cGr[(tri(j) + r) * nb + kb], cconj(vr));
-                cGl[(tri(j) + r) * nb + kb] = csub(cGl[(tri(j) + r) * nb + kb], cconj(vl));
-            }
+            const cplx v = cscal(W.C[l], x);
+            cplx* p = &dst[(j <= r ? tri(r) + j : tri(j) + r) * nb + kb];
+            *p = j <= r ? cadd(*p, v) : csub(*p, cconj(v));
         }
     }
 }
@@ -775,9 +796,10 @@ __global__ void __launch_bounds__(NG_BOOT_THREADS) k_adj_start(AdjBoot b) {
     extern __shared__ cplx dsm[];
     cplx* c = dsm;                          // [E] local cotangent of the slices
     cplx* rt = c + E;                       // [k][T+1] tv right-hand-side cotangents
-    __shared__ cplx red[32];
     __shared__ cplx M[NG_KMAX + 1][NG_KMAX + 1], cM[NG_KMAX + 1][NG_KMAX + 1];
     __shared__ cplx qsh[NG_KMAX + 1], crh[NG_KMAX + 1];
+    __shared__ cplx As[NG_KMAX * NG_KMAX], AHs[NG_KMAX * NG_KMAX], sol[NG_KMAX], cs[NG_KMAX], fs[NG_KMAX];
+    const int lane = t & 31, wid = t >> 5, nwp = blockDim.x >> 5;
     auto GR = [&](int n, int j) { return b.Gr[(tri(n) + j) * nb + kb]; };
     auto GRx = [&](int n, int j) { return j <= n ? GR(n, j) : cneg(cconj(GR(j, n))); };
     auto GL = [&](int j, int n) { return b.Gl[(tri(n) + j) * nb + kb]; };
@@ -804,62 +826,64 @@ __global__ void __launch_bounds__(NG_BOOT_THREADS) k_adj_start(AdjBoot b) {
     auto cmf = [&](int n) -> cplx& { return b.cmfx[(int64_t)(n + 1) * nb + kb]; };
 
     for (int64_t e = t; e < E; e += blockDim.x) c[e] = b.mu[e * nb + kb];
-    if (t == 0) {
-        // shared start matrix M[n][l] = D_{n,l}/h + h s_{n,l} i Sigma~^R(n,l) + delta i(eps_n - mu)
-        for (int n = 1; n <= k; ++n)
-            for (int l = 0; l <= k; ++l) {
-                cplx v = cadd(cr(W.D[n][l] / h), cscal(h * W.greg[n][l], cmuli(SRx(n, l))));
-                if (l == n) v = cadd(v, cmuli(EPS(n)));
-                M[n][l] = v;
-                cM[n][l] = cz();
-            }
+    // shared start matrix M[n][l] = D_{n,l}/h + h s_{n,l} i Sigma~^R(n,l) + delta i(eps_n - mu)
+    for (int p = t; p < k * (k + 1); p += blockDim.x) {
+        const int n = 1 + p / (k + 1), l = p % (k + 1);
+        cplx v = cadd(cr(W.D[n][l] / h), cscal(h * W.greg[n][l], cmuli(SRx(n, l))));
+        if (l == n) v = cadd(v, cmuli(EPS(n)));
+        M[n][l] = v;
+        cM[n][l] = cz();
     }
     __syncthreads();
     // ---- lesser columns n = k..0: y_0 = -conj(G^tv(n,0)), M[1:,1:] y = q_A - M[:,0] y_0 ----
     for (int n = k; n >= 0; --n) {
         // forward sources q_m = -i h c2 + xi htau c3, c2 = sum_{j<=k} s_{n,j} Sigma^<(m,j) conj(G~^R(n,j)),
         // c3 = sum_j w_{T,j} Sigma^tv(m,j) conj(G^tv(n,T-j))
-        for (int m = 1; m <= k; ++m) {
-            cplx p3 = cz();
-            for (int j = t; j <= T; j += blockDim.x) p3 = cfma(cscal(gw(W, T, j), ST(m, j)), cconj(GT(n, T - j)), p3);
-            p3 = block_csum(p3, red);
-            if (t == 0) {
-                cplx c2 = cz();
-                for (int j = 0; j <= k; ++j) c2 = cfma(cscal(W.greg[n][j], SL(m, j)), cconj(GRx(n, j)), c2);
-                qsh[m] = cadd(cmulmi(cscal(h, c2)), cscal(xi * ht, p3));
-            }
+        for (int m = 1 + wid; m <= k; m += nwp) {   // a warp per row
+            cplx p3 = cz(), c2 = cz();
+            for (int j = lane; j <= T; j += 32) p3 = cfma(cscal(gw(W, T, j), ST(m, j)), cconj(GT(n, T - j)), p3);
+            for (int j = lane; j <= k; j += 32) c2 = cfma(cscal(W.greg[n][j], SL(m, j)), cconj(GRx(n, j)), c2);
+            const cplx q = warp_sum(cadd(cmulmi(cscal(h, c2)), cscal(xi * ht, p3)));
+            if (lane == 0) qsh[m] = q;
         }
         __syncthreads();
-        if (t == 0) {
+        if (wid == 0) {
             const cplx y0 = GL(0, n);
-            cplx A[NG_KMAX * NG_KMAX], AH[NG_KMAX * NG_KMAX], sol[NG_KMAX], cs[NG_KMAX];
-            for (int m = 1; m <= k; ++m) {
+            for (int p = lane; p < k * k; p += 32) {
+                const int m = 1 + p / k, l = 1 + p % k;
+                As[(m - 1) * k + (l - 1)] = M[m][l];
+                AHs[(l - 1) * k + (m - 1)] = cconj(M[m][l]);
+            }
+            for (int m = 1 + lane; m <= k; m += 32) {
                 sol[m - 1] = csub(qsh[m], cmul(M[m][0], y0));
                 cs[m - 1] = (m <= n) ? cles(m, n) : cz();
-                for (int l = 1; l <= k; ++l) {
-                    A[(m - 1) * k + (l - 1)] = M[m][l];
-                    AH[(l - 1) * k + (m - 1)] = cconj(M[m][l]);
-                }
             }
-            dense_solve(A, k, sol, 1);      // full forward solution (components m > n are not stored)
-            dense_solve(AH, k, cs, 1);      // cotangent of the right-hand side
-            cplx cy0 = cles(0, n);
-            for (int m = 1; m <= k; ++m) {
-                for (int l = 1; l <= k; ++l) cM[m][l] = csub(cM[m][l], cmul(cs[m - 1], cconj(sol[l - 1])));
-                cM[m][0] = csub(cM[m][0], cmul(cconj(y0), cs[m - 1]));
-                cy0 = csub(cy0, cmul(cconj(M[m][0]), cs[m - 1]));
-                crh[m] = cs[m - 1];
+            __syncwarp();
+            warp_dense_solve(As, k, sol, 1, fs, lane);     // full forward solution (components m > n are not stored)
+            __syncwarp();
+            warp_dense_solve(AHs, k, cs, 1, fs, lane);     // cotangent of the right-hand side
+            __syncwarp();
+            for (int p = lane; p < k * (k + 1); p += 32) {
+                const int m = 1 + p / (k + 1), l = p % (k + 1);
+                cM[m][l] = csub(cM[m][l], l == 0 ? cmul(cconj(y0), cs[m - 1]) : cmul(cs[m - 1], cconj(sol[l - 1])));
+                if (l == 0) crh[m] = cs[m - 1];
             }
-            ctv(n, 0) = csub(ctv(n, 0), cconj(cy0));
-            // ret / les parts of the sources' transpose (j <= k)
+            __syncwarp();
+            if (lane == 0) {
+                cplx cy0 = cles(0, n);
+                for (int m = 1; m <= k; ++m) cy0 = csub(cy0, cmul(cconj(M[m][0]), crh[m]));
+                ctv(n, 0) = csub(ctv(n, 0), cconj(cy0));
+            }
+            // ret / les parts of the sources' transpose (j <= k): a row m at a time, whose targets differ
             for (int m = 1; m <= k; ++m) {
                 const cplx cc2 = cmuli(cscal(h, crh[m]));
-                for (int j = 0; j <= k; ++j) {
+                for (int j = lane; j <= k; j += 32) {
                     Ples(m, j, cmul(cscal(W.greg[n][j], GRx(n, j)), cc2));
                     const cplx v = cmul(cscal(W.greg[n][j], SL(m, j)), cconj(cc2));
                     if (j <= n) cret(n, j) = cadd(cret(n, j), v);
                     else cret(j, n) = csub(cret(j, n), cconj(v));
                 }
+                __syncwarp();
             }
         }
         __syncthreads();
@@ -875,25 +899,21 @@ __global__ void __launch_bounds__(NG_BOOT_THREADS) k_adj_start(AdjBoot b) {
         __syncthreads();
     }
     // ---- left-mixing rows 1..k: M[1:,1:] y(m) = q_tv(m) - M[:,0] y_0(m), y_0 = i xi G^M(T-m) ----
-    if (t == 0) {
-        cplx AH[NG_KMAX * NG_KMAX];
-        for (int r = 1; r <= k; ++r)
-            for (int l = 1; l <= k; ++l) AH[(l - 1) * k + (r - 1)] = cconj(M[r][l]);
-        for (int r = 0; r < k; ++r)
-            for (int m = 0; m <= T; ++m) rt[(int64_t)r * (T + 1) + m] = ctv(r + 1, m);
-        dense_solve(AH, k, rt, T + 1);
-    }
+    for (int e = t; e < k * (T + 1); e += blockDim.x) rt[e] = ctv(1 + e / (T + 1), e % (T + 1));
+    for (int p = t; p < k * k; p += blockDim.x) AHs[(p % k) * k + p / k] = cconj(M[1 + p / k][1 + p % k]);
     __syncthreads();
-    for (int r = 1; r <= k; ++r)
-        for (int l = 0; l <= k; ++l) {
-            cplx p = cz();
-            for (int m = t; m <= T; m += blockDim.x) {
-                const cplx y = (l == 0) ? cmuli(cscal(xi, GM(T - m))) : GT(l, m);
-                p = csub(p, cmul(cconj(y), rt[(int64_t)(r - 1) * (T + 1) + m]));
-            }
-            p = block_csum(p, red);
-            if (t == 0) cM[r][l] = cadd(cM[r][l], p);
+    if (wid == 0) warp_dense_solve(AHs, k, rt, T + 1, fs, lane);
+    __syncthreads();
+    for (int q = wid; q < k * (k + 1); q += nwp) {   // a warp per element of the start matrix
+        const int r = 1 + q / (k + 1), l = q % (k + 1);
+        cplx p = cz();
+        for (int m = lane; m <= T; m += 32) {
+            const cplx y = (l == 0) ? cmuli(cscal(xi, GM(T - m))) : GT(l, m);
+            p = csub(p, cmul(cconj(y), rt[(int64_t)(r - 1) * (T + 1) + m]));
         }
+        p = warp_sum(p);
+        if (lane == 0) cM[r][l] = cadd(cM[r][l], p);
+    }
     // Matsubara source q_tv = -i htau (C2 + C3) transposed, rows 1..k
     for (int64_t e = t; e < (int64_t)k * (T + 1); e += blockDim.x) {
         const int n = 1 + (int)(e / (T + 1)), p = (int)(e % (T + 1));
@@ -918,46 +938,45 @@ __global__ void __launch_bounds__(NG_BOOT_THREADS) k_adj_start(AdjBoot b) {
         Ptv(n, p) = cadd(Ptv(n, p), acc);
     }
     __syncthreads();
-    if (t != 0) return;
-    // start matrix cotangent -> Sigma~^R(n,l) and eps_n
+    if (wid != 0) return;
+    // start matrix cotangent -> Sigma~^R(n,l) and eps_n; one row n at a time, whose targets differ
     for (int n = 1; n <= k; ++n) {
-        for (int l = 0; l <= k; ++l) Pret(n, l, cmulmi(cscal(h * W.greg[n][l], cM[n][l])));
-        cmf(n) = cadd(cmf(n), cmulmi(cM[n][n]));
+        for (int l = lane; l <= k; l += 32) {
+            Pret(n, l, cmulmi(cscal(h * W.greg[n][l], cM[n][l])));
+            if (l == n) cmf(n) = cadd(cmf(n), cmulmi(cM[n][n]));
+        }
+        __syncwarp();
     }
     // ---- retarded columns m = k-1..0: Mf[n][l] y_l = 0 (n = m+1..k), y_m = -i,
     //      y_l = -conj(G^R(m,l)) for l < m; Mf = i D/h - h I_{m,n;l} Sigma~^R(n,l) - delta (eps_n - mu)
+    cplx(&Mf)[NG_KMAX + 1][NG_KMAX + 1] = M;   // the start matrix is done with
     for (int m = k - 1; m >= 0; --m) {
         const int N = k - m;
-        cplx y[NG_KMAX + 1], Mf[NG_KMAX + 1][NG_KMAX + 1], AH[NG_KMAX * NG_KMAX], cb[NG_KMAX], cyl[NG_KMAX + 1];
-        for (int l = 0; l < m; ++l) y[l] = cneg(cconj(GR(m, l)));
-        y[m] = make_double2(0.0, -1.0);
-        for (int l = m + 1; l <= k; ++l) y[l] = GR(l, m);
-        for (int n = m + 1; n <= k; ++n)
-            for (int l = 0; l <= k; ++l) {
-                cplx v = csub(cmuli(cr(W.D[n][l] / h)), cscal(h * W.I[m][n][l], SRx(n, l)));
-                if (l == n) v = csub(v, EPS(n));
-                Mf[n][l] = v;
-            }
-        for (int n = m + 1; n <= k; ++n) {
-            for (int l = m + 1; l <= k; ++l) AH[(l - m - 1) * N + (n - m - 1)] = cconj(Mf[n][l]);
-            cb[n - m - 1] = cret(n, m);
+        for (int p = lane; p < N * (k + 1); p += 32) {
+            const int n = m + 1 + p / (k + 1), l = p % (k + 1);
+            cplx v = csub(cmuli(cr(W.D[n][l] / h)), cscal(h * W.I[m][n][l], SRx(n, l)));
+            if (l == n) v = csub(v, EPS(n));
+            Mf[n][l] = v;
+            if (l > m) AHs[(l - m - 1) * N + (n - m - 1)] = cconj(v);
+            if (l == 0) cs[n - m - 1] = cret(n, m);
         }
-        dense_solve(AH, N, cb, 1);
-        for (int l = 0; l <= k; ++l) cyl[l] = cz();
-        for (int n = m + 1; n <= k; ++n) {
-            const cplx crn = cb[n - m - 1];
-            for (int l = 0; l <= k; ++l) {
-                cplx cMf;
-                if (l > m) cMf = cneg(cmul(crn, cconj(y[l])));
-                else {
-                    cMf = cneg(cmul(cconj(y[l]), crn));
-                    cyl[l] = csub(cyl[l], cmul(cconj(Mf[n][l]), crn));
-                }
+        __syncwarp();
+        warp_dense_solve(AHs, N, cs, 1, fs, lane);
+        __syncwarp();
+        if (lane <= k) {   // lane l: its column of every row n
+            const int l = lane;
+            const cplx y = l < m ? cneg(cconj(GR(m, l))) : (l == m ? make_double2(0.0, -1.0) : GR(l, m));
+            cplx cyl = cz();
+            for (int n = m + 1; n <= k; ++n) {
+                const cplx crn = cs[n - m - 1], cMf = cneg(cmul(crn, cconj(y)));
+                if (l <= m) cyl = csub(cyl, cmul(cconj(Mf[n][l]), crn));
                 Pret(n, l, cscal(-h * W.I[m][n][l], cMf));
                 if (l == n) cmf(n) = csub(cmf(n), cMf);
+                __syncwarp((1u << (k + 1)) - 1);   // rows one after the other: (n, l) and (l, n) share a target
             }
+            if (l < m) cret(m, l) = csub(cret(m, l), cconj(cyl));
         }
-        for (int l = 0; l < m; ++l) cret(m, l) = csub(cret(m, l), cconj(cyl[l]));
+        __syncwarp();
     }
 }
 

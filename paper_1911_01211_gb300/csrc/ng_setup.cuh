@@ -305,6 +305,7 @@ __global__ void k_mat_assemble(Grid g, const cplx* ws_g, const cplx* ws_K, cplx*
 // x_r for the W rows of a triangular block, lane (r, column) of one warp; A at the block's first element.
 // Lanes take the (row, right-hand side) pairs in turn; unit lower (FWD) or upper triangle.
 #define NG_LU_TRI 16
+#define NG_LU_STAGE 1024
 template <bool FWD>
 __device__ void lu_tri_block(const cplx* A, int ld, int w, cplx* B, int ldb, int nrhs, int lane) {
     const int r = lane & (NG_LU_TRI - 1);
@@ -338,13 +339,18 @@ __device__ __forceinline__ void lu_update_rows(const cplx* A, int ld, int c0, in
 }
 
 // Forward (FWD, unit lower) or backward (upper) substitution of B in blocks of NG_LU_TRI rows: a warp solves
-// the triangle, all threads subtract its columns from the other rows.  xs: NG_LU_TRI * nrhs values.
+// the triangle (staged in shared memory), all threads subtract its columns from the other rows.
+// xs: NG_LU_TRI * nrhs values.
 template <bool FWD>
 __device__ void lu_substitute(const cplx* A, int ld, int N, cplx* B, int ldb, int nrhs, cplx* xs) {
+    __shared__ cplx tri_s[NG_LU_TRI * NG_LU_TRI];
     const int nblk = (N + NG_LU_TRI - 1) / NG_LU_TRI;
     for (int q = 0; q < nblk; ++q) {
         const int c0 = (FWD ? q : nblk - 1 - q) * NG_LU_TRI, w = min(NG_LU_TRI, N - c0);
-        if (threadIdx.x < 32) lu_tri_block<FWD>(A + (int64_t)c0 * ld + c0, ld, w, B + (int64_t)c0 * ldb, ldb, nrhs, threadIdx.x);
+        for (int i = threadIdx.x; i < w * w; i += blockDim.x)
+            tri_s[(i / w) * NG_LU_TRI + i % w] = A[(int64_t)(c0 + i / w) * ld + c0 + i % w];
+        __syncthreads();
+        if (threadIdx.x < 32) lu_tri_block<FWD>(tri_s, NG_LU_TRI, w, B + (int64_t)c0 * ldb, ldb, nrhs, threadIdx.x);
         __syncthreads();
         for (int i = threadIdx.x; i < w * nrhs; i += blockDim.x) xs[i] = B[(int64_t)(c0 + i / nrhs) * ldb + i % nrhs];
         __syncthreads();
@@ -581,19 +587,28 @@ __global__ void __launch_bounds__(NG_LU_THREADS) k_lu_resolve(Grid g, int N, int
     const int* p = piv + (int64_t)blockIdx.x * N;
     cplx* r = ws_r + (int64_t)blockIdx.x * N * nrhs;
     const int t = threadIdx.x, nt = blockDim.x;
-    __shared__ cplx xs[NG_LU_TRI * 8];
+    __shared__ cplx xs[NG_LU_TRI * 8], rs[NG_LU_STAGE];
+    __shared__ int ps[NG_LU_STAGE];
+    const bool staged = N * nrhs <= NG_LU_STAGE;   // right-hand sides and interchanges fit shared memory
+    if (staged) {
+        for (int i = t; i < N * nrhs; i += nt) rs[i] = r[i];
+        for (int i = t; i < N; i += nt) ps[i] = p[i];
+    }
+    __syncthreads();
+    cplx* x_ = staged ? rs : r;
+    const int* p_ = staged ? ps : p;
     if (t < nrhs)   // row interchanges in factorisation order
         for (int c = 0; c < N; ++c) {
-            const int q = p[c];
-            if (q != c) { cplx x = r[c * nrhs + t]; r[c * nrhs + t] = r[q * nrhs + t]; r[q * nrhs + t] = x; }
+            const int q = p_[c];
+            if (q != c) { cplx x = x_[c * nrhs + t]; x_[c * nrhs + t] = x_[q * nrhs + t]; x_[q * nrhs + t] = x; }
         }
     __syncthreads();
-    lu_substitute<true>(A, ld, N, r, nrhs, nrhs, xs);
-    lu_substitute<false>(A, ld, N, r, nrhs, nrhs, xs);
+    lu_substitute<true>(A, ld, N, x_, nrhs, nrhs, xs);
+    lu_substitute<false>(A, ld, N, x_, nrhs, nrhs, xs);
     double s = 0.0;
     for (int64_t q = t; q < (int64_t)N * nrhs; q += nt) {
         const int64_t off = mat_offset(G.mat, nrhs, (int)(q / nrhs), (int)(q % nrhs), blockIdx.x);
-        const cplx x = r[q];
+        const cplx x = x_[q];
         G.mat.p[off] = cadd(G.mat.p[off], x);
         s += sqrt(cabs2(x));
     }
