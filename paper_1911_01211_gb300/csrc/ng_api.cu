@@ -14,6 +14,7 @@
 #include "ng_stepq.cuh"
 #include "ng_obs.cuh"
 #include "ng_ubatch.cuh"
+#include "ng_histu.cuh"
 #include "ng_stepdf.cuh"
 #include "ng_conv_launch.h"
 #include "ng_tvfft.h"
@@ -959,7 +960,50 @@ ng_status do_hartree(ng_ctx* c, const Grid& g, int tstp, const FuncV& mf, const 
 // ---------------------------------------------------------------------------------------
 struct UHost {
     int D, nt, ntau, k;
+    bool alone;   // stored for itself, not interleaved with other problems (ldk = 1)
 };
+
+// The history sums of problems active[c0..c1) as digit products (ng_histu.cuh); *ok = false without room for the
+// workspace: the step keeps k_ubulk
+ng_status histu_sums(ng_ctx* c, const UProb* d_probs, const std::vector<UHost>& info, const std::vector<int>& active,
+                     size_t c0, size_t c1, int n, HistUTab* tab, bool* ok, cudaStream_t s) {
+    *ok = false;
+    memset(tab, 0, sizeof(*tab));
+    HistUGeo q;
+    const size_t head = (sizeof(HistUProb) * (c1 - c0) + 255) / 256 * 256;
+    size_t need = head, off = head;
+    int lenp = 0;
+    for (size_t i = c0; i < c1; ++i) {   // room for the last step, so that the workspace does not grow on the way
+        const UHost& u = info[active[i]];
+        histu_geo(u.D, u.ntau, u.nt, q);
+        need += q.bytes;
+        const int j = (int)(i - c0);
+        histu_geo(u.D, u.ntau, n, q);
+        tab->prob[j] = active[i];
+        tab->off[j] = (int64_t)off;
+        tab->start[j] = tab->ntask;
+        tab->ntask += q.task0[NGU_SETS];
+        off += q.bytes;
+        lenp = std::max(lenp, q.lenp);
+    }
+    tab->np = (int)(c1 - c0);
+    tab->start[tab->np] = tab->ntask;
+    if (c->ws_hist_bytes < need && ensure(c, &c->ws_hist, &c->ws_hist_bytes, need)) return NG_OK;   // no room
+    tab->probs = (HistUProb*)c->ws_hist;
+    tab->base = (char*)c->ws_hist;
+    tab->src = d_probs;
+    tab->n = n;
+    tab->status = c->d_status;
+    k_histu_vec<<<dim3(lenp / 128, tab->np, 8 * (NGU_NVEC + 1)), 128, 0, s>>>(*tab);
+    ng_status st = check_launch(c, "k_histu_vec");
+    if (st) return st;
+    if (histu_launch(*tab, c->sms, s) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(c, NG_ECUDA, "launch of k_histu_mma failed");
+    }
+    *ok = true;
+    return NG_OK;
+}
 ng_status ustep(ng_ctx* c, const UProb* d_probs, const std::vector<UHost>& info, const std::vector<int>& active, int n,
                 int threads, cudaStream_t s) {
     ng_status st;
@@ -986,11 +1030,10 @@ ng_status ustep(ng_ctx* c, const UProb* d_probs, const std::vector<UHost>& info,
         }
         tab.np = (int)(c1 - c0);
         tab.start[tab.np] = blk;
-        // chunks of the (A) rows' source sums: max(n, k) + 1 + ntau + 1 summation indices
-        int nsum = 0;
-        for (size_t i = c0; i < c1; ++i) nsum = std::max(nsum, std::max(n, info[active[i]].k) + 2 + info[active[i]].ntau);
-        tab.chunk = 128;
-        tab.nchunk = (nsum + tab.chunk - 1) / tab.chunk;
+        for (size_t i = c0; i < c1; ++i) {
+            const UHost& u = info[active[i]];
+            tab.nchunk = std::max(tab.nchunk, usrc_chunks(u.D, u.k, u.ntau, n));
+        }
         {   // capacity for twice the current need, so the buffer grows a logarithmic number of times
             const size_t per = sizeof(cplx) * (size_t)NG_MAXQ * 2 * NG_UMAXD * NG_UMAXD;
             const size_t need = per * (size_t)tab.np * tab.nchunk;
@@ -1001,8 +1044,20 @@ ng_status ustep(ng_ctx* c, const UProb* d_probs, const std::vector<UHost>& info,
         if ((st = check_launch(c, "k_uminv"))) return st;
         long e0 = prof_pair(c, 0);
         if (e0 >= 0) cudaEventRecord(c->ev_pool[e0], s);
-        k_ubulk<<<blk, threads, sizeof(cplx) * threads, s>>>(d_probs, tab, c->d_status);
-        if ((st = check_launch(c, "k_ubulk"))) return st;
+        // Digit products (ng_histu.cu) wherever the formulas of a step inside the history hold: their three launches
+        // are the faster ones from the first steps on.  Whole steps in us, k_ubulk / digit products: problems of 1, 2,
+        // 4, 8 orbitals, n = 40, ntau = 50: 613 / 555, n = 200, ntau = 100: 1402 / 738; one of 2 orbitals, n = 100,
+        // ntau = 100: 225 / 190; four of 8, n = 500, ntau = 300: 14.7 / 3.5 ms.  Interleaved problems keep k_ubulk.
+        bool digits = c->bulk_split == NG_BULK_AUTO;
+        for (size_t i = c0; i < c1; ++i) {
+            const UHost& u = info[active[i]];
+            digits = digits && u.alone && n >= 2 * u.k + 2;
+        }
+        HistUTab ht;
+        if (digits && (st = histu_sums(c, d_probs, info, active, c0, c1, n, &ht, &digits, s))) return st;
+        if (digits) k_histu_close<<<blk, threads, sizeof(cplx) * threads, s>>>(ht.probs, tab, c->d_status);
+        else k_ubulk<<<blk, threads, sizeof(cplx) * threads, s>>>(d_probs, tab, c->d_status);
+        if ((st = check_launch(c, digits ? "k_histu_close" : "k_ubulk"))) return st;
         if (e0 >= 0) cudaEventRecord(c->ev_pool[e0 + 1], s);
         long e1 = prof_pair(c, 1);
         if (e1 >= 0) cudaEventRecord(c->ev_pool[e1], s);
@@ -1054,7 +1109,7 @@ ng_status utimestep_uniform(ng_ctx* c, const Grid& g, int n, const HermV& G, con
         c->uni_key_S = S.ret.p;
         c->uni_key_eps = eps.p;
     }
-    std::vector<UHost> info(g.nb, UHost{g.nf, g.nt, g.ntau, g.k});
+    std::vector<UHost> info(g.nb, UHost{g.nf, g.nt, g.ntau, g.k, g.nb == 1});
     std::vector<int> active(g.nb);
     for (int kb = 0; kb < g.nb; ++kb) active[kb] = kb;
     return ustep(c, d_probs, info, active, n, 128, s);
@@ -2219,7 +2274,7 @@ ng_status ng_batch_create(ng_ctx* c, int nprob, const ng_grid* grids, const ng_h
         b->G.push_back(Gv);
         b->S.push_back(Sv);
         b->eps.push_back(ev);
-        b->info.push_back(UHost{g.nf, g.nt, g.ntau, g.k});
+        b->info.push_back(UHost{g.nf, g.nt, g.ntau, g.k, true});
         h[p].g = g;
         h[p].G = Gv;
         h[p].S = Sv;

@@ -45,6 +45,28 @@ __device__ __forceinline__ uint64_t hist_fixed(double x, int F) {
     return ((b << 11) | 0x8000000000000000ull) >> s;
 }
 
+// Digits of element i (8 half + 2t + {0,1}) of its block of 16 on the scale F (2047: a non-finite vector, zeros),
+// balanced: -128..127, the leading one up to 128; layout of NGH_DIG_B
+__device__ __forceinline__ void hist_digits(cplx x, int F, bool conj, int i, __half (&dig)[2][8][4][2][2][2]) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const double v = c ? x.y : x.x;
+        const bool neg = v < 0.0;
+        const uint64_t M = F == 2047 ? 0 : hist_fixed(v, F) >> 1;
+        int carry = 0;
+#pragma unroll
+        for (int d = 7; d >= 0; --d) {
+            int b = (int)(M >> (56 - 8 * d) & 255) + carry;
+            carry = 0;
+            if (b >= 128 && d > 0) { b -= 256; carry = 1; }
+            const __half q = __int2half_rn(neg ? -b : b), m = __int2half_rn(neg ? b : -b);
+            auto at = [&](int part, int f) -> __half& { return dig[part][d][(i & 7) >> 1][i >> 3][f][i & 1]; };
+            if (c == 0) at(0, 0) = at(1, 1) = q;
+            else { at(1, 0) = conj ? m : q; at(0, 1) = conj ? q : m; }
+        }
+    }
+}
+
 // FP64 values, scale and digits of the row vectors.  A block takes 128 elements of one vector and of
 // KK problems (KK = 1: vectors shared by all problems); it finds the vector's largest exponent by
 // itself (a vector is a few 10 KB in L2, a second launch would cost more).
@@ -75,25 +97,7 @@ static __global__ void __launch_bounds__(256) k_hist_vec(HistWs w, HistRow S) {
         if (el < PE) {
             const cplx x = hist_vec_value(W, S, w.n, w.T, vec, j, kvc);
             if (kv < w.nv) w.vec[((int64_t)vec * w.nv + kv) * w.lenp + j] = x;
-            const int i = j & 15;   // element 8 half + 2t + {0,1} of its block of 16
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const double v = c ? x.y : x.x;
-                const bool neg = v < 0.0;
-                const uint64_t M = F == 2047 ? 0 : hist_fixed(v, F) >> 1;
-                int carry = 0;
-#pragma unroll
-                for (int d = 7; d >= 0; --d) {
-                    int b = (int)(M >> (56 - 8 * d) & 255) + carry;
-                    carry = 0;
-                    if (b >= 128 && d > 0) { b -= 256; carry = 1; }
-                    // the left-mixing row vector enters conjugated
-                    const __half q = __int2half_rn(neg ? -b : b), m = __int2half_rn(neg ? b : -b);
-                    auto at = [&](int part, int f) -> __half& { return dig[kk][el / 16][part][d][(i & 7) >> 1][i >> 3][f][i & 1]; };
-                    if (c == 0) at(0, 0) = at(1, 1) = q;
-                    else { at(1, 0) = vec == 3 ? m : q; at(0, 1) = vec == 3 ? q : m; }
-                }
-            }
+            hist_digits(x, F, vec == 3, j & 15, dig[kk][el / 16]);   // the left-mixing row vector enters conjugated
         }
         __syncthreads();
         constexpr int NU = KK * (PE / 16) * 64;   // uint4 of the pass

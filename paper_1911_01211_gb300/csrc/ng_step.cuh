@@ -316,36 +316,40 @@ __device__ inline int dense_solve(cplx* A, int N, cplx* B, int nrhs) {
         for (int r = c + 1; r < N; ++r) {
             cplx f = cmul(A[r * N + c], inv);
             if (f.x == 0.0 && f.y == 0.0) continue;
-            for (int j = c; j < N; ++j) A[r * N + j] = csub(A[r * N + j], cmul(f, A[c * N + j]));
-            for (int j = 0; j < nrhs; ++j) B[r * nrhs + j] = csub(B[r * nrhs + j], cmul(f, B[c * nrhs + j]));
+            for (int j = c; j < N; ++j) A[r * N + j] = cfma(cneg(f), A[c * N + j], A[r * N + j]);
+            for (int j = 0; j < nrhs; ++j) B[r * nrhs + j] = cfma(cneg(f), B[c * nrhs + j], B[r * nrhs + j]);
         }
     }
     for (int c = N - 1; c >= 0; --c) {
         cplx inv = cinv(A[c * N + c]);
         for (int j = 0; j < nrhs; ++j) {
             cplx s = B[c * nrhs + j];
-            for (int q = c + 1; q < N; ++q) s = csub(s, cmul(A[c * N + q], B[q * nrhs + j]));
+            for (int q = c + 1; q < N; ++q) s = cfma(cneg(A[c * N + q]), B[q * nrhs + j], s);
             B[c * nrhs + j] = cmul(s, inv);
         }
     }
     return 0;
 }
 
-// The same elimination by the 32 lanes of one warp (every lane calls it; A, B and the scratch
-// f[N] visible to the warp).  Per column the pivot is the first row of largest |A[r][c]|^2, as in
-// dense_solve; the lanes swap the rows, form the factors of the rows below once and update the
-// trailing elements, each element receiving the operations of dense_solve in the same order, so
-// the reduced system is bitwise that of dense_solve.  The back substitution runs column by
+// The same elimination by NT threads, one warp or a whole block (all call it; A, B and the scratch
+// f[N] visible to them).  Per column the pivot is the first row of largest |A[r][c]|^2, as in
+// dense_solve (every warp finds it for itself); the threads swap the rows, form the factors of the
+// rows below once and update the trailing elements, each element receiving the operations of
+// dense_solve in the same order, so the reduced system is bitwise that of dense_solve.  The back substitution runs column by
 // column (x_c = B[c] / A[c][c], then B[r] -= A[r][c] x_c for the rows r < c in parallel).
-// Returns 1 on every lane when a pivot vanishes.  FP64 on this part is issued per warp
-// instruction whatever the number of active lanes, so the lanes cost nothing over one thread.
-__device__ inline int warp_dense_solve(cplx* A, int N, cplx* B, int nrhs, cplx* f, int lane) {
+// Returns 1 on every thread when a pivot vanishes.  FP64 on this part is issued per warp
+// instruction whatever the number of active lanes, so the lanes cost nothing over one thread, and
+// each quarter of an SM has its own pipe: the start-up of 8 orbitals (40 x 40, 8 right-hand sides,
+// k_uboundary_ret) takes 600 us on one warp and 198 us on four.
+template <int NT>
+__device__ inline int group_dense_solve(cplx* A, int N, cplx* B, int nrhs, cplx* f, int t) {
     const unsigned full = 0xffffffffu;
+    auto sync = [] { if (NT == 32) __syncwarp(); else __syncthreads(); };
     for (int c = 0; c < N; ++c) {
         // squares of magnitudes compare as their bits, without the FP64 pipe
         long long best = -1;
         int p = N;
-        for (int r = c + lane; r < N; r += 32) {
+        for (int r = c + (t & 31); r < N; r += 32) {
             const long long v = __double_as_longlong(cabs2(A[r * N + c]));
             if (v > best) { best = v; p = r; }
         }
@@ -356,40 +360,44 @@ __device__ inline int warp_dense_solve(cplx* A, int N, cplx* B, int nrhs, cplx* 
             if (bo > best || (bo == best && po < p)) { best = bo; p = po; }
         }
         if (best == 0) return 1;
+        if (NT > 32) __syncthreads();   // every warp has read the column
         if (p != c) {
-            for (int j = lane; j < N; j += 32) {
+            for (int j = t; j < N; j += NT) {
                 const cplx t = A[c * N + j]; A[c * N + j] = A[p * N + j]; A[p * N + j] = t;
             }
-            for (int j = lane; j < nrhs; j += 32) {
+            for (int j = t; j < nrhs; j += NT) {
                 const cplx t = B[c * nrhs + j]; B[c * nrhs + j] = B[p * nrhs + j]; B[p * nrhs + j] = t;
             }
         }
-        __syncwarp();
+        sync();
         const cplx inv = cinv(A[c * N + c]);
-        for (int r = c + 1 + lane; r < N; r += 32) f[r] = cmul(A[r * N + c], inv);
-        __syncwarp();
-        if (lane == 0) A[c * N + c] = inv;   // for the back substitution (the factors in f are taken)
+        for (int r = c + 1 + t; r < N; r += NT) f[r] = cmul(A[r * N + c], inv);
+        sync();
+        if (t == 0) A[c * N + c] = inv;   // for the back substitution (the factors in f are taken)
         const int wa = N - c - 1, w = wa + nrhs, cnt = (N - c - 1) * w;
-        for (int e = lane; e < cnt; e += 32) {
+        for (int e = t; e < cnt; e += NT) {
             const int r = c + 1 + e / w, j = e % w;
             const cplx fr = f[r];
             if (fr.x == 0.0 && fr.y == 0.0) continue;
-            if (j < wa) A[r * N + c + 1 + j] = csub(A[r * N + c + 1 + j], cmul(fr, A[c * N + c + 1 + j]));
-            else B[r * nrhs + j - wa] = csub(B[r * nrhs + j - wa], cmul(fr, B[c * nrhs + j - wa]));
+            if (j < wa) A[r * N + c + 1 + j] = cfma(cneg(fr), A[c * N + c + 1 + j], A[r * N + c + 1 + j]);
+            else B[r * nrhs + j - wa] = cfma(cneg(fr), B[c * nrhs + j - wa], B[r * nrhs + j - wa]);
         }
-        __syncwarp();
+        sync();
     }
     for (int c = N - 1; c >= 0; --c) {
         const cplx inv = A[c * N + c];
-        for (int j = lane; j < nrhs; j += 32) B[c * nrhs + j] = cmul(B[c * nrhs + j], inv);
-        __syncwarp();
-        for (int e = lane; e < c * nrhs; e += 32) {
+        for (int j = t; j < nrhs; j += NT) B[c * nrhs + j] = cmul(B[c * nrhs + j], inv);
+        sync();
+        for (int e = t; e < c * nrhs; e += NT) {
             const int r = e / nrhs, j = e % nrhs;
-            B[r * nrhs + j] = csub(B[r * nrhs + j], cmul(A[r * N + c], B[c * nrhs + j]));
+            B[r * nrhs + j] = cfma(cneg(A[r * N + c]), B[c * nrhs + j], B[r * nrhs + j]);
         }
-        __syncwarp();
+        sync();
     }
     return 0;
+}
+__device__ inline int warp_dense_solve(cplx* A, int N, cplx* B, int nrhs, cplx* f, int lane) {
+    return group_dense_solve<32>(A, N, B, nrhs, f, lane);
 }
 
 // block-wide sum of a Mat<D> in a fixed order (deterministic); result valid in thread 0

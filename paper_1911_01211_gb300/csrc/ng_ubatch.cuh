@@ -6,9 +6,9 @@
 // Sec. "Time stepping", mixed schedule).
 #pragma once
 
+#include "ng_histu.h"
 #include "ng_step.cuh"
 
-#define NG_UMAXP 128    // problems per batch
 #define NG_UMAXD 8
 
 struct UProb {
@@ -28,11 +28,19 @@ struct UTable {
     int prob[NG_UMAXP];
     int nles[NG_UMAXP], ntv[NG_UMAXP];
     // partial sums of the (A) rows' sources and histories: src[((i * NG_MAXQ + r) * nchunk +
-    // c) * 2 + {0: source, 1: history}][a * D + b], chunks of `chunk` summation indices
+    // c) * 2 + {0: source, 1: history}][a * D + b], chunks of usrc_chunk(D) summation indices
     cplx* src;
-    int nchunk, chunk;
+    int nchunk;
 };
 #define NG_USRC_THREADS 256
+// Chunks of equal work for D >= 2 (an index costs D^3 multiply-adds, a block takes 256 / D^2 at a time), short
+// enough that the few problems of 8 orbitals spread over the GPU: 16 clusters, n = 500, ntau = 300: k_usrc 340 us with
+// chunks of 128 for every D, 125 us so
+__host__ __device__ __forceinline__ int usrc_chunk(int D) { return 256 / D; }
+__host__ __device__ __forceinline__ int usrc_chunks(int D, int k, int T, int n) {   // max(n, k) + 1 + T + 1 indices
+    const int c = usrc_chunk(D);
+    return ((n > k ? n : k) + 2 + T + c - 1) / c;
+}
 
 // element (a,b) of a stored d x d block
 __device__ __forceinline__ cplx uel(const Comp& c, int64_t e, int D, int a, int b, int kb) {
@@ -255,18 +263,18 @@ __device__ cplx u_qlesA_range(const NgWeights& W, const Grid& g, const HermV& G,
     const int k = W.k, T = g.ntau, T1 = g.ntau + 1;
     cplx c2 = cz(), c3 = cz();
     const int jmax = n <= k ? k : n;
-    for (int i = i0; i < i1; i += is) {
+    for (int i = i0; i < i1; i += is) {   // the weight once per index, not per c: a third of the arithmetic
+        cplx x = cz();
         if (i <= jmax) {
             const int j = i;
-            const double w = n <= k ? W.greg[n][j] : gw(W, n, j);
             for (int c = 0; c < D; ++c)   // Sigma^<(m,j) G^A(j,n), G^A(j,n)_cb = conj(G~^R(n,j)_bc)
-                c2 = cfma(cscal(w, ules(S, m, j, D, a, c, kb)), cconj(uretx(G, n, j, D, b, c, kb)), c2);
+                x = cfma(ules(S, m, j, D, a, c, kb), cconj(uretx(G, n, j, D, b, c, kb)), x);
+            c2 = cadd(c2, cscal(n <= k ? W.greg[n][j] : gw(W, n, j), x));
         } else {
             const int j = i - jmax - 1;
-            const double w = gw(W, T, j);
             for (int c = 0; c < D; ++c)   // Sigma^tv(m,j) [G^tv(n,T-j)]^dagger
-                c3 = cfma(cscal(w, uel(S.tv, (int64_t)m * T1 + j, D, a, c, kb)),
-                          cconj(uel(G.tv, (int64_t)n * T1 + T - j, D, b, c, kb)), c3);
+                x = cfma(uel(S.tv, (int64_t)m * T1 + j, D, a, c, kb), cconj(uel(G.tv, (int64_t)n * T1 + T - j, D, b, c, kb)), x);
+            c3 = cadd(c3, cscal(gw(W, T, j), x));
         }
     }
     return cadd(cscal(g.h, cmulmi(c2)), cscal((double)g.sig * g.htau, c3));
@@ -288,8 +296,8 @@ __device__ void u_stepmat(const NgWeights& W, const UProb& P, int m, cplx* out) 
 // The boundary of step n runs in three launches: k_uboundary_ret (retarded (A) start-up along
 // row n and G^<(0,n), one block per problem), k_usrc (sources and partial histories of the
 // lesser (A) rows, O((k+1)(n + ntau) nf^3) per problem, over many blocks), k_uboundary_les (the
-// serial lesser (A) steps, one block per problem).  The dense solves run on one warp
-// (warp_dense_solve) and the step matrices of the serial rows are inverted by the block's warps
+// serial lesser (A) steps, one block per problem).  The dense solves run on the
+// block's four warps (group_dense_solve) and the step matrices of the serial rows are inverted by the block's warps
 // before the serial chain, whose steps are then element-parallel products: FP64 is issued per
 // warp instruction on this part, so one thread doing them alone took as long as a whole warp.
 __global__ void __launch_bounds__(NG_UBND_THREADS) k_uboundary_ret(const UProb* probs, UTable tab, int* status) {
@@ -326,7 +334,7 @@ __global__ void __launch_bounds__(NG_UBND_THREADS) k_uboundary_ret(const UProb* 
         B[((j - 1) * D + a) * D + c] = cmuli(v);
     }
     __syncthreads();
-    if (t < 32 && warp_dense_solve(A, N, B, D, B + (NG_KMAX * NG_UMAXD) * NG_UMAXD, t) && t == 0)
+    if (group_dense_solve<NG_UBND_THREADS>(A, N, B, D, B + (NG_KMAX * NG_UMAXD) * NG_UMAXD, t) && t == 0)
         atomicOr(status, NGF_SINGULAR);
     __syncthreads();
     for (int q = t; q < (k + 1) * DD; q += blockDim.x) {
@@ -354,21 +362,22 @@ __global__ void __launch_bounds__(NG_USRC_THREADS) k_usrc(const UProb* probs, UT
     const bool full = (n <= 2 * k);
     const int m0 = full ? 1 : n - k;
     const int nq = n - m0 + 1;
-    if (r >= nq) return;
+    if (r >= nq || ch >= usrc_chunks(D, k, g.ntau, n)) return;
     const int m = m0 + r;
     const int jmax = n <= k ? k : n;
     const int nsum = jmax + 1 + g.ntau + 1;
-    const int i0 = ch * tab.chunk, i1 = min(nsum, i0 + tab.chunk);
+    const int i0 = ch * usrc_chunk(D), i1 = min(nsum, i0 + usrc_chunk(D));
     const int ngrp = NG_USRC_THREADS / DD, grp = t / DD, ab = t % DD, a = ab / D, b = ab % D;
     __shared__ cplx red[2][NG_USRC_THREADS];
     cplx qv = cz(), hv = cz();
     if (grp < ngrp && i0 < i1) {
         qv = u_qlesA_range(W, g, P.G, P.S, m, n, D, a, b, kb, i0 + grp, i1, ngrp);
         if (!full && m > k)
-            for (int l = i0 + grp; l < min(i1, m0); l += ngrp)
-                for (int c = 0; c < D; ++c)
-                    hv = cfma(cscal(gw(W, m, l), uel(P.S.ret, tri(m) + l, D, a, c, kb)),
-                              uel(P.G.les, tri(n) + l, D, c, b, kb), hv);
+            for (int l = i0 + grp; l < min(i1, m0); l += ngrp) {
+                cplx x = cz();
+                for (int c = 0; c < D; ++c) x = cfma(uel(P.S.ret, tri(m) + l, D, a, c, kb), uel(P.G.les, tri(n) + l, D, c, b, kb), x);
+                hv = cadd(hv, cscal(gw(W, m, l), x));
+            }
     }
     red[0][t] = qv;
     red[1][t] = hv;
@@ -409,7 +418,9 @@ __global__ void __launch_bounds__(NG_UBND_THREADS) k_uboundary_les(const UProb* 
         const int r = q / DD, ab = q % DD;
         const cplx* src = tab.src + ((int64_t)(blockIdx.x * NG_MAXQ + r) * tab.nchunk * 2) * (NG_UMAXD * NG_UMAXD);
         cplx sq = cz(), sh = cz();
-        for (int ch = 0; ch < tab.nchunk; ++ch) {
+        const int nch = usrc_chunks(D, k, g.ntau, n);
+#pragma unroll 4
+        for (int ch = 0; ch < nch; ++ch) {
             sq = cadd(sq, src[(2 * ch) * (NG_UMAXD * NG_UMAXD) + ab]);
             sh = cadd(sh, src[(2 * ch + 1) * (NG_UMAXD * NG_UMAXD) + ab]);
         }
@@ -442,7 +453,7 @@ __global__ void __launch_bounds__(NG_UBND_THREADS) k_uboundary_les(const UProb* 
             B[((m - 1) * D + aa) * D + cc] = acc;
         }
         __syncthreads();
-        if (t < 32 && warp_dense_solve(A, N, B, D, red, t) && t == 0) atomicOr(status, NGF_SINGULAR);
+        if (group_dense_solve<NG_UBND_THREADS>(A, N, B, D, red, t) && t == 0) atomicOr(status, NGF_SINGULAR);
         __syncthreads();
         for (int q = t; q < k * DD; q += blockDim.x) {
             const int m = 1 + q / DD, ab = q % DD, aa = ab / D, cc = ab % D;
