@@ -9,7 +9,7 @@
 //
 // Numbers.  X is taken as sign and a 64-bit fixed-point magnitude on the scale 2^E of the largest
 // element its warp has met in the unit (E grows in steps of 8 bits, so the window never holds less than
-// 56 bits below the largest element), and v as 63 bits on the scale of its largest element:
+// 56 bits below the largest element), and v as 63 bits on the scale of the largest element of its block of 128:
 //   X = +-sum_s d_s 2^(-8(s+1)) 2^(E-1022),  0 <= d_s <= 255,      s = 0..7
 //   v =   sum_t q_t 2^(-8(t+1)) 2^(F-1021),  -128 <= q_t <= 128,   t = 0..7
 // Products of equal weight u = s + t share an accumulator; the B operand for digit s of X holds the
@@ -342,7 +342,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_hist_mma(const Args a, const __g
         const int band = u.type == U_RET ? a.w.k : 0;
         const int cv = u.type == U_RET ? 0 : 1, rv = u.type == U_TV ? 3 : (u.type == U_LES ? 1 : 2);
         const uint4* ctab = a.w.tab + (((int64_t)cv * a.w.nv + kv) * (a.w.lenp / 16) + j0 / 16) * (DIG_B / 16);
-        const int fc = a.w.vexp[cv * a.w.nv + kv], fr = a.w.vexp[rv * a.w.nv + kv];
+        const int nblk = a.w.lenp / NGH_BLK;
+        const int fc = a.w.vexp[(cv * a.w.nv + kv) * nblk + u.bi], fr = a.w.vexp[(rv * a.w.nv + kv) * nblk + u.bj];
         cplx* colp = a.w.part + (u.id * 2) * NGH_BLK * a.w.nb + kb;
         cplx* rowp = colp + (int64_t)NGH_BLK * a.w.nb;
         bool bad = fc < 0 || fr < 0;
@@ -519,7 +520,7 @@ static HistWs layout(char* base, int n_max, int n, int T, int k, int nb, int nv,
     w.tab = (uint4*)(base + o);
     o += up256((size_t)NGH_NVEC * nv * (w.lenp / 16) * DIG_B);
     w.vexp = (int*)(base + o);
-    o += up256(sizeof(int) * (size_t)NGH_NVEC * nv);
+    o += up256(sizeof(int) * (size_t)NGH_NVEC * nv * (w.lenp / NGH_BLK));
     w.part = (cplx*)(base + o);
     w.nbr = pad_blk(n_max) / NGH_BLK;
     o += sizeof(cplx) * (size_t)hist_units(w) * 2 * NGH_BLK * nb;

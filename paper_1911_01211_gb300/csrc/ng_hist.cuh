@@ -67,44 +67,44 @@ __device__ __forceinline__ void hist_digits(cplx x, int F, bool conj, int i, __h
     }
 }
 
-// FP64 values, scale and digits of the row vectors.  A block takes 128 elements of one vector and of
-// KK problems (KK = 1: vectors shared by all problems); it finds the vector's largest exponent by
-// itself (a vector is a few 10 KB in L2, a second launch would cost more).
+// FP64 values, scale and digits of the row vectors.  A block takes 128 elements of one vector, with their own
+// scale, and of KK problems (KK = 1: vectors shared by all problems).
 template <int KK>
 static __global__ void __launch_bounds__(256) k_hist_vec(HistWs w, HistRow S) {
     const NgWeights& W = c_W[w.k - 1];
-    constexpr int NE = 256 / KK;            // elements in flight
-    constexpr int PE = KK == 1 ? NGH_BLK : NE;   // elements of a pass
+    constexpr int PE = KK == 1 ? NGH_BLK : 256 / KK, NP = NGH_BLK / PE;   // elements of a pass, passes
     __shared__ int smax[KK];
     __shared__ __align__(16) __half dig[KK][PE / 16][2][8][4][2][2][2];   // as NGH_DIG_B
     const int vec = blockIdx.z, tid = threadIdx.x, kk = tid % KK, el = tid / KK;
     const int kv = blockIdx.y * KK + kk, kvc = min(kv, w.nv - 1);
-    const int len = vec == 3 ? w.T + 1 : w.n;
-    if ((int)blockIdx.x * NGH_BLK >= (len + NGH_BLK - 1) / NGH_BLK * NGH_BLK) return;
+    const int len = vec == 3 ? w.T + 1 : w.n, j0 = blockIdx.x * NGH_BLK;
+    if (j0 >= len) return;
     if (tid < KK) smax[tid] = 0;
     __syncthreads();
+    cplx x[NP];
     int e = 0;
-    for (int j = el; j < len; j += NE) {
-        const cplx x = hist_vec_value(W, S, w.n, w.T, vec, j, kvc);
-        e = max(e, max(__double2hiint(x.x) >> 20 & 2047, __double2hiint(x.y) >> 20 & 2047));
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        x[p] = el < PE ? hist_vec_value(W, S, w.n, w.T, vec, j0 + p * PE + el, kvc) : cz();
+        e = max(e, max(__double2hiint(x[p].x) >> 20 & 2047, __double2hiint(x[p].y) >> 20 & 2047));
     }
     atomicMax(&smax[kk], e);
     __syncthreads();
     const int F = max(smax[kk], 128);
-    if (el == 0 && kv < w.nv) w.vexp[vec * w.nv + kv] = F == 2047 ? -1 : F;
-    for (int p = 0; p < NGH_BLK; p += PE) {
-        const int j = blockIdx.x * NGH_BLK + p + el;
+    if (el == 0 && kv < w.nv) w.vexp[(vec * w.nv + kv) * (w.lenp / NGH_BLK) + blockIdx.x] = F == 2047 ? -1 : F;
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        const int j = j0 + p * PE + el;
         if (el < PE) {
-            const cplx x = hist_vec_value(W, S, w.n, w.T, vec, j, kvc);
-            if (kv < w.nv) w.vec[((int64_t)vec * w.nv + kv) * w.lenp + j] = x;
-            hist_digits(x, F, vec == 3, j & 15, dig[kk][el / 16]);   // the left-mixing row vector enters conjugated
+            if (kv < w.nv) w.vec[((int64_t)vec * w.nv + kv) * w.lenp + j] = x[p];
+            hist_digits(x[p], F, vec == 3, j & 15, dig[kk][el / 16]);   // the left-mixing row vector enters conjugated
         }
         __syncthreads();
         constexpr int NU = KK * (PE / 16) * 64;   // uint4 of the pass
         for (int i = tid; i < NU; i += 256) {
             const int q = i / (PE / 16 * 64), r = i % (PE / 16 * 64), kq = blockIdx.y * KK + q;
             if (kq < w.nv)
-                w.tab[(((int64_t)vec * w.nv + kq) * (w.lenp / 16) + (blockIdx.x * NGH_BLK + p) / 16) * 64 + r] =
+                w.tab[(((int64_t)vec * w.nv + kq) * (w.lenp / 16) + (j0 + p * PE) / 16) * 64 + r] =
                     ((const uint4*)&dig[q][0][0][0][0][0][0][0])[r];
         }
         __syncthreads();
