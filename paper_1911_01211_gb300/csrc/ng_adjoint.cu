@@ -16,23 +16,24 @@ cudaError_t adj_pass(const AdjStep& a, SliceV Glc, const cplx* U, SliceV cLoc, d
     const int n = a.n, nb = a.g.nb, T = a.g.ntau, k = a.g.k;
     k_adj_lesA<<<nb, 128, 0, s>>>(a);
     k_adj_qA<<<nblk((int64_t)(std::max(n, T) + 1) * nb, 128), 128, 0, s>>>(a);
-    const int width = std::max(n + 1, T + 1);
-    k_adj_sigA<<<dim3(nblk((int64_t)a.nq * width * 32, 128), 4), 128, 0, s>>>(a, width);
     k_adj_bulk<<<dim3(nb, 2), 128, 0, s>>>(a);
-    const unsigned S = NG_ADJ_SPLIT;
-    k_adj_tvrow<<<dim3(n, S), 256, 0, s>>>(a);
-    k_adj_rrow<<<dim3(n, S), 256, 0, s>>>(a);
+    AdjHistGrid q{};
+    q.rrow = q.tvrow = n;
+    q.qtv = T + 1;
     if (!a.full) {
-        k_adj_tvcol<<<dim3(T + 1, S), 256, 0, s>>>(a);
-        k_adj_rcol<<<dim3(n - k, S), 256, 0, s>>>(a);
-        k_adj_lcol<<<dim3(n, S), 256, 0, s>>>(a);
-        if (n - k - 1 > 0) k_adj_lrow<<<dim3(n - k - 1, S), 256, 0, s>>>(a);
+        q.lcol = n;
+        q.tvcol = T + 1;
+        q.rcol = n - k;
+        q.lrow = std::max(0, n - k - 1);
     }
-    k_adj_qtv<<<dim3(T + 1, S), 256, 0, s>>>(a);
-    k_adj_cur<<<nblk(2 * (int64_t)(n + 1) + T + 1 + (int64_t)k * k, 128), 128, 0, s>>>(a);
+    q.width = std::max(n + 1, T + 1);
+    q.sigA = (int)nblk((int64_t)a.nq * q.width * 32, 256);
+    static_assert(NG_ADJ_SPLIT == 4, "one split per group of section 3");
+    k_adj_hist<<<dim3(q.rrow + q.lcol + q.tvrow + q.qtv + q.tvcol + q.rcol + q.lrow + q.sigA, NG_ADJ_SPLIT), 256, 0, s>>>(a, q);
+    const int64_t targets = 2 * (int64_t)(n + 1) + T + 1 + (int64_t)k * k + (nb + 31) / 32;
+    k_adj_cur<<<nblk(targets * 32, 128), 128, 0, s>>>(a, ce0_row);
     k_adj_sigma2b<<<nblk(std::max(n, T) + 1, 128), 128, 0, s>>>(a.g, n, Glc, a.cSw, a.cmfw, 1, FuncV{(cplx*)U, 1},
                                                                 cLoc);
-    k_adj_ce0<<<nblk(nb, 128), 128, 0, s>>>(nb, a.cmfw, 1, ce0_row);
     k_adj_bcast<<<nblk((2 * (int64_t)(n + 1) + T + 1) * nb, 256), 256, 0, s>>>(a.g, n, cLoc, a.cw, a.cSw, a.cmfw);
     return cudaGetLastError();
 }

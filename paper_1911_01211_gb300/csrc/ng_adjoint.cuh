@@ -178,11 +178,11 @@ __device__ __forceinline__ cplx* adj_tgt_tv(const AdjStep& a, int m, int j) {
     return m == a.n ? &a.cSw.tv[j] : &a.cSt[(int64_t)m * (a.g.ntau + 1) + j];
 }
 
-__global__ void k_adj_sigA(AdjStep a, int width) {
+__device__ __forceinline__ void adj_sigA(const AdjStep& a, int width, int blk) {
     const NgWeights& W = c_W[a.g.k - 1];
     const int k = W.k, n = a.n, nb = a.g.nb, T = a.g.ntau;
     const int lane = threadIdx.x & 31;
-    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t wid = ((int64_t)blk * blockDim.x + threadIdx.x) >> 5;
     const int grp = blockIdx.y;
     const int r = (int)(wid / width), q = (int)(wid % width);
     const double h = a.g.h, ht = a.g.htau, xi = (double)a.g.sig;
@@ -329,19 +329,18 @@ __global__ void __launch_bounds__(128) k_adj_bulk(AdjStep a) {
 // ======================================================================================
 // 5. History cotangents and the partial sums of the self-energy row / column cotangents.
 // ======================================================================================
-// The history kernels below run one block per history row (or column); each warp takes one
+// The history functions below run on one block per history row (or column); each warp takes one
 // index of the other time argument at a time and its lanes take the problems kb = lane,
 // lane + 32, ..., so the weights and self-energy values of that index are warp-uniform and the
 // per-problem arrays are read in contiguous 512-byte runs.
 
 // tv history row j < n: tv step (all tau), BDF, and the C^<_3 source of the lesser (B) row j.
-__global__ void __launch_bounds__(256) k_adj_tvrow(AdjStep a) {
+__device__ __forceinline__ void adj_tvrow(const AdjStep& a, int j, cplx* red) {
     const NgWeights& W = c_W[a.g.k - 1];
-    const int k = W.k, n = a.n, nb = a.g.nb, T = a.g.ntau, j = blockIdx.x;
+    const int k = W.k, n = a.n, nb = a.g.nb, T = a.g.ntau;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int m0 = blockIdx.y * nw + wp, ms = nw * gridDim.y;   // this block's share of the row
     const double h = a.g.h, ht = a.g.htau, xi = (double)a.g.sig;
-    __shared__ cplx red[32];
     const cplx coefA = cadd(cmuli(cscal(h * gw(W, n, j), cconj(a.Sc.ret[j]))),
                             cr(j >= n - k ? -W.a[n - j] / h : 0.0));
     const bool useB = !a.full && j >= 1 && j <= n - k - 1;
@@ -366,13 +365,12 @@ __global__ void __launch_bounds__(256) k_adj_tvrow(AdjStep a) {
 }
 
 // tv column m: cotangent of Sigma^tv(n, T-m) from the C^<_3 sources of the lesser (B) rows
-__global__ void __launch_bounds__(256) k_adj_tvcol(AdjStep a) {
+__device__ __forceinline__ void adj_tvcol(const AdjStep& a, int m, cplx* red) {
     const NgWeights& W = c_W[a.g.k - 1];
-    const int k = W.k, n = a.n, nb = a.g.nb, T = a.g.ntau, m = blockIdx.x;
+    const int k = W.k, n = a.n, nb = a.g.nb, T = a.g.ntau;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int j0 = blockIdx.y * nw + wp, js = nw * gridDim.y;
     const double ht = a.g.htau, xi = (double)a.g.sig;
-    __shared__ cplx red[32];
     cplx acc = cz();
     for (int j = 1 + j0; j <= n - k - 1; j += js) {
         const int64_t base = ((int64_t)j * (T + 1) + m) * nb;
@@ -388,14 +386,12 @@ __global__ void __launch_bounds__(256) k_adj_tvcol(AdjStep a) {
 // ret history row j < n: retarded (B) columns m <= n-k-1 (history term and BDF), and the
 // C^<_1 source of the lesser (B) rows (row j itself, and rows m < j <= k through the
 // modified retarded continuation).
-__global__ void __launch_bounds__(256) k_adj_rrow(AdjStep a) {
+__device__ __forceinline__ void adj_rrow(const AdjStep& a, int j, cplx* red) {
     const NgWeights& W = c_W[a.g.k - 1];
-    // rows in decreasing length (row j holds j + 1 entries): the longest are scheduled first
-    const int k = W.k, n = a.n, nb = a.g.nb, j = gridDim.x - 1 - blockIdx.x;
+    const int k = W.k, n = a.n, nb = a.g.nb;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int m0 = blockIdx.y * nw + wp, ms = nw * gridDim.y;
     const double h = a.g.h;
-    __shared__ cplx red[32];
     const cplx sRc = cconj(a.Sc.ret[j]);
     const double bdf = (j >= n - k) ? -W.a[n - j] / h : 0.0;
     const bool rowB = !a.full && j >= 1 && j <= n - k - 1;
@@ -433,13 +429,12 @@ __global__ void __launch_bounds__(256) k_adj_rrow(AdjStep a) {
 }
 
 // ret column b: cotangent of Sigma^<(b,n) from the C^<_1 sources of the lesser (B) rows
-__global__ void __launch_bounds__(256) k_adj_rcol(AdjStep a) {
+__device__ __forceinline__ void adj_rcol(const AdjStep& a, int b, cplx* red) {
     const NgWeights& W = c_W[a.g.k - 1];
-    const int k = W.k, n = a.n, nb = a.g.nb, b = blockIdx.x;
+    const int k = W.k, n = a.n, nb = a.g.nb;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int a0 = blockIdx.y * nw + wp, as = nw * gridDim.y;
     const double h = a.g.h;
-    __shared__ cplx red[32];
     cplx acc = cz();
     // rows ar >= max(1, b): R~(ar,b) = G^R(ar,b); rows 1 <= ar < b <= k: R~(ar,b) = -conj(G^R(b,ar))
     for (int ar = 1 + a0; ar <= n - k - 1; ar += as) {
@@ -466,14 +461,12 @@ __global__ void __launch_bounds__(256) k_adj_rcol(AdjStep a) {
 
 // les history column b < n: history term and BDF of the lesser (B) rows; partial of
 // Sigma^R(n,b) from rows m <= b
-__global__ void __launch_bounds__(256) k_adj_lcol(AdjStep a) {
+__device__ __forceinline__ void adj_lcol(const AdjStep& a, int b, cplx* red) {
     const NgWeights& W = c_W[a.g.k - 1];
-    // columns in decreasing length (column b holds b + 1 entries): the longest first
-    const int k = W.k, n = a.n, nb = a.g.nb, b = gridDim.x - 1 - blockIdx.x;
+    const int k = W.k, n = a.n, nb = a.g.nb;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int a0 = blockIdx.y * nw + wp, as = nw * gridDim.y;
     const double h = a.g.h;
-    __shared__ cplx red[32];
     const double wb = gw(W, n, b);
     const double bdf = (b >= n - k) ? -W.a[n - b] / h : 0.0;
     const bool colB = b >= 1 && b <= n - k - 1;
@@ -505,13 +498,12 @@ __global__ void __launch_bounds__(256) k_adj_lcol(AdjStep a) {
 }
 
 // les history row a: partial of Sigma^R(n,a) from the lesser (B) rows m > a
-__global__ void __launch_bounds__(256) k_adj_lrow(AdjStep a) {
+__device__ __forceinline__ void adj_lrow(const AdjStep& a, int ar, cplx* red) {
     const NgWeights& W = c_W[a.g.k - 1];
-    const int k = W.k, n = a.n, nb = a.g.nb, ar = blockIdx.x;
+    const int k = W.k, n = a.n, nb = a.g.nb;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int m0 = blockIdx.y * nw + wp, ms = nw * gridDim.y;
     const double h = a.g.h;
-    __shared__ cplx red[32];
     cplx acc = cz();
     for (int m = max(ar + 1, 1) + m0; m <= n - k - 1; m += ms) {
         const int64_t base = (tri(m) + ar) * nb;
@@ -527,13 +519,12 @@ __global__ void __launch_bounds__(256) k_adj_lrow(AdjStep a) {
 
 // Matsubara source of the tv row, q = -i htau (C2 + C3) (Eqs. ctv2, ctv3): cotangent of
 // Sigma^tv(n, tau_p), one block per p, sum over (m, problem).
-__global__ void __launch_bounds__(256) k_adj_qtv(AdjStep a) {
+__device__ __forceinline__ void adj_qtv(const AdjStep& a, int p, cplx* red) {
     const NgWeights& W = c_W[a.g.k - 1];
-    const int k = W.k, nb = a.g.nb, T = a.g.ntau, p = blockIdx.x;
+    const int k = W.k, nb = a.g.nb, T = a.g.ntau;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int m0 = blockIdx.y * nw + wp, ms = nw * gridDim.y;
     const double ht = a.g.htau, xi = (double)a.g.sig;
-    __shared__ cplx red[32];
     cplx acc = cz();
     for (int m = m0; m <= T; m += ms) {
         // C2 (with xi): m <= k: R[m][j][p] xi G^M(T-j), p <= k;  m > k: w_{m,m-p} xi G^M(T-m+p), p <= m
@@ -558,13 +549,35 @@ __global__ void __launch_bounds__(256) k_adj_qtv(AdjStep a) {
     if (threadIdx.x == 0) a.part[(P_QTV * NG_ADJ_SPLIT + blockIdx.y) * a.plen + p] = cmuli(cscal(ht, acc));
 }
 
+// All of them and the shared cotangents of the (A) part (section 3) in one launch: they read the work vectors of
+// the pass and write arrays of their own.  Each alone is a few hundred blocks waiting for memory (64 problems,
+// n <= 100, ntau = 80: 8 to 18 us each, 100 us in turn, 56 us together).  Blocks (index, split), the longest first; groups of
+// section 3 in blockIdx.y.
+struct AdjHistGrid {
+    int rrow, lcol, tvrow, qtv, tvcol, rcol, lrow, sigA;   // blocks of each kind
+    int width;
+};
+__global__ void __launch_bounds__(256) k_adj_hist(AdjStep a, AdjHistGrid q) {
+    __shared__ cplx red[32];
+    int b = blockIdx.x;
+    if (b < q.rrow) return adj_rrow(a, q.rrow - 1 - b, red);   // rows and columns in decreasing length
+    if ((b -= q.rrow) < q.lcol) return adj_lcol(a, q.lcol - 1 - b, red);
+    if ((b -= q.lcol) < q.tvrow) return adj_tvrow(a, b, red);
+    if ((b -= q.tvrow) < q.qtv) return adj_qtv(a, b, red);
+    if ((b -= q.qtv) < q.tvcol) return adj_tvcol(a, b, red);
+    if ((b -= q.tvcol) < q.rcol) return adj_rcol(a, b, red);
+    if ((b -= q.rcol) < q.lrow) return adj_lrow(a, b, red);
+    adj_sigA(a, q.width, b - q.lrow);
+}
+
 // Current self-energy slice: add the partial sums, the M_n term and the retarded (A) block.
-// Thread per target: ret slots 0..n, les slots 0..n, tv slots 0..T, then the (k+1)^2 entries
-// of the retarded (A) block in history rows n-1..n-k.
-__global__ void k_adj_cur(AdjStep a) {
+// Warp per target: ret slots 0..n, les slots 0..n, tv slots 0..T, then the (k+1)^2 entries
+// of the retarded (A) block in history rows n-1..n-k; then 32 problems each of the eps0 cotangent (real part of the
+// eps_mf cotangent).  The lanes share the sums over the problems, which a thread alone took 17 us for (64 problems).
+__global__ void __launch_bounds__(128) k_adj_cur(AdjStep a, double* ce0_row) {
     const NgWeights& W = c_W[a.g.k - 1];
-    const int k = W.k, n = a.n, nb = a.g.nb, T = a.g.ntau, K1 = k + 1;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = W.k, n = a.n, nb = a.g.nb, T = a.g.ntau, K1 = k + 1, lane = threadIdx.x & 31;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const double h = a.g.h;
     // the NG_ADJ_SPLIT block partials of a history sum, added in split order
     auto part = [&](int which, int64_t idx) {
@@ -572,11 +585,12 @@ __global__ void k_adj_cur(AdjStep a) {
         for (int sp = 0; sp < NG_ADJ_SPLIT; ++sp) v = cadd(v, a.part[(which * NG_ADJ_SPLIT + sp) * a.plen + idx]);
         return v;
     };
-    auto sumk = [&](int l, int j) {
+    auto sum = [&](const cplx* p) {
         cplx s = cz();
-        for (int kb = 0; kb < nb; ++kb) s = cadd(s, a.retA[(int64_t)(l * K1 + j) * nb + kb]);
-        return s;
+        for (int kb = lane; kb < nb; kb += 32) s = cadd(s, p[kb]);
+        return warp_sum(s);
     };
+    auto sumk = [&](int l, int j) { return sum(a.retA + (int64_t)(l * K1 + j) * nb); };
     if (i <= n) {
         const int j = (int)i;
         cplx v = cz();
@@ -585,18 +599,14 @@ __global__ void k_adj_cur(AdjStep a) {
             if (!a.full) v = cadd(v, part(P_LCOL, j));
             if (!a.full && j <= n - k - 2) v = cadd(v, part(P_LROW, j));
             if (j >= n - k) v = cadd(v, sumk(0, n - j));   // retarded (A) block, row n
-        } else {
-            cplx s = cz();
-            for (int kb = 0; kb < nb; ++kb) s = cadd(s, a.cMn[kb]);
-            v = cmulmi(cscal(h * gw(W, n, n), s));
-        }
-        a.cSw.ret[j] = cadd(a.cSw.ret[j], v);
+        } else v = cmulmi(cscal(h * gw(W, n, n), sum(a.cMn)));
+        if (lane == 0) cacc_to(&a.cSw.ret[j], v);
         return;
     }
     int64_t r = i - (n + 1);
     if (r <= n) {
         const int b = (int)r;
-        if (!a.full && b <= n - k - 1) a.cSw.les[b] = cadd(a.cSw.les[b], part(P_RCOL, b));
+        if (!a.full && b <= n - k - 1 && lane == 0) cacc_to(&a.cSw.les[b], part(P_RCOL, b));
         return;
     }
     r -= n + 1;
@@ -604,18 +614,21 @@ __global__ void k_adj_cur(AdjStep a) {
         const int p = (int)r;
         cplx v = part(P_QTV, p);
         if (!a.full) v = cadd(v, part(P_TVCOL, p));
-        a.cSw.tv[p] = cadd(a.cSw.tv[p], v);
+        if (lane == 0) cacc_to(&a.cSw.tv[p], v);
         return;
     }
     r -= T + 1;
+    if (r >= (int64_t)k * k) {
+        const int64_t kb = (r - k * k) * 32 + lane;
+        if (kb < nb) ce0_row[kb] += a.cmfw[kb].x;
+        return;
+    }
     // retarded (A) block, history rows: target (n-x, n-y), 1 <= x <= y <= k
-    if (r >= (int64_t)k * k) return;
     const int x = 1 + (int)(r / k), y = 1 + (int)(r % k);
     if (y < x) return;
     cplx v = sumk(x, y);                                   // l = x <= j = y
     if (y > x) v = csub(v, cconj(sumk(y, x)));             // l = y > j = x: continued
-    cplx* p = &a.cSr[tri(n - x) + (n - y)];
-    *p = cadd(*p, v);
+    if (lane == 0) cacc_to(&a.cSr[tri(n - x) + (n - y)], v);
 }
 
 // ======================================================================================
@@ -630,6 +643,17 @@ __global__ void k_adj_sigma2b(Grid g, int n, SliceV Lc /* ld 1 */, SliceV cS /* 
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const double xi = (double)g.sig;
     auto u = [&](int t) { return U.p[t + 1].x; };
+    __shared__ double hartree;   // sum over the problems for j = n, by a warp of its block
+    const int b0 = blockIdx.x * blockDim.x;
+    if (b0 <= n && n < b0 + (int)blockDim.x) {
+        if (threadIdx.x < 32) {
+            cplx s = cz();
+            for (int kb = threadIdx.x; kb < nb; kb += 32) s.x += cmfw[(int64_t)kb * ld_cmf].x;
+            s = warp_sum(s);
+            if (threadIdx.x == 0) hartree = s.x;
+        }
+        __syncthreads();
+    }
     if (i <= n) {
         const int j = i;
         const double uu = u(n) * u(j);
@@ -645,9 +669,7 @@ __global__ void k_adj_sigma2b(Grid g, int n, SliceV Lc /* ld 1 */, SliceV cS /* 
         cg = cfma(cconj(cmul(gl, gl)), cP, cg);
         cl = csub(cl, cconj(cg));
         if (j == n) {   // Hartree: eps_mf(n) = eps0(n) + U_n (Im G_loc^<(n,n) - nbar)
-            double s = 0.0;
-            for (int kb = 0; kb < nb; ++kb) s += cmfw[(int64_t)kb * ld_cmf].x;
-            cl = cadd(cl, cmuli(cr(u(n) * s)));
+            cl = cadd(cl, cmuli(cr(u(n) * hartree)));
         }
         out.ret[j] = cg;
         out.les[j] = cl;
@@ -660,12 +682,6 @@ __global__ void k_adj_sigma2b(Grid g, int n, SliceV Lc /* ld 1 */, SliceV cS /* 
         c = cfma(cscal(up, cmul(tvr, tvr)), cconj(cS.tv[T - m]), c);
         out.tv[m] = c;
     }
-}
-
-// eps0 cotangent of one step (real part of the eps_mf cotangent), thread per problem
-__global__ void k_adj_ce0(int nb, const cplx* cmfw, int ld_cmf, double* ce0_row) {
-    const int kb = blockIdx.x * blockDim.x + threadIdx.x;
-    if (kb < nb) ce0_row[kb] += cmfw[(int64_t)kb * ld_cmf].x;
 }
 
 // per-problem slice cotangent = (shared slice cotangent)/nb, thread per (element, problem);
