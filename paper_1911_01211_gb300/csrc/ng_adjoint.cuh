@@ -68,6 +68,7 @@ __device__ cplx block_csum(cplx v, cplx* sh /* >= 32 */) {
 //    - h sum_{l<m} w_{m,l} i Sigma^R(m,l) G^<(l,n).
 // ======================================================================================
 __global__ void __launch_bounds__(128) k_adj_lesA(AdjStep a) {
+    dep_wait();
     const NgWeights& W = c_W[a.g.k - 1];
     const int k = W.k, n = a.n, nb = a.g.nb, kb = blockIdx.x, t = threadIdx.x;
     const double h = a.g.h;
@@ -140,6 +141,7 @@ __global__ void __launch_bounds__(128) k_adj_lesA(AdjStep a) {
 //    -conj(G^tv(n,0)) (Eq. dyson_ini_les).  Thread per (j, problem).
 // ======================================================================================
 __global__ void k_adj_qA(AdjStep a) {
+    dep_wait();
     const NgWeights& W = c_W[a.g.k - 1];
     const int n = a.n, nb = a.g.nb, T = a.g.ntau;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -287,6 +289,7 @@ __device__ __forceinline__ void adj_retA_w(const AdjStep& a, int kb, int lane) {
 }
 
 __global__ void __launch_bounds__(128) k_adj_bulk(AdjStep a) {
+    dep_wait();
     const NgWeights& W = c_W[a.g.k - 1];
     const int k = W.k, n = a.n, nb = a.g.nb, T = a.g.ntau, kb = blockIdx.x, t = threadIdx.x;
     const double h = a.g.h;
@@ -558,6 +561,7 @@ struct AdjHistGrid {
     int width;
 };
 __global__ void __launch_bounds__(256) k_adj_hist(AdjStep a, AdjHistGrid q) {
+    dep_wait();
     __shared__ cplx red[32];
     int b = blockIdx.x;
     if (b < q.rrow) return adj_rrow(a, q.rrow - 1 - b, red);   // rows and columns in decreasing length
@@ -575,6 +579,7 @@ __global__ void __launch_bounds__(256) k_adj_hist(AdjStep a, AdjHistGrid q) {
 // of the retarded (A) block in history rows n-1..n-k; then 32 problems each of the eps0 cotangent (real part of the
 // eps_mf cotangent).  The lanes share the sums over the problems, which a thread alone took 17 us for (64 problems).
 __global__ void __launch_bounds__(128) k_adj_cur(AdjStep a, double* ce0_row) {
+    dep_wait();
     const NgWeights& W = c_W[a.g.k - 1];
     const int k = W.k, n = a.n, nb = a.g.nb, T = a.g.ntau, K1 = k + 1, lane = threadIdx.x & 31;
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -639,6 +644,7 @@ __global__ void __launch_bounds__(128) k_adj_cur(AdjStep a, double* ce0_row) {
 // ======================================================================================
 __global__ void k_adj_sigma2b(Grid g, int n, SliceV Lc /* ld 1 */, SliceV cS /* ld 1 */, const cplx* cmfw,
                               int ld_cmf, FuncV U, SliceV out /* ld 1 */) {
+    dep_wait();
     const int T = g.ntau, nb = g.nb;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const double xi = (double)g.sig;
@@ -687,6 +693,7 @@ __global__ void k_adj_sigma2b(Grid g, int n, SliceV Lc /* ld 1 */, SliceV cS /* 
 // per-problem slice cotangent = (shared slice cotangent)/nb, thread per (element, problem);
 // also clears the shared cotangent of the next pass and the eps_mf cotangent
 __global__ void k_adj_bcast(Grid g, int n, SliceV src, SliceV dst, SliceV sclear, cplx* cmfw) {
+    dep_wait();
     const int nb = g.nb, T = g.ntau;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t len = 2 * (int64_t)(n + 1) + T + 1;
@@ -710,6 +717,7 @@ __global__ void k_adj_bcast(Grid g, int n, SliceV src, SliceV dst, SliceV sclear
 
 // copy a slice (ld = nb or 1) between two slice views; thread per (element, problem)
 __global__ void k_slice_copy(int n, int T, int ld, SliceV src, SliceV dst) {
+    dep_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t len = 2 * (int64_t)(n + 1) + T + 1;
     if (i >= len * ld) return;
@@ -728,6 +736,7 @@ __global__ void k_slice_copy(int n, int T, int ld, SliceV src, SliceV dst) {
 // ======================================================================================
 // diagonals of ret and les and the tv rows: thread per (slice element, problem), loop over l
 __global__ void k_adj_extrap_diag(Grid g, int n, SliceV cw, cplx* cGr, cplx* cGl, cplx* cGt) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int k = W.k, nb = g.nb, T = g.ntau, Np = n - 1;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -770,6 +779,7 @@ __global__ void k_adj_extrap_diag(Grid g, int n, SliceV cw, cplx* cGr, cplx* cGl
 // columns j <= k of ret and rows j <= k of les (with the hermitian continuation): thread per (component, j,
 // problem) where no continued element meets another column's (n > 2k), else per (component, problem)
 __global__ void k_adj_extrap_cols(Grid g, int n, SliceV cw, cplx* cGr, cplx* cGl) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int k = W.k, nb = g.nb, Np = n - 1;
     const int i = blockIdx.x * blockDim.x + threadIdx.x, kb = i % nb, c = i / nb;
@@ -791,6 +801,7 @@ __global__ void k_adj_extrap_cols(Grid g, int n, SliceV cw, cplx* cGr, cplx* cGl
 
 // seed: c(G^<_k(n,n)) += seed[n][kb] for every n
 __global__ void k_adj_seed(Grid g, const cplx* seed, cplx* cGl) {
+    dep_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)(g.nt + 1) * g.nb) return;
     const int n = (int)(i / g.nb), kb = (int)(i % g.nb);
@@ -805,6 +816,7 @@ __global__ void k_adj_seed(Grid g, const cplx* seed, cplx* cGl) {
 
 
 __global__ void __launch_bounds__(NG_BOOT_THREADS) k_adj_start(AdjBoot b) {
+    dep_wait();
     const NgWeights& W = c_W[b.g.k - 1];
     const int k = W.k, T = b.g.ntau, nb = b.g.nb, kb = blockIdx.x, t = threadIdx.x;
     const double h = b.g.h, ht = b.g.htau, xi = (double)b.g.sig;
@@ -998,6 +1010,7 @@ __global__ void __launch_bounds__(NG_BOOT_THREADS) k_adj_start(AdjBoot b) {
 
 // shared Sigma cotangent of slices 0..k = sum over problems (fixed order); warp per entry
 __global__ void k_adj_boot_reduce(int64_t E, int nb, const cplx* Pk, cplx* out) {
+    dep_wait();
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (w >= E) return;
@@ -1009,6 +1022,7 @@ __global__ void k_adj_boot_reduce(int64_t E, int nb, const cplx* Pk, cplx* out) 
 
 // mu_new = ctot + bcast(cL)/nb over slices 0..k; dist[0] += |mu_new - mu|, dist[1] += |mu_new|
 __global__ void k_adj_boot_update(int64_t E, int nb, const cplx* ctot, const cplx* cL, cplx* mu, double* dist) {
+    dep_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     double d = 0.0, a = 0.0;
     if (i < E * nb) {
@@ -1030,6 +1044,7 @@ __global__ void k_adj_boot_update(int64_t E, int nb, const cplx* ctot, const cpl
 
 // gather the cotangent of slices 0..k of a herm (ld = nb or 1) into the compact layout
 __global__ void k_boot_gather(Grid g, const cplx* r, const cplx* l, const cplx* tv, int ld, cplx* out) {
+    dep_wait();
     const int k = g.k, T = g.ntau;
     const int64_t T3 = tri(k + 1), E = boot_E(k, T);
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1043,6 +1058,7 @@ __global__ void k_boot_gather(Grid g, const cplx* r, const cplx* l, const cplx* 
 
 // eps0 cotangent rows 0..k: ce0 += Re(cmf), thread per (row, problem)
 __global__ void k_adj_ce0_rows(int rows, int nb, const cplx* cmf, double* ce0) {
+    dep_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)rows * nb) return;
     ce0[nb + i] += cmf[nb + i].x;   // rows t = 0..rows-1 at index (t+1)

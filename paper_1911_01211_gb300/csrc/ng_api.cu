@@ -271,7 +271,7 @@ template <int D>
 ng_status launch_minv(ng_ctx* c, const Grid& g, int n, const HermV& S, const FuncV& eps, cudaStream_t s) {
     ng_status st = ensure(c, &c->ws_minv, &c->ws_minv_bytes, sizeof(cplx) * D * D * (size_t)g.nb);
     if (st) return st;
-    k_minv_step<D><<<nblocks(g.nb, 128), 128, 0, s>>>(g, n, S, eps, (cplx*)c->ws_minv, c->d_status);
+    dep_launch(k_minv_step<D>, nblocks(g.nb, 128), 128, 0, s)(g, n, S, eps, (cplx*)c->ws_minv, c->d_status);
     return check_launch(c, "k_minv_step");
 }
 
@@ -336,8 +336,8 @@ ng_status hist_sums(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV
     HistRow r{S.ret.p + tri(n) * S.ret.ldk, Scc.les.p + tri(n) * Scc.les.ldk,
               S.tv.p + (int64_t)n * (g.ntau + 1) * S.tv.ldk, S.ret.ldk, Scc.les.ldk, S.tv.ldk};
     const unsigned chunks = (unsigned)(w->lenp / NGH_BLK);
-    if (nv == 1) k_hist_vec<1><<<dim3(chunks, 1, NGH_NVEC), 256, 0, s>>>(*w, r);
-    else k_hist_vec<8><<<dim3(chunks, nblocks(nv, 8), NGH_NVEC), 256, 0, s>>>(*w, r);
+    if (nv == 1) dep_launch(k_hist_vec<1>, dim3(chunks, 1, NGH_NVEC), 256, 0, s)(*w, r);
+    else dep_launch(k_hist_vec<8>, dim3(chunks, nblocks(nv, 8), NGH_NVEC), 256, 0, s)(*w, r);
     ng_status st = check_launch(c, "k_hist_vec");
     if (st) return st;
     if (hist_launch(*w, G.ret.p, G.les.p, G.tv.p, c->sms, c->d_status, s) != cudaSuccess) {
@@ -361,12 +361,12 @@ ng_status boundary_spread(ng_ctx* c, const Grid& g, int n, const HermV& G, const
     const size_t need = sizeof(cplx) * (size_t)nq * g.nb * nchunk * 2 * D * D;
     if ((st = ensure(c, &c->ws_bnd, &c->ws_bnd_bytes, need))) return st;
     if (!pre_done) {
-        k_bnd_pre<D><<<g.nb, 32, 0, s>>>(g, n, G, S, eps, c->d_status);
+        dep_launch(k_bnd_pre<D>, g.nb, 32, 0, s)(g, n, G, S, eps, c->d_status);
         if ((st = check_launch(c, "k_bnd_pre"))) return st;
     }
-    k_bnd_src<D><<<dim3(nq, g.nb, nchunk), NG_BND_THREADS, 0, s>>>(g, n, G, S, nchunk, (cplx*)c->ws_bnd);
+    dep_launch(k_bnd_src<D>, dim3(nq, g.nb, nchunk), NG_BND_THREADS, 0, s)(g, n, G, S, nchunk, (cplx*)c->ws_bnd);
     if ((st = check_launch(c, "k_bnd_src"))) return st;
-    k_bnd_fin<D><<<g.nb, 32, 0, s>>>(g, n, G, S, eps, nchunk, (const cplx*)c->ws_bnd, c->d_status);
+    dep_launch(k_bnd_fin<D>, g.nb, 32, 0, s)(g, n, G, S, eps, nchunk, (const cplx*)c->ws_bnd, c->d_status);
     return check_launch(c, "k_bnd_fin");
 }
 
@@ -383,16 +383,16 @@ ng_status boundary1(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV
     const int len = std::max(4, (J + want - 1) / want), nchunk = (J + len - 1) / len;
     if ((st = ensure(c, &c->ws_bnd, &c->ws_bnd_bytes, sizeof(cplx) * (size_t)nchunk * 2 * NG_B1_ROWS * g.nb))) return st;
     if (!pre_done) {
-        k_bnd_pre<1><<<g.nb, 32, 0, s>>>(g, n, G, S, eps, c->d_status);
+        dep_launch(k_bnd_pre<1>, g.nb, 32, 0, s)(g, n, G, S, eps, c->d_status);
         if ((st = check_launch(c, "k_bnd_pre"))) return st;
     }
     const dim3 grid(groups, nchunk);
     if (S.ret.ldk == 1 && S.les.ldk == 1 && S.tv.ldk == 1)
-        k_bnd1_sums<true><<<grid, 128, 0, s>>>(g, n, G, S, len, (cplx*)c->ws_bnd);
+        dep_launch(k_bnd1_sums<true>, grid, 128, 0, s)(g, n, G, S, len, (cplx*)c->ws_bnd);
     else
-        k_bnd1_sums<false><<<grid, 128, 0, s>>>(g, n, G, S, len, (cplx*)c->ws_bnd);
+        dep_launch(k_bnd1_sums<false>, grid, 128, 0, s)(g, n, G, S, len, (cplx*)c->ws_bnd);
     if ((st = check_launch(c, "k_bnd1_sums"))) return st;
-    k_bnd1_fin<<<groups, 32 * NG_B1_WARPS, 0, s>>>(g, n, G, S, eps, nchunk, (const cplx*)c->ws_bnd, c->d_status);
+    dep_launch(k_bnd1_fin, groups, 32 * NG_B1_WARPS, 0, s)(g, n, G, S, eps, nchunk, (const cplx*)c->ws_bnd, c->d_status);
     return check_launch(c, "k_bnd1_fin");
 }
 
@@ -405,7 +405,7 @@ ng_status boundary_batch(ng_ctx* c, const Grid& g, int n, const HermV& G, const 
     if (D == 1 && bnd1_applies(g, n)) {
         st = boundary1(c, g, n, G, S, eps, false, s);
     } else {
-        k_step_boundary<D><<<g.nb, NG_BND_THREADS, 0, s>>>(g, n, G, S, eps, c->d_status);
+        dep_launch(k_step_boundary<D>, g.nb, NG_BND_THREADS, 0, s)(g, n, G, S, eps, c->d_status);
         st = check_launch(c, "k_step_boundary");
     }
     if (e >= 0) cudaEventRecord(c->ev_pool[e + 1], s);
@@ -454,19 +454,19 @@ ng_status launch_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const
     if (D == 1 && digits && (sm = hist_sums(c, g, n, G, S, S, &hw, &hist, s))) return sm;
     const int pre = hist && lanes ? (int)nblocks(g.nb, thr / 32) : 0;   // leading blocks: the retarded start-up
     if (hist) {
-        k_hist_close<<<pre + b_les + b_tv + b_ret, thr, 0, s>>>(g, n, G, S, eps, hw, (const cplx*)c->ws_minv, pre, b_les,
+        dep_launch(k_hist_close, pre + b_les + b_tv + b_ret, thr, 0, s)(g, n, G, S, eps, hw, (const cplx*)c->ws_minv, pre, b_les,
                                                                 b_tv, tvq, c->d_status);
     } else if (part) {
         const int c_les = it_les ? n - k - 1 : 0, c_tv = g.ntau + 1, c_ret = n - k, q = 32 / part;
         const int64_t warps = w_pre + (int64_t)(c_les + c_tv + c_ret) * nblocks(g.nb, q);
         auto kernel = part == 4 ? k_step_bulk_q<4> : k_step_bulk_q<8>;
-        kernel<<<nblocks(warps * 32, thr), thr, 0, s>>>(g, n, G, S, eps, (const cplx*)c->ws_minv, (int)w_pre, c_les, c_tv,
+        dep_launch(kernel, nblocks(warps * 32, thr), thr, 0, s)(g, n, G, S, eps, (const cplx*)c->ws_minv, (int)w_pre, c_les, c_tv,
                                                         c_ret, tvq, c->d_status);
     } else if (warp) {
-        k_step_bulk_w<D><<<nblocks((w_pre + items) * 32, thr), thr, 0, s>>>(g, n, G, S, eps, (const cplx*)c->ws_minv,
+        dep_launch(k_step_bulk_w<D>, nblocks((w_pre + items) * 32, thr), thr, 0, s)(g, n, G, S, eps, (const cplx*)c->ws_minv,
                                                                            w_pre, it_les, it_tv, it_ret, c->d_status);
     } else {
-        k_step_bulk<D><<<b_les + b_tv + b_ret, thr, 0, s>>>(g, n, G, S, eps, (const cplx*)c->ws_minv, b_les, b_tv,
+        dep_launch(k_step_bulk<D>, b_les + b_tv + b_ret, thr, 0, s)(g, n, G, S, eps, (const cplx*)c->ws_minv, b_les, b_tv,
                                                             b_ret, tvq, c->d_status);
     }
     ng_status st = check_launch(c, warp ? "k_step_bulk_w" : "k_step_bulk");
@@ -487,7 +487,7 @@ ng_status launch_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const
         if (e1 >= 0) cudaEventRecord(c->ev_pool[e1 + 1], s);
         return st;
     }
-    k_step_boundary<D><<<g.nb, NG_BND_THREADS, 0, s>>>(g, n, G, S, eps, c->d_status);
+    dep_launch(k_step_boundary<D>, g.nb, NG_BND_THREADS, 0, s)(g, n, G, S, eps, c->d_status);
     if (e1 >= 0) cudaEventRecord(c->ev_pool[e1 + 1], s);
     return check_launch(c, "k_step_boundary");
 }
@@ -517,7 +517,7 @@ ng_status update_shadow(ng_ctx* c, Shadow& sh, const Grid& g, const HermV& X, in
         const int a = n0 < 0 ? 0 : n0;
         const int64_t items = (2 * (tri(n1 + 1) - tri(a)) + (int64_t)(n1 - a + 1) * T1 + (n0 < 0 ? T1 : 0)) * dd * ldk;
         const unsigned blocks = (unsigned)std::min<int64_t>((items + 255) / 256, 152 * 16);
-        k_shadow<<<blocks, 256, 0, s>>>(g, n0, n1, X, sh.v, ldk);
+        dep_launch(k_shadow, blocks, 256, 0, s)(g, n0, n1, X, sh.v, ldk);
         return check_launch(c, "k_shadow");
     };
     ng_status st;
@@ -552,7 +552,7 @@ ng_status update_shadow_df(ng_ctx* c, ShadowDF& sh, const Grid& g, const HermV& 
         const int a = n0 < 0 ? 0 : n0;
         const int64_t items = (2 * (tri(n1 + 1) - tri(a)) + (int64_t)(n1 - a + 1) * T1 + (n0 < 0 ? T1 : 0)) * dd * ldk;
         const unsigned blocks = (unsigned)std::min<int64_t>((items + 255) / 256, 152 * 16);
-        k_shadow_df<<<blocks, 256, 0, s>>>(g, n0, n1, X, sh.v, ldk);
+        dep_launch(k_shadow_df, blocks, 256, 0, s)(g, n0, n1, X, sh.v, ldk);
         return check_launch(c, "k_shadow_df");
     };
     ng_status st;
@@ -583,7 +583,7 @@ ng_status launch_timestepdf(ng_ctx* c, const Grid& g, int n, const HermV& G, con
     if ((st = prep_tvfft(c, g, n, G, S, s, &tvq))) return st;
     long e0 = prof_pair(c, 0);
     if (e0 >= 0) cudaEventRecord(c->ev_pool[e0], s);
-    k_step_bulkdf<D><<<b_les + b_tv + b_ret, thr, 0, s>>>(g, n, G, S, c->dfG.v, c->dfS.v, (const cplx*)c->ws_minv,
+    dep_launch(k_step_bulkdf<D>, b_les + b_tv + b_ret, thr, 0, s)(g, n, G, S, c->dfG.v, c->dfS.v, (const cplx*)c->ws_minv,
                                                           b_les, b_tv, b_ret, tvq, c->d_status);
     if ((st = check_launch(c, "k_step_bulkdf"))) return st;
     if (e0 >= 0) {
@@ -614,10 +614,10 @@ ng_status launch_timestep32(ng_ctx* c, const Grid& g, int n, const HermV& G, con
         const int np = g.nb / 2;
         const int p_les = it_les ? (int)nblocks((int64_t)np * (n - k - 1), thr) : 0;
         const int p_tv = (int)nblocks((int64_t)np * (g.ntau + 1), thr), p_ret = (int)nblocks((int64_t)np * (n - k), thr);
-        k_step_bulk32p<<<p_les + p_tv + p_ret, thr, 0, s>>>(g, n, G, S, c->shG.v, c->shS.v, (const cplx*)c->ws_minv,
+        dep_launch(k_step_bulk32p, p_les + p_tv + p_ret, thr, 0, s)(g, n, G, S, c->shG.v, c->shS.v, (const cplx*)c->ws_minv,
                                                             p_les, p_tv, p_ret, tvq, c->d_status);
     } else {
-        k_step_bulk32<D><<<b_les + b_tv + b_ret, thr, 0, s>>>(g, n, G, S, c->shG.v, c->shS.v, eps,
+        dep_launch(k_step_bulk32<D>, b_les + b_tv + b_ret, thr, 0, s)(g, n, G, S, c->shG.v, c->shS.v, eps,
                                                               (const cplx*)c->ws_minv, b_les, b_tv, b_ret, tvq,
                                                               c->d_status);
     }
@@ -635,7 +635,7 @@ template <int PB>
 ng_status lu_solve_p(ng_ctx* c, int N, int nrhs, int nb, cplx* ws_A, int* ws_piv, cudaStream_t s) {
     const size_t smem = sizeof(cplx) * ((size_t)N * PB + NG_LU_TRI * nrhs);
     CUDA_TRY(c, cudaFuncSetAttribute(k_lu_solve<PB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_lu_solve<PB><<<nb, NG_LU_THREADS, smem, s>>>(N, nrhs, ws_A, ws_piv, c->d_status);
+    dep_launch(k_lu_solve<PB>, nb, NG_LU_THREADS, smem, s)(N, nrhs, ws_A, ws_piv, c->d_status);
     return check_launch(c, "k_lu_solve");
 }
 ng_status lu_solve(ng_ctx* c, int N, int nrhs, int nb, cplx* ws_A, int* ws_piv, cudaStream_t s) {
@@ -682,14 +682,14 @@ ng_status mat_solve(ng_ctx* c, const Grid& g, const HermV& G, const MatWs& w, bo
     ng_status st = NG_OK;
     auto refine = [&](double* dsum) -> ng_status {
         if constexpr (D <= 4) {
-            if (warp) k_mat_resid_w<D><<<nblocks(items * 32, 128), 128, 0, s>>>(g, w.g, w.K, G, w.r);
+            if (warp) dep_launch(k_mat_resid_w<D>, nblocks(items * 32, 128), 128, 0, s)(g, w.g, w.K, G, w.r);
         }
-        if (!warp) k_mat_resid<D><<<nblocks(items, 128), 128, 0, s>>>(g, w.g, w.K, G, w.r);
+        if (!warp) dep_launch(k_mat_resid<D>, nblocks(items, 128), 128, 0, s)(g, w.g, w.K, G, w.r);
         ng_status e = check_launch(c, "k_mat_resid");
         if (e) return e;
         CUDA_TRY(c, cudaMemsetAsync(dsum, 0, sizeof(double), s));
-        if (inverse) k_gj_apply<true><<<rows, 128, 0, s>>>(N, ld, D, inv, w.piv, w.r, G, dsum, c->d_status);
-        else k_lu_resolve<<<g.nb, NG_LU_THREADS, 0, s>>>(g, N, D, w.A, w.piv, w.r, G, dsum);
+        if (inverse) dep_launch(k_gj_apply<true>, rows, 128, 0, s)(N, ld, D, inv, w.piv, w.r, G, dsum, c->d_status);
+        else dep_launch(k_lu_resolve, g.nb, NG_LU_THREADS, 0, s)(g, N, D, w.A, w.piv, w.r, G, dsum);
         return check_launch(c, "Matsubara refinement");
     };
     if (refine_steps > 0) {
@@ -709,21 +709,21 @@ ng_status mat_solve(ng_ctx* c, const Grid& g, const HermV& G, const MatWs& w, bo
         }
         return NG_OK;
     }
-    k_mat_assemble<D><<<nblocks((int64_t)(T + 1) * (T + 2) * g.nb, 256), 256, 0, s>>>(g, w.g, w.K, w.A);
+    dep_launch(k_mat_assemble<D>, nblocks((int64_t)(T + 1) * (T + 2) * g.nb, 256), 256, 0, s)(g, w.g, w.K, w.A);
     if ((st = check_launch(c, "k_mat_assemble"))) return st;
     if (!inverse) {
         if ((st = lu_solve(c, N, D, g.nb, w.A, w.piv, s))) return st;
-        k_mat_store<D><<<nblocks(items, 128), 128, 0, s>>>(g, w.A, G, c->d_status);
+        dep_launch(k_mat_store<D>, nblocks(items, 128), 128, 0, s)(g, w.A, G, c->d_status);
         return check_launch(c, "k_mat_store");
     }
     CUDA_TRY(c, cudaMemsetAsync(w.keys, 0, 8 * (size_t)g.nb * (N + 1), s));
-    k_gj_first<<<dim3(nblocks(N, 128), g.nb), 128, 0, s>>>(N, ld, w.A, w.keys, w.piv);
+    dep_launch(k_gj_first, dim3(nblocks(N, 128), g.nb), 128, 0, s)(N, ld, w.A, w.keys, w.piv);
     const dim3 grid(nblocks(N, 32), nblocks(N, 4 * NG_GJ_ROWS), g.nb);
     for (int col = 0; col < N; ++col) {
-        k_gj_step<<<grid, 128, 0, s>>>(N, ld, col % 2 ? w.A2 : w.A, col % 2 ? w.A : w.A2, col, w.keys, w.piv, c->d_status);
+        dep_launch(k_gj_step, grid, 128, 0, s)(N, ld, col % 2 ? w.A2 : w.A, col % 2 ? w.A : w.A2, col, w.keys, w.piv, c->d_status);
         if (col % 256 == 0 && (st = check_launch(c, "k_gj_step"))) return st;
     }
-    k_gj_apply<false><<<rows, 128, 0, s>>>(N, ld, D, inv, w.piv, w.g, G, nullptr, c->d_status);
+    dep_launch(k_gj_apply<false>, rows, 128, 0, s)(N, ld, D, inv, w.piv, w.g, G, nullptr, c->d_status);
     if ((st = check_launch(c, "k_gj_apply"))) return st;
     return refine(c->d_scalar);   // the inverse's rounding: one step of refinement
 }
@@ -739,13 +739,13 @@ ng_status launch_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S, c
     if (!ws_ext && (st = ensure(c, &c->ws_mat, &c->ws_mat_bytes, need))) return st;
     mat_ws(ws_ext ? ws_ext : c->ws_mat, T, D, g.nb, inverse, &w);
     const int64_t items = (int64_t)(T + 1) * g.nb;
-    k_mat_g<D><<<nblocks(items, 128), 128, 0, s>>>(g, eps, w.g);
+    dep_launch(k_mat_g<D>, nblocks(items, 128), 128, 0, s)(g, eps, w.g);
     if ((st = check_launch(c, "k_mat_g"))) return st;
     const bool warp = D <= 4 && items < (int64_t)c->sms * 128;
     if constexpr (D <= 4) {
-        if (warp) k_mat_K_w<D><<<nblocks(items * 32, 128), 128, 0, s>>>(g, S, w.g, w.K);
+        if (warp) dep_launch(k_mat_K_w<D>, nblocks(items * 32, 128), 128, 0, s)(g, S, w.g, w.K);
     }
-    if (!warp) k_mat_K<D><<<nblocks(items, 128), 128, 0, s>>>(g, S, w.g, w.K);
+    if (!warp) dep_launch(k_mat_K<D>, nblocks(items, 128), 128, 0, s)(g, S, w.g, w.K);
     if ((st = check_launch(c, "k_mat_K"))) return st;
     return mat_solve<D>(c, g, G, w, inverse, s, refine_steps, ref_tol, refined_ok);
 }
@@ -762,20 +762,20 @@ ng_status launch_start(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S,
         // one warp per item: the dense solves while the warps fit the GPU at once, the left-mixing row while a thread
         // per item would leave SMs idle, the lesser columns always (k+1 items per problem)
         const bool ret_w = g.nb <= 4 * c->sms, tv_w = (int64_t)(g.ntau + 1) * g.nb < (int64_t)c->sms * 128;
-        if (ret_w) k_start_ret_w<D><<<g.nb, 32, 0, s>>>(g, G, S, eps, ws, c->d_status);
-        else k_start_ret<D><<<nblocks(g.nb, 64), 64, 0, s>>>(g, G, S, eps, ws, c->d_status);
+        if (ret_w) dep_launch(k_start_ret_w<D>, g.nb, 32, 0, s)(g, G, S, eps, ws, c->d_status);
+        else dep_launch(k_start_ret<D>, nblocks(g.nb, 64), 64, 0, s)(g, G, S, eps, ws, c->d_status);
         if ((st = check_launch(c, "k_start_ret"))) return st;
-        if (tv_w) k_start_tv_w<D><<<nblocks((int64_t)(g.ntau + 1) * g.nb * 32, 128), 128, 0, s>>>(g, G, S, ws, c->d_status);
-        else k_start_tv<D><<<nblocks((int64_t)(g.ntau + 1) * g.nb, 128), 128, 0, s>>>(g, G, S, ws, c->d_status);
+        if (tv_w) dep_launch(k_start_tv_w<D>, nblocks((int64_t)(g.ntau + 1) * g.nb * 32, 128), 128, 0, s)(g, G, S, ws, c->d_status);
+        else dep_launch(k_start_tv<D>, nblocks((int64_t)(g.ntau + 1) * g.nb, 128), 128, 0, s)(g, G, S, ws, c->d_status);
         if ((st = check_launch(c, "k_start_tv"))) return st;
-        k_start_les_w<D><<<(unsigned)((k + 1) * g.nb), 128, 0, s>>>(g, G, S, ws, c->d_status);
+        dep_launch(k_start_les_w<D>, (unsigned)((k + 1) * g.nb), 128, 0, s)(g, G, S, ws, c->d_status);
         return check_launch(c, "k_start_les");
     }
-    k_start_ret<D><<<nblocks(g.nb, 64), 64, 0, s>>>(g, G, S, eps, ws, c->d_status);
+    dep_launch(k_start_ret<D>, nblocks(g.nb, 64), 64, 0, s)(g, G, S, eps, ws, c->d_status);
     if ((st = check_launch(c, "k_start_ret"))) return st;
-    k_start_tv<D><<<nblocks((int64_t)(g.ntau + 1) * g.nb, 128), 128, 0, s>>>(g, G, S, ws, c->d_status);
+    dep_launch(k_start_tv<D>, nblocks((int64_t)(g.ntau + 1) * g.nb, 128), 128, 0, s)(g, G, S, ws, c->d_status);
     if ((st = check_launch(c, "k_start_tv"))) return st;
-    k_start_les<D><<<nblocks((int64_t)(k + 1) * g.nb, 64), 64, 0, s>>>(g, G, S, ws, c->d_status);
+    dep_launch(k_start_les<D>, nblocks((int64_t)(k + 1) * g.nb, 64), 64, 0, s)(g, G, S, ws, c->d_status);
     return check_launch(c, "k_start_les");
 }
 
@@ -784,6 +784,7 @@ ng_status launch_start(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S,
 // K = -F^M and right-hand side Q^M, solved by the same dense LU per problem.
 template <int D>
 __global__ void k_v2_mat_fill(Grid g, HermV F, HermV Q, cplx* ws_g, cplx* ws_K) {
+    dep_wait();
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (item >= (int64_t)(g.ntau + 1) * g.nb) return;
     const int kb = (int)(item % g.nb), m = (int)(item / g.nb);
@@ -808,7 +809,7 @@ ng_status launch_vie2_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV&
     ng_status st = ensure(c, ws, ws_bytes, mat_ws(nullptr, T, D, g.nb, inverse, &w));
     if (st) return st;
     mat_ws(*ws, T, D, g.nb, inverse, &w);
-    k_v2_mat_fill<D><<<nblocks((int64_t)(T + 1) * g.nb, 128), 128, 0, s>>>(g, F, Q, w.g, w.K);
+    dep_launch(k_v2_mat_fill<D>, nblocks((int64_t)(T + 1) * g.nb, 128), 128, 0, s)(g, F, Q, w.g, w.K);
     if ((st = check_launch(c, "k_v2_mat_fill"))) return st;
     return mat_solve<D>(c, g, G, w, inverse, s, refine_steps, ref_tol, refined_ok);
 }
@@ -833,7 +834,7 @@ ng_status vie2_mat_d(ng_ctx* c, const Grid& g, const HermV& G, const HermV& F, c
 template <int D>
 ng_status launch_free(ng_ctx* c, const Grid& g, const HermV& G, const cplx* eps_dev, double scale, cudaStream_t s) {
     const int64_t nel = (g.ntau + 1) + 2 * tri(g.nt + 1) + (int64_t)(g.nt + 1) * (g.ntau + 1);
-    k_free_gf<D><<<nblocks(nel * g.nb, 128), 128, 0, s>>>(g, G, eps_dev, scale);
+    dep_launch(k_free_gf<D>, nblocks(nel * g.nb, 128), 128, 0, s)(g, G, eps_dev, scale);
     return check_launch(c, "k_free_gf");
 }
 
@@ -841,7 +842,7 @@ ng_status do_kreduce(ng_ctx* c, const Grid& g, int tstp, const HermV& L, const H
                      const double* wk = nullptr) {
     const int cnt = tstp < 0 ? g.ntau + 1 : 2 * (tstp + 1) + g.ntau + 1;
     const int64_t warps = (int64_t)cnt * g.nf * g.nf;
-    k_kreduce<<<nblocks(warps * 32, 256), 256, 0, s>>>(g, tstp, L, Gk, wk);
+    dep_launch(k_kreduce, nblocks(warps * 32, 256), 256, 0, s)(g, tstp, L, Gk, wk);
     return check_launch(c, "k_kreduce");
 }
 
@@ -899,18 +900,18 @@ ng_status do_kreduce_rt(ng_ctx* c, const Grid& g, int tstp, const HermV& L, cons
     const int dd = g.nf * g.nf;
     const int nbl = rt->map.first[sh->rank + 1] - rt->map.first[sh->rank];
     const int64_t warps = (int64_t)nbl * cnt * dd;
-    k_kreduce_partial<<<nblocks(warps * 32, 256), 256, 0, s>>>(g, tstp, Gk, nullptr, rt->kb0, (cplx*)sh->send);
+    dep_launch(k_kreduce_partial, nblocks(warps * 32, 256), 256, 0, s)(g, tstp, Gk, nullptr, rt->kb0, (cplx*)sh->send);
     ng_status st = check_launch(c, "k_kreduce_partial");
     if (st) return st;
     if (sh->exchange(sh->user, (size_t)rt->maxb * cnt * dd * sizeof(cplx)) != 0)
         return fail(c, NG_ECOMM, "the exchange of the k-block sums failed (slice %d)", tstp);
-    k_kreduce_combine<<<nblocks((int64_t)cnt * dd, 128), 128, 0, s>>>(g, tstp, L, (const cplx*)sh->recv, sh->nk,
+    dep_launch(k_kreduce_combine, nblocks((int64_t)cnt * dd, 128), 128, 0, s)(g, tstp, L, (const cplx*)sh->recv, sh->nk,
                                                                       sh->nranks, rt->maxb, rt->map, 0);
     return check_launch(c, "k_kreduce_combine");
 }
 ng_status do_sigma(ng_ctx* c, const Grid& g, int tstp, const HermV& S, const HermV& L, const FuncV& U, cudaStream_t s) {
     const int cnt = tstp < 0 ? g.ntau + 1 : 2 * (tstp + 1) + g.ntau + 1;
-    k_sigma2b<<<nblocks((int64_t)cnt * g.nf * g.nf, 128), 128, 0, s>>>(g, tstp, S, L, U);
+    dep_launch(k_sigma2b, nblocks((int64_t)cnt * g.nf * g.nf, 128), 128, 0, s)(g, tstp, S, L, U);
     return check_launch(c, "k_sigma2b");
 }
 // GW launches on slice tstp: local (L = 1, whole-contour views) or on the ring of L momenta
@@ -920,13 +921,13 @@ inline SliceView compact(cplx* buf) { return SliceView{HermV{}, buf}; }
 ng_status do_gw_pol(ng_ctx* c, const Grid& g, int tstp, int L, const SliceView& P, const SliceView& K,
                     const SliceView& Kcc, const SliceView& G, const FuncV& U, cudaStream_t s) {
     const int cnt = tstp < 0 ? g.ntau + 1 : 2 * (tstp + 1) + g.ntau + 1;
-    k_gw_pol<<<nblocks((int64_t)cnt * g.nf * g.nf * L, 128), 128, 0, s>>>(g, tstp, L, P, K, Kcc, G, U);
+    dep_launch(k_gw_pol, nblocks((int64_t)cnt * g.nf * g.nf * L, 128), 128, 0, s)(g, tstp, L, P, K, Kcc, G, U);
     return check_launch(c, "k_gw_pol");
 }
 ng_status do_gw_sigma(ng_ctx* c, const Grid& g, int tstp, int L, const SliceView& S, const SliceView& G,
                       const SliceView& X, const FuncV& U, cudaStream_t s) {
     const int cnt = tstp < 0 ? g.ntau + 1 : 2 * (tstp + 1) + g.ntau + 1;
-    k_gw_sigma<<<nblocks((int64_t)cnt * g.nf * g.nf * L, 128), 128, 0, s>>>(g, tstp, L, S, G, X, U);
+    dep_launch(k_gw_sigma, nblocks((int64_t)cnt * g.nf * g.nf * L, 128), 128, 0, s)(g, tstp, L, S, G, X, U);
     return check_launch(c, "k_gw_sigma");
 }
 // lattice Fourier transform of every element of slice tstp along its L momenta / sites
@@ -946,12 +947,12 @@ ng_status do_kfft(ng_ctx* c, const Grid& g, int tstp, int L, const SliceView& in
     if (smem > 48 * 1024)
         CUDA_TRY(c, cudaFuncSetAttribute(k_kfft_slice, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int thr = std::min(256, std::max(64, vpb * L / 4 / 32 * 32));
-    k_kfft_slice<<<(unsigned)((nvec + vpb - 1) / vpb), thr, smem, s>>>(g, tstp, L, log2L, vpb, in, out, sign, scale);
+    dep_launch(k_kfft_slice, (unsigned)((nvec + vpb - 1) / vpb), thr, smem, s)(g, tstp, L, log2L, vpb, in, out, sign, scale);
     return check_launch(c, "k_kfft_slice");
 }
 ng_status do_hartree(ng_ctx* c, const Grid& g, int tstp, const FuncV& mf, const FuncV& e0, const HermV& L, const FuncV& U,
                      double nbar, cudaStream_t s) {
-    k_hartree<<<nblocks((int64_t)mf.ldk * g.nf * g.nf, 128), 128, 0, s>>>(g, tstp, mf, e0, L, U, nbar);
+    dep_launch(k_hartree, nblocks((int64_t)mf.ldk * g.nf * g.nf, 128), 128, 0, s)(g, tstp, mf, e0, L, U, nbar);
     return check_launch(c, "k_hartree");
 }
 // ---------------------------------------------------------------------------------------
@@ -994,7 +995,7 @@ ng_status histu_sums(ng_ctx* c, const UProb* d_probs, const std::vector<UHost>& 
     tab->src = d_probs;
     tab->n = n;
     tab->status = c->d_status;
-    k_histu_vec<<<dim3(lenp / 128, tab->np, 8 * (NGU_NVEC + 1)), 128, 0, s>>>(*tab);
+    dep_launch(k_histu_vec, dim3(lenp / 128, tab->np, 8 * (NGU_NVEC + 1)), 128, 0, s)(*tab);
     ng_status st = check_launch(c, "k_histu_vec");
     if (st) return st;
     if (histu_launch(*tab, c->sms, s) != cudaSuccess) {
@@ -1040,7 +1041,7 @@ ng_status ustep(ng_ctx* c, const UProb* d_probs, const std::vector<UHost>& info,
             if (need > c->ws_usrc_bytes && (st = ensure(c, &c->ws_usrc, &c->ws_usrc_bytes, 2 * need))) return st;
             tab.src = (cplx*)c->ws_usrc;
         }
-        k_uminv<<<tab.np, 32, 0, s>>>(d_probs, tab, c->d_status);
+        dep_launch(k_uminv, tab.np, 32, 0, s)(d_probs, tab, c->d_status);
         if ((st = check_launch(c, "k_uminv"))) return st;
         long e0 = prof_pair(c, 0);
         if (e0 >= 0) cudaEventRecord(c->ev_pool[e0], s);
@@ -1055,15 +1056,15 @@ ng_status ustep(ng_ctx* c, const UProb* d_probs, const std::vector<UHost>& info,
         }
         HistUTab ht;
         if (digits && (st = histu_sums(c, d_probs, info, active, c0, c1, n, &ht, &digits, s))) return st;
-        if (digits) k_histu_close<<<blk, threads, sizeof(cplx) * threads, s>>>(ht.probs, tab, c->d_status);
-        else k_ubulk<<<blk, threads, sizeof(cplx) * threads, s>>>(d_probs, tab, c->d_status);
+        if (digits) dep_launch(k_histu_close, blk, threads, sizeof(cplx) * threads, s)(ht.probs, tab, c->d_status);
+        else dep_launch(k_ubulk, blk, threads, sizeof(cplx) * threads, s)(d_probs, tab, c->d_status);
         if ((st = check_launch(c, digits ? "k_histu_close" : "k_ubulk"))) return st;
         if (e0 >= 0) cudaEventRecord(c->ev_pool[e0 + 1], s);
         long e1 = prof_pair(c, 1);
         if (e1 >= 0) cudaEventRecord(c->ev_pool[e1], s);
-        k_uboundary_ret<<<tab.np, NG_UBND_THREADS, NG_UBND_SMEM, s>>>(d_probs, tab, c->d_status);
-        k_usrc<<<dim3(tab.nchunk, NG_MAXQ, tab.np), NG_USRC_THREADS, 0, s>>>(d_probs, tab);
-        k_uboundary_les<<<tab.np, NG_UBND_THREADS, NG_UBND_SMEM, s>>>(d_probs, tab, c->d_status);
+        dep_launch(k_uboundary_ret, tab.np, NG_UBND_THREADS, NG_UBND_SMEM, s)(d_probs, tab, c->d_status);
+        dep_launch(k_usrc, dim3(tab.nchunk, NG_MAXQ, tab.np), NG_USRC_THREADS, 0, s)(d_probs, tab);
+        dep_launch(k_uboundary_les, tab.np, NG_UBND_THREADS, NG_UBND_SMEM, s)(d_probs, tab, c->d_status);
         if (e1 >= 0) cudaEventRecord(c->ev_pool[e1 + 1], s);
         if ((st = check_launch(c, "k_uboundary_ret/k_usrc/k_uboundary_les"))) return st;
         if (c->prof) {
@@ -1126,9 +1127,9 @@ ng_status launch_timestep_serial(ng_ctx* c, const Grid& g, int n, const HermV& G
     if (st) return st;
     const cplx* tvq = nullptr;
     if ((st = prep_tvfft(c, g, n, G, S, s, &tvq))) return st;
-    k_step_bulk<D><<<b_tv, thr, 0, s>>>(g, n, G, S, eps, (const cplx*)c->ws_minv, 0, b_tv, 0, tvq, c->d_status);
+    dep_launch(k_step_bulk<D>, b_tv, thr, 0, s)(g, n, G, S, eps, (const cplx*)c->ws_minv, 0, b_tv, 0, tvq, c->d_status);
     if ((st = check_launch(c, "k_step_bulk"))) return st;
-    k_step_serial<D><<<g.nb, NG_BND_THREADS, 0, s>>>(g, n, G, S, eps, c->d_status);
+    dep_launch(k_step_serial<D>, g.nb, NG_BND_THREADS, 0, s)(g, n, G, S, eps, c->d_status);
     return check_launch(c, "k_step_serial");
 }
 
@@ -1184,11 +1185,11 @@ ng_status do_start(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S, con
 }
 ng_status do_extrap(ng_ctx* c, const Grid& g, int n, const HermV& G, cudaStream_t s) {
     const int64_t items = (int64_t)(2 * (n + 2) + g.ntau + 1) * g.nf * g.nf * G.ret.ldk;
-    k_extrapolate<<<nblocks(items, 128), 128, 0, s>>>(g, n, G);
+    dep_launch(k_extrapolate, nblocks(items, 128), 128, 0, s)(g, n, G);
     return check_launch(c, "k_extrapolate");
 }
 ng_status do_distance(ng_ctx* c, const Grid& g, int tstp, const HermV& A, const HermV& B, double* out, cudaStream_t s) {
-    k_distance<<<4 * 152, 256, 0, s>>>(g, tstp, A, B, out);
+    dep_launch(k_distance, 4 * 152, 256, 0, s)(g, tstp, A, B, out);
     return check_launch(c, "k_distance");
 }
 
@@ -1490,10 +1491,10 @@ ng_status ng_observables(ng_ctx* c, const ng_grid* grid, int tstp, ng_herm G, ng
     if ((st = ensure(c, &c->ws_obs, &c->ws_obs_bytes, sizeof(double) * NG_NOBS * (size_t)g.nb))) return st;
     cudaStream_t s = (cudaStream_t)stream;
     if (g.nf > 2) return fail(c, NG_EUNSUPPORTED, "ng_observables supports nf <= 2");
-    if (g.nf == 1) k_observables<1><<<g.nb, NG_OBS_THREADS, 0, s>>>(g, tstp, Gv, Sv, e0, mf, (double*)c->ws_obs);
-    else k_observables<2><<<g.nb, NG_OBS_THREADS, 0, s>>>(g, tstp, Gv, Sv, e0, mf, (double*)c->ws_obs);
+    if (g.nf == 1) dep_launch(k_observables<1>, g.nb, NG_OBS_THREADS, 0, s)(g, tstp, Gv, Sv, e0, mf, (double*)c->ws_obs);
+    else dep_launch(k_observables<2>, g.nb, NG_OBS_THREADS, 0, s)(g, tstp, Gv, Sv, e0, mf, (double*)c->ws_obs);
     if ((st = check_launch(c, "k_observables"))) return st;
-    k_observables_reduce<<<1, NG_OBS_THREADS, 0, s>>>(g.nb, (const double*)c->ws_obs, out_dev);
+    dep_launch(k_observables_reduce, 1, NG_OBS_THREADS, 0, s)(g.nb, (const double*)c->ws_obs, out_dev);
     return check_launch(c, "k_observables_reduce");
 }
 
@@ -1557,7 +1558,7 @@ ng_status ng_kreduce_partial(ng_ctx* c, const ng_grid* grid, int tstp, void* par
     if (wk && ((uintptr_t)wk & 7u)) return fail(c, NG_EINVAL, "wk is not 8-byte aligned");
     const int cnt = tstp < 0 ? g.ntau + 1 : 2 * (tstp + 1) + g.ntau + 1;
     const int64_t warps = (int64_t)((g.nb + NG_KBLK - 1) / NG_KBLK) * cnt * g.nf * g.nf;
-    k_kreduce_partial<<<nblocks(warps * 32, 256), 256, 0, (cudaStream_t)stream>>>(g, tstp, K, wk, k_begin,
+    dep_launch(k_kreduce_partial, nblocks(warps * 32, 256), 256, 0, (cudaStream_t)stream)(g, tstp, K, wk, k_begin,
                                                                                   (cplx*)partial);
     return check_launch(c, "k_kreduce_partial");
 }
@@ -1577,7 +1578,7 @@ ng_status ng_kreduce_combine(ng_ctx* c, const ng_grid* grid, int tstp, ng_herm G
     BlkMap m;
     shard_map(nk, nranks, &m);
     const int cnt = tstp < 0 ? g.ntau + 1 : 2 * (tstp + 1) + g.ntau + 1;
-    k_kreduce_combine<<<nblocks((int64_t)cnt * g.nf * g.nf, 128), 128, 0, (cudaStream_t)stream>>>(
+    dep_launch(k_kreduce_combine, nblocks((int64_t)cnt * g.nf * g.nf, 128), 128, 0, (cudaStream_t)stream)(
         g, tstp, L, (const cplx*)gathered, nk, nranks, shard_maxb(m, nranks), m, weighted ? 1 : 0);
     return check_launch(c, "k_kreduce_combine");
 }
@@ -1862,7 +1863,7 @@ static ng_status run_2b_impl(ng_ctx* c, const ng_grid* grid, ng_herm G, ng_herm 
         if ((st = sigma_slices(-1, -1))) return st;
         // ---- bootstrapping ----
         for (int n = 0; n <= k; ++n) {
-            k_mf_init<<<nblocks((int64_t)dd * epsmf.ldk, 128), 128, 0, s>>>(g, n, mf, e0);
+            dep_launch(k_mf_init, nblocks((int64_t)dd * epsmf.ldk, 128), 128, 0, s)(g, n, mf, e0);
             if ((st = check_launch(c, "k_mf_init"))) return st;
         }
         if ((st = do_start(c, g, Gv, Sv, mf, s))) return st;
@@ -2114,11 +2115,11 @@ void* g_noalloc_addr[64] = {nullptr};
 template <int D>
 ng_status noalloc_start(const Grid& g, const HermV& G, const HermV& S, const FuncV& eps, cplx* ws, int* status,
                         cudaStream_t s) {
-    k_start_ret<D><<<nblocks(g.nb, 64), 64, 0, s>>>(g, G, S, eps, ws, status);
+    dep_launch(k_start_ret<D>, nblocks(g.nb, 64), 64, 0, s)(g, G, S, eps, ws, status);
     if (cudaGetLastError() != cudaSuccess) return NG_ECUDA;
-    k_start_tv<D><<<nblocks((int64_t)(g.ntau + 1) * g.nb, 128), 128, 0, s>>>(g, G, S, ws, status);
+    dep_launch(k_start_tv<D>, nblocks((int64_t)(g.ntau + 1) * g.nb, 128), 128, 0, s)(g, G, S, ws, status);
     if (cudaGetLastError() != cudaSuccess) return NG_ECUDA;
-    k_start_les<D><<<nblocks((int64_t)(g.k + 1) * g.nb, 64), 64, 0, s>>>(g, G, S, ws, status);
+    dep_launch(k_start_les<D>, nblocks((int64_t)(g.k + 1) * g.nb, 64), 64, 0, s)(g, G, S, ws, status);
     if (cudaGetLastError() != cudaSuccess) return NG_ECUDA;
     return NG_OK;
 }
@@ -2205,6 +2206,7 @@ struct ng_batch {
 
 namespace {
 __global__ void k_sandwich(Grid go, HermV O, Grid gi, HermV I, const cplx* V) {
+    dep_wait();
     const int Do = go.nf, Di = gi.nf;
     const int64_t T1 = go.ntau + 1, ntri = tri(go.nt + 1), ntv = (int64_t)(go.nt + 1) * T1;
     const int64_t nel = T1 + 2 * ntri + ntv;
@@ -2246,7 +2248,7 @@ ng_status ng_herm_sandwich(ng_ctx* c, const ng_grid* grid_out, ng_herm Out, cons
     cudaStream_t s = (cudaStream_t)stream;
     CUDA_TRY(c, cudaMemcpyAsync(c->d_eps, V_host, bytes, cudaMemcpyHostToDevice, s));
     const int64_t nel = (go.ntau + 1) + 2 * tri(go.nt + 1) + (int64_t)(go.nt + 1) * (go.ntau + 1);
-    k_sandwich<<<nblocks(nel * go.nf * go.nf, 256), 256, 0, s>>>(go, Ov, gi, Iv, c->d_eps);
+    dep_launch(k_sandwich, nblocks(nel * go.nf * go.nf, 256), 256, 0, s)(go, Ov, gi, Iv, c->d_eps);
     return check_launch(c, "k_sandwich");
 }
 

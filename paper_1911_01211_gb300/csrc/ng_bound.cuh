@@ -34,6 +34,7 @@ __device__ __forceinline__ void bnd1_values(const NgWeights& W, const Grid& g, c
 // NR + r: its partial history
 template <bool SHARED>
 static __global__ void __launch_bounds__(128) k_bnd1_sums(Grid g, int n, HermV G, HermV S, int len, cplx* part) {
+    dep_wait();
     constexpr int NR = NG_B1_ROWS;
     const NgWeights& W = c_W[g.k - 1];
     const int k = W.k, T = g.ntau, m0 = n - k, J = max(n, T) + 1;
@@ -97,6 +98,7 @@ static __global__ void __launch_bounds__(128) k_bnd1_sums(Grid g, int n, HermV G
 #define NG_B1_WARPS 12
 static __global__ void __launch_bounds__(32 * NG_B1_WARPS) k_bnd1_fin(Grid g, int n, HermV G, HermV S, FuncV eps, int nchunk,
                                                                       const cplx* part, int* status) {
+    dep_wait();
     constexpr int NR = NG_B1_ROWS;
     static_assert(NG_B1_WARPS == 2 * NR, "a warp per partial sum");
     const NgWeights& W = c_W[g.k - 1];

@@ -13,10 +13,10 @@ cudaError_t conv_launch(const Grid& g, int n, const HermV& C, const HermV& A, co
     const unsigned nblk = (unsigned)((items + 127) / 128);
     const FRef fr{f.p, f.ldk};
     switch (g.nf) {
-        case 1: k_conv_slice<1><<<nblk, 128, 0, s>>>(g, n, C, A, Acc, fr, B, Bcc, nbe, status); break;
-        case 2: k_conv_slice<2><<<nblk, 128, 0, s>>>(g, n, C, A, Acc, fr, B, Bcc, nbe, status); break;
-        case 4: k_conv_slice<4><<<nblk, 128, 0, s>>>(g, n, C, A, Acc, fr, B, Bcc, nbe, status); break;
-        default: k_conv_slice<8><<<nblk, 128, 0, s>>>(g, n, C, A, Acc, fr, B, Bcc, nbe, status); break;
+        case 1: dep_launch(k_conv_slice<1>, nblk, 128, 0, s)(g, n, C, A, Acc, fr, B, Bcc, nbe, status); break;
+        case 2: dep_launch(k_conv_slice<2>, nblk, 128, 0, s)(g, n, C, A, Acc, fr, B, Bcc, nbe, status); break;
+        case 4: dep_launch(k_conv_slice<4>, nblk, 128, 0, s)(g, n, C, A, Acc, fr, B, Bcc, nbe, status); break;
+        default: dep_launch(k_conv_slice<8>, nblk, 128, 0, s)(g, n, C, A, Acc, fr, B, Bcc, nbe, status); break;
     }
     return cudaGetLastError();
 }

@@ -252,6 +252,7 @@ __device__ __forceinline__ void row_store(const Comp& c, int64_t e, int a, int b
 template <int D>
 __global__ void __launch_bounds__(128) k_conv_slice(Grid g, int n, HermV C, HermV A, HermV Acc, FRef f, HermV B,
                                                     HermV Bcc, int nbe, int* status) {
+    dep_wait();
     constexpr int NW = ConvCols<D>::W, NB = D / NW;
     const NgWeights& W = c_W[g.k - 1];
     const int T = g.ntau;

@@ -76,6 +76,7 @@ struct GwAcc {
 // P, K and K^ddagger on slice tstp (-1: Matsubara) from the fermionic G (g.sig); P and the
 // kernels are bosonic.  L = 1 or the ring size.
 __global__ void k_gw_pol(Grid g, int tstp, int L, SliceView P, SliceView K, SliceView Kcc, SliceView G, FuncV U) {
+    dep_wait();
     const int nf = g.nf, dd = nf * nf;
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int cnt = slice_count(g, tstp);
@@ -143,6 +144,7 @@ __global__ void k_gw_pol(Grid g, int tstp, int L, SliceView P, SliceView K, Slic
 // Sigma on slice tstp (-1: Matsubara) from the fermionic G and the bosonic chi:
 // dW = U(t) chi U(t') formed on the fly, Sigma = Bubble2[G, dW] (same index r on both)
 __global__ void k_gw_sigma(Grid g, int tstp, int L, SliceView S, SliceView G, SliceView X, FuncV U) {
+    dep_wait();
     const int nf = g.nf, dd = nf * nf;
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int cnt = slice_count(g, tstp);
@@ -194,6 +196,7 @@ __global__ void k_gw_sigma(Grid g, int tstp, int L, SliceView S, SliceView G, Sl
 // tstp (whole-contour store or compact buffer).
 __global__ void k_kfft_slice(Grid g, int tstp, int L, int log2L, int vpb, SliceView in, SliceView out, int sign,
                              double scale) {
+    dep_wait();
     extern __shared__ cplx sm_all[];
     cplx* tw = sm_all;
     cplx* sm = sm_all + L;

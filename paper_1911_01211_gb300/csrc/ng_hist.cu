@@ -297,6 +297,7 @@ __device__ __noinline__ void unit_fp64(const Args& a, const Unit& u, int kb, int
 }
 
 __global__ void __launch_bounds__(THREADS, 1) k_hist_mma(const Args a, const __grid_constant__ Maps maps) {
+    dep_wait();
     extern __shared__ __align__(1024) unsigned char sm[];
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sm);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
@@ -576,6 +577,6 @@ cudaError_t hist_launch(const HistWs& ws, const cplx* ret, const cplx* les, cons
     cudaError_t e = cudaFuncSetAttribute(k_hist_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_BYTES);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)(a.nwork < sms ? a.nwork : sms);
-    k_hist_mma<<<grid, THREADS, SM_BYTES, s>>>(a, maps);
+    dep_launch(k_hist_mma, grid, THREADS, SM_BYTES, s)(a, maps);
     return cudaGetLastError();
 }

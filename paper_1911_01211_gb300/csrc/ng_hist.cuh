@@ -71,6 +71,7 @@ __device__ __forceinline__ void hist_digits(cplx x, int F, bool conj, int i, __h
 // scale, and of KK problems (KK = 1: vectors shared by all problems).
 template <int KK>
 static __global__ void __launch_bounds__(256) k_hist_vec(HistWs w, HistRow S) {
+    dep_wait();
     const NgWeights& W = c_W[w.k - 1];
     constexpr int PE = KK == 1 ? NGH_BLK : 256 / KK, NP = NGH_BLK / PE;   // elements of a pass, passes
     __shared__ int smax[KK];

@@ -10,6 +10,7 @@
 static __global__ void __launch_bounds__(128) k_hist_close(Grid g, int n, HermV G, HermV S, FuncV eps, HistWs w,
                                                            const cplx* minv_ws, int nb_pre, int nb_les, int nb_tv,
                                                            const cplx* tvq, int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int k = W.k;
     int blk = blockIdx.x, task;

@@ -371,6 +371,7 @@ __device__ __forceinline__ bool task_warp(const HistUTab& tab, const Task& t, un
 }
 
 __global__ void __launch_bounds__(THREADS, 1) k_histu_mma(const __grid_constant__ HistUTab tab) {
+    dep_wait();
     extern __shared__ __align__(1024) unsigned char sm[];
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sm);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -413,6 +414,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_histu_mma(const __grid_constant_
 cudaError_t histu_launch(const HistUTab& tab, int sms, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(k_histu_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_BYTES);
     if (e != cudaSuccess) return e;
-    k_histu_mma<<<tab.ntask < sms ? tab.ntask : sms, THREADS, SM_BYTES, s>>>(tab);
+    dep_launch(k_histu_mma, tab.ntask < sms ? tab.ntask : sms, THREADS, SM_BYTES, s)(tab);
     return cudaGetLastError();
 }

@@ -28,6 +28,7 @@ __device__ __forceinline__ cplx histu_vec_value(const NgWeights& W, const UProb&
 // block (chunk of 128 elements, problem, 8 vector + output): values, scale and digits; each block finds the
 // vector's largest exponent by itself.  Blocks of vector NGU_NVEC write Y.
 static __global__ void __launch_bounds__(128) k_histu_vec(const __grid_constant__ HistUTab tab) {
+    dep_wait();
     const UProb& p = tab.src[tab.prob[blockIdx.y]];
     const int D = p.g.nf, vec = blockIdx.z >> 3, o = blockIdx.z & 7, n = tab.n, tid = threadIdx.x;
     const int len = (vec == 3 || vec == 4 ? p.g.ntau + 1 : n) * D;
@@ -193,6 +194,7 @@ __device__ __forceinline__ void u_close_block(const HistUProb& P, int n, int lbl
     ust(dst, task == 1 ? (int64_t)n * (P.g.ntau + 1) + m : tri(n) + m, D, a, b, 0, y);
 }
 static __global__ void __launch_bounds__(256) k_histu_close(const HistUProb* probs, UTable tab, int* status) {
+    dep_wait();
     int i = 0;
     while (i + 1 < tab.np && (int)blockIdx.x >= tab.start[i + 1]) ++i;
     const HistUProb& P = probs[i];

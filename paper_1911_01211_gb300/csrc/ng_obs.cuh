@@ -17,6 +17,7 @@
 template <int D>
 __global__ void __launch_bounds__(NG_OBS_THREADS) k_observables(Grid g, int n, HermV G, HermV S, FuncV eps0,
                                                                 FuncV epsmf, double* ws) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int k = W.k;
     const int kb = blockIdx.x, t = threadIdx.x;
@@ -55,6 +56,7 @@ __global__ void __launch_bounds__(NG_OBS_THREADS) k_observables(Grid g, int n, H
 
 // batch average in a fixed order; one block
 __global__ void k_observables_reduce(int nb, const double* ws, double* out) {
+    dep_wait();
     __shared__ double red[NG_OBS_THREADS];
     for (int q = 0; q < NG_NOBS; ++q) {
         double s = 0.0;

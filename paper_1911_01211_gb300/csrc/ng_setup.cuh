@@ -66,6 +66,7 @@ __device__ __forceinline__ void fermi_terms(double e, double beta, double tau, d
 // ----------------------------------------------------------------------------------------
 template <int D>
 __global__ void k_free_gf(Grid g, HermV G, const cplx* eps_dev, double scale) {
+    dep_wait();
     const int64_t nel_tri = tri(g.nt + 1);
     const int64_t nel_tv = (int64_t)(g.nt + 1) * (g.ntau + 1);
     const int64_t nel = (g.ntau + 1) + 2 * nel_tri + nel_tv;
@@ -146,6 +147,7 @@ __global__ void k_free_gf(Grid g, HermV G, const cplx* eps_dev, double scale) {
 // ----------------------------------------------------------------------------------------
 template <int D>
 __global__ void k_mat_g(Grid g, FuncV eps, cplx* ws_g) {
+    dep_wait();
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (item >= (int64_t)(g.ntau + 1) * g.nb) return;
     const int kb = (int)(item % g.nb), m = (int)(item / g.nb);
@@ -238,6 +240,7 @@ __device__ __forceinline__ Mat<D> warp_sum_all(Mat<D> x) {
 
 template <int D>
 __global__ void k_mat_K(Grid g, HermV S, const cplx* ws_g, cplx* ws_K) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (item >= (int64_t)(g.ntau + 1) * g.nb) return;
@@ -252,6 +255,7 @@ __global__ void k_mat_K(Grid g, HermV S, const cplx* ws_g, cplx* ws_K) {
 // thread per (problem, block row m, block column c).
 template <int D>
 __global__ void k_mat_assemble(Grid g, const cplx* ws_g, const cplx* ws_K, cplx* ws_A) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int T = g.ntau, k = W.k;
     const int N = (T + 1) * D, ldA = N + D;
@@ -368,6 +372,7 @@ __device__ void lu_substitute(const cplx* A, int ld, int N, cplx* B, int ldb, in
 // Shared memory: panel N x PB, NG_LU_TRI * nrhs values, a reduction value and index per warp.
 template <int PB>
 __global__ void __launch_bounds__(NG_LU_THREADS) k_lu_solve(int N, int nrhs, cplx* ws_A, int* piv, int* status) {
+    dep_wait();
     const int ld = N + nrhs;
     cplx* A = ws_A + (int64_t)blockIdx.x * N * ld;
     int* pv = piv + (int64_t)blockIdx.x * N;
@@ -482,6 +487,7 @@ __device__ __forceinline__ unsigned long long gj_key(cplx x, int r) {
     return ((unsigned long long)__double_as_longlong(cabs2(x)) & ~0xffffull) | (unsigned)(0xffff - r);
 }
 __global__ void k_gj_first(int N, int ld, const cplx* ws_A, unsigned long long* keys, int* perm) {
+    dep_wait();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= N) return;
     perm[(int64_t)blockIdx.y * N + r] = r;
@@ -490,6 +496,7 @@ __global__ void k_gj_first(int N, int ld, const cplx* ws_A, unsigned long long* 
 #define NG_GJ_ROWS 8
 __global__ void __launch_bounds__(128) k_gj_step(int N, int ld, const cplx* src_, cplx* dst_, int c, unsigned long long* keys,
                                                  int* perm, int* status) {
+    dep_wait();
     const int pb = blockIdx.z, j = blockIdx.x * 32 + (threadIdx.x & 31);
     const int r0 = (blockIdx.y * 4 + (threadIdx.x >> 5)) * NG_GJ_ROWS;
     const cplx* src = src_ + (int64_t)pb * N * ld;
@@ -533,6 +540,7 @@ __global__ void __launch_bounds__(128) k_gj_step(int N, int ld, const cplx* src_
 __device__ __forceinline__ cplx mat_resid_el(cplx gg, cplx kg, cplx gm) { return csub(cadd(gg, kg), gm); }
 template <int D>
 __global__ void k_mat_resid(Grid g, const cplx* ws_g, const cplx* ws_K, HermV G, cplx* ws_r) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (item >= (int64_t)(g.ntau + 1) * g.nb) return;
@@ -550,6 +558,7 @@ __global__ void k_mat_resid(Grid g, const cplx* ws_g, const cplx* ws_K, HermV G,
 // serial sums on a few SMs (one problem, ntau = 200, nf = 2: 331 -> 20 us)
 template <int D>
 __global__ void __launch_bounds__(128) k_mat_resid_w(Grid g, const cplx* ws_g, const cplx* ws_K, HermV G, cplx* ws_r) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int64_t item = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (item >= (int64_t)(g.ntau + 1) * g.nb) return;
@@ -563,6 +572,7 @@ __global__ void __launch_bounds__(128) k_mat_resid_w(Grid g, const cplx* ws_g, c
 }
 template <int D>
 __global__ void __launch_bounds__(128) k_mat_K_w(Grid g, HermV S, const cplx* ws_g, cplx* ws_K) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int64_t item = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (item >= (int64_t)(g.ntau + 1) * g.nb) return;
@@ -582,6 +592,7 @@ __device__ __forceinline__ int64_t mat_offset(const Comp& mat, int nrhs, int row
 // *dsum += sum |x|
 __global__ void __launch_bounds__(NG_LU_THREADS) k_lu_resolve(Grid g, int N, int nrhs, const cplx* ws_A, const int* piv,
                                                               cplx* ws_r, HermV G, double* dsum) {
+    dep_wait();
     const int ld = N + nrhs;
     const cplx* A = ws_A + (int64_t)blockIdx.x * N * ld;
     const int* p = piv + (int64_t)blockIdx.x * N;
@@ -621,6 +632,7 @@ __global__ void __launch_bounds__(NG_LU_THREADS) k_lu_resolve(Grid g, int N, int
 template <bool ADD>
 __global__ void __launch_bounds__(128) k_gj_apply(int N, int ld, int nrhs, const cplx* inv_, const int* perm, const cplx* ws_r, HermV G,
                                                   double* dsum, int* status) {
+    dep_wait();
     const int64_t item = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (item >= (int64_t)N * nrhs) return;
     const int pb = blockIdx.y, lane = threadIdx.x & 31, row = (int)(item / nrhs), b = (int)(item % nrhs);
@@ -647,6 +659,7 @@ __global__ void __launch_bounds__(128) k_gj_apply(int N, int ld, int nrhs, const
 
 template <int D>
 __global__ void k_mat_store(Grid g, const cplx* ws_A, HermV G, int* status) {
+    dep_wait();
     const int T = g.ntau, N = (T + 1) * D, ld = N + D;
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (item >= (int64_t)(T + 1) * g.nb) return;
@@ -667,6 +680,7 @@ __global__ void k_mat_store(Grid g, const cplx* ws_A, HermV G, int* status) {
 // the workspace receives inv(M[1..k][1..k]) (kD x kD) and the blocks M[n][0].
 template <int D>
 __global__ void k_start_ret(Grid g, HermV G, HermV S, FuncV eps, cplx* ws_st, int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int kb = blockIdx.x * blockDim.x + threadIdx.x;
     if (kb >= g.nb) return;
@@ -754,6 +768,7 @@ __device__ void start_apply(const cplx* st_ws, int k, const Mat<D>* q, const Mat
 
 template <int D>
 __global__ void k_start_tv(Grid g, HermV G, HermV S, const cplx* ws_st, int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (item >= (int64_t)(g.ntau + 1) * g.nb) return;
@@ -772,6 +787,7 @@ __global__ void k_start_tv(Grid g, HermV G, HermV S, const cplx* ws_st, int* sta
 
 template <int D>
 __global__ void k_start_les(Grid g, HermV G, HermV S, const cplx* ws_st, int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int k = W.k, N = k * D;
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -808,6 +824,7 @@ __device__ __forceinline__ Mat<D> start_matrix_el(const NgWeights& W, const Grid
 
 template <int D>
 __global__ void __launch_bounds__(32) k_start_ret_w(Grid g, HermV G, HermV S, FuncV eps, cplx* ws_st, int* status) {
+    dep_wait();
     constexpr int NM = NG_KMAX * D;
     const NgWeights& W = c_W[g.k - 1];
     const int kb = blockIdx.x, lane = threadIdx.x, k = W.k, N = k * D;
@@ -911,6 +928,7 @@ __device__ inline int64_t start_el_les(const Grid&, int m, int n) { return tri(n
 
 template <int D>
 __global__ void __launch_bounds__(128) k_start_tv_w(Grid g, HermV G, HermV S, const cplx* ws_st, int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int64_t item = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (item >= (int64_t)(g.ntau + 1) * g.nb) return;
@@ -931,6 +949,7 @@ __global__ void __launch_bounds__(128) k_start_tv_w(Grid g, HermV G, HermV S, co
 
 template <int D>
 __global__ void __launch_bounds__(128) k_start_les_w(Grid g, HermV G, HermV S, const cplx* ws_st, int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int k = W.k, N = k * D, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int kb = blockIdx.x % g.nb, n = blockIdx.x / g.nb;   // one block: a warp per source row in turn

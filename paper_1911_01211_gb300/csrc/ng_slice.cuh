@@ -65,6 +65,7 @@ __device__ __forceinline__ cplx kblock_sum(const cplx* p, const double* wk, int 
 
 // Single GPU holding all nb problems: one warp per (slice element, a, b).
 __global__ void k_kreduce(Grid g, int tstp, HermV Gloc, HermV Gk, const double* wk) {
+    dep_wait();
     const int dd = g.nf * g.nf;
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -85,6 +86,7 @@ __global__ void k_kreduce(Grid g, int tstp, HermV Gloc, HermV Gk, const double* 
 // of NG_KBLK); out[(bl * cnt + i) * dd + ab] for the local blocks bl = 0..nblk_local-1.
 // One warp per (local block, slice element, a, b).
 __global__ void k_kreduce_partial(Grid g, int tstp, HermV Gk, const double* wk, int kb0, cplx* out) {
+    dep_wait();
     const int dd = g.nf * g.nf;
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -107,6 +109,7 @@ __global__ void k_kreduce_partial(Grid g, int tstp, HermV Gk, const double* wk, 
 // count, map.first[r]: first global block of rank r (r = 0..nranks).
 __global__ void k_kreduce_combine(Grid g, int tstp, HermV Gloc, const cplx* gathered, int nk, int nranks, int maxb,
                                   BlkMap map, int weighted) {
+    dep_wait();
     const int dd = g.nf * g.nf;
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int cnt = slice_count(g, tstp);
@@ -130,6 +133,7 @@ __global__ void k_kreduce_combine(Grid g, int tstp, HermV Gloc, const cplx* gath
 //   Sigma^M_ab(tau)  = -U_{-1}^2 G^M_ab(tau)^2 G^M_ba(-tau)
 // one thread per (slice element, a, b); G and Sigma have ldk = 1.
 __global__ void k_sigma2b(Grid g, int tstp, HermV S, HermV G, FuncV U) {
+    dep_wait();
     const int nf = g.nf, dd = nf * nf;
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int cnt = slice_count(g, tstp);
@@ -177,6 +181,7 @@ __global__ void k_sigma2b(Grid g, int tstp, HermV S, HermV G, FuncV U) {
 
 // eps_mf_kb(n) = eps0_kb(n) + U_n diag(Re rho_ii - nbar); one thread per (problem, a, b)
 __global__ void k_hartree(Grid g, int tstp, FuncV epsmf, FuncV eps0, HermV G, FuncV U, double nbar) {
+    dep_wait();
     const int nf = g.nf, dd = nf * nf;
     const int ldk = epsmf.ldk;
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -196,6 +201,7 @@ __global__ void k_hartree(Grid g, int tstp, FuncV epsmf, FuncV eps0, HermV G, Fu
 // Predictor (Eq. polyextrap): slice n+1 from slices n-k..n; one thread per
 // (slice element of n+1, a, b, problem).
 __global__ void k_extrapolate(Grid g, int n, HermV G) {
+    dep_wait();
     const int nf = g.nf, dd = nf * nf, k = g.k;
     const double* Cw = c_W[k - 1].C;
     const int N1 = n + 1;
@@ -249,6 +255,7 @@ __global__ void k_extrapolate(Grid g, int n, HermV G) {
 
 // out += sum |A - B| over slice tstp, all problems (Eq. distancenorm)
 __global__ void k_distance(Grid g, int tstp, HermV A, HermV B, double* out) {
+    dep_wait();
     const int dd = g.nf * g.nf;
     const int ldk = A.ret.ldk;
     const int cnt = slice_count(g, tstp);
@@ -270,6 +277,7 @@ __global__ void k_distance(Grid g, int tstp, HermV A, HermV B, double* out) {
 
 // bootstrapping initial guess eps_mf(n) = eps_mf(-1) - eps0(-1) + eps0(n)
 __global__ void k_mf_init(Grid g, int n, FuncV epsmf, FuncV eps0) {
+    dep_wait();
     const int dd = g.nf * g.nf, ldk = epsmf.ldk;
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (item >= (int64_t)dd * ldk) return;

@@ -252,6 +252,7 @@ __device__ __forceinline__ void les_item(const NgWeights& W, const Grid& g, cons
 // holds D x D complex per problem
 template <int D>
 __global__ void k_minv_step(Grid g, int n, HermV S, FuncV eps, cplx* minv_ws, int* status) {
+    dep_wait();
     const int kb = blockIdx.x * blockDim.x + threadIdx.x;
     if (kb >= g.nb) return;
     const NgWeights& W = c_W[g.k - 1];
@@ -277,6 +278,7 @@ __device__ __forceinline__ Mat<D> ld_minv(const cplx* minv_ws, int kb) {
 template <int D>
 __global__ void __launch_bounds__(128, D == 1 ? 6 : 1) k_step_bulk(Grid g, int n, HermV G, HermV S, FuncV eps, const cplx* minv_ws,
                                                    int nb_les, int nb_tv, int nb_ret, const cplx* tvq, int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     int blk = blockIdx.x;
     int task;
@@ -609,6 +611,7 @@ __device__ void les_steps_w(const NgWeights& W, const Grid& g, int n, const Herm
 template <int D>
 __global__ void __launch_bounds__(NG_BND_THREADS) k_step_boundary(Grid g, int n, HermV G, HermV S, FuncV eps,
                                                                   int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int k = W.k;
     const int kb = blockIdx.x;
@@ -669,6 +672,7 @@ __global__ void __launch_bounds__(NG_BND_THREADS) k_step_boundary(Grid g, int n,
 template <int D>
 __global__ void __launch_bounds__(NG_BND_THREADS) k_step_serial(Grid g, int n, HermV G, HermV S, FuncV eps,
                                                                 int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int k = W.k;
     const int kb = blockIdx.x;

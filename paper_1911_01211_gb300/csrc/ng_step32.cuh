@@ -233,6 +233,7 @@ template <int D>
 __global__ void __launch_bounds__(128) k_step_bulk32(Grid g, int n, HermV G, HermV S, HermV32 G32, HermV32 S32,
                                                      FuncV eps, const cplx* minv_ws, int nb_les, int nb_tv,
                                                      int nb_ret, const cplx* tvq, int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     int blk = blockIdx.x;
     int task;
@@ -256,6 +257,7 @@ __global__ void __launch_bounds__(128) k_step_bulk32(Grid g, int n, HermV G, Her
 // FP32 copies of slices [n0, n1] of a contour function (mat when n0 = -1); one thread per
 // (element, orbital pair, problem) over the slices' ret rows, les columns and tv rows.
 __global__ void k_shadow(Grid g, int n0, int n1, HermV X, HermV32 Y, int ldk) {
+    dep_wait();
     const int dd = g.nf * g.nf;
     const int T1 = g.ntau + 1;
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -450,6 +452,7 @@ __device__ __forceinline__ void les_item32p(const NgWeights& W, const Grid& g, c
 __global__ void __launch_bounds__(128, NG_F32P_MINB) k_step_bulk32p(Grid g, int n, HermV G, HermV S, HermV32 G32, HermV32 S32,
                                                       const cplx* minv_ws, int nb_les, int nb_tv, int nb_ret,
                                                       const cplx* tvq, int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     int blk = blockIdx.x;
     int task;

@@ -258,6 +258,7 @@ template <int D>
 __global__ void __launch_bounds__(128, D == 1 ? 6 : 1) k_step_bulkdf(Grid g, int n, HermV G, HermV S, HermVdf Gd, HermVdf Sd,
                                                      const cplx* minv_ws, int nb_les, int nb_tv, int nb_ret,
                                                      const cplx* tvq, int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     int blk = blockIdx.x;
     int task;
@@ -280,6 +281,7 @@ __global__ void __launch_bounds__(128, D == 1 ? 6 : 1) k_step_bulkdf(Grid g, int
 
 // double-float copies of slices [n0, n1] (mat when n0 = -1), layout as k_shadow
 __global__ void k_shadow_df(Grid g, int n0, int n1, HermV X, HermVdf Y, int ldk) {
+    dep_wait();
     const int dd = g.nf * g.nf;
     const int T1 = g.ntau + 1;
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

@@ -53,6 +53,7 @@ __device__ __forceinline__ cplx q_tv_lanes(const NgWeights& W, const Grid& g, co
 template <int P>
 static __global__ void __launch_bounds__(128) k_step_bulk_q(Grid g, int n, HermV G, HermV S, FuncV eps, const cplx* minv_ws,
                                                             int w_pre, int c_les, int c_tv, int c_ret, const cplx* tvq, int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     constexpr int Q = 32 / P;
     const int k = W.k, T = g.ntau, lane = threadIdx.x & 31, q = lane % Q, p = lane / Q;

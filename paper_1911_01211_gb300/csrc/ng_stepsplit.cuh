@@ -239,6 +239,7 @@ __host__ __device__ constexpr int bnd_pre_scratch() { return (NG_KMAX * D) * (NG
 // one warp (block of 32) per problem
 template <int D>
 __global__ void __launch_bounds__(32) k_bnd_pre(Grid g, int n, HermV G, HermV S, FuncV eps, int* status) {
+    dep_wait();
     __shared__ cplx sh[bnd_pre_scratch<D>()];
     bnd_pre_warp<D>(c_W[g.k - 1], g, n, G, S, eps, blockIdx.x, sh, threadIdx.x, status);
 }
@@ -252,6 +253,7 @@ template <int D>
 __global__ void __launch_bounds__(128, 1) k_step_bulk_w(Grid g, int n, HermV G, HermV S, FuncV eps,
                                                      const cplx* minv_ws, int64_t w_pre, int64_t w_les,
                                                      int64_t w_tv, int64_t w_ret, int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     int64_t item = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -277,6 +279,7 @@ __global__ void __launch_bounds__(128, 1) k_step_bulk_w(Grid g, int n, HermV G, 
 // part[((r nb + kb) nchunk + c) 2 D^2 ...]: the source, then the partial history over l < m0
 template <int D>
 __global__ void __launch_bounds__(NG_BND_THREADS) k_bnd_src(Grid g, int n, HermV G, HermV S, int nchunk, cplx* part) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int k = W.k;
     const bool full = (n <= 2 * k);
@@ -305,6 +308,7 @@ __global__ void __launch_bounds__(NG_BND_THREADS) k_bnd_src(Grid g, int n, HermV
 template <int D>
 __global__ void __launch_bounds__(32) k_bnd_fin(Grid g, int n, HermV G, HermV S, FuncV eps, int nchunk,
                                                 const cplx* part, int* status) {
+    dep_wait();
     const int kb = blockIdx.x, lane = threadIdx.x;
     const NgWeights& W = c_W[g.k - 1];
     const int k = W.k;

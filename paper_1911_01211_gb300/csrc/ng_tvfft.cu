@@ -27,6 +27,7 @@ namespace {
 constexpr int kThreads = 256;
 
 __global__ void k_twiddle(cplx* tw, int L) {
+    dep_wait();
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= L / 2) return;
     double s, c;
@@ -76,6 +77,7 @@ __device__ __forceinline__ cplx s_value(const NgWeights& W, const Grid& g, int64
 
 // spectra of the nf^2 elements of a shared S: FS[e L + frequency]
 __global__ void __launch_bounds__(1024) k_tvsrc_s(Grid g, NgWeights W, int n, Comp Stv, const cplx* tw, int L, cplx* FS) {
+    dep_wait();
     extern __shared__ cplx sm[];
     const int lg = 31 - __clz(L), e = blockIdx.x;
     for (int i = threadIdx.x; i < L; i += blockDim.x)
@@ -90,6 +92,7 @@ __global__ void __launch_bounds__(1024) k_tvsrc_s(Grid g, NgWeights W, int n, Co
 template <int D>
 __global__ void __launch_bounds__(kThreads) k_tvsrc_fft(Grid g, NgWeights W, int n, Comp Stv, Comp Gmat, const cplx* tw, int L,
                                                         const cplx* FSg, cplx* Q) {
+    dep_wait();
     extern __shared__ cplx sm[];
     constexpr int DD = D * D;
     cplx* FK = sm;            // [c b][L]: reversed K_cb, then the product P_ab in place
@@ -158,12 +161,12 @@ cudaError_t launch_d(const Grid& g, const NgWeights& W, int n, const Comp& Stv, 
     if (shared) {
         const size_t sm = sizeof(cplx) * (size_t)L;
         if ((e = cudaFuncSetAttribute(k_tvsrc_s, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
-        k_tvsrc_s<<<D * D, L >= 2048 ? 1024 : L / 2, sm, s>>>(g, W, n, Stv, tw, L, FS);
+        dep_launch(k_tvsrc_s, D * D, L >= 2048 ? 1024 : L / 2, sm, s)(g, W, n, Stv, tw, L, FS);
         if ((e = cudaGetLastError())) return e;
     }
     const size_t sm = shared ? one : 2 * one;
     if ((e = cudaFuncSetAttribute(k_tvsrc_fft<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
-    k_tvsrc_fft<D><<<g.nb, kThreads, sm, s>>>(g, W, n, Stv, Gmat, tw, L, FS, Q);
+    dep_launch(k_tvsrc_fft<D>, g.nb, kThreads, sm, s)(g, W, n, Stv, Gmat, tw, L, FS, Q);
     return cudaGetLastError();
 }
 
@@ -188,7 +191,7 @@ bool tvfft_supported(int nf, int ntau) {
 }
 
 cudaError_t tvfft_twiddles(cplx* tw, int L, cudaStream_t s) {
-    k_twiddle<<<(L / 2 + 255) / 256, 256, 0, s>>>(tw, L);
+    dep_launch(k_twiddle, (L / 2 + 255) / 256, 256, 0, s)(tw, L);
     return cudaGetLastError();
 }
 

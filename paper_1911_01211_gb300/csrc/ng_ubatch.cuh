@@ -65,6 +65,7 @@ __device__ __forceinline__ cplx ules(const HermV& X, int j, int n, int D, int a,
 
 // M_n^-1 of every active problem: one warp per problem builds M_n and solves M_n X = 1
 __global__ void __launch_bounds__(32) k_uminv(const UProb* probs, UTable tab, int* status) {
+    dep_wait();
     if (blockIdx.x >= tab.np) return;
     const UProb& P = probs[tab.prob[blockIdx.x]];
     const NgWeights& W = c_W[P.g.k - 1];
@@ -234,6 +235,7 @@ __device__ __forceinline__ void u_bulk_block(const UProb& P, int n, int lblk, in
 }
 
 __global__ void __launch_bounds__(256) k_ubulk(const UProb* probs, UTable tab, int* status) {
+    dep_wait();
     // find the problem of this block (tables are short)
     int i = 0;
     while (i + 1 < tab.np && (int)blockIdx.x >= tab.start[i + 1]) ++i;
@@ -301,6 +303,7 @@ __device__ void u_stepmat(const NgWeights& W, const UProb& P, int m, cplx* out) 
 // before the serial chain, whose steps are then element-parallel products: FP64 is issued per
 // warp instruction on this part, so one thread doing them alone took as long as a whole warp.
 __global__ void __launch_bounds__(NG_UBND_THREADS) k_uboundary_ret(const UProb* probs, UTable tab, int* status) {
+    dep_wait();
     const UProb& P = probs[tab.prob[blockIdx.x]];
     const NgWeights& W = c_W[P.g.k - 1];
     const Grid& g = P.g;
@@ -354,6 +357,7 @@ __global__ void __launch_bounds__(NG_UBND_THREADS) k_uboundary_ret(const UProb* 
 // of every active problem, spread over blocks (chunk, row, problem); within a block, groups of
 // D^2 threads take the summation indices in turn and are combined in a fixed order.
 __global__ void __launch_bounds__(NG_USRC_THREADS) k_usrc(const UProb* probs, UTable tab) {
+    dep_wait();
     const int i = blockIdx.z, r = blockIdx.y, ch = blockIdx.x;
     const UProb& P = probs[tab.prob[i]];
     const NgWeights& W = c_W[P.g.k - 1];
@@ -395,6 +399,7 @@ __global__ void __launch_bounds__(NG_USRC_THREADS) k_usrc(const UProb* probs, UT
 }
 
 __global__ void __launch_bounds__(NG_UBND_THREADS) k_uboundary_les(const UProb* probs, UTable tab, int* status) {
+    dep_wait();
     const UProb& P = probs[tab.prob[blockIdx.x]];
     const NgWeights& W = c_W[P.g.k - 1];
     const Grid& g = P.g;

@@ -298,6 +298,7 @@ template <int D>
 __global__ void __launch_bounds__(128, 1)
     k_v2_bulk_w(Grid g, int n, HermV G, HermV F, HermV Fcc, HermV Q, int64_t w_les, int64_t w_tv, int64_t w_ret,
                 int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     __shared__ cplx sh[4][D <= 2 ? 1 : 2 * D * D + D];   // blockDim.x = 128: four warps
     int64_t item = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -320,6 +321,7 @@ template <int D>
 __global__ void __launch_bounds__(128, D == 1 ? 6 : 1)
     k_v2_bulk(Grid g, int n, HermV G, HermV F, HermV Fcc, HermV Q, int nb_ret, int nb_tv, int nb_les, const cplx* tvq,
               int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     int blk = blockIdx.x, task;
     if (blk < nb_les) task = 0;
@@ -349,6 +351,7 @@ __global__ void __launch_bounds__(128, D == 1 ? 6 : 1)
 static __global__ void __launch_bounds__(128)
     k_v2_hist_close(Grid g, int n, HermV G, HermV F, HermV Fcc, HermV Q, HistWs w, int nb_tv, int nb_les, const cplx* tvq,
                     int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int k = W.k;
     int blk = blockIdx.x, task;
@@ -401,6 +404,7 @@ static __global__ void __launch_bounds__(128)
 template <int D>
 __global__ void __launch_bounds__(NG_BND_THREADS) k_v2_diag(Grid g, int n, HermV G, HermV F, HermV Fcc, HermV Q,
                                                              int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int kb = blockIdx.x, t = threadIdx.x;
     __shared__ cplx red[NG_BND_THREADS * D * D];
@@ -429,6 +433,7 @@ __global__ void __launch_bounds__(NG_BND_THREADS) k_v2_diag(Grid g, int n, HermV
 // lesser start-up: the workspace receives inv(M[1..k][1..k]) (kD x kD) and the blocks M[n][0].
 template <int D>
 __global__ void k_v2_start_ret(Grid g, HermV G, HermV F, HermV Fcc, HermV Q, cplx* ws, int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int kb = blockIdx.x * blockDim.x + threadIdx.x;
     if (kb >= g.nb) return;
@@ -510,6 +515,7 @@ __device__ void v2_start_apply(const cplx* ws, int k, const Mat<D>* q, const Mat
 // sources Q^tv(n,m) - (C^tv_2 + C^tv_3)[F, 1, G^M](n,m)
 template <int D>
 __global__ void k_v2_start_tv(Grid g, HermV G, HermV F, HermV Q, const cplx* ws, int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (item >= (int64_t)(g.ntau + 1) * g.nb) return;
@@ -531,6 +537,7 @@ __global__ void k_v2_start_tv(Grid g, HermV G, HermV F, HermV Q, const cplx* ws,
 // m > n); rows m <= n are stored
 template <int D>
 __global__ void k_v2_start_les(Grid g, HermV G, HermV F, HermV Fcc, HermV Q, const cplx* ws, int* status) {
+    dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     const int k = W.k, N = k * D;
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
