@@ -463,7 +463,7 @@ ng_status launch_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const
         dep_launch(kernel, nblocks(warps * 32, thr), thr, 0, s)(g, n, G, S, eps, (const cplx*)c->ws_minv, (int)w_pre, c_les, c_tv,
                                                         c_ret, tvq, c->d_status);
     } else if (warp) {
-        dep_launch(k_step_bulk_w<D>, nblocks((w_pre + items) * 32, thr), thr, 0, s)(g, n, G, S, eps, (const cplx*)c->ws_minv,
+        dep_launch(k_step_bulk_w<D>, nblocks((w_pre + (w_pre & 1) + items + it_les) * 32, thr), thr, 0, s)(g, n, G, S, eps, (const cplx*)c->ws_minv,
                                                                            w_pre, it_les, it_tv, it_ret, c->d_status);
     } else {
         dep_launch(k_step_bulk<D>, b_les + b_tv + b_ret, thr, 0, s)(g, n, G, S, eps, (const cplx*)c->ws_minv, b_les, b_tv,

@@ -166,25 +166,36 @@ __device__ __forceinline__ void tv_item_w(const NgWeights& W, const Grid& g, con
     }
 }
 
+// The lesser item has three sums, the others one or two, and a small batch has about one warp for each FP64 pipe: two
+// warps share it, one (half 0) taking the history and the closing step, the other C^<_1 and C^<_3, which it
+// leaves at xq[lane] (barrier `bar` of the two).  Run of the dimer to n = 200, ntau = 200: 63.5 -> 62.1 ms.
 template <int D>
 __device__ __forceinline__ void les_item_w(const NgWeights& W, const Grid& g, const HermV& G, const HermV& S,
-                                           const cplx* minv_ws, int n, int m, int kb, int lane, int* status) {
+                                           const cplx* minv_ws, int n, int m, int kb, int lane, int half, cplx* xq, int bar,
+                                           int* status) {
     const int k = W.k, T = g.ntau;
-    // C^<_1[G,1,Sigma](m,n) = int_0^{t_m} G^R(m,s) Sigma^<(s,n)
-    Mat<D> c1 = mzero<D>();
-    if (m <= k) {
-        for (int j = lane; j <= k; j += 32)
-            mfma<D>(c1, mscal<D>(W.greg[m][j], gretx<D>(G, m, j, kb)), ld<D>(S.les, tri(n) + j, kb));
-    } else {
-        greg_for_lanes(W, m, m, lane, [&](int j, double w) {
-            mfma<D>(c1, mscal<D>(w, gret<D>(G, m, j, kb)), ld<D>(S.les, tri(n) + j, kb));
+    auto sync = [&] { asm volatile("bar.sync %0, 64;" ::"r"(bar) : "memory"); };
+    if (half == 1) {
+        // C^<_1[G,1,Sigma](m,n) = int_0^{t_m} G^R(m,s) Sigma^<(s,n)
+        Mat<D> c1 = mzero<D>();
+        if (m <= k) {
+            for (int j = lane; j <= k; j += 32)
+                mfma<D>(c1, mscal<D>(W.greg[m][j], gretx<D>(G, m, j, kb)), ld<D>(S.les, tri(n) + j, kb));
+        } else {
+            greg_for_lanes(W, m, m, lane, [&](int j, double w) {
+                mfma<D>(c1, mscal<D>(w, gret<D>(G, m, j, kb)), ld<D>(S.les, tri(n) + j, kb));
+            });
+        }
+        // sum_j w_{T,j} G^tv(m,j) [Sigma^tv(n,T-j)]^dagger
+        Mat<D> c3 = mzero<D>();
+        greg_for_lanes(W, T, T, lane, [&](int j, double w) {
+            mfma_db<D>(c3, mscal<D>(w, gtv<D>(G, g, m, j, kb)), gtv<D>(S, g, n, T - j, kb));
         });
+        const cplx c1e = warp_rsum<D>(c1, lane), c3e = warp_rsum<D>(c3, lane);
+        xq[lane] = csub(cscal(g.h, cmuli(c1e)), cscal((double)g.sig * g.htau, c3e));
+        sync();
+        return;
     }
-    // sum_j w_{T,j} G^tv(m,j) [Sigma^tv(n,T-j)]^dagger
-    Mat<D> c3 = mzero<D>();
-    greg_for_lanes(W, T, T, lane, [&](int j, double w) {
-        mfma_db<D>(c3, mscal<D>(w, gtv<D>(G, g, m, j, kb)), gtv<D>(S, g, n, T - j, kb));
-    });
     // history sum_{l<n} w_{n,l} G^<(m,l) [Sigma^R(n,l)]^dagger
     Mat<D> hist = mzero<D>();
     greg_for_lanes(W, n, n - 1, lane, [&](int l, double w) {
@@ -193,12 +204,12 @@ __device__ __forceinline__ void les_item_w(const NgWeights& W, const Grid& g, co
     });
     // closing step, one element (a, b) per lane: rhs = h i c1 - xi htau c3 - bdf / h + h i hist,
     // y = rhs [M_n^-1]^dagger
-    const cplx c1e = warp_rsum<D>(c1, lane), c3e = warp_rsum<D>(c3, lane), he = warp_rsum<D>(hist, lane);
+    const cplx he = warp_rsum<D>(hist, lane);
     const int e = rs_elem<D>(lane), a = e / D, b = e % D;
-    const cplx q = csub(cscal(g.h, cmuli(c1e)), cscal((double)g.sig * g.htau, c3e));
     cplx bdf = cz();
     for (int l = 1; l <= k; ++l) bdf = cadd(bdf, cscal(W.a[l], elw(G.les, tri(n - l) + m, a, b, D, kb)));
-    cplx rhs = csub(q, cscal(1.0 / g.h, bdf));
+    sync();
+    cplx rhs = csub(xq[lane], cscal(1.0 / g.h, bdf));
     rhs = cadd(rhs, cscal(g.h, cmuli(he)));
     cplx y = cz();
 #pragma unroll
@@ -244,7 +255,7 @@ __global__ void __launch_bounds__(32) k_bnd_pre(Grid g, int n, HermV G, HermV S,
     bnd_pre_warp<D>(c_W[g.k - 1], g, n, G, S, eps, blockIdx.x, sh, threadIdx.x, status);
 }
 
-// One warp per item, items ordered as in k_step_bulk (lesser, left-mixing, retarded; problem
+// One warp per item, two per lesser item, items ordered as in k_step_bulk (lesser, left-mixing, retarded; problem
 // fastest); w_les, w_tv, w_ret: the items of each task.  With w_pre = nb the first nb warps
 // run the boundary's retarded start-up of problem kb = warp (bnd_pre_warp), which reads only
 // Sigma and eps and writes G^R(n, n-k..n), which no bulk item reads, so that it overlaps the
@@ -256,21 +267,22 @@ __global__ void __launch_bounds__(128, 1) k_step_bulk_w(Grid g, int n, HermV G, 
     dep_wait();
     const NgWeights& W = c_W[g.k - 1];
     int64_t item = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, half = warp & 1;
+    __shared__ cplx xq[2][32];
     if (item < w_pre) {
         __shared__ cplx sh[4][bnd_pre_scratch<D>()];   // blockDim.x = 128: four warps
-        bnd_pre_warp<D>(W, g, n, G, S, eps, (int)item, sh[threadIdx.x >> 5], lane, status);
+        bnd_pre_warp<D>(W, g, n, G, S, eps, (int)item, sh[warp], lane, status);
         return;
     }
-    item -= w_pre;
+    if ((item -= w_pre + (w_pre & 1)) < 0) return;   // pairs start on an even warp
     int task;
-    if (item < w_les) task = 0;
-    else if ((item -= w_les) < w_tv) task = 1;
+    if (item < 2 * w_les) { task = 0; item >>= 1; }
+    else if ((item -= 2 * w_les) < w_tv) task = 1;
     else if ((item -= w_tv) < w_ret) task = 2;
     else return;
     const int kb = (int)(item % g.nb);
     const int col = (int)(item / g.nb);
-    if (task == 0) les_item_w<D>(W, g, G, S, minv_ws, n, col + 1, kb, lane, status);
+    if (task == 0) les_item_w<D>(W, g, G, S, minv_ws, n, col + 1, kb, lane, half, xq[warp >> 1], 1 + (warp >> 1), status);
     else if (task == 1) tv_item_w<D>(W, g, G, S, minv_ws, n, col, kb, lane, status);
     else ret_item_w<D>(W, g, G, S, minv_ws, n, col, kb, lane, status);
 }

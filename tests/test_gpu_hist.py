@@ -159,3 +159,27 @@ def test_fft_source_edges(ng, nk, shared, T, k):
         ctx.dyson_timestep(g, n, G, S, eps)
         out.append({q: v.clone() for q, v in _slice(G, g, n).items()})
     _check(*out)
+
+
+@pytest.mark.parametrize("nf,nk,n,T,k", [(2, 1, 40, 25, 5), (2, 3, 12, 33, 5), (2, 2, 97, 12, 4), (1, 1, 64, 40, 3), (1, 5, 33, 31, 5),
+                                         (2, 1, 11, 12, 5)])
+def test_warp_items(ng, nf, nk, n, T, k):
+    """A warp per item, two per lesser item (one or a few problems, an odd and an even number of start-up
+    warps before them, the first step inside the history), against a thread per item."""
+    g = ng.Grid(nt=max(n, 2 * k + 2), ntau=T, nf=nf, nbatch=nk, korder=k, h=0.02, beta=4.0, mu=0.1)
+    G, S, eps = ng.Herm(g), ng.Herm(g), ng.Func(g)
+    _random(G, 1, 0.3)
+    _random(S, 2, 0.1)
+    torch.view_as_real(eps.val)[..., 0].normal_()
+    ctx = ng.Context(k)
+    out = []
+    for mode in (ng.NG_BULK_THREAD, ng.NG_BULK_WARP):
+        ctx.set_bulk_split(mode)
+        for v in _slice(G, g, n).values():
+            v.zero_()
+        ctx.dyson_timestep(g, n, G, S, eps)
+        assert ctx.status_sync()[1] == 0
+        out.append({q: v.clone() for q, v in _slice(G, g, n).items()})
+    for q in out[0]:
+        x, y = out[0][q], out[1][q]
+        assert ((x - y).abs().amax((0, 1, 2)) <= TOL * x.abs().amax((0, 1, 2))).all(), q
