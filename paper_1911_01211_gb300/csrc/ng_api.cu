@@ -971,7 +971,7 @@ ng_status histu_sums(ng_ctx* c, const UProb* d_probs, const std::vector<UHost>& 
     *ok = false;
     memset(tab, 0, sizeof(*tab));
     HistUGeo q;
-    const size_t head = (sizeof(HistUProb) * (c1 - c0) + 255) / 256 * 256;
+    const size_t head = (sizeof(HistUProb) * (c1 - c0) + 255) / 256 * 256 + 256;   // descriptors, the task counter
     size_t need = head, off = head;
     int lenp = 0;
     for (size_t i = c0; i < c1; ++i) {   // room for the last step, so that the workspace does not grow on the way
@@ -992,6 +992,7 @@ ng_status histu_sums(ng_ctx* c, const UProb* d_probs, const std::vector<UHost>& 
     if (c->ws_hist_bytes < need && ensure(c, &c->ws_hist, &c->ws_hist_bytes, need)) return NG_OK;   // no room
     tab->probs = (HistUProb*)c->ws_hist;
     tab->base = (char*)c->ws_hist;
+    tab->next = (int*)((char*)c->ws_hist + head - 256);
     tab->src = d_probs;
     tab->n = n;
     tab->status = c->d_status;

@@ -48,7 +48,8 @@ constexpr int SM_U = ST * TILE_B;              // digits of the row-sum vector: 
 constexpr int SM_COL = SM_U + ST * NGH_KG * U_B;       // column accumulators: [warp][8][2][32] int4
 constexpr int SM_ROW = SM_COL + 8 * 16 * 32 * 16;      // row accumulators: [warp][2][32] int4
 constexpr int SM_BAR = SM_ROW + 8 * 2 * 32 * 16;       // full[ST], empty[ST]
-constexpr int SM_BYTES = SM_BAR + 2 * ST * 8;
+constexpr int SM_WQ = SM_BAR + 2 * ST * 8;             // work queue: full[2], empty[2], two items
+constexpr int SM_BYTES = SM_WQ + 4 * 8 + 2 * 4;
 constexpr int E_MIN = 128;                     // smallest scale: everything below 2^-1000 counts as zero
 constexpr int WAIT_LIMIT = 1 << 22;            // polls of a barrier before the kernel gives up
 
@@ -106,37 +107,6 @@ __device__ __forceinline__ int64_t row_offset(const Args& a, int type, int j) {
     return type == U_TV ? (int64_t)j * (a.w.T + 1) : tri(j);
 }
 
-// the order of the tiles: (work item, strip of 16 rows, column tile); run ahead by the loads
-struct Tiles {
-    int64_t wk;
-    Unit u;
-    int jr0, jend, mt, mtn;
-    __device__ __forceinline__ void open(const Args& a) {   // first strip with tiles from (wk, jr0) on
-        while (wk < a.nwork) {
-            while (jr0 < jend) {
-                mtn = (strip_cols(a, u, jr0) + 15) >> 4;
-                if (mtn > 0) return;
-                jr0 += 16;
-            }
-            wk += gridDim.x;
-            start(a);
-        }
-    }
-    __device__ __forceinline__ void start(const Args& a) {
-        mt = 0;
-        if (wk >= a.nwork) return;
-        u = unit_of(a, wk);
-        jr0 = u.bi * NGH_BLK;
-        jend = min(jr0 + NGH_BLK, a.w.n);
-    }
-    __device__ __forceinline__ void next(const Args& a) {
-        if (++mt < mtn) return;
-        mt = 0;
-        jr0 += 16;
-        open(a);
-    }
-};
-
 __device__ __forceinline__ void mbar_init(uint32_t bar, int count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
@@ -158,45 +128,62 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, int parity) {
     return false;
 }
 
-// The producer warp: all tiles of the block in order; lane r < 16 copies row r of the tile, lanes from
-// 16 on the row-sum vector's digits of a problem each.
-__device__ __forceinline__ void produce(const Args& a, const Maps& maps, uint32_t sbase, int lane) {
-    Tiles t;
-    t.wk = blockIdx.x;
-    t.start(a);
-    t.open(a);
+// The producer warp: takes items of work from the counter a.w.next, hands them to the consumers through a
+// queue of two, and issues the copies of all their tiles in order; lane r < 16 copies row r of the tile, lanes from
+// 16 on the row-sum vector's digits of a problem each.  The next item is fetched while the copies of one are issued.
+// Items differ in size (triangles and edges hold less): with a fixed share per block the SMs were busy for 81 %
+// of a launch for 256 problems, n = 590, ntau = 400; steps 9.89 -> 9.14 ms for 512 problems, n = 1600, ntau = 800,
+// 1.42 -> 1.33 ms for 251, n = 777, ntau = 401.
+__device__ __forceinline__ void produce(const Args& a, const Maps& maps, uint32_t sbase, int* wq, int lane) {
     const int64_t blk = (int64_t)(a.w.lenp / 16) * DIG_B;   // digits of one vector
-    int slot = 0, ph = 1;   // an empty stage's first wait passes
-    while (t.wk < a.nwork) {
-        const uint32_t full = sbase + SM_BAR + slot * 8, empty = full + ST * 8;
-        if (!mbar_wait(empty, ph)) {
-            if (lane == 0) atomicOr(a.status, NGF_TIMEOUT);
-            for (int i = 0; i < ST; ++i) {   // the copies in flight
-                const int sl = (slot + i) % ST;
-                mbar_wait(sbase + SM_BAR + sl * 8, sl >= slot ? ph : ph ^ 1);
+    int slot = 0, ph = 1, q = 0, qph = 1;   // an empty stage's first wait passes
+    auto give_up = [&] {
+        if (lane == 0) atomicOr(a.status, NGF_TIMEOUT);
+        for (int i = 0; i < ST; ++i) {   // the copies in flight
+            const int sl = (slot + i) % ST;
+            mbar_wait(sbase + SM_BAR + sl * 8, sl >= slot ? ph : ph ^ 1);
+        }
+    };
+    int next = lane == 0 ? atomicAdd(a.w.next, 1) : 0;
+    while (true) {
+        const int wk = __shfl_sync(0xffffffffu, next, 0);
+        const bool more = wk < a.nwork;
+        if (!mbar_wait(sbase + SM_WQ + 16 + q * 8, qph)) return give_up();
+        if (lane == 0) {
+            wq[q] = more ? wk : -1;
+            mbar_arrive(sbase + SM_WQ + q * 8);
+        }
+        if (!more) return;
+        if (lane == 0) next = atomicAdd(a.w.next, 1);
+        if (++q == 2) { q = 0; qph ^= 1; }
+        const Unit u = unit_of(a, wk);
+        const int k0 = u.grp * NGH_KG, type = u.type, rv = type == U_TV ? 3 : (type == U_LES ? 1 : 2);
+        const int ndig = a.w.nv == 1 ? 1 : min(NGH_KG, a.w.nb - k0);
+        for (int jr0 = u.bi * NGH_BLK; jr0 < min(u.bi * NGH_BLK + NGH_BLK, a.w.n); jr0 += 16) {
+            const int mtn = (strip_cols(a, u, jr0) + 15) >> 4, rows = min(16, a.w.n - jr0);
+            for (int mt = 0; mt < mtn; ++mt) {
+                const uint32_t full = sbase + SM_BAR + slot * 8, empty = full + ST * 8;
+                if (!mbar_wait(empty, ph)) return give_up();
+                const int m0 = u.bj * NGH_BLK + mt * 16;
+                if (lane == 0) mbar_expect(full, rows * (TILE_B / 16) + ndig * DIG_B);
+                __syncwarp();
+                if (lane < rows) {
+                    const CUtensorMap* map = type == U_TV ? &maps.tv : (type == U_LES ? &maps.les : &maps.ret);
+                    const int y = (int)(row_offset(a, type, jr0 + lane) + m0);
+                    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                                 ::"r"(sbase + slot * TILE_B + lane * (TILE_B / 16)), "l"(map), "r"(2 * k0), "r"(y), "r"(full)
+                                 : "memory");
+                } else if (lane >= 16 && lane - 16 < ndig) {
+                    const int p = lane - 16;
+                    const char* src = (const char*)a.w.tab + ((int64_t)rv * a.w.nv + (a.w.nv == 1 ? 0 : k0 + p)) * blk + (m0 / 16) * DIG_B;
+                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                 ::"r"(sbase + SM_U + (slot * NGH_KG + p) * U_B), "l"(src), "r"(DIG_B), "r"(full)
+                                 : "memory");
+                }
+                __syncwarp();
+                if (++slot == ST) { slot = 0; ph ^= 1; }
             }
-            return;
         }
-        const int type = t.u.type, m0 = t.u.bj * NGH_BLK + t.mt * 16, k0 = t.u.grp * NGH_KG;
-        const int rows = min(16, a.w.n - t.jr0), ndig = a.w.nv == 1 ? 1 : min(NGH_KG, a.w.nb - k0);
-        if (lane == 0) mbar_expect(full, rows * (TILE_B / 16) + ndig * DIG_B);
-        __syncwarp();
-        if (lane < rows) {
-            const CUtensorMap* map = type == U_TV ? &maps.tv : (type == U_LES ? &maps.les : &maps.ret);
-            const int y = (int)(row_offset(a, type, t.jr0 + lane) + m0);
-            asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                         ::"r"(sbase + slot * TILE_B + lane * (TILE_B / 16)), "l"(map), "r"(2 * k0), "r"(y), "r"(full)
-                         : "memory");
-        } else if (lane >= 16 && lane - 16 < ndig) {
-            const int rv = type == U_TV ? 3 : (type == U_LES ? 1 : 2), q = lane - 16;
-            const char* src = (const char*)a.w.tab + ((int64_t)rv * a.w.nv + (a.w.nv == 1 ? 0 : k0 + q)) * blk + (m0 / 16) * DIG_B;
-            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                         ::"r"(sbase + SM_U + (slot * NGH_KG + q) * U_B), "l"(src), "r"(DIG_B), "r"(full)
-                         : "memory");
-        }
-        __syncwarp();
-        if (++slot == ST) { slot = 0; ph ^= 1; }
-        t.next(a);
     }
 }
 
@@ -307,15 +294,20 @@ __global__ void __launch_bounds__(THREADS, 1) k_hist_mma(const Args a, const __g
             mbar_init(sbase + SM_BAR + i * 8, 1);
             mbar_init(sbase + SM_BAR + (ST + i) * 8, NGH_KG);
         }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(sbase + SM_WQ + i * 8, 1);
+            mbar_init(sbase + SM_WQ + 16 + i * 8, NGH_KG);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (threadIdx.x < ST * NGH_KG * 4)
         ((uint4*)(sm + SM_U + (threadIdx.x >> 2) * U_B + DIG_B))[threadIdx.x & 3] = make_uint4(0, 0, 0, 0);
+    int* wq = (int*)(sm + SM_WQ + 32);
     __syncthreads();
     // registers of the launch: 12 x 32 x 168; the consumers take 224, the others keep 40
     if (warp >= NGH_KG) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
-        if (warp == NGH_KG) produce(a, maps, sbase, lane);
+        if (warp == NGH_KG) produce(a, maps, sbase, wq, lane);
         return;
     }
     asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
@@ -334,7 +326,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_hist_mma(const Args a, const __g
         uo[i] = SM_U + warp * (a.w.nv == 1 ? 0 : U_B) + ((g & 3) >= i ? (g >> 2) * 512 + ((g & 3) - i) * 64 : DIG_B) + t * 16;
 
 #pragma unroll 1
-    for (int64_t wk = blockIdx.x; wk < a.nwork; wk += gridDim.x) {
+    for (int q = 0, qph = 0;;) {
+        if (!mbar_wait(sbase + SM_WQ + q * 8, qph)) {
+            if (lane == 0) atomicOr(a.status, NGF_TIMEOUT);
+            return;
+        }
+        const int wk = ((volatile int*)wq)[q];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(sbase + SM_WQ + 16 + q * 8);
+        if (++q == 2) { q = 0; qph ^= 1; }
+        if (wk < 0) return;
         const Unit u = unit_of(a, wk);
         const int kb = u.grp * NGH_KG + warp;
         const bool act = kb < a.w.nb;
@@ -522,6 +523,8 @@ static HistWs layout(char* base, int n_max, int n, int T, int k, int nb, int nv,
     o += up256((size_t)NGH_NVEC * nv * (w.lenp / 16) * DIG_B);
     w.vexp = (int*)(base + o);
     o += up256(sizeof(int) * (size_t)NGH_NVEC * nv * (w.lenp / NGH_BLK));
+    w.next = (int*)(base + o);
+    o += 256;
     w.part = (cplx*)(base + o);
     w.nbr = pad_blk(n_max) / NGH_BLK;
     o += sizeof(cplx) * (size_t)hist_units(w) * 2 * NGH_BLK * nb;

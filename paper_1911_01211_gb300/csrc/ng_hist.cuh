@@ -80,6 +80,7 @@ static __global__ void __launch_bounds__(256) k_hist_vec(HistWs w, HistRow S) {
     const int kv = blockIdx.y * KK + kk, kvc = min(kv, w.nv - 1);
     const int len = vec == 3 ? w.T + 1 : w.n, j0 = blockIdx.x * NGH_BLK;
     if (j0 >= len) return;
+    if (tid == 0 && blockIdx.x + blockIdx.y + blockIdx.z == 0) *w.next = 0;
     if (tid < KK) smax[tid] = 0;
     __syncthreads();
     cplx x[NP];

@@ -17,6 +17,7 @@ struct HistWs {
     cplx* vec;          // [NGH_NVEC][nv][lenp] row vectors with their quadrature weights, FP64
     uint4* tab;         // [NGH_NVEC][nv][lenp/16][64] their digits, see below
     int* vexp;          // [NGH_NVEC][nv][lenp/NGH_BLK] exponent of a block's largest element, -1: a non-finite one
+    int* next;          // next unit of work, zeroed by k_hist_vec
     cplx* part;         // [unit][2][NGH_BLK][nb] column sums, row sums of each unit
     int nv, lenp;       // problems of the row vectors (1: shared by all), padded length
     int nbr, nct;       // row blocks of the history, column blocks of the left-mixing rows

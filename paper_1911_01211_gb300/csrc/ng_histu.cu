@@ -35,7 +35,8 @@ constexpr int U_B = NGH_DIG_B + 64;                  // digits of a vector, a ro
 constexpr int SM_U = ST * TILE_B;                    // [stage][output][U_B]
 constexpr int SM_INT = SM_U + ST * 8 * U_B;          // integer accumulators: [warp][output][lo, hi][32] int4
 constexpr int SM_BAR = SM_INT + 8 * 8 * 2 * 32 * 16;
-constexpr int SM_BYTES = SM_BAR + 2 * ST * 8;
+constexpr int SM_WQ = SM_BAR + 2 * ST * 8;             // task queue: full[2], empty[2], two tasks
+constexpr int SM_BYTES = SM_WQ + 4 * 8 + 2 * 4;
 
 struct Task {
     const HistUProb* p;
@@ -106,22 +107,34 @@ __device__ __forceinline__ Span span_of(const Task& t, int kt) {
     return s;
 }
 
-__device__ __forceinline__ void produce(const HistUTab& tab, uint32_t sbase, int lane) {
-    int slot = 0, ph = 1;
-    for (int tk = blockIdx.x; tk < tab.ntask; tk += gridDim.x) {
+// The producer warp; tasks, which differ by the orbitals and the triangles, come from a counter as in ng_hist.cu
+__device__ __forceinline__ void produce(const HistUTab& tab, uint32_t sbase, int* wq, int lane) {
+    int slot = 0, ph = 1, w = 0, wph = 1;
+    auto give_up = [&] {
+        if (lane == 0) atomicOr(tab.status, NGF_TIMEOUT);
+        for (int i = 0; i < ST; ++i) {   // the copies in flight
+            const int sl = (slot + i) % ST;
+            mbar_wait(sbase + SM_BAR + sl * 8, sl >= slot ? ph : ph ^ 1);
+        }
+    };
+    int next = lane == 0 ? atomicAdd(tab.next, 1) : 0;
+    while (true) {
+        const int tk = __shfl_sync(0xffffffffu, next, 0);
+        const bool more = tk < tab.ntask;
+        if (!mbar_wait(sbase + SM_WQ + 16 + w * 8, wph)) return give_up();
+        if (lane == 0) {
+            wq[w] = more ? tk : -1;
+            mbar_arrive(sbase + SM_WQ + w * 8);
+        }
+        if (!more) return;
+        if (lane == 0) next = atomicAdd(tab.next, 1);
+        if (++w == 2) { w = 0; wph ^= 1; }
         const Task t = task_of(tab, tk);
         const int D = t.D, DD16 = D * D * 16;
         const char* base = (const char*)histu_base(*t.p, t.s.type);
         for (int kt = t.kt0; kt < t.kt1; ++kt) {
             const uint32_t full = sbase + SM_BAR + slot * 8, empty = full + ST * 8;
-            if (!mbar_wait(empty, ph)) {
-                if (lane == 0) atomicOr(tab.status, NGF_TIMEOUT);
-                for (int i = 0; i < ST; ++i) {   // the copies in flight
-                    const int sl = (slot + i) % ST;
-                    mbar_wait(sbase + SM_BAR + sl * 8, sl >= slot ? ph : ph ^ 1);
-                }
-                return;
-            }
+            if (!mbar_wait(empty, ph)) return give_up();
             const Span s = span_of(t, kt);
             auto bytes_of = [&](int i) {   // stored elements of row j0 + i inside the span
                 const int j = s.j0 + i;
@@ -380,22 +393,36 @@ __global__ void __launch_bounds__(THREADS, 1) k_histu_mma(const __grid_constant_
             mbar_init(sbase + SM_BAR + i * 8, 1);
             mbar_init(sbase + SM_BAR + (ST + i) * 8, 8);
         }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(sbase + SM_WQ + i * 8, 1);
+            mbar_init(sbase + SM_WQ + 16 + i * 8, 8);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (threadIdx.x < ST * 8 * 4)
         ((uint4*)(sm + SM_U + (threadIdx.x >> 2) * U_B + NGH_DIG_B))[threadIdx.x & 3] = make_uint4(0, 0, 0, 0);
+    int* wq = (int*)(sm + SM_WQ + 32);
     __syncthreads();
     // registers of the launch: 12 x 32 x 168; the consumers take 224, the others keep 40
     if (warp >= 8) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
-        if (warp == 8) produce(tab, sbase, lane);
+        if (warp == 8) produce(tab, sbase, wq, lane);
         return;
     }
     asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
     int slot = 0, ph = 0;
-    for (int tk = blockIdx.x; tk < tab.ntask; tk += gridDim.x) {
+    for (int w = 0, wph = 0;;) {
+        bool ok = mbar_wait(sbase + SM_WQ + w * 8, wph);
+        if (!ok) {
+            if (lane == 0) atomicOr(tab.status, NGF_TIMEOUT);
+            return;
+        }
+        const int tk = ((volatile int*)wq)[w];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(sbase + SM_WQ + 16 + w * 8);
+        if (++w == 2) { w = 0; wph ^= 1; }
+        if (tk < 0) return;
         const Task t = task_of(tab, tk);
-        bool ok;
         switch (t.D) {
             case 1: ok = task_warp<1>(tab, t, sm, sbase, warp, lane, slot, ph); break;
             case 2: ok = task_warp<2>(tab, t, sm, sbase, warp, lane, slot, ph); break;

@@ -53,6 +53,7 @@ static __global__ void __launch_bounds__(128) k_histu_vec(const __grid_constant_
     char* base = tab.base + tab.off[blockIdx.y];
     if (tid == 0) {
         smax = 0;
+        if (blockIdx.x + blockIdx.y + blockIdx.z == 0) *tab.next = 0;
         if (blockIdx.x == 0 && blockIdx.z == 0)
             tab.probs[blockIdx.y] = HistUProb{p.G, p.S, p.g, p.minv, (cplx*)base, (uint4*)(base + q.tab), (int*)(base + q.vexp),
                                               (cplx*)(base + q.conv), (cplx*)(base + q.part), q};

@@ -55,7 +55,7 @@ struct HistUTab {
     HistUProb* probs;    // first in the workspace; a problem's part at base + off[i]
     const UProb* src;
     char* base;
-    int* status;
+    int *status, *next;   // next task, zeroed by k_histu_vec
     int np, n, ntask;
     int prob[NG_UMAXP], start[NG_UMAXP + 1];   // index into src, first task
     int64_t off[NG_UMAXP];
