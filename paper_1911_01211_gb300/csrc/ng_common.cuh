@@ -228,14 +228,18 @@ __host__ __device__ __forceinline__ Mat<D> minv(const Mat<D>& x, int* sing) {
                 cplx t = a.v[c][j]; a.v[c][j] = a.v[p][j]; a.v[p][j] = t;
                 t = r.v[c][j]; r.v[c][j] = r.v[p][j]; r.v[p][j] = t;
             }
-        cplx inv = cdiv(cr(1.0), a.v[c][c]);
+#ifdef __CUDA_ARCH__
+        const cplx inv = cinv(a.v[c][c]);
+#else
+        const cplx inv = cdiv(cr(1.0), a.v[c][c]);
+#endif
         for (int j = 0; j < D; ++j) { a.v[c][j] = cmul(a.v[c][j], inv); r.v[c][j] = cmul(r.v[c][j], inv); }
         for (int i = 0; i < D; ++i) {
             if (i == c) continue;
             cplx f = a.v[i][c];
             for (int j = 0; j < D; ++j) {
-                a.v[i][j] = csub(a.v[i][j], cmul(f, a.v[c][j]));
-                r.v[i][j] = csub(r.v[i][j], cmul(f, r.v[c][j]));
+                a.v[i][j] = cfma(cneg(f), a.v[c][j], a.v[i][j]);
+                r.v[i][j] = cfma(cneg(f), r.v[c][j], r.v[i][j]);
             }
         }
     }

@@ -521,7 +521,7 @@ __device__ void les_col_startup_w(const NgWeights& W, const Grid& g, int n, cons
     __syncwarp();
 }
 
-// scratch of les_steps_w: the weighted Sigma^R(m, l) of the chain's rows (at most k+1 rows of at
+// scratch of les_steps_w: -i h w_{m,l} Sigma^R(m, l) of the chain's rows (at most k+1 rows of at
 // most 2k terms) and the column values G^<(l, n) it reads (at most 2k+1)
 #define NG_LS_ROWS (NG_KMAX + 1)
 #define NG_LS_TERMS (2 * NG_KMAX)
@@ -532,10 +532,13 @@ __host__ __device__ constexpr int les_steps_scratch() { return (NG_LS_ROWS * NG_
 // Serial VIDE steps (Eq. MBCVSAMx_t) of column n in the first argument, rows m = mstep..n, with
 // the sources qsrc[m - m0] and the partial histories hsrc[m - m0] over l < lfrom.  One warp: the
 // inverse step matrices of all rows first, one lane per row (they do not depend on the column),
-// and every value the chain reads from memory (w_{m,l} Sigma^R(m,l), the column below mstep) is
+// and every value the chain reads from memory (-i h w_{m,l} Sigma^R(m,l), the column below mstep) is
 // staged in shared memory at once, so that the serial part waits on no global load; then per row,
-// lane (grp, a, b) sums element (a, b) of the history and BDF terms l = grp, grp + 32/D^2, ...,
-// the groups are added by a butterfly, and the lanes of group 0 store the elements of G^<(m, n).
+// lane (grp, a, b) sums element (a, b) of the history and BDF terms l = grp, grp + 32/D^2, ... into one
+// number, the groups are added by a butterfly, and the lanes of group 0 store the elements of G^<(m, n).
+// The chain is FP64 instructions of one warp, 64 clocks each: with the factors staged and one sum 26 a row
+// for D = 2, with the sums apart and scaled afterwards 46 (run of the dimer, n = 200, ntau = 200: 62.0 -> 59.2 ms with
+// the cheaper inverses of minv).
 // Mi: NG_MAXQ + 1 blocks; scr: les_steps_scratch<D>() values.
 template <int D>
 __device__ void les_steps_w(const NgWeights& W, const Grid& g, int n, const HermV& G, const HermV& S,
@@ -558,37 +561,39 @@ __device__ void les_steps_w(const NgWeights& W, const Grid& g, int n, const Herm
     for (int i = lane; i < (n - mstep + 1) * NG_LS_TERMS * E; i += 32) {
         const int r = i / (NG_LS_TERMS * E), rem = i % (NG_LS_TERMS * E), l = lfrom + rem / E, e = rem % E;
         const int m = mstep + r;
-        if (l < m) wS[i] = cscal(gw(W, m, l), cel(S.ret, tri(m) + l, e / D, e % D, D, kb));
+        if (l < m) {
+            const cplx x = cel(S.ret, tri(m) + l, e / D, e % D, D, kb);
+            const double hw = g.h * gw(W, m, l);
+            wS[i] = make_double2(hw * x.y, -hw * x.x);
+        }
     }
     for (int i = lane; i < (mstep - lo) * E; i += 32)
         col[i] = cel(G.les, tri(n) + lo + i / E, (i % E) / D, (i % E) % D, D, kb);
     __syncwarp();
     const int grp = lane / E, e = lane % E, a = e / D, b = e % D;
-    const double hinv = 1.0 / g.h;
+    const double hinv = -1.0 / g.h, a1 = grp < k ? hinv * W.a[1 + grp] : 0.0;
     for (int m = mstep; m <= n; ++m) {
         const int r = m - m0;
         const cplx* wrow = wS + (m - mstep) * NG_LS_TERMS * E;
-        cplx hs = cr(0.0), bd = cr(0.0);
+        cplx acc = cr(0.0);   // - bdf / h - h i h_rows
         for (int l = lfrom + grp; l < m; l += NGR) {
 #pragma unroll
             for (int c = 0; c < D; ++c)
-                hs = cfma(wrow[(l - lfrom) * E + a * D + c], col[(l - lo) * E + c * D + b], hs);
+                acc = cfma(wrow[(l - lfrom) * E + a * D + c], col[(l - lo) * E + c * D + b], acc);
         }
         for (int l = 1 + grp; l <= k; l += NGR) {
             const cplx x = col[(m - l - lo) * E + e];
-            bd = cadd(bd, make_double2(W.a[l] * x.x, W.a[l] * x.y));
+            const double f = l <= NGR ? a1 : hinv * W.a[l];
+            acc = make_double2(fma(f, x.x, acc.x), fma(f, x.y, acc.y));
         }
 #pragma unroll
         for (int o = E; o < 32; o <<= 1) {
-            hs.x += __shfl_xor_sync(full, hs.x, o);
-            hs.y += __shfl_xor_sync(full, hs.y, o);
-            bd.x += __shfl_xor_sync(full, bd.x, o);
-            bd.y += __shfl_xor_sync(full, bd.y, o);
+            acc.x += __shfl_xor_sync(full, acc.x, o);
+            acc.y += __shfl_xor_sync(full, acc.y, o);
         }
-        // acc = q - bdf / h - h i (h_partial + h_rows)
-        const cplx h0 = cadd(hsrc[r][a][b], hs);
-        cplx acc = csub(qsrc[r][a][b], make_double2(hinv * bd.x, hinv * bd.y));
-        acc = csub(acc, make_double2(-g.h * h0.y, g.h * h0.x));
+        // + q - h i h_partial
+        const cplx q = qsrc[r][a][b], hp = hsrc[r][a][b];
+        acc = cadd(acc, make_double2(fma(g.h, hp.y, q.x), fma(-g.h, hp.x, q.y)));
         cplx y = cr(0.0);
 #pragma unroll
         for (int c = 0; c < D; ++c) {
