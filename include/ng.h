@@ -98,7 +98,8 @@ typedef struct {
  * compensation (rounded once to FP64); BDF terms, the per-step matrix inverses, the (A)
  * boundary steps, the start-up and the Matsubara solve stay FP64.  NG_DF64: the same sums in
  * double-float arithmetic (each value an FP32 pair, 48 significand bits; products with their
- * cross terms, TwoSum accumulation), FP64-class accuracy on the FP32 pipes. */
+ * cross terms, TwoSum accumulation), FP64-class accuracy on the FP32 pipes; nf = 1 steps large enough
+ * for the exact digit products of NG_FP64 take these. */
 typedef enum { NG_FP64 = 0, NG_F32C = 1, NG_DF64 = 2 } ng_precision;
 
 /* Evaluation of the left-mixing Matsubara source -i (C^tv_2 + C^tv_3)[Sigma, 1, G^M](n, tau_m) of
@@ -119,10 +120,13 @@ typedef enum { NG_TVSRC_AUTO = 0, NG_TVSRC_DIRECT = 1 } ng_tv_source;
  * that leaves one element of the nf x nf result per lane for the closing solve, the
  * boundary's (A)-row sums spread over (row, problem, chunk) blocks added in chunk order, and
  * the boundary's retarded start-up run by extra warps of the bulk launch (small batches: a
- * dimer, a real-space cluster); NG_BULK_AUTO (default), each warp/spread form when the batch
- * has fewer than 128 bulk items per SM, resp. fewer than 2 boundary rows per SM.  In every
- * mode the boundary's dense solves and serial steps run on one warp per problem.  The forms
- * differ by the order of additions only.  nf = 4, 8 always run the element-wise form. */
+ * dimer, a real-space cluster; two warps for a lesser item); NG_BULK_AUTO (default), each warp/spread form when the batch
+ * has fewer than 128 bulk items per SM, resp. fewer than 2 boundary rows per SM, and for nf = 1 from 16
+ * problems on 4 or 8 lanes per item and a boundary with a lane per problem.  Where a step is large enough (nf = 1,
+ * at least 8 problems), and for nf = 4, 8 and the uneven batch inside the history, NG_BULK_AUTO forms the history
+ * sums on the tensor cores as exact products of 8-bit digits, rounded once per block of the history.  In every
+ * mode the boundary's dense solves and serial steps run on the warps of one block per problem.  The forms
+ * differ by rounding only.  nf = 4, 8 otherwise run the element-wise form. */
 typedef enum { NG_BULK_AUTO = 0, NG_BULK_THREAD = 1, NG_BULK_WARP = 2 } ng_bulk_split;
 
 /* Schedule of a time step (Sec. "Time stepping"): NG_MIXED is the paper's parallel variant

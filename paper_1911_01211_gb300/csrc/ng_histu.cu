@@ -20,8 +20,8 @@
 // instructions of 8 slots; the two directions are separate tasks, which reads X twice but needs no
 // transposition and keeps no column sums.
 //
-// Measured (16 clusters, one of 8, four of 4, five of 2 orbitals, n = 500, ntau = 300): 1.31 ms, with
-// k_histu_close 0.19 and k_histu_vec 0.05 against 6.3 ms of k_ubulk.  The issue slots alone are 0.6 ms; the
+// Measured (16 clusters, one of 8, four of 4, five of 2 orbitals, n = 500, ntau = 300): 1.14 ms (1.31 with a fixed
+// share of tasks per block), with k_histu_close 0.19 and k_histu_vec 0.05 against 6.3 ms of k_ubulk.  The issue slots alone are 0.6 ms; the
 // rest is shared memory (per tile and output 8 loads of 512 bytes of digits, and the elements, whose
 // orbital stride of 128 bytes at nf = 8 puts four lanes of eight on one bank in half the sets) and the
 // latency of two warps per quarter of an SM.

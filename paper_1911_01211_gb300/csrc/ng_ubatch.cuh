@@ -282,19 +282,6 @@ __device__ cplx u_qlesA_range(const NgWeights& W, const Grid& g, const HermV& G,
     return cadd(cscal(g.h, cmulmi(c2)), cscal((double)g.sig * g.htau, c3));
 }
 
-// M_m = a_0/h + i(eps_m - mu) + h w_{m,m} i Sigma^R(m,m) into out[D*D]
-__device__ void u_stepmat(const NgWeights& W, const UProb& P, int m, cplx* out) {
-    const int D = P.g.nf;
-    for (int a = 0; a < D; ++a)
-        for (int b = 0; b < D; ++b) {
-            cplx e = ufunc(P.eps, m, D, a, b, P.kb);
-            if (a == b) e.x -= P.g.mu;
-            cplx v = cadd(cmuli(e), cscal(P.g.h * gw(W, m, m), cmuli(uel(P.S.ret, tri(m) + m, D, a, b, P.kb))));
-            if (a == b) v.x += W.a[0] / P.g.h;
-            out[a * D + b] = v;
-        }
-}
-
 // The boundary of step n runs in three launches: k_uboundary_ret (retarded (A) start-up along
 // row n and G^<(0,n), one block per problem), k_usrc (sources and partial histories of the
 // lesser (A) rows, O((k+1)(n + ntau) nf^3) per problem, over many blocks), k_uboundary_les (the
