@@ -396,24 +396,27 @@ def run_ours(a):
     e2e_window = nk * K / max_over_ranks(r["window_s"])
     prof, clk = r["prof"], r["clk"]
     # per step: extrapolation, then per corrector pass k-reduce (or partial + combine), Hartree,
-    # 2B, M_n^-1 (+ bulk, boundary)
+    # 2B, M_n^-1 (+ bulk, boundary); a lower bound: the bulk of a step is three launches with the digit
+    # products, the boundary two
     launches = int(prof["bulk_launches"] + prof["boundary_launches"] + prof["tvfft_launches"]) + \
         K * (1 + 3 * (4 + (1 if dist else 0)))
-    achieved = prof["bulk_flops"] / (prof["bulk_ms"] / 1e3) / 1e12
-    peak = fp64_peak_tflops(clk.get("sm_mhz"), sms)
     bulk_launches = max(1, prof["bulk_launches"])
-    cmac_per_launch = prof["bulk_flops"] / 8.0 / w.nf ** 3 / bulk_launches
+    fp64_equiv = prof["bulk_flops"] / (prof["bulk_ms"] / 1e3) / 1e12
+    # the history once per corrector pass: left-mixing rows, retarded and lesser triangles of slices < n
+    window_bytes = 3 * 16.0 * w.nf ** 2 * nkl * sum(n * (w.ntau + 1) + n * (n + 1) for n in range(n_first_timed, w.nt + 1))
+    achieved = window_bytes / (prof["bulk_ms"] / 1e3) / 1e9
+    peak = measured_hbm_gbs()
     traffic, traffic_note = None, None
     try:
         import hashlib
         with open(os.path.join(ROOT, "profiles", "traffic.json")) as f:
             tr = json.load(f)
-        src = open(os.path.join(ROOT, "paper_1911_01211_gb300", "csrc", "ng_step.cuh"), "rb").read()
-        if tr.get("ng_step_sha1") == hashlib.sha1(src).hexdigest():
-            traffic = tr["captured"]["dram_bytes_per_cmac"] * cmac_per_launch
-            traffic_note = (f"{tr['captured']['dram_bytes_per_cmac']:.2f} DRAM bytes per complex multiply-add "
-                            f"(ncu capture: {tr['captured']['launch']}) x {cmac_per_launch:.4g} multiply-adds per "
-                            f"launch of this window")
+        src = open(os.path.join(ROOT, "paper_1911_01211_gb300", "csrc", "ng_hist.cu"), "rb").read()
+        if tr.get("ng_hist_sha1") == hashlib.sha1(src).hexdigest():
+            per = tr["captured"]["dram_bytes_per_history_byte"]
+            traffic = per * window_bytes / bulk_launches
+            traffic_note = (f"{per:.3f} DRAM bytes per byte of history (ncu capture: {tr['captured']['launch']}) x "
+                            f"{window_bytes / bulk_launches:.4g} bytes of history per launch of this window")
         else:
             traffic_note = "null: the time-step kernels changed since the ncu capture"
     except (OSError, ValueError, KeyError):
@@ -446,9 +449,8 @@ def run_ours(a):
         sl = lambda: {"ret": G.ret[ng.tri(nt):ng.tri(nt) + nt + 1], "les": G.les[ng.tri(nt):ng.tri(nt) + nt + 1],
                       "tv": G.tv[nt * (w.ntau + 1):(nt + 1) * (w.ntau + 1)]}
         ref = {c: x.clone() for c, x in sl().items()}
-        bytes_per_elem = {"f32c": 8, "df64": 16}
         k32 = "k_step_bulk32p (two k-points per thread)" if w.nbatch % 2 == 0 else "k_step_bulk32<1>"
-        for name, prec, kern in (("f32c", ng.NG_F32C, k32), ("df64", ng.NG_DF64, "k_step_bulkdf<1>")):
+        for name, prec, kern in (("f32c", ng.NG_F32C, k32), ("df64", ng.NG_DF64, "k_hist_mma + k_hist_close")):
             rm = propagate(prec, False)
             stm, flagsm = ctx.status_sync()
             submit_check(name)
@@ -463,7 +465,8 @@ def run_ours(a):
                 "e2e_window": {"value": nk * K / max_over_ranks(rm["window_s"]), "unit": "k-point timesteps/s"},
                 "bulk_kernel": {"kernel": kern,
                                 "algorithmic_fp64_equiv_tflops": profm["bulk_flops"] / (profm["bulk_ms"] / 1e3) / 1e12,
-                                "history_gbs": cmacs * bytes_per_elem[name] / (profm["bulk_ms"] / 1e3) / 1e9,
+                                # F32C: 8 B of FP32 copy per multiply-add; DF64: as FP64
+                                "history_gbs": (cmacs * 8 if name == "f32c" else window_bytes) / (profm["bulk_ms"] / 1e3) / 1e9,
                                 "hbm_frac_of_measured": None,
                                 "avg_launch_ms": profm["bulk_ms"] / max(1, profm["bulk_launches"]),
                                 "share_of_timed": profm["bulk_ms"] / rm["ms"]},
@@ -498,12 +501,16 @@ def run_ours(a):
                          "memory to the device and Gloc^<(t_n, t_n) back",
                 "window": {"value": e2e_window, "unit": "k-point timesteps/s",
                            "scope": "the timed window's steps only, same call, host clock"}},
-        "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                     "frac": achieved / peak, "traffic": traffic, "traffic_note": traffic_note,
-                     "kernel": "k_step_bulk<1>",
-                     "peak_source": f"FP64 DFMA from unit counts: {sms} SMs (device property) x "
-                                    f"{FP64_FLOP_PER_CLK_PER_SM} flop/clk x median SM clock {clk.get('sm_mhz')} MHz; "
-                                    f"measured by ng_fp64_probe in this run: {probe}",
+        "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+                     "frac": achieved / peak if peak else None, "traffic": traffic, "traffic_note": traffic_note,
+                     "kernel": "k_hist_mma (with k_minv_step, k_hist_vec and k_hist_close in its time)",
+                     "peak_source": "measured copy bandwidth; achieved: the FP64 history of slices < n read once per "
+                                    "corrector pass",
+                     "fp64_equivalent_tflops": fp64_equiv,
+                     "fp64_peak_tflops": fp64_peak_tflops(clk.get("sm_mhz"), sms),
+                     "fp64_peak_source": f"FP64 DFMA from unit counts: {sms} SMs (device property) x "
+                                         f"{FP64_FLOP_PER_CLK_PER_SM} flop/clk x median SM clock {clk.get('sm_mhz')} MHz; "
+                                         f"measured by ng_fp64_probe in this run: {probe}",
                      "avg_launch_ms": prof["bulk_ms"] / bulk_launches,
                      "share_of_timed": prof["bulk_ms"] / r["ms"],
                      "tv_source_fft_share_of_timed": prof["tvfft_ms"] / r["ms"],
@@ -680,16 +687,19 @@ def run_gw(a):
         v = obs.cpu().numpy()
         N.append(v[0])
         E.append(v[4])
-    peak = fp64_peak_tflops(clk.get("sm_mhz") or 2070.0)
-    bulk_tf = prof["bulk_flops"] / (prof["bulk_ms"] * 1e-3) / 1e12 if prof["bulk_ms"] > 0 else None
+    peak = measured_hbm_gbs()
+    # the history once per Dyson solve, one per corrector pass
+    hist_bytes = w.corrector * 16.0 * w.nbatch * sum(n * (w.ntau + 1) + n * (n + 1) for n in range(n_w + 1, n_to + 1))
+    bulk_gbs = hist_bytes / (prof["bulk_ms"] * 1e-3) / 1e9 if prof["bulk_ms"] > 0 else None
     line = {"metric": "k-point timesteps/s (k-space GW chain)", "value": w.nbatch * K / (ms / 1e3),
             "unit": "k-point timesteps/s", "n_gpus": 1, "steps": K, "warmup": W, "ms_per_step": ms / K,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": {"workload": f"chain_kspace GW nk={w.nbatch} nt={w.nt} ntau={w.ntau} h={w.h} beta={w.beta} "
                                    f"U=2 k={w.korder} corrector={w.corrector} (k-space GW, Eqs. Sigmak/Pol, Peierls "
                                    f"pulse)", "timed": f"steps {n_w + 1}..{n_to} (setup and {W} warm-up steps untimed)"},
-            "roofline": {"bound": "alu", "achieved": bulk_tf, "peak": peak, "unit": "TFLOP/s",
-                         "frac": bulk_tf / peak if bulk_tf else None, "traffic": None, "kernel": "k_step_bulk<1>",
+            "roofline": {"bound": "hbm", "achieved": bulk_gbs, "peak": peak, "unit": "GB/s",
+                         "frac": bulk_gbs / peak if bulk_gbs and peak else None, "traffic": None,
+                         "kernel": "k_hist_mma (with k_minv_step, k_hist_vec and k_hist_close in its time)",
                          "share_of_timed": prof["bulk_ms"] / ms},
             "gw_chain_share_of_timed": prof["gw_ms"] / ms, "gw_chain_ms_per_eval": prof["gw_ms"] / max(prof["gw_evals"], 1),
             "setup": {"s": t_setup, "iterations": its},
@@ -749,7 +759,9 @@ def run_uneven(a):
                        "nf_counts": {str(d): sum(1 for p in probs if p["nf"] == d) for d in (1, 2, 4, 8)},
                        "timed": "whole batch solve: setup of every problem, block-size tuning, all global steps"},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                         "frac": achieved / peak, "traffic": None, "kernel": "k_ubulk",
+                         "frac": achieved / peak, "traffic": None,
+                         "kernel": "k_histu_mma with k_histu_close (digit products on the tensor cores: FP64-equivalent "
+                                   "rate against the FP64 pipe's peak)",
                          "share_of_timed": prof["bulk_ms"] / ms},
             "tuned_threads": threads, "clocks": clk, "device_status": {"status": st, "flags": flags}}
     if a.compare_plain:
