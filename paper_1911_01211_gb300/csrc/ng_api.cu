@@ -989,6 +989,7 @@ ng_status histu_sums(ng_ctx* c, const UProb* d_probs, const std::vector<UHost>& 
     }
     tab->np = (int)(c1 - c0);
     tab->start[tab->np] = tab->ntask;
+    if (off > need) return fail(c, NG_EINVAL, "the digit sums of step %d need %zu bytes, their workspace holds %zu", n, off, need);
     if (c->ws_hist_bytes < need && ensure(c, &c->ws_hist, &c->ws_hist_bytes, need)) return NG_OK;   // no room
     tab->probs = (HistUProb*)c->ws_hist;
     tab->base = (char*)c->ws_hist;

@@ -9,11 +9,15 @@ struct UProb;
 
 #define NGU_M 128        // free indices of a task
 #define NGU_KT 16        // tiles of a task: at least 16, at most 256 (the integer accumulators), 24 tasks to a contraction
+#define NGU_CHUNKS 24
 #define NGU_SETS 7
 #define NGU_NVEC 6
 
 // Sizes of one problem at step n: padded vector length; per set the padded free indices, tiles of a task, chunks of
-// the contraction, the first task and the first partial sum; bytes of the problem's part of the workspace.
+// the contraction, the first task and the first partial sum; bytes of the problem's part of the workspace.  The
+// chunks fall from 24 to 23 and rise again as n grows (the tiles of a task are whole), so the partial sums are laid
+// out for the largest number of chunks of any step up to n: no step needs more bytes than a later one, and a
+// workspace sized for the last step holds them all.
 struct HistUGeo {
     int lenp, free_[NGU_SETS], kt[NGU_SETS], chunks[NGU_SETS], task0[NGU_SETS + 1];
     int64_t poff[NGU_SETS], tab, vexp, conv, part, bytes;
@@ -26,12 +30,13 @@ __host__ __device__ inline void histu_geo(int D, int T, int n, HistUGeo& q) {
     for (int s = 0; s < NGU_SETS; ++s) {
         const int64_t rows = s >> 1 == 3 ? T + 1 : n, cols = s >> 1 >= 2 ? T + 1 : n, fr = (s & 1) ? rows : cols, con = (s & 1) ? cols : rows;
         q.free_[s] = pad(fr * D);
-        const int tiles = (int)((con * D + 15) / 16), kt = (tiles + 23) / 24;
+        const int tiles = (int)((con * D + 15) / 16), kt = (tiles + NGU_CHUNKS - 1) / NGU_CHUNKS;
         q.kt[s] = kt < NGU_KT ? NGU_KT : (kt > 256 ? 256 : kt);
         q.chunks[s] = (tiles + q.kt[s] - 1) / q.kt[s];
+        const int most = kt <= NGU_KT || q.chunks[s] > NGU_CHUNKS ? q.chunks[s] : NGU_CHUNKS;
         q.task0[s + 1] = q.task0[s] + q.free_[s] / NGU_M * q.chunks[s];
         q.poff[s] = el;
-        el += (int64_t)q.free_[s] * q.chunks[s] * D;
+        el += (int64_t)q.free_[s] * most * D;
     }
     q.tab = (int64_t)NGU_NVEC * D * q.lenp * sizeof(cplx);
     q.vexp = q.tab + (int64_t)NGU_NVEC * D * (q.lenp / 16) * NGH_DIG_B;
