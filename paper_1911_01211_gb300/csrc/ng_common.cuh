@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "ng_weights.h"
 
@@ -36,6 +37,19 @@ __host__ __device__ __forceinline__ cplx cfma(cplx a, cplx b, cplx c) {
     return c;
 }
 __host__ __device__ __forceinline__ double cabs2(cplx a) { return a.x * a.x + a.y * a.y; }
+// |a|^2 for the search of a pivot: squares of magnitudes compare as their bits, without the FP64 pipe.  -1 for a
+// NaN of either sign, which a finite element therefore always beats: a search that starts with the diagonal
+// row at -1 ends on a row of the matrix whatever the column holds.
+__host__ __device__ __forceinline__ long long pivot_key(cplx a) {
+    const double v = cabs2(a);
+#ifdef __CUDA_ARCH__
+    const long long b = __double_as_longlong(v);
+#else
+    long long b;
+    memcpy(&b, &v, sizeof(b));
+#endif
+    return (b & 0x7fffffffffffffffll) > 0x7ff0000000000000ll ? -1 : b;
+}
 __host__ __device__ __forceinline__ cplx cdiv(cplx a, cplx b) {
     // Smith's algorithm (R. L. Smith, CACM 1962) for a / b
     if (fabs(b.x) >= fabs(b.y)) {

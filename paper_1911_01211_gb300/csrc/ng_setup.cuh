@@ -390,11 +390,11 @@ __global__ void __launch_bounds__(NG_LU_THREADS) k_lu_solve(int N, int nrhs, cpl
         }
         __syncthreads();
         for (int c = 0; c < w; ++c) {
-            // pivot: the first row of largest magnitude (squares compare as their bits)
+            // pivot: the first row of largest magnitude; the diagonal row when none compares (a column of NaN)
             long long best = -1;
-            int bi = N;
+            int bi = c0 + c;
             for (int r = c0 + c + t; r < N; r += nt) {
-                const long long v = __double_as_longlong(cabs2(P[(size_t)r * PB + c]));
+                const long long v = pivot_key(P[(size_t)r * PB + c]);
                 if (v > best) { best = v; bi = r; }
             }
 #pragma unroll
@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(NG_LU_THREADS) k_lu_solve(int N, int nrhs, cpl
             for (int q = 1; q < nw; ++q)
                 if (rv[q] > best || (rv[q] == best && ri[q] < bi)) { best = rv[q]; bi = ri[q]; }
             if (t == 0) {
-                if (best == 0) atomicOr(status, NGF_SINGULAR);
+                if (best <= 0) atomicOr(status, NGF_SINGULAR);
                 pv[c0 + c] = prow[c] = bi;
             }
             if (bi != c0 + c && t < PB) {
@@ -480,11 +480,12 @@ __global__ void __launch_bounds__(NG_LU_THREADS) k_lu_solve(int N, int nrhs, cpl
 // A few problems: the inverse of A by Gauss-Jordan elimination with partial pivoting, one launch per
 // column over the whole GPU (a few microseconds each: one pass over an L2-resident matrix), from one
 // buffer to the other so that the row interchange needs no second pass.  Each launch also finds the
-// next column's pivot: key = magnitude's leading 48 bits, then the smallest row.  With the inverse, a
+// next column's pivot: key = magnitude's leading 48 bits (none for a NaN), then the smallest row.  With the inverse, a
 // solve is a product (k_gj_apply) instead of 2 N dependent steps of one block: for 402 unknowns and 2
 // right-hand sides 1775 -> 9 us, a factorisation with its solve 9.4 -> 2.9 ms.
 __device__ __forceinline__ unsigned long long gj_key(cplx x, int r) {
-    return ((unsigned long long)__double_as_longlong(cabs2(x)) & ~0xffffull) | (unsigned)(0xffff - r);
+    const long long v = pivot_key(x);
+    return ((unsigned long long)(v < 0 ? 0 : v) & ~0xffffull) | (unsigned)(0xffff - r);
 }
 __global__ void k_gj_first(int N, int ld, const cplx* ws_A, unsigned long long* keys, int* perm) {
     dep_wait();
@@ -504,7 +505,7 @@ __global__ void __launch_bounds__(128) k_gj_step(int N, int ld, const cplx* src_
     const unsigned long long key = keys[(int64_t)pb * (N + 1) + c];
     const int p = 0xffff - (int)(key & 0xffff);
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
-        if (src[(int64_t)p * ld + c].x == 0.0 && src[(int64_t)p * ld + c].y == 0.0) atomicOr(status, NGF_SINGULAR);
+        if (pivot_key(src[(int64_t)p * ld + c]) <= 0) atomicOr(status, NGF_SINGULAR);
         int* pm = perm + (int64_t)pb * N;
         const int x = pm[c];
         pm[c] = pm[p];

@@ -348,11 +348,10 @@ __device__ inline int group_dense_solve(cplx* A, int N, cplx* B, int nrhs, cplx*
     const unsigned full = 0xffffffffu;
     auto sync = [] { if (NT == 32) __syncwarp(); else __syncthreads(); };
     for (int c = 0; c < N; ++c) {
-        // squares of magnitudes compare as their bits, without the FP64 pipe
         long long best = -1;
-        int p = N;
+        int p = c;   // kept when no entry compares (a column of NaN), as dense_solve does
         for (int r = c + (t & 31); r < N; r += 32) {
-            const long long v = __double_as_longlong(cabs2(A[r * N + c]));
+            const long long v = pivot_key(A[r * N + c]);
             if (v > best) { best = v; p = r; }
         }
 #pragma unroll
