@@ -21,6 +21,14 @@
 // is rounded once per unit.  Dropped are the products of weight 8 and more, below 2^-60 of the
 // largest product.
 //
+// Small sums.  All of this is relative to the largest element of the unit, so a sum that is small beside it (the tail
+// of a damped function, a column far down the tau axis, a cancellation) would keep fewer bits than on the FP64 pipe.
+// With X and v on the scales above, a sum of 128 terms is off by less than 2^-53.8 (the dropped products 2^-54.2, the
+// cut of v 2^-56, that of X 2^-57), and by about 2^-60 for errors of random sign.  Where its result is 2^-8 and
+// more that is at most 2^-45.8 of it, below the FP64 kernels' bound (256 roundings, 2^-45 of sum |v X|), and 2^-52 for
+// random signs, as theirs.  Every sum below 2^-8 whose terms are not all zero is done again on the FP64 pipe
+// (k_hist_small), so that no element of a step has less precision than there.
+//
 // Work.  A unit is 128 x 128 elements of 8 neighbouring problems (128 contiguous bytes per element);
 // a warp owns a problem, a ninth warp issues the copies.  16 x 16 tiles of all 8 problems pass through
 // a ring of 32 KB stages filled by TMA, one 16-element row per copy, with the 128-byte swizzle: a
@@ -71,6 +79,28 @@ struct Unit {
     int64_t id;
 };
 
+__device__ __forceinline__ Unit unit_at(const Args& a, int64_t id) {
+    Unit u;
+    u.id = id;
+    u.grp = 0;
+    int64_t r = id;
+    const int64_t ntv = (int64_t)a.w.nbr * a.w.nct, nt = tri(a.w.nbr);
+    if (r < ntv) {
+        u.type = U_TV;
+        u.bi = (int)(r / a.w.nct);
+        u.bj = (int)(r - (int64_t)u.bi * a.w.nct);
+        return u;
+    }
+    r -= ntv;
+    u.type = U_LES;
+    if (r >= nt) { r -= nt; u.type = U_RET; }
+    int b = (int)((sqrtf(8.0f * (float)r + 1.0f) - 1.0f) * 0.5f);
+    while (tri(b + 1) <= r) ++b;
+    while (tri(b) > r) --b;
+    u.bi = b;
+    u.bj = (int)(r - tri(b));
+    return u;
+}
 __device__ __forceinline__ Unit unit_of(const Args& a, int64_t wk) {
     Unit u;
     u.id = wk / a.ngrp;
@@ -346,7 +376,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_hist_mma(const Args a, const __g
         const uint4* ctab = a.w.tab + (((int64_t)cv * a.w.nv + kv) * (a.w.lenp / 16) + j0 / 16) * (DIG_B / 16);
         const int nblk = a.w.lenp / NGH_BLK;
         const int fc = a.w.vexp[(cv * a.w.nv + kv) * nblk + u.bi], fr = a.w.vexp[(rv * a.w.nv + kv) * nblk + u.bj];
-        cplx* colp = a.w.part + (u.id * 2) * NGH_BLK * a.w.nb + kb;
+        cplx* colp = a.w.part + u.id * NGH_PART * a.w.nb + kb;
         cplx* rowp = colp + (int64_t)NGH_BLK * a.w.nb;
         bool bad = fc < 0 || fr < 0;
         int E = 0;
@@ -406,7 +436,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_hist_mma(const Args a, const __g
                     const int emax = E + __reduce_max_sync(full, -lo);
                     bad = bad || emax == 2047;
                     int dE;
-                    if (E == 0) dE = max(emax, E_MIN);
+                    if (E == 0) dE = max(emax + 1, E_MIN);   // a bit of room: the parts of a value that turns grow by up to sqrt(2)
                     else {
                         const int q = (emax - E + 7) >> 3, qs = min(q, 8);
                         dE = 8 * q;
@@ -499,10 +529,90 @@ __global__ void __launch_bounds__(THREADS, 1) k_hist_mma(const Args a, const __g
         }
         if (!act) continue;
         __syncwarp();
+        if (lane == 0) rowp[(int64_t)NGH_BLK * a.w.nb].x = bad ? 0.0 : E;
         const double sc = bad ? 0.0 : pow2(max(E, E_MIN) - 1022 - 20) * pow2(fc - 1021 - 20);
         for (int i = lane; i < NGH_BLK; i += 32) colp[(int64_t)i * a.w.nb] = digits_value(colacc + (i >> 4) * 64, i & 15, sc);
         __syncwarp();
         if (bad) unit_fp64(a, u, kb, cv, rv, colp, rowp, lane);   // a non-finite element or vector
+    }
+}
+
+// The sums that are small on the scale of their unit, again on the FP64 pipe.  A warp takes SMALL_Q sums of 32
+// neighbouring problems at a time: it reads the results, whole lines, compares their exponents with the scales, and does
+// the small ones four at once, eight lanes to a sum (70 FP64 instructions for the four, which bound the kernel where many
+// are small; else it is the read of the results).  In a kernel of its own because small sums lie in a few problems, and
+// the ring of k_hist_mma goes at the pace of its slowest warp: done there, 0.2 % of the sums took the step of 251
+// problems, n = 777, ntau = 401 from 1.28 to 2.18 ms.  Here, of whole steps: 512 problems, n = 1600, ntau = 800 (0.02 % of
+// the sums) 0.16 ms of 9.4; the 251 problems 0.06 of 1.36; 256 problems, n = 900, ntau = 400 (0.6 %) 0.08 of 1.76; a
+// second-Born run of 128 problems, n = 160, ntau = 200 (8 %, most of them columns far down the tau axis) 106 -> 115 ms.
+template <int SMALL_Q>
+__global__ void __launch_bounds__(128) k_hist_small(const Args a) {
+    dep_wait();
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, nb = a.w.nb, nkb = (nb + 31) / 32, nblk = a.w.lenp / NGH_BLK;
+    const int64_t items = hist_units(a.w) * (2 * NGH_BLK / SMALL_Q) * nkb, step = (int64_t)gridDim.x * blockDim.x >> 5;
+    for (int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += step) {
+        const int64_t r = it / nkb, id = r / (2 * NGH_BLK / SMALL_Q);
+        const int kb0 = (int)(it - r * nkb) * 32, kb = min(kb0 + lane, nb - 1), i0 = (int)(r % (2 * NGH_BLK / SMALL_Q)) * SMALL_Q;
+        const bool row = i0 >= NGH_BLK;
+        cplx* p = a.w.part + (id * NGH_PART + i0) * nb;
+        const int E = (int)p[(int64_t)(2 * NGH_BLK - i0) * nb + kb].x;
+        int ex[SMALL_Q];
+#pragma unroll
+        for (int q = 0; q < SMALL_Q; ++q) {
+            const cplx x = p[(int64_t)q * nb + kb];
+            ex[q] = max(__double2hiint(x.x) >> 20 & 2047, __double2hiint(x.y) >> 20 & 2047);
+        }
+        const Unit u = unit_at(a, id);
+        const int vec = row ? (u.type == U_TV ? 3 : (u.type == U_LES ? 1 : 2)) : (u.type == U_RET ? 0 : 1);
+        const int F = a.w.vexp[(vec * a.w.nv + (a.w.nv == 1 ? 0 : kb)) * nblk + (row ? u.bj : u.bi)];
+        const int low = max(E + F - 2043 - 8 + 1023, 1);   // exponent of 2^-8 on the scale 2^(E-1022) 2^(F-1021)
+        const int j0 = u.bi * NGH_BLK, m0 = u.bj * NGH_BLK, j1 = min(j0 + NGH_BLK, a.w.n), band = u.type == U_RET ? a.w.k : 0;
+        // terms [c0, c1) of sum i0 + q: row j0 + i over its columns, or column m0 + i over its rows
+        auto range = [&](int q, int& c0, int& c1) {
+            const int i = (i0 + q) % NGH_BLK;
+            if (row) {
+                c0 = m0;
+                c1 = j0 + i >= j1 ? 0 : min(m0 + NGH_BLK, u.type == U_TV ? a.w.T + 1 : j0 + i - band);
+            } else {
+                c0 = u.type == U_TV ? j0 : max(j0, m0 + i + band + 1);
+                c1 = u.type == U_TV && m0 + i > a.w.T ? 0 : j1;
+            }
+        };
+        unsigned left[SMALL_Q];
+        int total = 0;
+#pragma unroll
+        for (int q = 0; q < SMALL_Q; ++q) {
+            int c0, c1;
+            range(q, c0, c1);
+            // scales above E_MIN: neither the history's unit nor the vector's block is zero
+            left[q] = __ballot_sync(full, kb0 + lane < nb && E > E_MIN && F > E_MIN && ex[q] < low && c0 < c1);
+            total += __popc(left[q]);
+        }
+        const bool conj = u.type == (row ? U_TV : U_LES);
+        const cplx* X = u.type == U_TV ? a.tv : (u.type == U_LES ? a.les : a.ret);
+        for (int base = 0; base < total; base += 4) {
+            int at = base + (lane >> 3), q = 0;   // this group's sum: the at-th of the masks in turn
+            const bool mine = at < total;
+            if (!mine) at = total - 1;
+            while (q < SMALL_Q - 1 && at >= __popc(left[q])) at -= __popc(left[q++]);
+            const int k = kb0 + (int)__fns(left[q], 0, at + 1), i = (i0 + q) % NGH_BLK;
+            int c0, c1;
+            range(q, c0, c1);
+            const cplx* v = a.w.vec + ((int64_t)vec * a.w.nv + (a.w.nv == 1 ? 0 : k)) * a.w.lenp;
+            cplx s = cz();
+#pragma unroll 4
+            for (int c = c0 + (lane & 7); c < c1; c += 8) {
+                const int64_t el = row ? row_offset(a, u.type, j0 + i) + c : row_offset(a, u.type, c) + m0 + i;
+                s = cfma(X[el * nb + k], conj ? cconj(v[c]) : v[c], s);
+            }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) {
+                s.x += __shfl_xor_sync(full, s.x, o);
+                s.y += __shfl_xor_sync(full, s.y, o);
+            }
+            if (mine && (lane & 7) == 0) p[(int64_t)q * nb + k] = s;
+        }
     }
 }
 
@@ -527,7 +637,7 @@ static HistWs layout(char* base, int n_max, int n, int T, int k, int nb, int nv,
     o += 256;
     w.part = (cplx*)(base + o);
     w.nbr = pad_blk(n_max) / NGH_BLK;
-    o += sizeof(cplx) * (size_t)hist_units(w) * 2 * NGH_BLK * nb;
+    o += sizeof(cplx) * (size_t)hist_units(w) * NGH_PART * nb;
     w.nbr = pad_blk(n) / NGH_BLK;
     if (bytes) *bytes = o;
     return w;
@@ -581,5 +691,11 @@ cudaError_t hist_launch(const HistWs& ws, const cplx* ret, const cplx* les, cons
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)(a.nwork < sms ? a.nwork : sms);
     dep_launch(k_hist_mma, grid, THREADS, SM_BYTES, s)(a, maps);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // sums of 32 problems; one at a time while these are fewer than four for each warp the GPU holds
+    const int64_t sums = hist_units(ws) * 2 * NGH_BLK * ((ws.nb + 31) / 32);
+    const unsigned most = 16 * (unsigned)sms;
+    if (sums < 16 * (int64_t)most) dep_launch(k_hist_small<1>, (unsigned)(sums < 4 * (int64_t)most ? (sums + 3) / 4 : most), 128, 0, s)(a);
+    else dep_launch(k_hist_small<4>, most, 128, 0, s)(a);
     return cudaGetLastError();
 }

@@ -115,10 +115,10 @@ static __global__ void __launch_bounds__(256) k_hist_vec(HistWs w, HistRow S) {
 
 // column c, row r of a unit's sums
 __device__ __forceinline__ cplx hist_col(const HistWs& w, int64_t unit, int c, int kb) {
-    return w.part[(unit * 2 * NGH_BLK + c) * w.nb + kb];
+    return w.part[(unit * NGH_PART + c) * w.nb + kb];
 }
 __device__ __forceinline__ cplx hist_row(const HistWs& w, int64_t unit, int r, int kb) {
-    return w.part[((unit * 2 + 1) * NGH_BLK + r) * w.nb + kb];
+    return w.part[(unit * NGH_PART + NGH_BLK + r) * w.nb + kb];
 }
 
 // sum_{j<n} of the retarded column m (n - m > k): unit weights of the interior, Gregory weights at

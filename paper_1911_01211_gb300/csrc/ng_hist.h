@@ -5,6 +5,7 @@
 #include "ng_common.cuh"
 
 #define NGH_BLK 128     // rows and columns of a unit of work
+#define NGH_PART (2 * NGH_BLK + 1)   // results of a unit and problem
 #define NGH_KG 8        // problems of a unit (one warp each)
 #define NGH_NVEC 4      // row vectors of a step, see k_hist_vec
 #define NGH_DIG_B 1024  // bytes of the digits of 16 elements of a row vector v:
@@ -18,7 +19,7 @@ struct HistWs {
     uint4* tab;         // [NGH_NVEC][nv][lenp/16][64] their digits, see below
     int* vexp;          // [NGH_NVEC][nv][lenp/NGH_BLK] exponent of a block's largest element, -1: a non-finite one
     int* next;          // next unit of work, zeroed by k_hist_vec
-    cplx* part;         // [unit][2][NGH_BLK][nb] column sums, row sums of each unit
+    cplx* part;         // [unit][NGH_PART][nb] column sums, row sums, scale of each unit (0: done on the FP64 pipe)
     int nv, lenp;       // problems of the row vectors (1: shared by all), padded length
     int nbr, nct;       // row blocks of the history, column blocks of the left-mixing rows
     int n, T, k, nb;
