@@ -972,20 +972,27 @@ ng_status histu_sums(ng_ctx* c, const UProb* d_probs, const std::vector<UHost>& 
     memset(tab, 0, sizeof(*tab));
     HistUGeo q;
     const size_t head = (sizeof(HistUProb) * (c1 - c0) + 255) / 256 * 256 + 256;   // descriptors, the task counter
-    size_t need = head, off = head;
+    size_t need = head + 256, off = head;   // then the scales of the tasks, then each problem's part
     int lenp = 0;
     for (size_t i = c0; i < c1; ++i) {   // room for the last step, so that the workspace does not grow on the way
         const UHost& u = info[active[i]];
         histu_geo(u.D, u.ntau, u.nt, q);
-        need += q.bytes;
+        need += q.bytes + q.slots * sizeof(int);
         const int j = (int)(i - c0);
         histu_geo(u.D, u.ntau, n, q);
         tab->prob[j] = active[i];
-        tab->off[j] = (int64_t)off;
+        tab->dmax = std::max(tab->dmax, u.D);
+        off += q.slots * sizeof(int);
         tab->start[j] = tab->ntask;
         tab->ntask += q.task0[NGU_SETS];
-        off += q.bytes;
         lenp = std::max(lenp, q.lenp);
+    }
+    off = (off + 255) / 256 * 256;
+    for (size_t i = c0; i < c1; ++i) {
+        const UHost& u = info[active[i]];
+        histu_geo(u.D, u.ntau, n, q);
+        tab->off[i - c0] = (int64_t)off;
+        off += q.bytes;
     }
     tab->np = (int)(c1 - c0);
     tab->start[tab->np] = tab->ntask;
@@ -994,6 +1001,7 @@ ng_status histu_sums(ng_ctx* c, const UProb* d_probs, const std::vector<UHost>& 
     tab->probs = (HistUProb*)c->ws_hist;
     tab->base = (char*)c->ws_hist;
     tab->next = (int*)((char*)c->ws_hist + head - 256);
+    tab->uexp = (int*)((char*)c->ws_hist + head);
     tab->src = d_probs;
     tab->n = n;
     tab->status = c->d_status;

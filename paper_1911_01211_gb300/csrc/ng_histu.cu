@@ -1,5 +1,8 @@
 // History sums of the uneven batch (problems of 1, 2, 4 or 8 orbitals, each with its own storage) by
-// exact digit products on the tensor cores; numbers, digits and scales as in ng_hist.cu.
+// exact digit products on the tensor cores; numbers and digits as in ng_hist.cu, with a scale of X for a warp's 16 free
+// indices in a task, of a vector for each chunk of the contraction.  A sum below 2^-8 on these scales (a weak
+// coupling between orbitals, a damped tail, a cancellation) is done again on the FP64 pipe, for the reason given there
+// (its bounds are per term, those of the FP64 kernels too).
 //
 // With orbitals the stored history of a component is a matrix X over (time, orbital) pairs, and the
 // sums of a step are products of X or its transpose with nf row vectors each (vectors: k_histu_vec):
@@ -21,7 +24,7 @@
 // transposition and keeps no column sums.
 //
 // Measured (16 clusters, one of 8, four of 4, five of 2 orbitals, n = 500, ntau = 300): 1.14 ms (1.31 with a fixed
-// share of tasks per block), with k_histu_close 0.19 and k_histu_vec 0.05 against 6.3 ms of k_ubulk.  The issue slots alone are 0.6 ms; the
+// share of tasks per block), with k_histu_close 0.19, k_histu_small 0.22 and k_histu_vec 0.02 against 6.3 ms of k_ubulk.  The issue slots alone are 0.6 ms; the
 // rest is shared memory (per tile and output 8 loads of 512 bytes of digits, and the elements, whose
 // orbital stride of 128 bytes at nf = 8 puts four lanes of eight on one bank in half the sets) and the
 // latency of two warps per quarter of an SM.
@@ -36,7 +39,8 @@ constexpr int SM_U = ST * TILE_B;                    // [stage][output][U_B]
 constexpr int SM_INT = SM_U + ST * 8 * U_B;          // integer accumulators: [warp][output][lo, hi][32] int4
 constexpr int SM_BAR = SM_INT + 8 * 8 * 2 * 32 * 16;
 constexpr int SM_WQ = SM_BAR + 2 * ST * 8;             // task queue: full[2], empty[2], two tasks
-constexpr int SM_BYTES = SM_WQ + 4 * 8 + 2 * 4;
+constexpr int SM_TASK = SM_WQ + 4 * 8 + 2 * 4;         // the task of each warp
+constexpr int SM_BYTES = SM_TASK + 8 * 4;
 
 struct Task {
     const HistUProb* p;
@@ -45,10 +49,8 @@ struct Task {
 };
 
 // task tk; kt1 <= kt0 when the history has no element there
-__device__ __forceinline__ Task task_of(const HistUTab& tab, int tk) {
+__device__ __forceinline__ Task task_at(const HistUTab& tab, int tk, int i) {   // of problem i
     Task t;
-    int i = 0;
-    while (tk >= tab.start[i + 1]) ++i;
     t.p = &tab.probs[i];
     int r = tk - tab.start[i];
     t.set = 0;
@@ -70,6 +72,12 @@ __device__ __forceinline__ Task task_of(const HistUTab& tab, int tk) {
         }
     }
     return t;
+}
+
+__device__ __forceinline__ Task task_of(const HistUTab& tab, int tk) {
+    int i = 0;
+    while (tk >= tab.start[i + 1]) ++i;
+    return task_at(tab, tk, i);
 }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, int count) {
@@ -182,6 +190,87 @@ __device__ __forceinline__ double digits_value(int4 lo, int4 hi, double sc) {
     return fma((double)l, 0x1p-32, (double)h) * sc;
 }
 
+__device__ __forceinline__ bool nonzero(cplx x) {   // on the integer pipe
+    return ((unsigned)(__double2hiint(x.x) << 1) | (unsigned)__double2loint(x.x) | (unsigned)(__double2hiint(x.y) << 1) |
+            (unsigned)__double2loint(x.y)) != 0;
+}
+// contracted times [lo, hi) of free time f in a task (all that the matrix holds; set 6 has gaps)
+__device__ __forceinline__ void task_range(const Task& t, int f, int& lo, int& hi) {
+    const HistUSet& s = t.s;
+    lo = t.kt0 * 16 / t.D;
+    hi = min(t.kt1 * 16 / t.D, s.rowc ? s.rows : s.cols);
+    if (f >= (s.rowc ? s.cols : s.rows)) hi = 0;
+    else if (s.type < 2) {
+        if (s.rowc) lo = max(lo, f + s.band + 1);
+        else hi = min(hi, histu_mend(s, f));
+    }
+}
+
+// The sums that are small on their scale, again on the FP64 pipe, in a kernel of its own as in ng_hist.cu: a warp takes
+// 16 free indices and an output of a task and does the small sums four at once, eight lanes to a sum, four terms of a lane
+// in flight; terms whose couplings are zero cost no arithmetic.  Whole steps without and with it: 16 clusters of 1 to 8
+// orbitals, n = 500, ntau = 300 1.87 / 2.05 ms; one of 8, n = 250, ntau = 60 (no small sums) 0.65 / 0.67.
+__global__ void __launch_bounds__(128) k_histu_small(const __grid_constant__ HistUTab tab) {
+    dep_wait();
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < tab.ntask * 8 * tab.dmax; i += gridDim.x * blockDim.x >> 5) {
+        const int tw = i / tab.dmax, o = i - tw * tab.dmax, code = tab.uexp[tw], E = code & 0xfff, D = code >> 12 & 15;
+        if (E <= 128 || o >= D) continue;
+        const Task t = task_at(tab, tw >> 3, code >> 16);
+        const HistUSet& s = t.s;
+        const int f0 = t.f0 + (tw & 7) * 16;
+        cplx* out = t.p->part + t.p->q.poff[t.set] + ((int64_t)t.chunk * t.p->q.free_[t.set] + f0) * D + o;
+        const int F = t.p->vexp[(s.vec * D + o) * t.p->q.vch + t.chunk];
+        bool is = false;
+        if (lane < 16) {
+            const cplx x = out[lane * D];
+            int lo, hi;
+            task_range(t, (f0 + lane) / D, lo, hi);
+            // 2^-8 on the scale 2^(E-1022) 2^(F-1021); scales of 128: zeros
+            const int ex = max(__double2hiint(x.x) >> 20 & 2047, __double2hiint(x.y) >> 20 & 2047);
+            is = lo < hi && F > 128 && ex < max(E + F - 2043 - 8 + 1023, 1);
+        }
+        const cplx* v = t.p->vec + ((int64_t)s.vec * D + o) * t.p->q.lenp;
+        for (unsigned left = __ballot_sync(full, is); left;) {
+            unsigned rest = left;   // this group's sum: the bit number lane / 8, else the first
+            for (int z = lane >> 3; z > 0; --z) rest &= rest - 1;
+            const bool mine = rest != 0;
+            const int r = __ffs(mine ? rest : left) - 1, f = (f0 + r) / D, fo = (f0 + r) % D;
+            for (int z = 0; z < 4; ++z) left &= left - 1;
+            int lo, hi;
+            task_range(t, f, lo, hi);
+            const int steps = (__reduce_max_sync(full, hi - lo) + 7) / 8;   // of an orbital
+            cplx x = cz();
+            for (int q0 = 0; q0 < D * steps; q0 += 4) {
+                cplx w[4], e[4];
+                bool any = false;
+#pragma unroll
+                for (int z = 0; z < 4; ++z) {
+                    const int co = (q0 + z) / steps, c = lo + (lane & 7) + 8 * (q0 + z - co * steps);
+                    const int j = s.rowc ? c : f, m = s.rowc ? f : c;
+                    w[z] = e[z] = cz();
+                    if (co < D && c < hi && histu_has(s, j, m)) {
+                        w[z] = v[c * D + co];
+                        e[z] = histu_el(*t.p, s, D, j, m, s.rowc ? co : fo, s.rowc ? fo : co);
+                    }
+                }
+#pragma unroll
+                for (int z = 0; z < 4; ++z) any = any || (nonzero(w[z]) && nonzero(e[z]));
+                if (!__any_sync(full, any)) continue;
+#pragma unroll
+                for (int z = 0; z < 4; ++z) x = cfma(e[z], histu_conj(s.vec) ? cconj(w[z]) : w[z], x);
+            }
+#pragma unroll
+            for (int b = 4; b > 0; b >>= 1) {
+                x.x += __shfl_xor_sync(full, x.x, b);
+                x.y += __shfl_xor_sync(full, x.y, b);
+            }
+            if (mine && (lane & 7) == 0) out[r * D] = x;
+        }
+    }
+}
+
 // one warp's 16 free indices of a task; false when a wait ran out
 template <int D>
 __device__ __forceinline__ bool task_warp(const HistUTab& tab, const Task& t, unsigned char* sm, uint32_t sbase, int warp, int lane,
@@ -190,10 +279,10 @@ __device__ __forceinline__ bool task_warp(const HistUTab& tab, const Task& t, un
     const unsigned full = 0xffffffffu;
     int4* acc = (int4*)(sm + SM_INT) + warp * 8 * 2 * 32 + lane;   // [output][lo, hi][32]
     const HistUSet s = t.s;
-    const int* vexp = t.p->vexp + s.vec * D;
+    auto vexp = [&](int o) { return t.p->vexp[(s.vec * D + o) * t.p->q.vch + t.chunk]; };
     bool bad = false;
 #pragma unroll
-    for (int o = 0; o < D; ++o) bad = bad || vexp[o] < 0;
+    for (int o = 0; o < D; ++o) bad = bad || vexp(o) < 0;
     // byte offsets of this lane's free indices (g, g + 8) and contracted ones (2t, 2t+1, 2t+8, 2t+9) in a tile
     constexpr int DD16 = D * D * 16;
     const int row_b = (s.rowc ? NGU_M / D : 16 / D) * DD16 + 16;
@@ -239,7 +328,7 @@ __device__ __forceinline__ bool task_warp(const HistUTab& tab, const Task& t, un
     auto take = [&]() {   // the sums so far, at their scale
 #pragma unroll
         for (int o = 0; o < D; ++o) {
-            const double sc = bad ? 0.0 : pow2(max(E, 128) - 1022 - 20) * pow2(vexp[o] - 1021 - 20);
+            const double sc = bad ? 0.0 : pow2(max(E, 128) - 1022 - 20) * pow2(vexp(o) - 1021 - 20);
             val[o] += digits_value(acc[o * 64], acc[o * 64 + 32], sc);
             acc[o * 64] = acc[o * 64 + 32] = make_int4(0, 0, 0, 0);
         }
@@ -288,7 +377,7 @@ __device__ __forceinline__ bool task_warp(const HistUTab& tab, const Task& t, un
             for (int i = 0; i < 16; ++i) low = min(low, (&sh[0][0][0])[i]);
             const int emax = E + __reduce_max_sync(full, -low);
             bad = bad || emax == 2047;
-            const int dE = E == 0 ? max(emax, 128) : emax - E + 3;   // three bits of room: the sums so far are set aside
+            const int dE = E == 0 ? max(emax + 1, 128) : emax - E + 3;   // a bit of room, then three: the sums so far are set aside
             if (E != 0) { flush(); take(); }
             E += dE;
 #pragma unroll
@@ -363,9 +452,11 @@ __device__ __forceinline__ bool task_warp(const HistUTab& tab, const Task& t, un
     if (!bad) {
 #pragma unroll
         for (int o = 0; o < D; ++o) ((double*)(out + (g + 8 * (tt & 1)) * D + o))[tt >> 1] = val[o];
+        if (lane == 0) tab.uexp[((int*)(sm + SM_TASK))[warp] * 8 + warp] = (int)(t.p - tab.probs) << 16 | D << 12 | E;
         return true;
     }
     // a non-finite element or vector: the sums on the FP64 pipe, lane -> (free index, output)
+    if (lane == 0) tab.uexp[((int*)(sm + SM_TASK))[warp] * 8 + warp] = 0;
     const cplx* v = t.p->vec + (int64_t)s.vec * D * t.p->q.lenp;
     for (int q = lane; q < 16 * D; q += 32) {
         const int f = (f0 + q / D) / D, fo = (f0 + q / D) % D, o = q % D;
@@ -423,6 +514,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_histu_mma(const __grid_constant_
         if (++w == 2) { w = 0; wph ^= 1; }
         if (tk < 0) return;
         const Task t = task_of(tab, tk);
+        if (lane == 0) ((int*)(sm + SM_TASK))[warp] = tk;
         switch (t.D) {
             case 1: ok = task_warp<1>(tab, t, sm, sbase, warp, lane, slot, ph); break;
             case 2: ok = task_warp<2>(tab, t, sm, sbase, warp, lane, slot, ph); break;
@@ -442,5 +534,8 @@ cudaError_t histu_launch(const HistUTab& tab, int sms, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(k_histu_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_BYTES);
     if (e != cudaSuccess) return e;
     dep_launch(k_histu_mma, tab.ntask < sms ? tab.ntask : sms, THREADS, SM_BYTES, s)(tab);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const int64_t blocks = (int64_t)tab.ntask * 2 * tab.dmax;
+    dep_launch(k_histu_small, (unsigned)(blocks < 16 * sms ? blocks : 16 * sms), 128, 0, s)(tab);
     return cudaGetLastError();
 }

@@ -25,8 +25,9 @@ __device__ __forceinline__ cplx histu_vec_value(const NgWeights& W, const UProb&
     return j >= n - k ? cscal(W.omega[n - j], x) : x;
 }
 
-// block (chunk of 128 elements, problem, 8 vector + output): values, scale and digits; each block finds the
-// vector's largest exponent by itself.  Blocks of vector NGU_NVEC write Y.
+// block (128 elements, problem, 8 vector + output): values, scales and digits.  Each chunk of the contraction (the kt
+// tiles of a task) has the scale of its largest element, which every block of 128 elements finds by itself; it
+// touches two chunks at most (16 tiles and more each).  Blocks of vector NGU_NVEC write Y.
 static __global__ void __launch_bounds__(128) k_histu_vec(const __grid_constant__ HistUTab tab) {
     dep_wait();
     const UProb& p = tab.src[tab.prob[blockIdx.y]];
@@ -46,30 +47,33 @@ static __global__ void __launch_bounds__(128) k_histu_vec(const __grid_constant_
     }
     if (o >= D || (int)blockIdx.x * 128 >= (len + 127) / 128 * 128) return;
     const NgWeights& W = c_W[p.g.k - 1];
-    __shared__ int smax;
+    __shared__ int smax[2];
     __shared__ __align__(16) __half dig[8][2][8][4][2][2][2];   // as NGH_DIG_B
     HistUGeo q;
     histu_geo(D, p.g.ntau, n, q);
     char* base = tab.base + tab.off[blockIdx.y];
     if (tid == 0) {
-        smax = 0;
+        smax[0] = smax[1] = 0;
         if (blockIdx.x + blockIdx.y + blockIdx.z == 0) *tab.next = 0;
         if (blockIdx.x == 0 && blockIdx.z == 0)
             tab.probs[blockIdx.y] = HistUProb{p.G, p.S, p.g, p.minv, (cplx*)base, (uint4*)(base + q.tab), (int*)(base + q.vexp),
                                               (cplx*)(base + q.conv), (cplx*)(base + q.part), q};
     }
     __syncthreads();
-    int e = 0;
+    const int ke = histu_vec_kt(q, vec) * 16, ch0 = (int)blockIdx.x * 128 / ke, ch1 = ((int)blockIdx.x * 128 + 127) / ke;
+    for (int ch = ch0; ch <= ch1; ++ch) {
+        int e = 0;
 #pragma unroll 4
-    for (int i = tid; i < len; i += 128) {
-        const cplx x = histu_vec_value(W, p, n, vec, o, i);
-        e = max(e, max(__double2hiint(x.x) >> 20 & 2047, __double2hiint(x.y) >> 20 & 2047));
+        for (int i = ch * ke + tid; i < min(len, (ch + 1) * ke); i += 128) {
+            const cplx x = histu_vec_value(W, p, n, vec, o, i);
+            e = max(e, max(__double2hiint(x.x) >> 20 & 2047, __double2hiint(x.y) >> 20 & 2047));
+        }
+        atomicMax(&smax[ch - ch0], e);
     }
-    atomicMax(&smax, e);
     __syncthreads();
-    const int F = max(smax, 128);
-    if (tid == 0) ((int*)(base + q.vexp))[vec * D + o] = F == 2047 ? -1 : F;
-    const int i0 = blockIdx.x * 128 + tid;
+    if (tid <= ch1 - ch0 && (ch0 + tid) * ke < len)   // each block of a chunk writes the same value
+        ((int*)(base + q.vexp))[(vec * D + o) * q.vch + ch0 + tid] = smax[tid] == 2047 ? -1 : max(smax[tid], 128);
+    const int i0 = blockIdx.x * 128 + tid, F = max(smax[i0 / ke - ch0], 128);
     const cplx x = i0 < len ? histu_vec_value(W, p, n, vec, o, i0) : cz();
     ((cplx*)base)[((int64_t)vec * D + o) * q.lenp + i0] = x;
     hist_digits(x, F, histu_conj(vec), tid & 15, dig[tid >> 4]);

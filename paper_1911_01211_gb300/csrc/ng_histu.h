@@ -13,19 +13,20 @@ struct UProb;
 #define NGU_SETS 7
 #define NGU_NVEC 6
 
-// Sizes of one problem at step n: padded vector length; per set the padded free indices, tiles of a task, chunks of
+// Sizes of one problem at step n: padded vector length, chunks of a vector (room for them); per set the padded free indices, tiles of a task, chunks of
 // the contraction, the first task and the first partial sum; bytes of the problem's part of the workspace.  The
 // chunks fall from 24 to 23 and rise again as n grows (the tiles of a task are whole), so the partial sums are laid
 // out for the largest number of chunks of any step up to n: no step needs more bytes than a later one, and a
 // workspace sized for the last step holds them all.
 struct HistUGeo {
-    int lenp, free_[NGU_SETS], kt[NGU_SETS], chunks[NGU_SETS], task0[NGU_SETS + 1];
-    int64_t poff[NGU_SETS], tab, vexp, conv, part, bytes;
+    int lenp, vch, free_[NGU_SETS], kt[NGU_SETS], chunks[NGU_SETS], task0[NGU_SETS + 1];
+    int64_t poff[NGU_SETS], tab, vexp, conv, part, bytes, slots;   // slots: entries of HistUTab::uexp
 };
 __host__ __device__ inline void histu_geo(int D, int T, int n, HistUGeo& q) {
     auto pad = [](int64_t x) { return (int)((x + NGU_M - 1) / NGU_M * NGU_M); };
     q.lenp = pad((n > T + 1 ? n : T + 1) * (int64_t)D);
-    q.task0[0] = 0;
+    q.task0[0] = q.vch = 0;
+    q.slots = 0;
     int64_t el = 0;
     for (int s = 0; s < NGU_SETS; ++s) {
         const int64_t rows = s >> 1 == 3 ? T + 1 : n, cols = s >> 1 >= 2 ? T + 1 : n, fr = (s & 1) ? rows : cols, con = (s & 1) ? cols : rows;
@@ -34,13 +35,15 @@ __host__ __device__ inline void histu_geo(int D, int T, int n, HistUGeo& q) {
         q.kt[s] = kt < NGU_KT ? NGU_KT : (kt > 256 ? 256 : kt);
         q.chunks[s] = (tiles + q.kt[s] - 1) / q.kt[s];
         const int most = kt <= NGU_KT || q.chunks[s] > NGU_CHUNKS ? q.chunks[s] : NGU_CHUNKS;
+        if (q.vch < most) q.vch = most;
+        q.slots += (int64_t)q.free_[s] / NGU_M * most * 8;   // an entry per warp of a task
         q.task0[s + 1] = q.task0[s] + q.free_[s] / NGU_M * q.chunks[s];
         q.poff[s] = el;
         el += (int64_t)q.free_[s] * most * D;
     }
     q.tab = (int64_t)NGU_NVEC * D * q.lenp * sizeof(cplx);
     q.vexp = q.tab + (int64_t)NGU_NVEC * D * (q.lenp / 16) * NGH_DIG_B;
-    q.conv = q.vexp + 256;   // NGU_NVEC D <= 48 exponents
+    q.conv = q.vexp + ((int64_t)NGU_NVEC * D * q.vch * (int64_t)sizeof(int) + 255) / 256 * 256;
     q.part = q.conv + (2 * T + 1) * D * D * (int64_t)sizeof(cplx);
     q.bytes = (q.part + el * (int64_t)sizeof(cplx) + 255) / 256 * 256;
 }
@@ -51,7 +54,7 @@ struct HistUProb {       // written by k_histu_vec
     cplx* minv;
     cplx* vec;           // [NGU_NVEC][nf][lenp]
     uint4* tab;          // [NGU_NVEC][nf][lenp/16][64]
-    int* vexp;           // [NGU_NVEC][nf]
+    int* vexp;           // [NGU_NVEC][nf][vch] exponent of a chunk's largest element, -1: a non-finite one
     cplx* conv;          // Y(i) at i + ntau
     cplx* part;          // per set: [chunk][padded free index][nf]
     HistUGeo q;
@@ -64,6 +67,9 @@ struct HistUTab {
     int np, n, ntask;
     int prob[NG_UMAXP], start[NG_UMAXP + 1];   // index into src, first task
     int64_t off[NG_UMAXP];
+    int* uexp;             // [task][8] scale of the history of a warp's free indices (0: zeros, or done on the FP64 pipe),
+                           // nf at bit 12, problem at bit 16
+    int dmax;              // largest nf
 };
 
 // rows (time indices) and columns of the matrix of a set; band: j - m above it
@@ -87,6 +93,8 @@ __device__ __forceinline__ const cplx* histu_base(const HistUProb& p, int type) 
 __device__ __forceinline__ int64_t histu_row(const Grid& g, int type, int j) {
     return type == 3 ? g.ntau - j : (type == 2 ? (int64_t)j * (g.ntau + 1) : tri(j));
 }
+// tiles of a chunk of a vector: vectors 3 and 4 run over the tau axis, the others over the history
+__host__ __device__ __forceinline__ int histu_vec_kt(const HistUGeo& q, int vec) { return q.kt[vec == 3 || vec == 4 ? 5 : 0]; }
 // vectors 3 and 5 enter conjugated
 __host__ __device__ __forceinline__ bool histu_conj(int vec) { return vec == 3 || vec == 5; }
 // last column + 1 of row j in memory
