@@ -70,7 +70,7 @@ cudaError_t adj_boot_gather(const Grid& g, const cplx* r, const cplx* l, const c
 
 cudaError_t adj_boot_start(const AdjBoot& b, cudaStream_t s) {
     const size_t smem = sizeof(cplx) * (size_t)(boot_E(b.g.k, b.g.ntau) + (int64_t)b.g.k * (b.g.ntau + 1));
-    cudaError_t e = cudaFuncSetAttribute(k_adj_start, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = smem_limit(k_adj_start);
     if (e != cudaSuccess) return e;
     dep_launch(k_adj_start, b.g.nb, NG_BOOT_THREADS, smem, s)(b);
     return cudaGetLastError();

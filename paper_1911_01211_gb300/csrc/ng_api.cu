@@ -634,7 +634,7 @@ ng_status launch_timestep32(ng_ctx* c, const Grid& g, int n, const HermV& G, con
 template <int PB>
 ng_status lu_solve_p(ng_ctx* c, int N, int nrhs, int nb, cplx* ws_A, int* ws_piv, cudaStream_t s) {
     const size_t smem = sizeof(cplx) * ((size_t)N * PB + NG_LU_TRI * nrhs);
-    CUDA_TRY(c, cudaFuncSetAttribute(k_lu_solve<PB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CUDA_TRY(c, smem_limit(k_lu_solve<PB>));
     dep_launch(k_lu_solve<PB>, nb, NG_LU_THREADS, smem, s)(N, nrhs, ws_A, ws_piv, c->d_status);
     return check_launch(c, "k_lu_solve");
 }
@@ -944,8 +944,7 @@ ng_status do_kfft(ng_ctx* c, const Grid& g, int tstp, int L, const SliceView& in
     const int64_t fill = std::max<int64_t>(1, nvec / (2 * (int64_t)c->sms));
     const int vpb = (int)std::max<int64_t>(1, std::min<int64_t>(std::max(1, 1024 / L), fill));
     const size_t smem = sizeof(cplx) * (size_t)(vpb + 1) * L;
-    if (smem > 48 * 1024)
-        CUDA_TRY(c, cudaFuncSetAttribute(k_kfft_slice, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 48 * 1024) CUDA_TRY(c, smem_limit(k_kfft_slice));
     const int thr = std::min(256, std::max(64, vpb * L / 4 / 32 * 32));
     dep_launch(k_kfft_slice, (unsigned)((nvec + vpb - 1) / vpb), thr, smem, s)(g, tstp, L, log2L, vpb, in, out, sign, scale);
     return check_launch(c, "k_kfft_slice");

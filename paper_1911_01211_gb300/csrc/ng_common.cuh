@@ -109,6 +109,17 @@ DepLaunch<P...> dep_launch(void (*k)(P...), dim3 grid, dim3 block, size_t smem, 
     return {k, grid, block, smem, s};
 }
 
+// Before a launch with more than 48 KB of dynamic shared memory that depends on the problem: the kernel's limit to all
+// that a block can have (227 KB).  The limit belongs to the process: set to the need of one launch it would be lowered
+// between the two calls of another thread, whose context has a larger problem.
+template <class... P>
+cudaError_t smem_limit(void (*k)(P...)) {
+    cudaFuncAttributes f;
+    const cudaError_t e = cudaFuncGetAttributes(&f, k);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - (int)f.sharedSizeBytes);
+}
+
 // ---------------------------------------------------------------------------------------
 // d x d complex matrices in registers
 // ---------------------------------------------------------------------------------------

@@ -160,12 +160,12 @@ cudaError_t launch_d(const Grid& g, const NgWeights& W, int n, const Comp& Stv, 
     cudaError_t e;
     if (shared) {
         const size_t sm = sizeof(cplx) * (size_t)L;
-        if ((e = cudaFuncSetAttribute(k_tvsrc_s, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
+        if ((e = smem_limit(k_tvsrc_s))) return e;
         dep_launch(k_tvsrc_s, D * D, L >= 2048 ? 1024 : L / 2, sm, s)(g, W, n, Stv, tw, L, FS);
         if ((e = cudaGetLastError())) return e;
     }
     const size_t sm = shared ? one : 2 * one;
-    if ((e = cudaFuncSetAttribute(k_tvsrc_fft<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
+    if ((e = smem_limit(k_tvsrc_fft<D>))) return e;
     dep_launch(k_tvsrc_fft<D>, g.nb, kThreads, sm, s)(g, W, n, Stv, Gmat, tw, L, FS, Q);
     return cudaGetLastError();
 }
