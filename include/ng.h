@@ -501,9 +501,11 @@ ng_status ng_run_2b_host(ng_ctx *ctx, const ng_grid *grid, ng_herm G, ng_herm Gl
  * eps_mf hold the rank's own k-points (k_begin .. k_begin + k_count - 1 of ng_shard_plan); Gloc,
  * Sigma and U are full copies on every rank.  Every k-reduction goes through the exchange, so
  * Gloc, Sigma and the rank's G_k are bitwise those of a single-GPU ng_run_2b over all nk
- * k-points (up to the rounding of the convergence distances, which are summed per rank, so a
- * setup loop could stop one iteration apart when its distance lands within rounding of the
- * tolerance).  NG_ECOMM if the callback fails. */
+ * k-points: the forms of the steps and solves, which differ by rounding, and the chunks of their
+ * sums are those of nk problems on every rank (up to the rounding of the convergence distances and of
+ * the Matsubara refinement's updates, which are summed per rank, so a setup loop could stop one
+ * iteration apart when its distance lands within rounding of the tolerance).  NG_ECOMM if the
+ * callback fails. */
 ng_status ng_run_2b_sharded(ng_ctx *ctx, const ng_grid *grid, ng_herm G, ng_herm Gloc, ng_herm Sigma,
                             ng_func eps0, ng_func eps_mf, ng_func U, const ng_run_params *p, const ng_shard *shard,
                             int *iters_out, void *stream);

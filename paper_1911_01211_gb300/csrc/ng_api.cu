@@ -23,6 +23,7 @@
 #include "ng_histclose.cuh"
 #include "ng_adjoint_types.h"
 #include <cmath>
+#include <functional>
 
 // double-float copy of one contour function (NG_DF64 time steps), as Shadow
 struct ShadowDF {
@@ -100,6 +101,7 @@ struct ng_ctx {
     std::vector<std::pair<std::vector<int>, int>> tune_cache;
     int tvsrc = NG_TVSRC_AUTO;       // evaluation of the left-mixing Matsubara source
     int bulk_split = NG_BULK_AUTO;   // one thread or one warp per bulk item (ng_set_bulk_split)
+    int run_nk = 0;                  // k-points of all ranks while a sharded run is on, else 0
     void* ws_tvq = nullptr;          // FFT correlation of the source, [m][a][b][kb]
     size_t ws_tvq_bytes = 0;
     void* ws_hist = nullptr;         // digit-product history sums: row vectors, digits, unit sums
@@ -165,6 +167,11 @@ ng_status ensure(ng_ctx* c, void** p, size_t* have, size_t need) {
     *have = need;
     return NG_OK;
 }
+
+// The number of problems that chooses between the forms of a step or a solve and the chunks of their sums, which
+// differ by rounding: the batch's own, or in a sharded run that of all ranks, so that every rank adds in the order
+// of one GPU.  Sizes of launches and workspaces take the batch's own.
+int form_nb(const ng_ctx* c, const Grid& g) { return c->run_nk ? c->run_nk : g.nb; }
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
@@ -311,12 +318,12 @@ ng_status prep_tvfft(ng_ctx* c, const Grid& g, int n, const HermV& G, const Herm
 // 128 problems, ntau = 400, n = 64 (7.6e6) 185 / 165; 256 problems, ntau = 250, n = 16 (2.2e6) 138 / 118, ntau = 30,
 // n = 64 (3.1e6) 85 / 97 (with plain launches: the programmatic ones take 5 to 10 us off both sides).
 bool hist_form(const ng_ctx* c, const Grid& g, int n) {
-    return g.nf == 1 && g.nb >= NGH_KG && c->bulk_split == NG_BULK_AUTO && n >= 2 * g.k + 2;
+    return g.nf == 1 && form_nb(c, g) >= NGH_KG && c->bulk_split == NG_BULK_AUTO && n >= 2 * g.k + 2;
 }
 bool hist_applies(const ng_ctx* c, const Grid& g, int n) {
-    const double work = 2.0 * g.nb * n * ((double)n + g.ntau);
-    return hist_form(c, g, n) &&
-           work >= (g.nb < 128 ? 14e6 : g.nb < 256 ? 7e6 : g.ntau >= 100 ? 1.8e6 : 4e6);
+    const int nb = form_nb(c, g);
+    const double work = 2.0 * nb * n * ((double)n + g.ntau);
+    return hist_form(c, g, n) && work >= (nb < 128 ? 14e6 : nb < 256 ? 7e6 : g.ntau >= 100 ? 1.8e6 : 4e6);
 }
 // vie2 step: against a warp or a thread per item, with the left-mixing source's direct sums (ntau^2 multiply-adds per
 // problem) in the work: 16e6 where the warp form is the alternative, else 8e6.  Step in us, FP64 kernels / digit
@@ -356,7 +363,7 @@ ng_status boundary_spread(ng_ctx* c, const Grid& g, int n, const HermV& G, const
     ng_status st;
     const int k = g.k, nq = (n <= 2 * k) ? n : k + 1;
     const int64_t terms = std::max(n, g.ntau) + 1;
-    const int64_t want = (4 * (int64_t)c->sms + (int64_t)nq * g.nb - 1) / ((int64_t)nq * g.nb);
+    const int64_t rows = (int64_t)nq * form_nb(c, g), want = (4 * (int64_t)c->sms + rows - 1) / rows;
     const int nchunk = (int)std::max<int64_t>(1, std::min<int64_t>({want, (terms + NG_BND_THREADS - 1) / NG_BND_THREADS, 64}));
     const size_t need = sizeof(cplx) * (size_t)nq * g.nb * nchunk * 2 * D * D;
     if ((st = ensure(c, &c->ws_bnd, &c->ws_bnd_bytes, need))) return st;
@@ -373,13 +380,13 @@ ng_status boundary_spread(ng_ctx* c, const Grid& g, int n, const HermV& G, const
 // The boundary with one lane per problem: nf = 1, batches of 16 and more, n > 2k.  pre_done: the retarded
 // start-up ran with the bulk launch.  Below 16 problems most lanes would be idle and the per-problem forms
 // stay.
-bool bnd1_applies(const Grid& g, int n) { return g.nf == 1 && g.nb >= 16 && n > 2 * g.k; }
+bool bnd1_applies(const ng_ctx* c, const Grid& g, int n) { return g.nf == 1 && form_nb(c, g) >= 16 && n > 2 * g.k; }
 ng_status boundary1(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV& S, const FuncV& eps, bool pre_done,
                     cudaStream_t s) {
     ng_status st;
-    const int J = std::max(n, g.ntau) + 1, groups = (g.nb + 31) / 32;
+    const int J = std::max(n, g.ntau) + 1, groups = (g.nb + 31) / 32, all = (form_nb(c, g) + 31) / 32;
     // two blocks a SM, chunks of four indices (one a warp) or more, at most 48 partial sums to add
-    const int want = std::min(48, std::max(1, (2 * c->sms + groups - 1) / groups));
+    const int want = std::min(48, std::max(1, (2 * c->sms + all - 1) / all));
     const int len = std::max(4, (J + want - 1) / want), nchunk = (J + len - 1) / len;
     if ((st = ensure(c, &c->ws_bnd, &c->ws_bnd_bytes, sizeof(cplx) * (size_t)nchunk * 2 * NG_B1_ROWS * g.nb))) return st;
     if (!pre_done) {
@@ -402,7 +409,7 @@ ng_status boundary_batch(ng_ctx* c, const Grid& g, int n, const HermV& G, const 
     ng_status st;
     const long e = prof_pair(c, 1);
     if (e >= 0) cudaEventRecord(c->ev_pool[e], s);
-    if (D == 1 && bnd1_applies(g, n)) {
+    if (D == 1 && bnd1_applies(c, g, n)) {
         st = boundary1(c, g, n, G, S, eps, false, s);
     } else {
         dep_launch(k_step_boundary<D>, g.nb, NG_BND_THREADS, 0, s)(g, n, G, S, eps, c->d_status);
@@ -422,28 +429,28 @@ ng_status launch_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const
     const int b_les = (int)nblocks(it_les, thr), b_tv = (int)nblocks(it_tv, thr), b_ret = (int)nblocks(it_ret, thr);
     // small batches: one warp per item when one thread per item would not give each SM a block;
     // the warp form splits the left-mixing source over its lanes instead of the FFT pre-pass
-    const int64_t items = it_les + it_tv + it_ret;
+    const int64_t items = it_les + it_tv + it_ret, nb = form_nb(c, g), form_items = items / g.nb * nb;
     const bool digits = hist_applies(c, g, n);
     const bool warp = c->bulk_split == NG_BULK_WARP ||
-                      (c->bulk_split == NG_BULK_AUTO && !digits && items < (int64_t)c->sms * thr);
+                      (c->bulk_split == NG_BULK_AUTO && !digits && form_items < (int64_t)c->sms * thr);
     // small batches: the boundary's (A)-row sums spread over (row, problem, chunk) blocks, and
     // with the warp bulk its retarded start-up in the bulk launch's leading warps
     const int nq = (n <= 2 * k) ? n : k + 1;
     const bool spread = c->bulk_split == NG_BULK_WARP ||
-                        (c->bulk_split == NG_BULK_AUTO && (int64_t)nq * g.nb < 2 * (int64_t)c->sms);
-    const bool lanes = D == 1 && c->bulk_split == NG_BULK_AUTO && bnd1_applies(g, n);
+                        (c->bulk_split == NG_BULK_AUTO && nq * nb < 2 * (int64_t)c->sms);
+    const bool lanes = D == 1 && c->bulk_split == NG_BULK_AUTO && bnd1_applies(c, g, n);
     // lanes per item of k_step_bulk_q (0: not used): below 16 problems the warp form's boundary is the faster one, and
     // above 1000 items a SM a thread per item fills the GPU.  Whole steps in us, warp or thread per item / 8
     // lanes: 16 problems, ntau = 100, n = 300: 126 / 91; 64 problems, ntau = 100, n = 40: 97 / 62; 256 problems,
     // ntau = 30, n = 96: 144 / 124 (4 lanes 128); 4 lanes win from 256 items a SM on.
     int part = 0;
-    if (D == 1 && c->bulk_split == NG_BULK_AUTO && !digits && g.nb >= 16 && items < 1000 * (int64_t)c->sms)
-        part = items < 256 * (int64_t)c->sms ? 8 : 4;
+    if (D == 1 && c->bulk_split == NG_BULK_AUTO && !digits && nb >= 16 && form_items < 1000 * (int64_t)c->sms)
+        part = form_items < 256 * (int64_t)c->sms ? 8 : 4;
     const int64_t w_pre = (part ? lanes : warp && (spread || lanes)) ? g.nb : 0;
     const cplx* tvq = nullptr;
     // its left-mixing source: direct sums while these are below the cost of the FFT's launch (32 problems, ntau = 400,
     // n = 16: 97 against 103 us; ntau = 900: 260 against 167)
-    const bool direct = part ? (double)g.nb * g.ntau * g.ntau < 6e6 : warp;
+    const bool direct = part ? (double)nb * g.ntau * g.ntau < 6e6 : warp;
     ng_status sm = direct ? NG_OK : prep_tvfft(c, g, n, G, S, s, &tvq);
     if (sm) return sm;
     long e0 = prof_pair(c, 0);
@@ -609,7 +616,7 @@ ng_status launch_timestep32(ng_ctx* c, const Grid& g, int n, const HermV& G, con
     long e0 = prof_pair(c, 0);
     if (e0 >= 0) cudaEventRecord(c->ev_pool[e0], s);
     if ((st = launch_minv<D>(c, g, n, S, eps, s))) return st;
-    if (D == 1 && g.nb % 2 == 0) {
+    if (D == 1 && g.nb % 2 == 0 && form_nb(c, g) % 2 == 0) {
         // two problems per thread (16-byte loads of the FP32 copies)
         const int np = g.nb / 2;
         const int p_les = it_les ? (int)nblocks((int64_t)np * (n - k - 1), thr) : 0;
@@ -651,6 +658,8 @@ ng_status lu_solve(ng_ctx* c, int N, int nrhs, int nb, cplx* ws_A, int* ws_piv, 
 // sum below ref_tol), otherwise the caller solves afresh.  Few problems (less than a quarter of the SMs)
 // keep the inverse (k_gj_step) unless the solves run side by side on streams (spread = false): one block per
 // problem would leave the GPU idle.
+// (read: the sum of the updates over all ranks of a sharded run from c->d_scalar, so that all stop together)
+typedef std::function<ng_status(double*)> ReadSum;
 struct MatWs {
     cplx *g, *K, *r, *A, *A2;
     int* piv;
@@ -673,10 +682,10 @@ size_t mat_ws(void* base, int T, int D, int nb, bool inverse, MatWs* w) {
 
 template <int D>
 ng_status mat_solve(ng_ctx* c, const Grid& g, const HermV& G, const MatWs& w, bool inverse, cudaStream_t s, int refine_steps,
-                    double ref_tol, bool* refined_ok) {
+                    double ref_tol, bool* refined_ok, const ReadSum* read) {
     const int T = g.ntau, N = (T + 1) * D, ld = N + D;
     const int64_t items = (int64_t)(T + 1) * g.nb;
-    const bool warp = D <= 4 && items < (int64_t)c->sms * 128;   // as for the bulk items: a warp per item where threads are few
+    const bool warp = D <= 4 && (int64_t)(T + 1) * form_nb(c, g) < (int64_t)c->sms * 128;   // as for the bulk items: a warp per item where threads are few
     const dim3 rows(nblocks((int64_t)N * D * 32, 128), g.nb);
     const cplx* inv = N % 2 ? w.A2 : w.A;   // where the last of N passes ends
     ng_status st = NG_OK;
@@ -698,8 +707,12 @@ ng_status mat_solve(ng_ctx* c, const Grid& g, const HermV& G, const MatWs& w, bo
         for (int r = 0; r < refine_steps; ++r) {
             if ((st = refine(c->d_scalar))) return st;
             double dsum = 0.0;
-            CUDA_TRY(c, cudaMemcpyAsync(&dsum, c->d_scalar, sizeof(double), cudaMemcpyDeviceToHost, s));
-            CUDA_TRY(c, cudaStreamSynchronize(s));
+            if (read) {
+                if ((st = (*read)(&dsum))) return st;
+            } else {
+                CUDA_TRY(c, cudaMemcpyAsync(&dsum, c->d_scalar, sizeof(double), cudaMemcpyDeviceToHost, s));
+                CUDA_TRY(c, cudaStreamSynchronize(s));
+            }
             if (!(dsum == dsum)) return NG_OK;               // non-finite: a fresh solve follows
             if (dsum == 0.0 || dsum > 0.5 * prev) {           // at the round-off floor, or stalled
                 *refined_ok = dsum < ref_tol;
@@ -730,9 +743,10 @@ ng_status mat_solve(ng_ctx* c, const Grid& g, const HermV& G, const MatWs& w, bo
 
 template <int D>
 ng_status launch_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S, const FuncV& eps, cudaStream_t s,
-                     int refine_steps = 0, double ref_tol = 0.0, bool* refined_ok = nullptr, void* ws_ext = nullptr) {
+                     int refine_steps = 0, double ref_tol = 0.0, bool* refined_ok = nullptr, void* ws_ext = nullptr,
+                     const ReadSum* read = nullptr) {
     const int T = g.ntau, N = (T + 1) * D;
-    const bool inverse = mat_inverse(c, N, g.nb, ws_ext == nullptr);
+    const bool inverse = mat_inverse(c, N, form_nb(c, g), ws_ext == nullptr);
     MatWs w;
     const size_t need = mat_ws(nullptr, T, D, g.nb, inverse, &w);
     ng_status st = NG_OK;
@@ -741,13 +755,13 @@ ng_status launch_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S, c
     const int64_t items = (int64_t)(T + 1) * g.nb;
     dep_launch(k_mat_g<D>, nblocks(items, 128), 128, 0, s)(g, eps, w.g);
     if ((st = check_launch(c, "k_mat_g"))) return st;
-    const bool warp = D <= 4 && items < (int64_t)c->sms * 128;
+    const bool warp = D <= 4 && (int64_t)(T + 1) * form_nb(c, g) < (int64_t)c->sms * 128;
     if constexpr (D <= 4) {
         if (warp) dep_launch(k_mat_K_w<D>, nblocks(items * 32, 128), 128, 0, s)(g, S, w.g, w.K);
     }
     if (!warp) dep_launch(k_mat_K<D>, nblocks(items, 128), 128, 0, s)(g, S, w.g, w.K);
     if ((st = check_launch(c, "k_mat_K"))) return st;
-    return mat_solve<D>(c, g, G, w, inverse, s, refine_steps, ref_tol, refined_ok);
+    return mat_solve<D>(c, g, G, w, inverse, s, refine_steps, ref_tol, refined_ok, read);
 }
 
 template <int D>
@@ -761,7 +775,8 @@ ng_status launch_start(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S,
     if constexpr (D <= 4) {
         // one warp per item: the dense solves while the warps fit the GPU at once, the left-mixing row while a thread
         // per item would leave SMs idle, the lesser columns always (k+1 items per problem)
-        const bool ret_w = g.nb <= 4 * c->sms, tv_w = (int64_t)(g.ntau + 1) * g.nb < (int64_t)c->sms * 128;
+        const int64_t nb = form_nb(c, g);
+        const bool ret_w = nb <= 4 * c->sms, tv_w = (g.ntau + 1) * nb < (int64_t)c->sms * 128;
         if (ret_w) dep_launch(k_start_ret_w<D>, g.nb, 32, 0, s)(g, G, S, eps, ws, c->d_status);
         else dep_launch(k_start_ret<D>, nblocks(g.nb, 64), 64, 0, s)(g, G, S, eps, ws, c->d_status);
         if ((st = check_launch(c, "k_start_ret"))) return st;
@@ -804,14 +819,14 @@ ng_status launch_vie2_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV&
                           void** ws, size_t* ws_bytes, int refine_steps = 0, double ref_tol = 0.0,
                           bool* refined_ok = nullptr) {
     const int T = g.ntau, N = (T + 1) * D;
-    const bool inverse = mat_inverse(c, N, g.nb, true);
+    const bool inverse = mat_inverse(c, N, form_nb(c, g), true);
     MatWs w;
     ng_status st = ensure(c, ws, ws_bytes, mat_ws(nullptr, T, D, g.nb, inverse, &w));
     if (st) return st;
     mat_ws(*ws, T, D, g.nb, inverse, &w);
     dep_launch(k_v2_mat_fill<D>, nblocks((int64_t)(T + 1) * g.nb, 128), 128, 0, s)(g, F, Q, w.g, w.K);
     if ((st = check_launch(c, "k_v2_mat_fill"))) return st;
-    return mat_solve<D>(c, g, G, w, inverse, s, refine_steps, ref_tol, refined_ok);
+    return mat_solve<D>(c, g, G, w, inverse, s, refine_steps, ref_tol, refined_ok, nullptr);
 }
 
 // one warp per vie2 bulk item: forced, or for batches with fewer items than 128 per SM
@@ -1119,7 +1134,7 @@ ng_status utimestep_uniform(ng_ctx* c, const Grid& g, int n, const HermV& G, con
         c->uni_key_S = S.ret.p;
         c->uni_key_eps = eps.p;
     }
-    std::vector<UHost> info(g.nb, UHost{g.nf, g.nt, g.ntau, g.k, g.nb == 1});
+    std::vector<UHost> info(g.nb, UHost{g.nf, g.nt, g.ntau, g.k, g.nb == 1 && form_nb(c, g) == 1});
     std::vector<int> active(g.nb);
     for (int kb = 0; kb < g.nb; ++kb) active[kb] = kb;
     return ustep(c, d_probs, info, active, n, 128, s);
@@ -1175,12 +1190,12 @@ size_t start_ws_bytes(const Grid& g) {
     return sizeof(cplx) * g.nb * (N * N + g.k * D * D);
 }
 ng_status do_mat_refine(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S, const FuncV& eps, cudaStream_t s,
-                        int steps, double tol, bool* ok) {
+                        int steps, double tol, bool* ok, const ReadSum* read) {
     switch (g.nf) {
-        case 1: return launch_mat<1>(c, g, G, S, eps, s, steps, tol, ok);
-        case 2: return launch_mat<2>(c, g, G, S, eps, s, steps, tol, ok);
-        case 4: return launch_mat<4>(c, g, G, S, eps, s, steps, tol, ok);
-        default: return launch_mat<8>(c, g, G, S, eps, s, steps, tol, ok);
+        case 1: return launch_mat<1>(c, g, G, S, eps, s, steps, tol, ok, nullptr, read);
+        case 2: return launch_mat<2>(c, g, G, S, eps, s, steps, tol, ok, nullptr, read);
+        case 4: return launch_mat<4>(c, g, G, S, eps, s, steps, tol, ok, nullptr, read);
+        default: return launch_mat<8>(c, g, G, S, eps, s, steps, tol, ok, nullptr, read);
     }
 }
 ng_status do_start(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S, const FuncV& eps, cudaStream_t s,
@@ -1714,6 +1729,11 @@ static ng_status run_2b_impl(ng_ctx* c, const ng_grid* grid, ng_herm G, ng_herm 
         if ((st = check_shard(c, g, sh, &rt))) return st;
         rtp = &rt;
     }
+    struct RunNk {   // forms and chunks by the k-points of all ranks until the run returns
+        ng_ctx* c;
+        ~RunNk() { c->run_nk = 0; }
+    } run_nk{c};
+    if (sh) c->run_nk = sh->nk;
     // problems summed by the convergence distances (all ranks')
     const double nk_all = sh ? (double)sh->nk : (double)G.ldk;
     cudaStream_t s = (cudaStream_t)stream;
@@ -1733,6 +1753,7 @@ static ng_status run_2b_impl(ng_ctx* c, const ng_grid* grid, ng_herm G, ng_herm 
         for (int r = 0; r < sh->nranks; ++r) *err += per[r];
         return NG_OK;
     };
+    const ReadSum read_sum = read_distance;
     const int k = g.k, dd = g.nf * g.nf, T = g.ntau;
     // Sigma slices from..to from Gloc: from = to = -1 the Matsubara slice, 0..k the start-up
     // slices, n > k one time step.  GW: P, K and K^ddagger on those slices, then the chi
@@ -1858,7 +1879,7 @@ static ng_status run_2b_impl(ng_ctx* c, const ng_grid* grid, ng_herm G, ng_herm 
             // after two fresh solves the operator changes little between iterations: refine the
             // current iterate with the kept LU factors, refactor only if that stalls
             bool refined = false;
-            if (mats_it >= 2 && (st = do_mat_refine(c, g, Gv, Sv, mf, s, 30, 1e-13 * nel_mat, &refined))) return st;
+            if (mats_it >= 2 && (st = do_mat_refine(c, g, Gv, Sv, mf, s, 30, 1e-13 * nel_mat, &refined, &read_sum))) return st;
             if (!refined && (st = do_mat(c, g, Gv, Sv, mf, s))) return st;
             CUDA_TRY(c, cudaMemsetAsync(c->d_scalar, 0, sizeof(double), s));
             if ((st = do_distance(c, g, -1, Gv, Pv, c->d_scalar, s))) return st;
