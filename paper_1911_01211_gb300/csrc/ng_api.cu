@@ -106,6 +106,8 @@ struct ng_ctx {
     size_t ws_tvq_bytes = 0;
     void* ws_hist = nullptr;         // digit-product history sums: row vectors, digits, unit sums
     size_t ws_hist_bytes = 0;
+    size_t hist_refused = 0;         // bytes the device had no room for at step hist_refused_n (0: none refused)
+    int hist_refused_n = 0;
     void* ws_tw = nullptr;           // twiddle table of length tw_L
     size_t ws_tw_bytes = 0;
     int tw_L = 0;
@@ -332,13 +334,44 @@ bool hist_applies_vie2(const ng_ctx* c, const Grid& g, int n) {
     const double N = n, T = g.ntau, work = g.nb * (2.0 * N * (N + T) + T * T);
     return hist_form(c, g, n) && work >= ((double)g.nb * (2.0 * N + T) < 128.0 * c->sms ? 16e6 : 8e6);
 }
-// *w describes the sums; *ok = false without room for the workspace: the step keeps the FP64 kernels
-ng_status hist_sums(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV& S, const HermV& Scc, HistWs* w, bool* ok,
+// Whether the digit products of step n have their workspace of `need` bytes.  They can be done without: where the device
+// has no room the call takes the form it would take otherwise, leaves no message, and the later steps of the
+// run do not ask again (an earlier step, of another run, does).
+bool hist_room(ng_ctx* c, size_t need, int n) {
+    if (c->ws_hist_bytes >= need) return true;
+    if (c->hist_refused && need >= c->hist_refused && n >= c->hist_refused_n) return false;
+    void* p = nullptr;
+    cudaError_t e = cudaMalloc(&p, need);
+    if (e != cudaSuccess && c->ws_hist) {   // again with the smaller one given back
+        cudaGetLastError();
+        cudaFree(c->ws_hist);
+        c->ws_hist = nullptr;
+        c->ws_hist_bytes = 0;
+        e = cudaMalloc(&p, need);
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        c->hist_refused = need;
+        c->hist_refused_n = n;
+        return false;
+    }
+    cudaFree(c->ws_hist);
+    c->ws_hist = p;
+    c->ws_hist_bytes = need;
+    c->hist_refused = 0;
+    return true;
+}
+// problems of the row vectors: 1 when S and Scc are shared by all
+int hist_nv(const Grid& g, const HermV& S, const HermV& Scc) {
+    return (S.ret.ldk == 1 && Scc.les.ldk == 1 && S.tv.ldk == 1) ? 1 : g.nb;
+}
+bool hist_ready(ng_ctx* c, const Grid& g, int n, const HermV& S, const HermV& Scc) {
+    return hist_room(c, hist_ws_bytes(g.nt, g.ntau, g.nb, hist_nv(g, S, Scc)), n);
+}
+// the sums into the workspace (hist_ready), which *w describes
+ng_status hist_sums(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV& S, const HermV& Scc, HistWs* w,
                     cudaStream_t s) {
-    const int nv = (S.ret.ldk == 1 && Scc.les.ldk == 1 && S.tv.ldk == 1) ? 1 : g.nb;
-    *ok = false;
-    const size_t need = hist_ws_bytes(g.nt, g.ntau, g.nb, nv);
-    if (c->ws_hist_bytes < need && ensure(c, &c->ws_hist, &c->ws_hist_bytes, need)) return NG_OK;   // no room: FP64 kernels
+    const int nv = hist_nv(g, S, Scc);
     *w = hist_ws_layout(c->ws_hist, g.nt, n, g.ntau, g.k, g.nb, nv);
     HistRow r{S.ret.p + tri(n) * S.ret.ldk, Scc.les.p + tri(n) * Scc.les.ldk,
               S.tv.p + (int64_t)n * (g.ntau + 1) * S.tv.ldk, S.ret.ldk, Scc.les.ldk, S.tv.ldk};
@@ -351,7 +384,6 @@ ng_status hist_sums(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV
         cudaGetLastError();
         return fail(c, NG_ECUDA, "launch of k_hist_mma failed");
     }
-    *ok = true;
     return NG_OK;
 }
 
@@ -430,7 +462,7 @@ ng_status launch_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const
     // small batches: one warp per item when one thread per item would not give each SM a block;
     // the warp form splits the left-mixing source over its lanes instead of the FFT pre-pass
     const int64_t items = it_les + it_tv + it_ret, nb = form_nb(c, g), form_items = items / g.nb * nb;
-    const bool digits = hist_applies(c, g, n);
+    const bool digits = hist_applies(c, g, n) && hist_ready(c, g, n, S, S);
     const bool warp = c->bulk_split == NG_BULK_WARP ||
                       (c->bulk_split == NG_BULK_AUTO && !digits && form_items < (int64_t)c->sms * thr);
     // small batches: the boundary's (A)-row sums spread over (row, problem, chunk) blocks, and
@@ -456,11 +488,10 @@ ng_status launch_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const
     long e0 = prof_pair(c, 0);
     if (e0 >= 0) cudaEventRecord(c->ev_pool[e0], s);
     if ((sm = launch_minv<D>(c, g, n, S, eps, s))) return sm;
-    bool hist = false;   // their sums are per unit and problem: k_hist_close finishes the items
-    HistWs hw;
-    if (D == 1 && digits && (sm = hist_sums(c, g, n, G, S, S, &hw, &hist, s))) return sm;
-    const int pre = hist && lanes ? (int)nblocks(g.nb, thr / 32) : 0;   // leading blocks: the retarded start-up
-    if (hist) {
+    HistWs hw;   // their sums are per unit and problem: k_hist_close finishes the items
+    if (D == 1 && digits && (sm = hist_sums(c, g, n, G, S, S, &hw, s))) return sm;
+    const int pre = digits && lanes ? (int)nblocks(g.nb, thr / 32) : 0;   // leading blocks: the retarded start-up
+    if (digits) {
         dep_launch(k_hist_close, pre + b_les + b_tv + b_ret, thr, 0, s)(g, n, G, S, eps, hw, (const cplx*)c->ws_minv, pre, b_les,
                                                                 b_tv, tvq, c->d_status);
     } else if (part) {
@@ -577,7 +608,7 @@ ng_status launch_timestepdf(ng_ctx* c, const Grid& g, int n, const HermV& G, con
     ng_status st;
     // the digit products are exact and read half the bytes of the double-float sums (16 B per element for
     // two multiply-adds): a step of 256 problems, n = 900, ntau = 400: 2.07 -> 1.59 ms
-    if (hist_applies(c, g, n)) return launch_timestep<D>(c, g, n, G, S, eps, s);
+    if (hist_applies(c, g, n) && hist_ready(c, g, n, S, S)) return launch_timestep<D>(c, g, n, G, S, eps, s);
     if ((st = update_shadow_df(c, c->dfG, g, G, n, false, s))) return st;
     if ((st = update_shadow_df(c, c->dfS, g, S, n, true, s))) return st;
     const int k = g.k, thr = 128;
@@ -830,9 +861,9 @@ ng_status launch_vie2_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV&
 }
 
 // one warp per vie2 bulk item: forced, or for batches with fewer items than 128 per SM
-bool vie2_warp(const ng_ctx* c, const Grid& g, int n) {
+bool vie2_warp(const ng_ctx* c, const Grid& g, int n, bool digits) {
     const int64_t items = (int64_t)g.nb * ((n - 1) + (g.ntau + 1) + n);
-    if (hist_applies_vie2(c, g, n)) return false;
+    if (digits) return false;
     return c->bulk_split == NG_BULK_WARP || (c->bulk_split == NG_BULK_AUTO && items < (int64_t)c->sms * 128);
 }
 
@@ -1011,7 +1042,7 @@ ng_status histu_sums(ng_ctx* c, const UProb* d_probs, const std::vector<UHost>& 
     tab->np = (int)(c1 - c0);
     tab->start[tab->np] = tab->ntask;
     if (off > need) return fail(c, NG_EINVAL, "the digit sums of step %d need %zu bytes, their workspace holds %zu", n, off, need);
-    if (c->ws_hist_bytes < need && ensure(c, &c->ws_hist, &c->ws_hist_bytes, need)) return NG_OK;   // no room
+    if (!hist_room(c, need, n)) return NG_OK;
     tab->probs = (HistUProb*)c->ws_hist;
     tab->base = (char*)c->ws_hist;
     tab->next = (int*)((char*)c->ws_hist + head - 256);
@@ -1460,11 +1491,10 @@ ng_status ng_vie2_timestep(ng_ctx* c, const ng_grid* grid, int tstp, ng_herm G, 
     if (schedule == NG_SERIAL) return fail(c, NG_EUNSUPPORTED, "the vie2 time step runs the mixed schedule only");
     if (schedule != NG_MIXED) return fail(c, NG_EINVAL, "unknown schedule %d", schedule);
     const cplx* tvq = nullptr;
-    const bool w = vie2_warp(c, g, tstp);
+    const bool hist = hist_applies_vie2(c, g, tstp) && hist_ready(c, g, tstp, Fv, Fccv), w = vie2_warp(c, g, tstp, hist);
     if (!w && (st = prep_tvfft(c, g, tstp, Gv, Fv, (cudaStream_t)stream, &tvq))) return st;
-    bool hist = false;
     HistWs hw;
-    if (!w && hist_applies_vie2(c, g, tstp) && (st = hist_sums(c, g, tstp, Gv, Fv, Fccv, &hw, &hist, (cudaStream_t)stream))) return st;
+    if (hist && (st = hist_sums(c, g, tstp, Gv, Fv, Fccv, &hw, (cudaStream_t)stream))) return st;
     if (vie2_step_launch(g, tstp, Gv, Fv, Fccv, Qv, tvq, w, hist ? &hw : nullptr, c->d_status, (cudaStream_t)stream) !=
         cudaSuccess) {
         cudaGetLastError();
@@ -1804,12 +1834,11 @@ static ng_status run_2b_impl(ng_ctx* c, const ng_grid* grid, ng_herm G, ng_herm 
         } else {
             for (int n = from; n <= to && e == cudaSuccess; ++n) {
                 const cplx* tvq = nullptr;
-                const bool w = vie2_warp(c, gw->gb, n);
+                const bool hist = hist_applies_vie2(c, gw->gb, n) && hist_ready(c, gw->gb, n, gw->K, gw->Kcc);
+                const bool w = vie2_warp(c, gw->gb, n, hist);
                 if (!w && (r = prep_tvfft(c, gw->gb, n, gw->X, gw->K, s, &tvq, false))) return r;
-                bool hist = false;
                 HistWs hw;
-                if (!w && hist_applies_vie2(c, gw->gb, n) && (r = hist_sums(c, gw->gb, n, gw->X, gw->K, gw->Kcc, &hw, &hist, s)))
-                    return r;
+                if (hist && (r = hist_sums(c, gw->gb, n, gw->X, gw->K, gw->Kcc, &hw, s))) return r;
                 e = vie2_step_launch(gw->gb, n, gw->X, gw->K, gw->Kcc, gw->P, tvq, w, hist ? &hw : nullptr, c->d_status, s);
             }
         }
