@@ -285,13 +285,11 @@ ng_status launch_minv(ng_ctx* c, const Grid& g, int n, const HermV& S, const Fun
 }
 
 // FFT pre-pass of the left-mixing source of step n (*tvq = nullptr when the direct sums are
-// used: NG_TVSRC_DIRECT, or nf / ntau outside what the transforms support)
+// used: NG_TVSRC_DIRECT, or nf / ntau outside what the transforms support); tvfft_room: its buffer and twiddles
 // prof: record the pre-pass as its own profile entry (not inside a GW evaluation, which is
 // timed as a whole)
-ng_status prep_tvfft(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV& S, cudaStream_t s,
-                     const cplx** tvq, bool prof = true) {
-    *tvq = nullptr;
-    if (c->tvsrc == NG_TVSRC_DIRECT || !tvfft_supported(g.nf, g.ntau)) return NG_OK;
+bool tvfft_used(const ng_ctx* c, const Grid& g) { return c->tvsrc != NG_TVSRC_DIRECT && tvfft_supported(g.nf, g.ntau); }
+ng_status tvfft_room(ng_ctx* c, const Grid& g, const HermV& S, cudaStream_t s) {
     ng_status st;
     const int L = tvfft_length(g.ntau);
     if (c->tw_L != L) {
@@ -299,8 +297,14 @@ ng_status prep_tvfft(ng_ctx* c, const Grid& g, int n, const HermV& G, const Herm
         if (tvfft_twiddles((cplx*)c->ws_tw, L, s) != cudaSuccess) return check_launch(c, "k_twiddle");
         c->tw_L = L;
     }
-    const size_t need = tvfft_out_bytes(g, S.tv.ldk);
-    if ((st = ensure(c, &c->ws_tvq, &c->ws_tvq_bytes, need))) return st;
+    return ensure(c, &c->ws_tvq, &c->ws_tvq_bytes, tvfft_out_bytes(g, S.tv.ldk));
+}
+ng_status prep_tvfft(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV& S, cudaStream_t s,
+                     const cplx** tvq, bool prof = true) {
+    *tvq = nullptr;
+    if (!tvfft_used(c, g)) return NG_OK;
+    ng_status st = tvfft_room(c, g, S, s);
+    if (st) return st;
     long e = prof ? prof_pair(c, 2) : -1;
     if (e >= 0) cudaEventRecord(c->ev_pool[e], s);
     if (tvfft_launch(g, c->W, n, S.tv, G.mat, (const cplx*)c->ws_tw, (cplx*)c->ws_tvq, s) != cudaSuccess) {
@@ -336,9 +340,15 @@ bool hist_applies_vie2(const ng_ctx* c, const Grid& g, int n) {
 }
 // Whether the digit products of step n have their workspace of `need` bytes.  They can be done without: where the device
 // has no room the call takes the form it would take otherwise, leaves no message, and the later steps of the
-// run do not ask again (an earlier step, of another run, does).
-bool hist_room(ng_ctx* c, size_t need, int n) {
+// run do not ask again (an earlier step, of another run, does).  A step under stream capture, which cannot allocate,
+// takes what is there.
+bool hist_room(ng_ctx* c, size_t need, int n, cudaStream_t s) {
     if (c->ws_hist_bytes >= need) return true;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
     if (c->hist_refused && need >= c->hist_refused && n >= c->hist_refused_n) return false;
     void* p = nullptr;
     cudaError_t e = cudaMalloc(&p, need);
@@ -365,8 +375,8 @@ bool hist_room(ng_ctx* c, size_t need, int n) {
 int hist_nv(const Grid& g, const HermV& S, const HermV& Scc) {
     return (S.ret.ldk == 1 && Scc.les.ldk == 1 && S.tv.ldk == 1) ? 1 : g.nb;
 }
-bool hist_ready(ng_ctx* c, const Grid& g, int n, const HermV& S, const HermV& Scc) {
-    return hist_room(c, hist_ws_bytes(g.nt, g.ntau, g.nb, hist_nv(g, S, Scc)), n);
+bool hist_ready(ng_ctx* c, const Grid& g, int n, const HermV& S, const HermV& Scc, cudaStream_t s) {
+    return hist_room(c, hist_ws_bytes(g.nt, g.ntau, g.nb, hist_nv(g, S, Scc)), n, s);
 }
 // the sums into the workspace (hist_ready), which *w describes
 ng_status hist_sums(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV& S, const HermV& Scc, HistWs* w,
@@ -413,14 +423,26 @@ ng_status boundary_spread(ng_ctx* c, const Grid& g, int n, const HermV& G, const
 // start-up ran with the bulk launch.  Below 16 problems most lanes would be idle and the per-problem forms
 // stay.
 bool bnd1_applies(const ng_ctx* c, const Grid& g, int n) { return g.nf == 1 && form_nb(c, g) >= 16 && n > 2 * g.k; }
+constexpr int B1_CHUNKS = 48;   // partial sums to add, at most
+ng_status bnd1_room(ng_ctx* c, const Grid& g) {
+    return ensure(c, &c->ws_bnd, &c->ws_bnd_bytes, sizeof(cplx) * (size_t)B1_CHUNKS * 2 * NG_B1_ROWS * g.nb);
+}
+// What the forms of any step of this grid need beyond the first one's, so that the steps after an eager one allocate
+// nothing for a form that sets in later (steps captured into a graph)
+ng_status step_room(ng_ctx* c, const Grid& g, const HermV& S, cudaStream_t s) {
+    if (g.nf != 1 || form_nb(c, g) < 16) return NG_OK;
+    ng_status st = bnd1_room(c, g);
+    if (st == NG_OK && tvfft_used(c, g)) st = tvfft_room(c, g, S, s);
+    return st;
+}
 ng_status boundary1(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV& S, const FuncV& eps, bool pre_done,
                     cudaStream_t s) {
     ng_status st;
     const int J = std::max(n, g.ntau) + 1, groups = (g.nb + 31) / 32, all = (form_nb(c, g) + 31) / 32;
-    // two blocks a SM, chunks of four indices (one a warp) or more, at most 48 partial sums to add
-    const int want = std::min(48, std::max(1, (2 * c->sms + all - 1) / all));
+    // two blocks a SM, chunks of four indices (one a warp) or more
+    const int want = std::min(B1_CHUNKS, std::max(1, (2 * c->sms + all - 1) / all));
     const int len = std::max(4, (J + want - 1) / want), nchunk = (J + len - 1) / len;
-    if ((st = ensure(c, &c->ws_bnd, &c->ws_bnd_bytes, sizeof(cplx) * (size_t)nchunk * 2 * NG_B1_ROWS * g.nb))) return st;
+    if ((st = bnd1_room(c, g))) return st;
     if (!pre_done) {
         dep_launch(k_bnd_pre<1>, g.nb, 32, 0, s)(g, n, G, S, eps, c->d_status);
         if ((st = check_launch(c, "k_bnd_pre"))) return st;
@@ -462,7 +484,7 @@ ng_status launch_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const
     // small batches: one warp per item when one thread per item would not give each SM a block;
     // the warp form splits the left-mixing source over its lanes instead of the FFT pre-pass
     const int64_t items = it_les + it_tv + it_ret, nb = form_nb(c, g), form_items = items / g.nb * nb;
-    const bool digits = hist_applies(c, g, n) && hist_ready(c, g, n, S, S);
+    const bool digits = hist_applies(c, g, n) && hist_ready(c, g, n, S, S, s);
     const bool warp = c->bulk_split == NG_BULK_WARP ||
                       (c->bulk_split == NG_BULK_AUTO && !digits && form_items < (int64_t)c->sms * thr);
     // small batches: the boundary's (A)-row sums spread over (row, problem, chunk) blocks, and
@@ -608,7 +630,7 @@ ng_status launch_timestepdf(ng_ctx* c, const Grid& g, int n, const HermV& G, con
     ng_status st;
     // the digit products are exact and read half the bytes of the double-float sums (16 B per element for
     // two multiply-adds): a step of 256 problems, n = 900, ntau = 400: 2.07 -> 1.59 ms
-    if (hist_applies(c, g, n) && hist_ready(c, g, n, S, S)) return launch_timestep<D>(c, g, n, G, S, eps, s);
+    if (hist_applies(c, g, n) && hist_ready(c, g, n, S, S, s)) return launch_timestep<D>(c, g, n, G, S, eps, s);
     if ((st = update_shadow_df(c, c->dfG, g, G, n, false, s))) return st;
     if ((st = update_shadow_df(c, c->dfS, g, S, n, true, s))) return st;
     const int k = g.k, thr = 128;
@@ -1042,7 +1064,7 @@ ng_status histu_sums(ng_ctx* c, const UProb* d_probs, const std::vector<UHost>& 
     tab->np = (int)(c1 - c0);
     tab->start[tab->np] = tab->ntask;
     if (off > need) return fail(c, NG_EINVAL, "the digit sums of step %d need %zu bytes, their workspace holds %zu", n, off, need);
-    if (!hist_room(c, need, n)) return NG_OK;
+    if (!hist_room(c, need, n, s)) return NG_OK;
     tab->probs = (HistUProb*)c->ws_hist;
     tab->base = (char*)c->ws_hist;
     tab->next = (int*)((char*)c->ws_hist + head - 256);
@@ -1196,6 +1218,7 @@ ng_status do_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const Her
         // ran the 4-site chain's step at half this form's speed)
         return utimestep_uniform(c, g, n, G, S, eps, s);
     }
+    if (ng_status st = step_room(c, g, S, s)) return st;
     if (precision == NG_DF64)
         return g.nf == 1 ? launch_timestepdf<1>(c, g, n, G, S, eps, s) : launch_timestepdf<2>(c, g, n, G, S, eps, s);
     if (precision == NG_F32C)
@@ -1491,7 +1514,7 @@ ng_status ng_vie2_timestep(ng_ctx* c, const ng_grid* grid, int tstp, ng_herm G, 
     if (schedule == NG_SERIAL) return fail(c, NG_EUNSUPPORTED, "the vie2 time step runs the mixed schedule only");
     if (schedule != NG_MIXED) return fail(c, NG_EINVAL, "unknown schedule %d", schedule);
     const cplx* tvq = nullptr;
-    const bool hist = hist_applies_vie2(c, g, tstp) && hist_ready(c, g, tstp, Fv, Fccv), w = vie2_warp(c, g, tstp, hist);
+    const bool hist = hist_applies_vie2(c, g, tstp) && hist_ready(c, g, tstp, Fv, Fccv, (cudaStream_t)stream), w = vie2_warp(c, g, tstp, hist);
     if (!w && (st = prep_tvfft(c, g, tstp, Gv, Fv, (cudaStream_t)stream, &tvq))) return st;
     HistWs hw;
     if (hist && (st = hist_sums(c, g, tstp, Gv, Fv, Fccv, &hw, (cudaStream_t)stream))) return st;
@@ -1834,7 +1857,7 @@ static ng_status run_2b_impl(ng_ctx* c, const ng_grid* grid, ng_herm G, ng_herm 
         } else {
             for (int n = from; n <= to && e == cudaSuccess; ++n) {
                 const cplx* tvq = nullptr;
-                const bool hist = hist_applies_vie2(c, gw->gb, n) && hist_ready(c, gw->gb, n, gw->K, gw->Kcc);
+                const bool hist = hist_applies_vie2(c, gw->gb, n) && hist_ready(c, gw->gb, n, gw->K, gw->Kcc, s);
                 const bool w = vie2_warp(c, gw->gb, n, hist);
                 if (!w && (r = prep_tvfft(c, gw->gb, n, gw->X, gw->K, s, &tvq, false))) return r;
                 HistWs hw;
