@@ -70,7 +70,8 @@ struct ng_ctx {
     void* ws_gwk = nullptr;          // k-space GW: compact real-space slice buffers
     size_t ws_gwk_bytes = 0;
     void* ws_gwmat = nullptr;        // GW driver: Matsubara workspace of the chi solve (ws_mat
-    size_t ws_gwmat_bytes = 0;       // keeps the LU factors of G^M between iterations)
+    size_t ws_gwmat_bytes = 0;       // keeps what refines G^M between iterations)
+    bool mat_kept = false, gwmat_kept = false;   // what the last fresh solve left there: the inverse, else LU factors
     // per-launch timing of the time-step kernels (ng_profile_enable / ng_profile_read)
     bool prof = false;
     std::vector<cudaEvent_t> ev_pool;
@@ -698,7 +699,19 @@ ng_status lu_solve_p(ng_ctx* c, int N, int nrhs, int nb, cplx* ws_A, int* ws_piv
     dep_launch(k_lu_solve<PB>, nb, NG_LU_THREADS, smem, s)(N, nrhs, ws_A, ws_piv, c->d_status);
     return check_launch(c, "k_lu_solve");
 }
-ng_status lu_solve(ng_ctx* c, int N, int nrhs, int nb, cplx* ws_A, int* ws_piv, cudaStream_t s) {
+// spread: column by column with the updates over the GPU
+ng_status lu_solve(ng_ctx* c, int N, int nrhs, int nb, cplx* ws_A, int* ws_piv, bool spread, cudaStream_t s) {
+    if (spread) {
+        ng_status st;
+        for (int col = 0; col < N; ++col) {
+            dep_launch(k_lu_col, nb, NG_LU_THREADS, 0, s)(N, nrhs, ws_A, ws_piv, col, c->d_status);
+            const int64_t items = (int64_t)(N - col - 1) * (N + nrhs - col - 1);
+            if (items > 0) dep_launch(k_lu_rank1, dim3(nblocks(items, 256), nb), 256, 0, s)(N, nrhs, ws_A, col);
+            if (col % 256 == 0 && (st = check_launch(c, "k_lu_col/k_lu_rank1"))) return st;
+        }
+        dep_launch(k_lu_backsub, nb, NG_LU_THREADS, 0, s)(N, nrhs, ws_A);
+        return check_launch(c, "k_lu_backsub");
+    }
     if (N <= 800) return lu_solve_p<16>(c, N, nrhs, nb, ws_A, ws_piv, s);
     if (N <= 1600) return lu_solve_p<8>(c, N, nrhs, nb, ws_A, ws_piv, s);
     if (N <= 3200) return lu_solve_p<4>(c, N, nrhs, nb, ws_A, ws_piv, s);
@@ -708,9 +721,8 @@ ng_status lu_solve(ng_ctx* c, int N, int nrhs, int nb, cplx* ws_A, int* ws_piv, 
 // The discretised Matsubara equation X = g + [K * X]^M for the right-hand sides and kernels in ws (as laid out
 // by mat_ws): refine_steps = 0: a fresh solve; > 0: refinement of the current G^M with what the last fresh solve
 // kept in ws (its LU factors, or the inverse), at most refine_steps steps; *refined_ok reports convergence (update
-// sum below ref_tol), otherwise the caller solves afresh.  Few problems (less than a quarter of the SMs)
-// keep the inverse (k_gj_step) unless the solves run side by side on streams (spread = false): one block per
-// problem would leave the GPU idle.
+// sum below ref_tol), otherwise the caller solves afresh.  Few problems (less than a quarter of the SMs) spread over
+// the GPU unless the solves run side by side on streams (ws_ext): one block per problem would leave it idle.
 // (read: the sum of the updates over all ranks of a sharded run from c->d_scalar, so that all stop together)
 typedef std::function<ng_status(double*)> ReadSum;
 struct MatWs {
@@ -718,7 +730,31 @@ struct MatWs {
     int* piv;
     unsigned long long* keys;
 };
-bool mat_inverse(const ng_ctx* c, int N, int nb, bool spread) { return spread && 4 * (int64_t)nb < c->sms && N < 0xffff; }
+bool mat_spread(const ng_ctx* c, int nb, bool alone) { return alone && 4 * (int64_t)nb < c->sms; }
+// Of these a solve whose result is refined (again) keeps the inverse (k_gj_step), with which a refinement is a product:
+// 9 us for 402 unknowns, where the two substitutions take half a millisecond, tens of times in a set-up.  A solve
+// for itself takes the faster of the two, the inverse while its passes are short (nb N^2 <= 4e5), else the LU, of a
+// third of its arithmetic, in ms LU / inverse: 1 problem of 402 unknowns (1.6e5) 5 / 2.9; 37 of 101 (3.8e5) about 1.3 / 1.3;
+// 8 of 401 (1.3e6) 5 / 9.7, 16 of 401 (2.6e6) 5.3 / 19.3, 37 of 401 8.4 / 41, 4 of 801 11 / 38, 1 of 1501 21 / 58, 1 of 3001
+// 96 / 435.  8 orbitals take the LU: the refinement step that follows the inverse costs them more than it saves.
+bool mat_inverse(const ng_ctx* c, int D, int N, int nb, bool alone, bool again) {
+    return mat_spread(c, nb, alone) && N < 0xffff && (again || (D <= 4 && (double)nb * N * N <= 4e5));
+}
+// room for the inverse of a solve that is refined; without it the LU is kept
+bool mat_room(void** p, size_t* have, size_t need) {
+    if (*have >= need) return true;
+    void* q = nullptr;
+    if (*p) cudaFree(*p);
+    *p = nullptr;
+    *have = 0;
+    if (cudaMalloc(&q, need) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    *p = q;
+    *have = need;
+    return true;
+}
 size_t mat_ws(void* base, int T, int D, int nb, bool inverse, MatWs* w) {
     const size_t N = (size_t)(T + 1) * D, b_g = (size_t)nb * N * D, b_A = (size_t)nb * N * (N + D);
     cplx* p = (cplx*)base;
@@ -734,7 +770,7 @@ size_t mat_ws(void* base, int T, int D, int nb, bool inverse, MatWs* w) {
 }
 
 template <int D>
-ng_status mat_solve(ng_ctx* c, const Grid& g, const HermV& G, const MatWs& w, bool inverse, cudaStream_t s, int refine_steps,
+ng_status mat_solve(ng_ctx* c, const Grid& g, const HermV& G, const MatWs& w, bool inverse, bool spread, cudaStream_t s, int refine_steps,
                     double ref_tol, bool* refined_ok, const ReadSum* read) {
     const int T = g.ntau, N = (T + 1) * D, ld = N + D;
     const int64_t items = (int64_t)(T + 1) * g.nb;
@@ -778,7 +814,7 @@ ng_status mat_solve(ng_ctx* c, const Grid& g, const HermV& G, const MatWs& w, bo
     dep_launch(k_mat_assemble<D>, nblocks((int64_t)(T + 1) * (T + 2) * g.nb, 256), 256, 0, s)(g, w.g, w.K, w.A);
     if ((st = check_launch(c, "k_mat_assemble"))) return st;
     if (!inverse) {
-        if ((st = lu_solve(c, N, D, g.nb, w.A, w.piv, s))) return st;
+        if ((st = lu_solve(c, N, D, g.nb, w.A, w.piv, spread, s))) return st;
         dep_launch(k_mat_store<D>, nblocks(items, 128), 128, 0, s)(g, w.A, G, c->d_status);
         return check_launch(c, "k_mat_store");
     }
@@ -797,13 +833,16 @@ ng_status mat_solve(ng_ctx* c, const Grid& g, const HermV& G, const MatWs& w, bo
 template <int D>
 ng_status launch_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S, const FuncV& eps, cudaStream_t s,
                      int refine_steps = 0, double ref_tol = 0.0, bool* refined_ok = nullptr, void* ws_ext = nullptr,
-                     const ReadSum* read = nullptr) {
+                     const ReadSum* read = nullptr, bool again = false) {
     const int T = g.ntau, N = (T + 1) * D;
-    const bool inverse = mat_inverse(c, N, form_nb(c, g), ws_ext == nullptr);
+    bool inverse = refine_steps > 0 ? c->mat_kept : mat_inverse(c, D, N, form_nb(c, g), ws_ext == nullptr, again);
     MatWs w;
-    const size_t need = mat_ws(nullptr, T, D, g.nb, inverse, &w);
     ng_status st = NG_OK;
-    if (!ws_ext && (st = ensure(c, &c->ws_mat, &c->ws_mat_bytes, need))) return st;
+    if (!ws_ext) {
+        if (again && inverse) inverse = mat_room(&c->ws_mat, &c->ws_mat_bytes, mat_ws(nullptr, T, D, g.nb, true, &w));
+        if ((st = ensure(c, &c->ws_mat, &c->ws_mat_bytes, mat_ws(nullptr, T, D, g.nb, inverse, &w)))) return st;
+        c->mat_kept = inverse;
+    }
     mat_ws(ws_ext ? ws_ext : c->ws_mat, T, D, g.nb, inverse, &w);
     const int64_t items = (int64_t)(T + 1) * g.nb;
     dep_launch(k_mat_g<D>, nblocks(items, 128), 128, 0, s)(g, eps, w.g);
@@ -814,7 +853,7 @@ ng_status launch_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S, c
     }
     if (!warp) dep_launch(k_mat_K<D>, nblocks(items, 128), 128, 0, s)(g, S, w.g, w.K);
     if ((st = check_launch(c, "k_mat_K"))) return st;
-    return mat_solve<D>(c, g, G, w, inverse, s, refine_steps, ref_tol, refined_ok, read);
+    return mat_solve<D>(c, g, G, w, inverse, mat_spread(c, form_nb(c, g), ws_ext == nullptr), s, refine_steps, ref_tol, refined_ok, read);
 }
 
 template <int D>
@@ -869,17 +908,19 @@ __global__ void k_v2_mat_fill(Grid g, HermV F, HermV Q, cplx* ws_g, cplx* ws_K) 
 // self-consistency loop changes little between iterations), as the Dyson Matsubara solve does
 template <int D>
 ng_status launch_vie2_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV& F, const HermV& Q, cudaStream_t s,
-                          void** ws, size_t* ws_bytes, int refine_steps = 0, double ref_tol = 0.0,
+                          void** ws, size_t* ws_bytes, bool* kept, bool again, int refine_steps = 0, double ref_tol = 0.0,
                           bool* refined_ok = nullptr) {
     const int T = g.ntau, N = (T + 1) * D;
-    const bool inverse = mat_inverse(c, N, form_nb(c, g), true);
+    bool inverse = refine_steps > 0 ? *kept : mat_inverse(c, D, N, form_nb(c, g), true, again);
     MatWs w;
+    if (again && inverse) inverse = mat_room(ws, ws_bytes, mat_ws(nullptr, T, D, g.nb, true, &w));
     ng_status st = ensure(c, ws, ws_bytes, mat_ws(nullptr, T, D, g.nb, inverse, &w));
     if (st) return st;
+    *kept = inverse;
     mat_ws(*ws, T, D, g.nb, inverse, &w);
     dep_launch(k_v2_mat_fill<D>, nblocks((int64_t)(T + 1) * g.nb, 128), 128, 0, s)(g, F, Q, w.g, w.K);
     if ((st = check_launch(c, "k_v2_mat_fill"))) return st;
-    return mat_solve<D>(c, g, G, w, inverse, s, refine_steps, ref_tol, refined_ok, nullptr);
+    return mat_solve<D>(c, g, G, w, inverse, mat_spread(c, form_nb(c, g), true), s, refine_steps, ref_tol, refined_ok, nullptr);
 }
 
 // one warp per vie2 bulk item: forced, or for batches with fewer items than 128 per SM
@@ -890,11 +931,12 @@ bool vie2_warp(const ng_ctx* c, const Grid& g, int n, bool digits) {
 }
 
 ng_status vie2_mat_d(ng_ctx* c, const Grid& g, const HermV& G, const HermV& F, const HermV& Q, cudaStream_t s,
-                     void** ws, size_t* ws_bytes, int refine_steps = 0, double ref_tol = 0.0, bool* ok = nullptr) {
+                     void** ws, size_t* ws_bytes, bool* kept, bool again, int refine_steps = 0, double ref_tol = 0.0,
+                     bool* ok = nullptr) {
     switch (g.nf) {
-    case 1: return launch_vie2_mat<1>(c, g, G, F, Q, s, ws, ws_bytes, refine_steps, ref_tol, ok);
-    case 2: return launch_vie2_mat<2>(c, g, G, F, Q, s, ws, ws_bytes, refine_steps, ref_tol, ok);
-    case 4: return launch_vie2_mat<4>(c, g, G, F, Q, s, ws, ws_bytes, refine_steps, ref_tol, ok);
+    case 1: return launch_vie2_mat<1>(c, g, G, F, Q, s, ws, ws_bytes, kept, again, refine_steps, ref_tol, ok);
+    case 2: return launch_vie2_mat<2>(c, g, G, F, Q, s, ws, ws_bytes, kept, again, refine_steps, ref_tol, ok);
+    case 4: return launch_vie2_mat<4>(c, g, G, F, Q, s, ws, ws_bytes, kept, again, refine_steps, ref_tol, ok);
     default: return fail(c, NG_EUNSUPPORTED, "the vie2 solver supports nf = 1, 2, 4");
     }
 }
@@ -1226,12 +1268,12 @@ ng_status do_timestep(ng_ctx* c, const Grid& g, int n, const HermV& G, const Her
     return g.nf == 1 ? launch_timestep<1>(c, g, n, G, S, eps, s) : launch_timestep<2>(c, g, n, G, S, eps, s);
 }
 ng_status do_mat(ng_ctx* c, const Grid& g, const HermV& G, const HermV& S, const FuncV& eps, cudaStream_t s,
-                 void* ws = nullptr) {
+                 void* ws = nullptr, bool again = false) {   // again: refinement of this solve follows
     switch (g.nf) {
-        case 1: return launch_mat<1>(c, g, G, S, eps, s, 0, 0.0, nullptr, ws);
-        case 2: return launch_mat<2>(c, g, G, S, eps, s, 0, 0.0, nullptr, ws);
-        case 4: return launch_mat<4>(c, g, G, S, eps, s, 0, 0.0, nullptr, ws);
-        default: return launch_mat<8>(c, g, G, S, eps, s, 0, 0.0, nullptr, ws);
+        case 1: return launch_mat<1>(c, g, G, S, eps, s, 0, 0.0, nullptr, ws, nullptr, again);
+        case 2: return launch_mat<2>(c, g, G, S, eps, s, 0, 0.0, nullptr, ws, nullptr, again);
+        case 4: return launch_mat<4>(c, g, G, S, eps, s, 0, 0.0, nullptr, ws, nullptr, again);
+        default: return launch_mat<8>(c, g, G, S, eps, s, 0, 0.0, nullptr, ws, nullptr, again);
     }
 }
 // workspace bytes of one Matsubara solve and of one start-up (nb problems of grid g)
@@ -1488,7 +1530,7 @@ ng_status ng_vie2_mat(ng_ctx* c, const ng_grid* grid, ng_herm G, ng_herm F, ng_h
     ng_status st;
     if ((st = vie2_args(c, grid, G, F, F, Q, false, &g, &Gv, &Fv, &Fccv, &Qv))) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    return vie2_mat_d(c, g, Gv, Fv, Qv, s, &c->ws_mat, &c->ws_mat_bytes);
+    return vie2_mat_d(c, g, Gv, Fv, Qv, s, &c->ws_mat, &c->ws_mat_bytes, &c->mat_kept, false);
 }
 
 ng_status ng_vie2_start(ng_ctx* c, const ng_grid* grid, ng_herm G, ng_herm F, ng_herm Fcc, ng_herm Q, void* stream) {
@@ -1846,10 +1888,11 @@ static ng_status run_2b_impl(ng_ctx* c, const ng_grid* grid, ng_herm G, ng_herm 
             bool refined = false;
             const double nel = (double)(T + 1) * dd * gw->gb.nb;
             if (gw_mats_calls >= 2 &&
-                (r = vie2_mat_d(c, gw->gb, gw->X, gw->K, gw->P, s, &c->ws_gwmat, &c->ws_gwmat_bytes, 30, 1e-13 * nel,
+                (r = vie2_mat_d(c, gw->gb, gw->X, gw->K, gw->P, s, &c->ws_gwmat, &c->ws_gwmat_bytes, &c->gwmat_kept, true, 30, 1e-13 * nel,
                                 &refined)))
                 return r;
-            if (!refined && (r = vie2_mat_d(c, gw->gb, gw->X, gw->K, gw->P, s, &c->ws_gwmat, &c->ws_gwmat_bytes)))
+            if (!refined && (r = vie2_mat_d(c, gw->gb, gw->X, gw->K, gw->P, s, &c->ws_gwmat, &c->ws_gwmat_bytes, &c->gwmat_kept,
+                                            gw_mats_calls >= 1)))
                 return r;
             ++gw_mats_calls;
         } else if (from == 0) {
@@ -1932,7 +1975,7 @@ static ng_status run_2b_impl(ng_ctx* c, const ng_grid* grid, ng_herm G, ng_herm 
             // current iterate with the kept LU factors, refactor only if that stalls
             bool refined = false;
             if (mats_it >= 2 && (st = do_mat_refine(c, g, Gv, Sv, mf, s, 30, 1e-13 * nel_mat, &refined, &read_sum))) return st;
-            if (!refined && (st = do_mat(c, g, Gv, Sv, mf, s))) return st;
+            if (!refined && (st = do_mat(c, g, Gv, Sv, mf, s, nullptr, mats_it >= 1))) return st;
             CUDA_TRY(c, cudaMemsetAsync(c->d_scalar, 0, sizeof(double), s));
             if ((st = do_distance(c, g, -1, Gv, Pv, c->d_scalar, s))) return st;
             if ((st = read_distance(&err))) return st;

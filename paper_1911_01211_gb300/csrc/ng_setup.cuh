@@ -302,7 +302,8 @@ __global__ void k_mat_assemble(Grid g, const cplx* ws_g, const cplx* ws_K, cplx*
 
 // ----------------------------------------------------------------------------------------
 // Dense solves of the Matsubara systems.  Batches: LU, one block per problem (k_lu_solve,
-// k_lu_resolve).  A few problems: the inverse by Gauss-Jordan elimination over the whole GPU.
+// k_lu_resolve).  A few problems: the inverse by Gauss-Jordan elimination over the whole GPU, or for larger
+// systems LU with the updates over the whole GPU (k_lu_col, k_lu_rank1, k_lu_backsub).
 // ----------------------------------------------------------------------------------------
 #define NG_LU_THREADS 512
 
@@ -474,6 +475,64 @@ __global__ void __launch_bounds__(NG_LU_THREADS) k_lu_solve(int N, int nrhs, cpl
         }
         __syncthreads();
     }
+    lu_substitute<false>(A, ld, N, A + N, ld, nrhs, xs);
+}
+
+// The same factorisation for a few larger systems: per column the pivot search, row interchange and multipliers in one
+// block per problem (blockIdx.x), then the rank-1 update of the trailing rows and columns over the GPU (problem
+// blockIdx.y), at the end the back substitution.  It needs a third of the arithmetic of the inverse.
+__global__ void __launch_bounds__(NG_LU_THREADS) k_lu_col(int N, int nrhs, cplx* ws_A, int* piv, int c, int* status) {
+    dep_wait();
+    const int ld = N + nrhs, t = threadIdx.x, nt = blockDim.x;
+    cplx* A = ws_A + (int64_t)blockIdx.x * N * ld;
+    __shared__ long long rv[NG_LU_THREADS / 32];
+    __shared__ int ri[NG_LU_THREADS / 32];
+    long long best = -1;
+    int p = c;
+    for (int r = c + t; r < N; r += nt) {
+        const long long v = pivot_key(A[(int64_t)r * ld + c]);
+        if (v > best) { best = v; p = r; }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const long long bo = __shfl_xor_sync(0xffffffffu, best, o);
+        const int po = __shfl_xor_sync(0xffffffffu, p, o);
+        if (bo > best || (bo == best && po < p)) { best = bo; p = po; }
+    }
+    if ((t & 31) == 0) { rv[t >> 5] = best; ri[t >> 5] = p; }
+    __syncthreads();
+    best = rv[0];
+    p = ri[0];
+    for (int q = 1; q < nt / 32; ++q)
+        if (rv[q] > best || (rv[q] == best && ri[q] < p)) { best = rv[q]; p = ri[q]; }
+    if (t == 0) {
+        if (best <= 0) atomicOr(status, NGF_SINGULAR);
+        piv[(int64_t)blockIdx.x * N + c] = p;
+    }
+    if (p != c)
+        for (int j = t; j < ld; j += nt) {
+            const cplx x = A[(int64_t)p * ld + j];
+            A[(int64_t)p * ld + j] = A[(int64_t)c * ld + j];
+            A[(int64_t)c * ld + j] = x;
+        }
+    __syncthreads();
+    const cplx inv = cinv(A[(int64_t)c * ld + c]);
+    for (int r = c + 1 + t; r < N; r += nt) A[(int64_t)r * ld + c] = cmul(A[(int64_t)r * ld + c], inv);
+}
+__global__ void k_lu_rank1(int N, int nrhs, cplx* ws_A, int c) {
+    dep_wait();
+    const int ld = N + nrhs, w = ld - c - 1;
+    cplx* A = ws_A + (int64_t)blockIdx.y * N * ld;
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= (int64_t)(N - c - 1) * w) return;
+    const int r = c + 1 + (int)(q / w), j = c + 1 + (int)(q % w);
+    A[(int64_t)r * ld + j] = cfma(cneg(A[(int64_t)r * ld + c]), A[(int64_t)c * ld + j], A[(int64_t)r * ld + j]);
+}
+__global__ void __launch_bounds__(NG_LU_THREADS) k_lu_backsub(int N, int nrhs, cplx* ws_A) {
+    dep_wait();
+    const int ld = N + nrhs;
+    cplx* A = ws_A + (int64_t)blockIdx.x * N * ld;
+    __shared__ cplx xs[NG_LU_TRI * 8];
     lu_substitute<false>(A, ld, N, A + N, ld, nrhs, xs);
 }
 
