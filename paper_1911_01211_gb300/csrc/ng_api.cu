@@ -86,8 +86,8 @@ struct ng_ctx {
     size_t ws_minv_bytes = 0;
     void* ws_uni = nullptr;          // problem table of the element-wise step (nf = 4, 8)
     size_t ws_uni_bytes = 0;
-    int uni_key_nb = -1;
-    const void *uni_key_G = nullptr, *uni_key_S = nullptr, *uni_key_eps = nullptr;
+    std::vector<char> uni_table;     // its first entry, as last copied to the device (empty: none)
+    int uni_nb = 0;
     void* ws_usrc = nullptr;         // element-wise step: chunk partials of the (A) sources
     size_t ws_usrc_bytes = 0;
     void* ws_adj = nullptr;          // adjoint: iterate store, work vectors, start-slice buffers
@@ -1211,23 +1211,28 @@ ng_status utimestep_uniform(ng_ctx* c, const Grid& g, int n, const HermV& G, con
     if (st) return st;
     UProb* d_probs = (UProb*)c->ws_uni;
     cplx* d_minv = (cplx*)((char*)c->ws_uni + off_minv);
-    if (c->uni_key_nb != g.nb || c->uni_key_G != G.ret.p || c->uni_key_S != S.ret.p || c->uni_key_eps != eps.p) {
-        std::vector<UProb> h(g.nb);
+    // the table holds the whole grid and every pointer: an entry that differs in any of them is copied anew (buffers are
+    // used again with another step or chemical potential, and another grid's buffers may begin at the same address)
+    UProb first;
+    memset((void*)&first, 0, sizeof(first));
+    first.g = g;
+    first.g.nb = 1;
+    first.G = G;
+    first.S = S;
+    first.eps.p = eps.p;
+    first.eps.ldk = eps.ldk;
+    first.minv = d_minv;
+    if (c->uni_nb != g.nb || c->uni_table.size() != sizeof(first) || memcmp(c->uni_table.data(), &first, sizeof(first)) != 0) {
+        std::vector<UProb> h(g.nb, first);
         for (int kb = 0; kb < g.nb; ++kb) {
-            h[kb].g = g;
-            h[kb].g.nb = 1;
-            h[kb].G = G;
-            h[kb].S = S;
-            h[kb].eps = eps;
             h[kb].kb = kb;
             h[kb].minv = d_minv + 64 * (size_t)kb;
         }
+        c->uni_table.clear();
         CUDA_TRY(c, cudaMemcpyAsync(d_probs, h.data(), sizeof(UProb) * h.size(), cudaMemcpyHostToDevice, s));
         CUDA_TRY(c, cudaStreamSynchronize(s));
-        c->uni_key_nb = g.nb;
-        c->uni_key_G = G.ret.p;
-        c->uni_key_S = S.ret.p;
-        c->uni_key_eps = eps.p;
+        c->uni_nb = g.nb;
+        c->uni_table.assign((const char*)&first, (const char*)&first + sizeof(first));
     }
     std::vector<UHost> info(g.nb, UHost{g.nf, g.nt, g.ntau, g.k, g.nb == 1 && form_nb(c, g) == 1});
     std::vector<int> active(g.nb);
