@@ -288,7 +288,7 @@ ng_status launch_minv(ng_ctx* c, const Grid& g, int n, const HermV& S, const Fun
 // FFT pre-pass of the left-mixing source of step n (*tvq = nullptr when the direct sums are
 // used: NG_TVSRC_DIRECT, or nf / ntau outside what the transforms support); tvfft_room: its buffer and twiddles
 // prof: record the pre-pass as its own profile entry (not inside a GW evaluation, which is
-// timed as a whole)
+// timed as a whole); ends: q_tv_sums in place of q_tv_fft
 bool tvfft_used(const ng_ctx* c, const Grid& g) { return c->tvsrc != NG_TVSRC_DIRECT && tvfft_supported(g.nf, g.ntau); }
 ng_status tvfft_room(ng_ctx* c, const Grid& g, const HermV& S, cudaStream_t s) {
     ng_status st;
@@ -301,14 +301,14 @@ ng_status tvfft_room(ng_ctx* c, const Grid& g, const HermV& S, cudaStream_t s) {
     return ensure(c, &c->ws_tvq, &c->ws_tvq_bytes, tvfft_out_bytes(g, S.tv.ldk));
 }
 ng_status prep_tvfft(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV& S, cudaStream_t s,
-                     const cplx** tvq, bool prof = true) {
+                     const cplx** tvq, bool prof = true, bool ends = false) {
     *tvq = nullptr;
     if (!tvfft_used(c, g)) return NG_OK;
     ng_status st = tvfft_room(c, g, S, s);
     if (st) return st;
     long e = prof ? prof_pair(c, 2) : -1;
     if (e >= 0) cudaEventRecord(c->ev_pool[e], s);
-    if (tvfft_launch(g, c->W, n, S.tv, G.mat, (const cplx*)c->ws_tw, (cplx*)c->ws_tvq, s) != cudaSuccess) {
+    if (tvfft_launch(g, c->W, n, S.tv, G.mat, (const cplx*)c->ws_tw, (cplx*)c->ws_tvq, ends, s) != cudaSuccess) {
         cudaGetLastError();
         return fail(c, NG_ECUDA, "launch of k_tvsrc_fft failed");
     }
@@ -666,7 +666,7 @@ ng_status launch_timestep32(ng_ctx* c, const Grid& g, int n, const HermV& G, con
     const int64_t it_ret = (int64_t)g.nb * (n - k);
     const int b_les = (int)nblocks(it_les, thr), b_tv = (int)nblocks(it_tv, thr), b_ret = (int)nblocks(it_ret, thr);
     const cplx* tvq = nullptr;
-    if ((st = prep_tvfft(c, g, n, G, S, s, &tvq))) return st;
+    if ((st = prep_tvfft(c, g, n, G, S, s, &tvq, true, true))) return st;
     long e0 = prof_pair(c, 0);
     if (e0 >= 0) cudaEventRecord(c->ev_pool[e0], s);
     if ((st = launch_minv<D>(c, g, n, S, eps, s))) return st;

@@ -149,6 +149,17 @@ __device__ Mat<D> q_tv_fft(const NgWeights& W, const Grid& g, const HermV& G, co
     return mscal<D>(g.htau, mmuli<D>(mscal<D>(-1.0, F)));
 }
 
+// The same, -i h_tau F(m), where the pre-pass has added the ends
+template <int D>
+__device__ __forceinline__ Mat<D> q_tv_sums(const Grid& g, int m, int kb, const cplx* Q) {
+    Mat<D> F;
+#pragma unroll
+    for (int a = 0; a < D; ++a)
+#pragma unroll
+        for (int b = 0; b < D; ++b) F.v[a][b] = Q[((int64_t)m * (D * D) + a * D + b) * g.nb + kb];
+    return mscal<D>(g.htau, mmuli<D>(mscal<D>(-1.0, F)));
+}
+
 // Partial sums of the (A)-source of the lesser column, -i (C^<_2 + C^<_3)[Sigma,1,G](m,n)
 // (Eqs. cles2, cles3), over the terms j = j0, j0+js, ...  (j0 = 0, js = 1 for the full sum).
 template <int D>

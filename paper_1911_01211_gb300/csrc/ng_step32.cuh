@@ -182,7 +182,7 @@ __device__ __forceinline__ void tv_item32(const NgWeights& W, const Grid& g, con
     });
     Mat<D> bdf = mzero<D>();
     for (int l = 1; l <= W.k; ++l) bdf = madd<D>(bdf, mscal<D>(W.a[l], gtv<D>(G, g, n - l, m, kb)));
-    Mat<D> rhs = tvq ? q_tv_fft<D>(W, g, G, S, n, m, kb, tvq) : q_tv32<D>(W, g, G32, S32, n, m, kb);
+    Mat<D> rhs = tvq ? q_tv_sums<D>(g, m, kb, tvq) : q_tv32<D>(W, g, G32, S32, n, m, kb);
     rhs = msub<D>(rhs, mscal<D>(1.0 / g.h, bdf));
     rhs = msub<D>(rhs, mscal<D>(g.h, mmuli<D>(kval<D>(acc))));
     Mat<D> y = mmul<D>(Minv, rhs);
@@ -399,7 +399,7 @@ __device__ __forceinline__ void tv_item32p(const NgWeights& W, const Grid& g, co
     for (int i = 0; i < 2; ++i) {
         Mat<1> bdf = mzero<1>();
         for (int l = 1; l <= W.k; ++l) bdf = madd<1>(bdf, mscal<1>(W.a[l], gtv<1>(G, g, n - l, m, kb + i)));
-        Mat<1> rhs = tvq ? q_tv_fft<1>(W, g, G, S, n, m, kb + i, tvq) : q_tv32<1>(W, g, G32, S32, n, m, kb + i);
+        Mat<1> rhs = tvq ? q_tv_sums<1>(g, m, kb + i, tvq) : q_tv32<1>(W, g, G32, S32, n, m, kb + i);
         rhs = msub<1>(rhs, mscal<1>(1.0 / g.h, bdf));
         rhs = msub<1>(rhs, mscal<1>(g.h, mmuli<1>(kpval(acc, i))));
         Mat<1> y = mmul<1>(ld_minv<1>(minv_ws, kb + i), rhs);

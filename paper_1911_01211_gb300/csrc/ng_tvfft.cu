@@ -11,7 +11,10 @@
 // frequency, one inverse transform.  In the 2k+2 columns next to either end the quadrature differs
 // from F by O(k) terms (short rows, boundary formulas), which the time-step kernels add (q_tv_fft in
 // ng_step.cuh).  (With unit weights here every column needed 4(k+1) correction terms: 144 FP64
-// instructions of the closing of each left-mixing item.)
+// instructions of the closing of each left-mixing item.)  For the F32C kernels the warps here add them (`ends`), a column
+// each in turn: with them k_step_bulk32p lost the schedule of its main loops (128 problems, n = 100, ntau = 900: 0.46 ms, 0.31
+// without, whole steps 634 / 464 us; 12 problems 551 / 452).  Not for the others: the lanes of a warp per column are not
+// as well used as those of a thread per item, and steps of 512 problems, n = 40, ntau = 100 took 175 instead of 149 us.
 //
 // One block per problem; the transforms are radix-2 decimation in time in shared memory, bit-reversed
 // in, natural out; the spectra are multiplied and put back into bit-reversed order in one pass.  They
@@ -25,6 +28,10 @@
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kMaxThreads = 768;
+// With the ends a warp for each of the 24 columns while every block has an SM to itself (152; 48 registers let an SM hold
+// one block of 768 threads or two of 512), else as many blocks as fit
+inline int fft_threads(int nb, bool ends) { return !ends || nb > 304 ? kThreads : nb <= 152 ? kMaxThreads : 512; }
 
 __global__ void k_twiddle(cplx* tw, int L) {
     dep_wait();
@@ -88,10 +95,10 @@ __global__ void __launch_bounds__(1024) k_tvsrc_s(Grid g, NgWeights W, int n, Co
 }
 
 // Q[(m nf^2 + a nf + b) nb + kb] = F_ab(m), m = 0..ntau, for problem kb = blockIdx.x; FSg: the spectra of a
-// shared S, or NULL
+// shared S, or NULL; ends: with the corrections of the columns next to the ends
 template <int D>
-__global__ void __launch_bounds__(kThreads) k_tvsrc_fft(Grid g, NgWeights W, int n, Comp Stv, Comp Gmat, const cplx* tw, int L,
-                                                        const cplx* FSg, cplx* Q) {
+__global__ void __launch_bounds__(kMaxThreads) k_tvsrc_fft(Grid g, NgWeights W, int n, Comp Stv, Comp Gmat, const cplx* tw, int L,
+                                                        const cplx* FSg, bool ends, cplx* Q) {
     dep_wait();
     extern __shared__ cplx sm[];
     constexpr int DD = D * D;
@@ -145,14 +152,67 @@ __global__ void __launch_bounds__(kThreads) k_tvsrc_fft(Grid g, NgWeights W, int
     __syncthreads();
     for (int e = 0; e < DD; ++e) fft_dit<true>(FK + e * L, tw, L);
     const double inv = 1.0 / (double)L;
+    const int k = g.k, edge = 2 * k + 2, lane = threadIdx.x & 31;
     for (int e = 0; e < DD; ++e)
         for (int m = threadIdx.x; m <= T; m += blockDim.x)
-            Q[((int64_t)m * DD + e) * g.nb + kb] = cscal(inv, FK[e * L + m]);
+            if (!ends || min(m, T - m) >= edge) Q[((int64_t)m * DD + e) * g.nb + kb] = cscal(inv, FK[e * L + m]);
+    const int ncol = ends ? min(T + 1, 2 * edge) : 0;
+    for (int c = threadIdx.x >> 5; c < ncol; c += blockDim.x >> 5) {
+        const int m = c < edge ? c : T - (ncol - 1 - c), L3 = T - m;
+        auto om = [&](int l) { return l <= k ? W.omega[l] : 1.0; };
+        auto ws = [&](int j) { return om(min(j, T - j)); };   // F's weight of S(j)
+        cplx x[D][D];
+#pragma unroll
+        for (int a = 0; a < D; ++a)
+#pragma unroll
+            for (int b = 0; b < D; ++b) x[a][b] = cz();
+        auto add = [&](double w, int js, int jg) {   // w S(js) G^M(jg)
+#pragma unroll
+            for (int a = 0; a < D; ++a)
+#pragma unroll
+                for (int q = 0; q < D; ++q) {
+                    const cplx v = cscal(w, el(Stv, rowS + js, a * D + q, kb));
+#pragma unroll
+                    for (int b = 0; b < D; ++b) x[a][b] = cfma(v, el(Gmat, jg, q * D + b, kb), x[a][b]);
+                }
+        };
+        // C2: sum_l w_{m,l} S(m-l) xi G^M(T-l)
+        auto t2 = [&](int l, double w) { add(xi * (w - om(l) * ws(m - l)), m - l, T - l); };
+        if (m <= k) {
+            for (int i = lane; i < (k + 1) * (k + 1); i += 32) add(xi * W.R[m][i / (k + 1)][i % (k + 1)], i % (k + 1), T - i / (k + 1));
+            for (int l = lane; l <= m; l += 32) t2(l, 0.0);
+        } else if (m <= 2 * k + 1) {
+            for (int l = lane; l <= m; l += 32) t2(l, W.greg[m][l]);
+        } else {
+            for (int l = lane; l <= m - T + k; l += 32) t2(l, gw(W, m, l));   // the weights of the end j = T
+        }
+        // C3: sum_l w_{T-m,l} S(m+l) G^M(l)
+        auto t3 = [&](int l, double w) { add(w - om(l) * ws(m + l), m + l, l); };
+        if (L3 <= k) {
+            for (int i = lane; i < (k + 1) * (k + 1); i += 32) add(W.R[L3][i / (k + 1)][i % (k + 1)], T - i % (k + 1), i / (k + 1));
+            for (int l = lane; l <= L3; l += 32) t3(l, 0.0);
+        } else if (L3 <= 2 * k + 1) {
+            for (int l = lane; l <= L3; l += 32) t3(l, W.greg[L3][l]);
+        } else {
+            for (int l = lane; l <= k - m; l += 32) t3(l, gw(W, L3, l));      // the weights of the end j = 0
+        }
+#pragma unroll
+        for (int a = 0; a < D; ++a)
+#pragma unroll
+            for (int b = 0; b < D; ++b) {
+                cplx y = x[a][b];
+                for (int o = 16; o > 0; o >>= 1) {
+                    y.x += __shfl_xor_sync(0xffffffffu, y.x, o);
+                    y.y += __shfl_xor_sync(0xffffffffu, y.y, o);
+                }
+                if (lane == 0) Q[((int64_t)m * DD + a * D + b) * g.nb + kb] = cadd(cscal(inv, FK[(a * D + b) * L + m]), y);
+            }
+    }
 }
 
 template <int D>
 cudaError_t launch_d(const Grid& g, const NgWeights& W, int n, const Comp& Stv, const Comp& Gmat, const cplx* tw, cplx* Q,
-                     cudaStream_t s) {
+                     bool ends, cudaStream_t s) {
     const int L = tvfft_length(g.ntau);
     const size_t one = sizeof(cplx) * (size_t)D * D * L;
     const bool shared = tvfft_shared(g, Stv.ldk);
@@ -166,7 +226,7 @@ cudaError_t launch_d(const Grid& g, const NgWeights& W, int n, const Comp& Stv, 
     }
     const size_t sm = shared ? one : 2 * one;
     if ((e = smem_limit(k_tvsrc_fft<D>))) return e;
-    dep_launch(k_tvsrc_fft<D>, g.nb, kThreads, sm, s)(g, W, n, Stv, Gmat, tw, L, FS, Q);
+    dep_launch(k_tvsrc_fft<D>, g.nb, fft_threads(g.nb, ends), sm, s)(g, W, n, Stv, Gmat, tw, L, FS, ends, Q);
     return cudaGetLastError();
 }
 
@@ -196,6 +256,6 @@ cudaError_t tvfft_twiddles(cplx* tw, int L, cudaStream_t s) {
 }
 
 cudaError_t tvfft_launch(const Grid& g, const NgWeights& W, int n, const Comp& Stv, const Comp& Gmat, const cplx* tw, cplx* Q,
-                         cudaStream_t s) {
-    return g.nf == 1 ? launch_d<1>(g, W, n, Stv, Gmat, tw, Q, s) : launch_d<2>(g, W, n, Stv, Gmat, tw, Q, s);
+                         bool ends, cudaStream_t s) {
+    return g.nf == 1 ? launch_d<1>(g, W, n, Stv, Gmat, tw, Q, ends, s) : launch_d<2>(g, W, n, Stv, Gmat, tw, Q, ends, s);
 }

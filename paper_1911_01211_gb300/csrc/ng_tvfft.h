@@ -17,6 +17,7 @@ cudaError_t tvfft_twiddles(cplx* tw, int L, cudaStream_t s);
 // of Q with those spectra behind it
 bool tvfft_shared(const Grid& g, int ldk);
 size_t tvfft_out_bytes(const Grid& g, int ldk);
-// Q[(m nf^2 + a nf + b) nb + kb] = the correlation F_ab(m) of step n, every problem; W: weights of order g.k
+// Q[(m nf^2 + a nf + b) nb + kb] = the correlation F_ab(m) of step n, every problem; W: weights of order g.k;
+// ends: with the corrections of the columns next to the ends of the axis
 cudaError_t tvfft_launch(const Grid& g, const NgWeights& W, int n, const Comp& Stv, const Comp& Gmat, const cplx* tw, cplx* Q,
-                         cudaStream_t s);
+                         bool ends, cudaStream_t s);
