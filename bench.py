@@ -396,7 +396,7 @@ def run_ours(a):
     e2e_window = nk * K / max_over_ranks(r["window_s"])
     prof, clk = r["prof"], r["clk"]
     # per step: extrapolation, then per corrector pass k-reduce (or partial + combine), Hartree,
-    # 2B, M_n^-1 (+ bulk, boundary); a lower bound: the bulk of a step is three launches with the digit
+    # 2B, M_n^-1 (+ bulk, boundary); a lower bound: the bulk of a step is four launches with the digit
     # products, the boundary two
     launches = int(prof["bulk_launches"] + prof["boundary_launches"] + prof["tvfft_launches"]) + \
         K * (1 + 3 * (4 + (1 if dist else 0)))
@@ -503,7 +503,7 @@ def run_ours(a):
                            "scope": "the timed window's steps only, same call, host clock"}},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak if peak else None, "traffic": traffic, "traffic_note": traffic_note,
-                     "kernel": "k_hist_mma (with k_minv_step, k_hist_vec and k_hist_close in its time)",
+                     "kernel": "k_hist_mma (with k_minv_step, k_hist_vec, k_hist_small and k_hist_close in its time)",
                      "peak_source": "measured copy bandwidth; achieved: the FP64 history of slices < n read once per "
                                     "corrector pass",
                      "fp64_equivalent_tflops": fp64_equiv,
@@ -699,7 +699,7 @@ def run_gw(a):
                                    f"pulse)", "timed": f"steps {n_w + 1}..{n_to} (setup and {W} warm-up steps untimed)"},
             "roofline": {"bound": "hbm", "achieved": bulk_gbs, "peak": peak, "unit": "GB/s",
                          "frac": bulk_gbs / peak if bulk_gbs and peak else None, "traffic": None,
-                         "kernel": "k_hist_mma (with k_minv_step, k_hist_vec and k_hist_close in its time)",
+                         "kernel": "k_hist_mma (with k_minv_step, k_hist_vec, k_hist_small and k_hist_close in its time)",
                          "share_of_timed": prof["bulk_ms"] / ms},
             "gw_chain_share_of_timed": prof["gw_ms"] / ms, "gw_chain_ms_per_eval": prof["gw_ms"] / max(prof["gw_evals"], 1),
             "setup": {"s": t_setup, "iterations": its},

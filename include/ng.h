@@ -99,7 +99,7 @@ typedef struct {
  * boundary steps, the start-up and the Matsubara solve stay FP64.  NG_DF64: the same sums in
  * double-float arithmetic (each value an FP32 pair, 48 significand bits; products with their
  * cross terms, TwoSum accumulation), FP64-class accuracy on the FP32 pipes; nf = 1 steps large enough
- * for the exact digit products of NG_FP64 take these. */
+ * for the digit products of NG_FP64 take these. */
 typedef enum { NG_FP64 = 0, NG_F32C = 1, NG_DF64 = 2 } ng_precision;
 
 /* Evaluation of the left-mixing Matsubara source -i (C^tv_2 + C^tv_3)[Sigma, 1, G^M](n, tau_m) of
@@ -124,7 +124,8 @@ typedef enum { NG_TVSRC_AUTO = 0, NG_TVSRC_DIRECT = 1 } ng_tv_source;
  * has fewer than 128 bulk items per SM, resp. fewer than 2 boundary rows per SM, and for nf = 1 from 16
  * problems on 4 or 8 lanes per item and a boundary with a lane per problem.  Where a step is large enough (nf = 1,
  * at least 8 problems), and for nf = 4, 8 and the uneven batch inside the history, NG_BULK_AUTO forms the history
- * sums on the tensor cores as exact products of 8-bit digits, rounded once per block of the history.  In every
+ * sums on the tensor cores as products of 8-bit digits on the scale of a block of the history, and in FP64 those
+ * that are small on it (where the device has no room for their workspace, as with NG_BULK_THREAD).  In every
  * mode the boundary's dense solves and serial steps run on the warps of one block per problem.  The forms
  * differ by rounding only.  nf = 4, 8 otherwise run the element-wise form. */
 typedef enum { NG_BULK_AUTO = 0, NG_BULK_THREAD = 1, NG_BULK_WARP = 2 } ng_bulk_split;

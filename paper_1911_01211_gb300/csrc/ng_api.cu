@@ -323,7 +323,8 @@ ng_status prep_tvfft(ng_ctx* c, const Grid& g, int n, const HermV& G, const Herm
 // units fill the GPU.  Whole steps, lanes / digit products in us: 16 problems, ntau = 250, n = 300 (5.3e6)
 // 106 / 179, n = 800 (27e6) 308 / 201; 64 problems, ntau = 100, n = 200 (7.7e6) 130 / 168, n = 300 (15e6) 196 / 189;
 // 128 problems, ntau = 400, n = 64 (7.6e6) 185 / 165; 256 problems, ntau = 250, n = 16 (2.2e6) 138 / 118, ntau = 30,
-// n = 64 (3.1e6) 85 / 97 (with plain launches: the programmatic ones take 5 to 10 us off both sides).
+// n = 64 (3.1e6) 85 / 97 (with plain launches: the programmatic ones take 5 to 10 us off both sides, k_hist_small adds as much to
+// the digits).
 bool hist_form(const ng_ctx* c, const Grid& g, int n) {
     return g.nf == 1 && form_nb(c, g) >= NGH_KG && c->bulk_split == NG_BULK_AUTO && n >= 2 * g.k + 2;
 }
@@ -629,8 +630,8 @@ template <int D>
 ng_status launch_timestepdf(ng_ctx* c, const Grid& g, int n, const HermV& G, const HermV& S, const FuncV& eps,
                             cudaStream_t s) {
     ng_status st;
-    // the digit products are exact and read half the bytes of the double-float sums (16 B per element for
-    // two multiply-adds): a step of 256 problems, n = 900, ntau = 400: 2.07 -> 1.59 ms
+    // the digit products read half the bytes of the double-float sums (16 B per element for
+    // two multiply-adds): a step of 256 problems, n = 900, ntau = 400: 2.07 -> 1.72 ms
     if (hist_applies(c, g, n) && hist_ready(c, g, n, S, S, s)) return launch_timestep<D>(c, g, n, G, S, eps, s);
     if ((st = update_shadow_df(c, c->dfG, g, G, n, false, s))) return st;
     if ((st = update_shadow_df(c, c->dfS, g, S, n, true, s))) return st;
@@ -1167,7 +1168,8 @@ ng_status ustep(ng_ctx* c, const UProb* d_probs, const std::vector<UHost>& info,
         // Digit products (ng_histu.cu) wherever the formulas of a step inside the history hold: their three launches
         // are the faster ones from the first steps on.  Whole steps in us, k_ubulk / digit products: problems of 1, 2,
         // 4, 8 orbitals, n = 40, ntau = 50: 613 / 555, n = 200, ntau = 100: 1402 / 738; one of 2 orbitals, n = 100,
-        // ntau = 100: 225 / 190; four of 8, n = 500, ntau = 300: 14.7 / 3.5 ms (before the tasks came from a counter, which takes a tenth off).  Interleaved problems keep k_ubulk.
+        // ntau = 100: 225 / 190; four of 8, n = 500, ntau = 300: 14.7 / 3.5 ms.  Nearest for 100 problems of one orbital, ntau = 100,
+        // which fill the GPU either way: n = 12 332 / 329, n = 250 677 / 673, n = 600 1533 / 1559.  Interleaved problems keep k_ubulk.
         bool digits = c->bulk_split == NG_BULK_AUTO;
         for (size_t i = c0; i < c1; ++i) {
             const UHost& u = info[active[i]];

@@ -37,7 +37,7 @@
 // the A operand with the columns contracted (row sums), and transposes them by movmatrix for the
 // column sums.
 //
-// Measured (512 problems, n = 1600, ntau = 800, 31.5 GB of history): about 8.5 ms, 3.7 TB/s, of a step of 9.1,
+// Measured (512 problems, n = 1600, ntau = 800, 31.5 GB of history): about 8.5 ms, 3.7 TB/s, of a step of 9.4,
 // against 28 ms of k_step_bulk, which is bound by the FP64 pipe, of a step of 28.7.  What bounds it is the issue
 // of instructions: per tile and warp about 600, and 48 tensor instructions that take 8 issue slots each (mma.sync
 // runs at 1024 multiply-adds per clock and SM on this part), with two warps on a scheduler to hide their latency.
