@@ -17,6 +17,7 @@ pytestmark = pytest.mark.gpu
     (250, 4, 24, 200, 0),   # digit products from n = 18 for all 250, later or not at all for 58 or 64; 38 chunks against 48
     (33, 2, 20, 30, 0),     # lanes per item against a warp per item; a rank of one k-point
     (97, 3, 18, 100, 1),    # FP32 copies: two problems a thread for 32 but not for 97
+    (129, 5, 80, 300, 0),   # digit products from n = 75 on, on a rank of one k-point too
 ])
 def test_ranks_equal_one_gpu(nk, nranks, nt, ntau, precision):
     import paper_1911_01211_gb300 as ng
